@@ -127,13 +127,17 @@ class _Draw:
         return torch.clamp(torch.round(w / s), -127, 127).to(torch.int8).contiguous(), s.reshape(-1).contiguous()
 
 
-def _linear(d, rows, K, N, G, in_type):
+def _linear_inputs(d, rows, K, N):
     x, cal, xs = d.activations(rows, K)
     Wq, ws = d.weights(d.normal(K, N) * 0.02, 1)
     bias = d.normal(N) * 0.02
-    perm, shift, _ = calib.static_preparation_device(cal, xs, Wq, G)
     y = torch.clamp(torch.round(cal / xs), -128, 127) @ Wq.float() * (xs * ws) + bias
-    ys = float(np.float32(float(y.abs().max()) / 127.0))
+    return x, cal, xs, Wq, ws, bias, float(np.float32(float(y.abs().max()) / 127.0))
+
+
+def _linear(d, rows, K, N, G, in_type):
+    x, cal, xs, Wq, ws, bias, ys = _linear_inputs(d, rows, K, N)
+    perm, shift, _ = calib.static_preparation_device(cal, xs, Wq, G)
     return {"layer": fx.Layer(Wq, ws, bias, perm, shift, G), "X": x.to(in_type), "xs": xs, "ys": ys, "rows": rows}
 
 
@@ -269,6 +273,82 @@ def run(state):
         return perm, shift, info
     dist = state["fit"].distances(state["pop"])
     return dist, state["fit"].Y[-1]
+
+
+# ---------------------------------------------------------------------------------------------- the same in 64 bits
+def _bits(lo, hi):
+    """Lowest bit position that keeps four bits of every integer in [lo, hi] (lo <= 0 <= hi)."""
+    m = torch.maximum(hi, -lo - 1)
+    return sum((m >= 8 << b).long() for b in range(4))
+
+
+def _quantized(x, xs):
+    scale = torch.full((), xs, dtype=torch.float32, device=x.device)      # a tensor: a scalar divisor becomes a multiplication
+    return torch.clamp(torch.round(x.float() / scale), -128, 127).double()
+
+
+def _positions(q, Wmax, G):
+    """Order of the channel groups (ascending activation range x weight range) and their positions, from quantized rows."""
+    lo, hi = q.amin(0).clamp(max=0), q.amax(0).clamp(min=0)
+    score = (torch.maximum(hi, -lo) * Wmax).reshape(-1, G).amax(1)
+    return torch.sort(score, stable=True).indices, _bits(lo, hi).reshape(-1, G).amax(1)
+
+
+def _lowered(v, s):
+    """Integers v clipped to what four bits hold at position s, with the bits below it cleared."""
+    return torch.floor(torch.minimum(torch.maximum(v, -(8 << s).double()), ((8 << s) - 1).double()) / (1 << s).double()) * (1 << s).double()
+
+
+def _operands(x, cal, xs, W, G, ratio, dynamic=False):
+    """8-bit activations [rows, K] and weights [taps, K, N] with the selected groups at 4 bits; the positions in slab order."""
+    q = _quantized(x, xs)
+    n_g = W.shape[1] // G
+    order, pos = _positions(_quantized(cal, xs), W.abs().amax((0, 2)), G)
+    if dynamic:
+        pos = _bits(q.amin(0).clamp(max=0), q.amax(0).clamp(min=0)).reshape(-1, G).amax(1)
+    low = torch.zeros(n_g, dtype=torch.bool, device=q.device)
+    low[order[:math.ceil(ratio * n_g - 1e-4)]] = True
+    ch = low.repeat_interleave(G)
+    Wg = W.reshape(W.shape[0], n_g, G, -1)
+    sw = _bits(Wg.amin((0, 2)).clamp(max=0), Wg.amax((0, 2)).clamp(min=0))
+    q = torch.where(ch, _lowered(q, pos.repeat_interleave(G)), q)
+    return q, torch.where(ch[None, :, None], _lowered(W, sw.repeat_interleave(G, 0)[None]), W), pos[order].to(torch.uint8)
+
+
+def _finished(acc, case, xs, ws, bias, ys):
+    if case["out"] == "i32":
+        return acc
+    y = acc.mul_(xs * ws.double()).add_(bias.double())
+    return torch.clamp(torch.round(y / ys), -128, 127) if case["out"] == "i8" else y
+
+
+def exact(case, seed):
+    """Sums and scaling in 64 bits (Eq. 1's division is fp32 by definition); the other kinds return integers throughout."""
+    d = _Draw(seed)
+    G, kind = case["G"], case["kind"]
+    if kind in ("linear", "linears"):
+        D, out = case.get("D"), []
+        shapes = [(case["K"], case["N"])] if kind == "linear" else [(D, 3 * D), (D, D), (D, 4 * D), (4 * D, D)] * case["blocks"]
+        inputs = [_linear_inputs(d, case["rows"], K, N) for K, N in shapes]
+        for ratio in ([case["ratio"]] if kind == "linear" else [float(r) for r in case["ratios"].split(",")]):
+            for x, cal, xs, Wq, ws, bias, ys in inputs:
+                q, W, pos = _operands(x.to(IN_TYPES[case["in"]]), cal, xs, Wq.double()[None], G, ratio, case.get("dynamic", False))
+                out.append(_finished(q @ W[0], case, xs, ws, bias, ys))
+        if kind == "linears":
+            return out if sum(y.numel() for y in out) < 2.5e9 else None
+        return (out[0], pos) if case["dynamic"] else out[0]
+    if kind == "conv":
+        R, stride, H, W_ = case["R"], case["stride"], case["H"], case["W"]
+        x, cal, xs = d.activations(case["images"] * H * W_, case["C"], half=True)
+        Wq, ws, bias = _conv_weights(d, case["C"], case["N"], R)
+        taps = Wq.double().permute(1, 2, 3, 0).reshape(R * R, case["C"], case["N"])
+        q, W, _ = _operands(x.to(IN_TYPES[case["in"]]), cal, xs, taps, G, case["ratio"])
+        p = R // 2
+        q = torch.nn.functional.pad(q.reshape(case["images"], H, W_, case["C"]), (0, 0, p, p, p, p))
+        P, Q = (H + 2 * p - R) // stride + 1, (W_ + 2 * p - R) // stride + 1
+        acc = sum(q[:, t // R:t // R + (P - 1) * stride + 1:stride, t % R:t % R + (Q - 1) * stride + 1:stride] @ W[t] for t in range(R * R))
+        return _finished(acc, case, xs, ws, bias, _conv_scale(cal, xs, Wq, ws, bias))
+    return None
 
 
 # ---------------------------------------------------------------------------------------------- work and tolerance
