@@ -174,49 +174,217 @@ int make_map_2d(CUtensorMap *map, const void *base, uint64_t row_bytes, uint64_t
 int choose_bk(const Layer *L) { return L->C >= 128 ? 128 : 64; }
 
 // ---------------------------------------------------------------------------------
-// Weight preparation.  One thread per (slab group j, output channel n): finds the
-// extraction position of the group's G weights (x all taps), then writes the three
-// slab-order weight forms.  Runs once per layer.
-__global__ void prep_weights_kernel(const int8_t *__restrict__ Wq, int is_conv, int C, int N, int G,
-                                    int T, const int32_t *__restrict__ perm, int8_t *__restrict__ w8,
-                                    int8_t *__restrict__ w8m, uint8_t *__restrict__ w4, int w4_pitch,
-                                    uint8_t *__restrict__ sw)
+// Weight preparation (Sec. 5, Sec. 4.1): the slab-order weight forms of a handle for a group order, and the
+// tables that go with the order.  A selection search lays a layer out once per chromosome, so this runs between
+// forward passes and not only once per layer.
+//
+// Bound by bytes: Wq is read once (K N), w8 and w8m (K N each), w4 (K N / 2) and sw (K N / G) are written, mostly
+// in L2.  The original weights of a linear layer are [K][N] and the slab rows [N][K], so a byte transpose lies in
+// between: done in registers (4 x 4 bytes by byte permutes) and through a shared-memory tile whose rows leave as
+// whole 128-byte segments.  One thread per (group, output channel) with byte loads and byte stores, each store 32
+// rows apart from its neighbour lane's, took 59.5 us for 768 x 3072 (2.4 MB in, 6.2 MB out).
+
+// The group order and the activation positions travel in the launch's parameters (at most 4 KB of them) up to
+// this many groups, i.e. 16,384 channels at the smallest group size; beyond it they are uploaded beforehand.
+constexpr int kInlineGroups = 1024;
+struct InlineOrder {
+    uint16_t perm[kInlineGroups];
+    uint8_t sx[kInlineGroups];   // slab order
+};
+struct PrepArgs {
+    const int8_t *Wq;
+    int aligned;          // Wq allows 4-byte (linear) or 16-byte (convolution) loads
+    int C, N, G, T;
+    int inline_order;     // the order is in InlineOrder and the tables are still to be written, else perm is on the device
+    int32_t *perm, *inv_perm, *chunk_ent, *chunk_ent_slab;
+    uint8_t *sx;
+    int8_t *w8, *w8m;
+    uint8_t *w4;
+    int w4_pitch;
+    uint8_t *sw;
+};
+
+// bytes with their sign folded away (v >= 0 ? v : ~v): the OR of a range's folded values has the bit length of the
+// range's used magnitude bits
+__device__ __forceinline__ uint32_t fold_signs(uint32_t w)
 {
-    const int n_g = C / G;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)n_g * N) return;
-    const int j = (int)(idx / N), n = (int)(idx % N);
-    const int g = perm[j];
-    const long long Kw = (long long)T * C;
-    int lo = 0, hi = 0;
-    for (int t = 0; t < T; ++t)
-        for (int i = 0; i < G; ++i) {
-            const long long src = is_conv ? ((long long)n * T + t) * C + g * G + i
-                                          : (long long)(g * G + i) * N + n;
-            const int v = Wq[src];
-            lo = min(lo, v);
-            hi = max(hi, v);
+    uint32_t sign;
+    asm("prmt.b32 %0, %1, 0, 0xba98;" : "=r"(sign) : "r"(w));   // 0xff where the byte is negative
+    return w ^ sign;
+}
+// extraction position of a group whose folded values OR to o: sign + 3 bits are kept
+__device__ __forceinline__ int position_of(uint32_t o)
+{
+    const int used = 32 - __clz(o);
+    return used > 3 ? used - 3 : 0;
+}
+// 16 weights of one slab row at position s: w8 as they are, w8m with the bits below s cleared, w4 the nibbles
+__device__ __forceinline__ void write_forms(const PrepArgs &a, long long row8, long long row4, int col, const uint4 &v, int s)
+{
+    const uint32_t mask = ((0xffu << s) & 0xffu) * 0x01010101u;
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t h[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t n = (w[k] >> s) & 0x0f0f0f0fu;   // one nibble per byte
+        h[k] = n | (n >> 4);                             // bytes 0 and 2 hold two nibbles each
+    }
+    *reinterpret_cast<uint4 *>(a.w8 + row8 + col) = v;
+    *reinterpret_cast<uint4 *>(a.w8m + row8 + col) = make_uint4(w[0] & mask, w[1] & mask, w[2] & mask, w[3] & mask);
+    *reinterpret_cast<uint2 *>(a.w4 + row4 + (col >> 1)) = make_uint2(__byte_perm(h[0], h[1], 0x6420), __byte_perm(h[2], h[3], 0x6420));
+}
+// the tables of an inline order, by one block
+__device__ __forceinline__ void write_tables(const PrepArgs &a, const InlineOrder &o)
+{
+    const int n_g = a.C / a.G, cpg = a.G / 16;
+    for (int j = threadIdx.x; j < n_g; j += blockDim.x) {
+        const int g = o.perm[j];
+        const int sx = o.sx[j];
+        a.perm[j] = g;
+        a.inv_perm[g] = j;
+        a.sx[j] = (uint8_t)sx;
+        // chunk table: original chunk c lies in original group c * 16 / G, which is slab group j with perm[j] = that group
+        for (int i = 0; i < cpg; ++i) {
+            const int ent = (j * cpg + i) | (sx << 24);
+            a.chunk_ent[g * cpg + i] = ent;
+            a.chunk_ent_slab[j * cpg + i] = ent;
         }
-    // magnitude bits in use: bit length of hi and of ~lo; keep sign + 3 bits
-    int used = 0;
-    if (hi > 0) used = max(used, 32 - __clz(hi));
-    if (lo < 0) used = max(used, 32 - __clz(~lo));
-    const int s = used > 3 ? used - 3 : 0;
-    sw[(long long)j * N + n] = (uint8_t)s;
-    for (int t = 0; t < T; ++t)
-        for (int i = 0; i < G; i += 2) {
-            const long long src0 = is_conv ? ((long long)n * T + t) * C + g * G + i
-                                           : (long long)(g * G + i) * N + n;
-            const long long src1 = is_conv ? src0 + 1 : src0 + N;
-            const int v0 = Wq[src0], v1 = Wq[src1];
-            const long long dst = (long long)n * Kw + (long long)t * C + j * G + i;
-            w8[dst] = (int8_t)v0;
-            w8[dst + 1] = (int8_t)v1;
-            const int a = v0 >> s, b = v1 >> s;  // arithmetic shift: floor
-            w8m[dst] = (int8_t)(a << s);
-            w8m[dst + 1] = (int8_t)(b << s);
-            w4[(long long)n * w4_pitch + (((long long)t * C + j * G + i) >> 1)] = (uint8_t)((a & 15) | ((b & 15) << 4));
+    }
+}
+
+// Linear weights [K][N].  A block transposes 128 slab channels x 64 output channels: thread (chunk, quad) loads 16
+// channels of 4 output channels, so that 16 lanes cover 64 contiguous bytes of a row.  64 and not 128 output channels: 288 blocks
+// instead of 144 for 768 x 3072, and 18 for 384 x 384.
+constexpr int kPrepN = 64, kPrepChunks = 8;
+__global__ void __launch_bounds__(kPrepN / 4 * kPrepChunks)
+prep_linear_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ InlineOrder order)
+{
+    __shared__ uint4 tile[kPrepN * kPrepChunks];      // [n][chunk ^ (n / 4)]: neither the writes nor the reads share a bank
+    __shared__ uint32_t fold_s[kPrepChunks][kPrepN / 4];
+    const int quad = threadIdx.x % (kPrepN / 4), chunk = threadIdx.x / (kPrepN / 4);
+    const int n0 = blockIdx.x * kPrepN + 4 * quad, c16 = blockIdx.y * kPrepChunks + chunk;
+    const int cpg = a.G / 16, j = c16 / cpg;
+    if (a.inline_order && blockIdx.x == 0 && blockIdx.y == 0) write_tables(a, order);
+    uint32_t r[16];
+    uint32_t o = 0;
+    const bool live = c16 < a.C / 16 && n0 < a.N;
+    if (live) {
+        const int g = a.inline_order ? (int)order.perm[j] : a.perm[j];
+        const int8_t *src = a.Wq + (long long)(g * a.G + (c16 % cpg) * 16) * a.N + n0;
+        if (a.aligned) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) r[i] = __ldg(reinterpret_cast<const uint32_t *>(src + (long long)i * a.N));
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const uint8_t *b = reinterpret_cast<const uint8_t *>(src + (long long)i * a.N);
+                r[i] = (uint32_t)b[0] | (uint32_t)b[1] << 8 | (uint32_t)b[2] << 16 | (uint32_t)b[3] << 24;
+            }
         }
+        uint32_t t[4][4];                               // [output channel][word of 4 channels]
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t *q = r + 4 * i;
+            const uint32_t lo01 = __byte_perm(q[0], q[1], 0x5140), lo23 = __byte_perm(q[2], q[3], 0x5140);
+            const uint32_t hi01 = __byte_perm(q[0], q[1], 0x7362), hi23 = __byte_perm(q[2], q[3], 0x7362);
+            t[0][i] = __byte_perm(lo01, lo23, 0x5410);
+            t[1][i] = __byte_perm(lo01, lo23, 0x7632);
+            t[2][i] = __byte_perm(hi01, hi23, 0x5410);
+            t[3][i] = __byte_perm(hi01, hi23, 0x7632);
+            o |= fold_signs(q[0]) | fold_signs(q[1]) | fold_signs(q[2]) | fold_signs(q[3]);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) tile[(4 * quad + e) * kPrepChunks + (chunk ^ (quad & 7))] = make_uint4(t[e][0], t[e][1], t[e][2], t[e][3]);
+    }
+    fold_s[chunk][quad] = o;
+    __syncthreads();
+    // the whole group's folded OR, one byte per output channel (a group's chunks never span two blocks: 128 % G == 0)
+    uint32_t go = 0;
+    for (int i = 0; i < cpg; ++i) go |= fold_s[chunk - chunk % cpg + i][quad];
+    __syncthreads();
+    uint32_t pos = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) pos |= (uint32_t)position_of((go >> (8 * e)) & 0xffu) << (8 * e);
+    fold_s[chunk][quad] = pos;
+    if (live && chunk % cpg == 0) *reinterpret_cast<uint32_t *>(a.sw + (long long)j * a.N + n0) = pos;
+    __syncthreads();
+    // eight lanes write 128 contiguous bytes of one slab row
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+        const int u = threadIdx.x + it * (kPrepN / 4 * kPrepChunks);
+        const int nl = u / kPrepChunks, ch = u % kPrepChunks;
+        const int n = blockIdx.x * kPrepN + nl, c = blockIdx.y * kPrepChunks + ch;
+        if (n < a.N && c < a.C / 16) {
+            const uint4 v = tile[nl * kPrepChunks + (ch ^ ((nl >> 2) & 7))];
+            const int s = (int)((fold_s[ch][nl >> 2] >> (8 * (nl & 3))) & 0xffu);
+            write_forms(a, (long long)n * a.C, (long long)n * a.w4_pitch, c * 16, v, s);
+        }
+    }
+}
+
+// Convolution weights [N][T][C]: the slab rows have the same orientation, so 16-byte chunks move whole.  A block owns
+// nb output channels and a window of groups; a position needs the group's chunks of every tap, so the chunks are
+// folded first and read again (from L1 or L2) when they are written.
+constexpr int kPrepGroups = 2048;   // groups per window: bounds the shared memory; one window up to 32,768 channels
+__global__ void __launch_bounds__(256) prep_conv_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ InlineOrder order, int nb)
+{
+    extern __shared__ uint32_t prep_s[];                // folded OR [nb][window], then the window's order
+    const int g0 = blockIdx.y * kPrepGroups, n_g = min(kPrepGroups, a.C / a.G - g0);
+    const int cpg = a.G / 16, n_c16 = n_g * cpg, units = a.T * n_c16;
+    const int n_first = blockIdx.x * nb, n_here = min(nb, a.N - n_first);
+    uint32_t *perm_s = prep_s + nb * n_g;
+    if (a.inline_order && blockIdx.x == 0) write_tables(a, order);   // an inline order is one window
+    for (int i = threadIdx.x; i < nb * n_g; i += blockDim.x) prep_s[i] = 0;
+    for (int i = threadIdx.x; i < n_g; i += blockDim.x) perm_s[i] = a.inline_order ? (uint32_t)order.perm[i] : (uint32_t)a.perm[g0 + i];
+    __syncthreads();
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int idx = threadIdx.x; idx < n_here * units; idx += blockDim.x) {
+            const int nl = idx / units, u = idx - nl * units, t = u / n_c16, c = u - t * n_c16, j = c / cpg;
+            const int8_t *src = a.Wq + ((long long)(n_first + nl) * a.T + t) * a.C + perm_s[j] * a.G + (c % cpg) * 16;
+            uint4 v;
+            if (a.aligned) v = __ldg(reinterpret_cast<const uint4 *>(src));
+            else {
+                uint32_t w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const uint8_t *b = reinterpret_cast<const uint8_t *>(src + 4 * k);
+                    w[k] = (uint32_t)b[0] | (uint32_t)b[1] << 8 | (uint32_t)b[2] << 16 | (uint32_t)b[3] << 24;
+                }
+                v = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            if (pass == 0) {
+                uint32_t o = fold_signs(v.x) | fold_signs(v.y) | fold_signs(v.z) | fold_signs(v.w);
+                o |= o >> 16;
+                o = (o | o >> 8) & 0xffu;
+                if (o) atomicOr(&prep_s[nl * n_g + j], o);
+            } else {
+                write_forms(a, (long long)(n_first + nl) * a.T * a.C, (long long)(n_first + nl) * a.w4_pitch, t * a.C + g0 * a.G + c * 16, v,
+                            position_of(prep_s[nl * n_g + j]));
+            }
+        }
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < n_here * n_g; i += blockDim.x) {
+        const int j = i / n_here, nl = i - j * n_here;
+        a.sw[(long long)(g0 + j) * a.N + n_first + nl] = (uint8_t)position_of(prep_s[nl * n_g + j]);
+    }
+}
+
+static cudaError_t launch_prep(const Layer *L, const PrepArgs &a, const InlineOrder &order, cudaStream_t stream)
+{
+    if (!L->is_conv) {
+        const dim3 grid((a.N + kPrepN - 1) / kPrepN, (a.C / 16 + kPrepChunks - 1) / kPrepChunks);
+        prep_linear_kernel<<<grid, kPrepN / 4 * kPrepChunks, 0, stream>>>(a, order);
+        return cudaGetLastError();
+    }
+    // as many output channels per block as give every thread a chunk, but blocks enough for the machine
+    const int sms = device_sm_count(L->device), window = L->n_g < kPrepGroups ? L->n_g : kPrepGroups;
+    int nb = 256 / (a.T * window * (a.G / 16));
+    if (nb > (a.N + sms - 1) / sms) nb = (a.N + sms - 1) / sms;
+    if (nb < 1) nb = 1;
+    const dim3 grid((a.N + nb - 1) / nb, (L->n_g + kPrepGroups - 1) / kPrepGroups);
+    prep_conv_kernel<<<grid, 256, sizeof(uint32_t) * (size_t)(nb + 1) * window, stream>>>(a, order, nb);
+    return cudaGetLastError();
 }
 
 static int validate_perm(const int32_t *perm, int n_g)
@@ -254,7 +422,6 @@ static void free_layer(Layer *L)
     cudaFree(L->tables); cudaFree(L->w_scale); cudaFree(L->bias); cudaFree(L->factor_mem);
     if (L->tables_host) cudaFreeHost(L->tables_host);
     if (L->tables_event) cudaEventDestroy(L->tables_event);
-    free(L->perm_host); free(L->sx_host);
     L->magic = 0;
     free(L);
 }
@@ -278,38 +445,47 @@ int encode_weight_maps(Layer *L)
     return FLEXIQ_OK;
 }
 
-// The layout post-processing of a handle for a group order (Sec. 5): uploads the order, the
-// activation positions in slab order and the chunk tables, and rebuilds the slab-order weights, their
-// positions and the 4-bit cache from the original-order weights.  Stream-ordered, allocates nothing
-// on the device, does not wait for the stream: the tables go up in one copy from a pinned mirror.
+// The layout post-processing of a handle for a group order (Sec. 5): the order, the activation positions in slab
+// order and the chunk tables, the slab-order weights, their positions and the 4-bit cache, all from the
+// original-order weights.  Stream-ordered, allocates nothing on the device, does not wait for the stream: one launch
+// that carries the order in its parameters, or beyond kInlineGroups groups an upload from a pinned mirror before it.
 static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const uint8_t *x_shift, cudaStream_t stream)
 {
-    const int n_g = L->n_g, C = L->C, G = L->G, N = L->N;
-    // the pinned mirror is free again once the previous upload has read it (normally long ago)
-    if (L->tables_in_flight) FLEXIQ_CUDA_TRY(cudaEventSynchronize(L->tables_event));
-    memcpy(L->perm_host, perm, sizeof(int32_t) * n_g);
-    for (int j = 0; j < n_g; ++j) L->sx_host[j] = x_shift ? x_shift[perm[j]] : 0;  // slab order
-    const int n_c = C / 16, cpg = G / 16;
-    int32_t *h_perm = static_cast<int32_t *>(L->tables_host), *h_inv = h_perm + n_g, *h_ent = h_inv + n_g, *h_ent_slab = h_ent + n_c;
-    uint8_t *h_sx = reinterpret_cast<uint8_t *>(h_ent_slab + n_c);
-    // chunk table: original chunk c lies in original group c*16/G, which is slab group j with perm[j] = that group
-    for (int j = 0; j < n_g; ++j) {
-        h_perm[j] = perm[j];
-        h_inv[perm[j]] = j;
-        h_sx[j] = L->sx_host[j];
-        for (int i = 0; i < cpg; ++i) {
-            h_ent[perm[j] * cpg + i] = (j * cpg + i) | ((int32_t)L->sx_host[j] << 24);
-            h_ent_slab[j * cpg + i] = (j * cpg + i) | ((int32_t)L->sx_host[j] << 24);
+    const int n_g = L->n_g, C = L->C, G = L->G;
+    InlineOrder order;
+    PrepArgs a{};
+    a.Wq = Wq;
+    a.aligned = (reinterpret_cast<uintptr_t>(Wq) & (L->is_conv ? 15u : 3u)) == 0;
+    a.C = C; a.N = L->N; a.G = G; a.T = L->R * L->S;
+    a.perm = L->perm; a.inv_perm = L->inv_perm; a.chunk_ent = L->chunk_ent; a.chunk_ent_slab = L->chunk_ent_slab; a.sx = L->sx;
+    a.w8 = L->w8; a.w8m = L->w8m; a.w4 = L->w4; a.w4_pitch = L->w4_pitch; a.sw = L->sw;
+    a.inline_order = n_g <= kInlineGroups;
+    if (a.inline_order) {
+        for (int j = 0; j < n_g; ++j) {
+            order.perm[j] = (uint16_t)perm[j];
+            order.sx[j] = x_shift ? x_shift[perm[j]] : 0;
         }
+    } else {
+        // the pinned mirror is free again once the previous upload has read it (normally long ago)
+        if (L->tables_in_flight) FLEXIQ_CUDA_TRY(cudaEventSynchronize(L->tables_event));
+        const int n_c = C / 16, cpg = G / 16;
+        int32_t *h_perm = static_cast<int32_t *>(L->tables_host), *h_inv = h_perm + n_g, *h_ent = h_inv + n_g, *h_ent_slab = h_ent + n_c;
+        uint8_t *h_sx = reinterpret_cast<uint8_t *>(h_ent_slab + n_c);
+        // chunk table: original chunk c lies in original group c*16/G, which is slab group j with perm[j] = that group
+        for (int j = 0; j < n_g; ++j) {
+            h_perm[j] = perm[j];
+            h_inv[perm[j]] = j;
+            h_sx[j] = x_shift ? x_shift[perm[j]] : 0;  // slab order
+            for (int i = 0; i < cpg; ++i) {
+                h_ent[perm[j] * cpg + i] = (j * cpg + i) | ((int32_t)h_sx[j] << 24);
+                h_ent_slab[j * cpg + i] = (j * cpg + i) | ((int32_t)h_sx[j] << 24);
+            }
+        }
+        FLEXIQ_CUDA_TRY(cudaMemcpyAsync(L->tables, L->tables_host, L->tables_bytes, cudaMemcpyHostToDevice, stream));
+        FLEXIQ_CUDA_TRY(cudaEventRecord(L->tables_event, stream));
+        L->tables_in_flight = 1;
     }
-    FLEXIQ_CUDA_TRY(cudaMemcpyAsync(L->tables, L->tables_host, L->tables_bytes, cudaMemcpyHostToDevice, stream));
-    FLEXIQ_CUDA_TRY(cudaEventRecord(L->tables_event, stream));
-    L->tables_in_flight = 1;
-    const long long total = (long long)n_g * N;
-    const int threads = 128;
-    prep_weights_kernel<<<(unsigned)((total + threads - 1) / threads), threads, 0, stream>>>(
-        Wq, L->is_conv, C, N, G, L->R * L->S, L->perm, L->w8, L->w8m, L->w4, L->w4_pitch, L->sw);
-    FLEXIQ_CUDA_TRY(cudaGetLastError());
+    FLEXIQ_CUDA_TRY(launch_prep(L, a, order, stream));
     L->st_K_lo = -1;   // the straddle block was cut from the previous order's weights
     L->st_cap_id = 0;
     L->slab_next = 0;  // slabs written for the previous order are no longer this layer's
@@ -340,8 +516,6 @@ static int create_common(flexiq_layer_t *out, int is_conv, int C, int N, int R, 
     L->R = R; L->S = S; L->stride = stride; L->pad = pad;
     L->Kw = R * S * C; L->w4_pitch = ((L->Kw / 2 + 15) / 16) * 16; L->K_lo = 0; L->lowbit_path = FLEXIQ_LOWBIT_MASKED_I8;
     cudaGetDevice(&L->device);
-    L->perm_host = (int32_t *)malloc(sizeof(int32_t) * n_g);
-    L->sx_host = (uint8_t *)malloc(n_g);
     const size_t wbytes = (size_t)N * L->Kw;
 #define TRY_OR_FREE(expr)                                                                        \
     do {                                                                                         \
@@ -362,8 +536,10 @@ static int create_common(flexiq_layer_t *out, int is_conv, int C, int N, int R, 
         const int n_c = C / 16;
         L->tables_bytes = sizeof(int32_t) * (2 * (size_t)n_g + 2 * (size_t)n_c) + (size_t)n_g;
         TRY_OR_FREE(cudaMalloc(&L->tables, L->tables_bytes));
-        TRY_OR_FREE(cudaMallocHost(&L->tables_host, L->tables_bytes));
-        TRY_OR_FREE(cudaEventCreateWithFlags(&L->tables_event, cudaEventDisableTiming));
+        if (n_g > kInlineGroups) {
+            TRY_OR_FREE(cudaMallocHost(&L->tables_host, L->tables_bytes));
+            TRY_OR_FREE(cudaEventCreateWithFlags(&L->tables_event, cudaEventDisableTiming));
+        }
         L->perm = static_cast<int32_t *>(L->tables);
         L->inv_perm = L->perm + n_g;
         L->chunk_ent = L->inv_perm + n_g;

@@ -1,0 +1,69 @@
+"""Layout post-processing of a handle: the slab-order weights, their 4-bit form and the positions of every
+(group, output channel) against the oracle and a plain gather, at the edges of the kernels' tiles (64 output
+channels x 128 input channels; whole convolution rows), for every group size, for weights at odd addresses and
+for more groups than a launch's parameters carry."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2510_02822_b200 import binding as fx
+from paper_2510_02822_b200 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def draw(seed, shape):
+    w = (inputs.uniform(seed, 0, int(np.prod(shape))) * 256).astype(np.int64) - 128
+    narrow = np.repeat((inputs.uniform(seed, 1, -(-w.size // 32)) * 6).astype(np.int64), 32)[:w.size]   # every position occurs
+    return (w >> narrow).astype(np.int8).reshape(shape)
+
+
+@pytest.mark.parametrize("shape, G, offset", [
+    ((16, 16), 16, 0), ((128, 64), 16, 0), ((144, 80), 16, 0), ((112, 48), 16, 1), ((192, 208), 64, 0), ((320, 64), 32, 2),
+    ((1025 * 16, 16), 16, 0),                                                  # linear [K, N]
+    ((16, 1, 1, 16), 16, 0), ((48, 3, 3, 80), 16, 0), ((64, 3, 3, 64), 64, 4), ((160, 1, 1, 544), 32, 0), ((16, 5, 3, 272), 16, 0),
+    ((32, 1, 1, 1025 * 16), 16, 0), ((16, 1, 1, 2049 * 16), 16, 0)])           # convolution [N, R, S, C]
+def test_layout_matches_oracle(shape, G, offset):
+    dev = torch.device("cuda:0")
+    conv = len(shape) == 4
+    W = draw(500 + G + shape[0], shape)
+    C, N = (shape[3], shape[0]) if conv else shape
+    T, n_g = W.size // (C * N), C // G
+    raw = torch.empty(W.size + 16, dtype=torch.int8, device=dev)
+    Wd = raw[offset:offset + W.size].view(shape)
+    Wd.copy_(torch.from_numpy(W))
+    ones = torch.ones(N, device=dev)
+    L = fx.Layer(Wd, ones, None, np.arange(n_g, dtype=np.int32), None, G, conv=(1, 0) if conv else None)
+    sx = (np.arange(n_g) % 5).astype(np.uint8)
+    for perm in (np.arange(n_g, dtype=np.int32)[::-1].copy(), np.argsort(inputs.uniform(7, 2, n_g), kind="stable").astype(np.int32)):
+        L.set_group_perm(Wd, perm, sx)
+        cols = (perm[:, None].astype(np.int64) * G + np.arange(G)).reshape(-1)
+        slab = (W[..., cols] if conv else W[cols].T).reshape(N, T, C)
+        sw = oracle.weight_positions_conv(W, G, perm) if conv else oracle.weight_positions_linear(W, G, perm)
+        s = np.repeat(sw.reshape(n_g, N).T.astype(np.int64), G, axis=1)[:, None, :]
+        nib = ((slab.astype(np.int64) >> s) & 15).astype(np.uint8).reshape(N, T * C)
+        sw_g, w8, w4 = np.empty((n_g, N), np.uint8), np.empty((N, T * C), np.int8), np.empty((N, T * C // 2), np.uint8)
+        fx.flexiq_layer_export(L.h, sw_g, w8, w4)
+        assert np.array_equal(sw_g, sw.reshape(n_g, N))
+        assert np.array_equal(w8, slab.reshape(N, T * C))
+        assert np.array_equal(w4, nib[:, 0::2] | (nib[:, 1::2] << 4))
+        # the masked weights, the order and the activation positions through the mixed kernel itself (one tap of input)
+        if not conv:
+            X = draw(900, (5, C))
+            for ratio in (1.0, 0.5):
+                L.set_lowbit_ratio(ratio)
+                x4, x8, _ = L.quantize_lower(torch.from_numpy(X).to(dev), 1.0)
+                acc = L.mixed_gemm(x4, x8, 5, 1.0, 1.0, fx.OUT_ACC_I32)
+                assert np.array_equal(acc.cpu().numpy(), oracle.mixed_gemm_acc(X, W, G, perm, sx[perm].copy(), sw, oracle.n_low(ratio, n_g)))
+        else:
+            R, S = shape[1], shape[2]
+            X = draw(901, (1, R, S, C))
+            for ratio in (1.0, 0.5):
+                L.set_lowbit_ratio(ratio)
+                x4, x8, _ = L.quantize_lower(torch.from_numpy(X).to(dev), 1.0)
+                acc = L.mixed_conv(x4, x8, 1, R, S, 1.0, 1.0, fx.OUT_ACC_I32)
+                ref = oracle.mixed_conv_acc(X, W, 1, 0, G, perm, sx[perm].copy(), sw, oracle.n_low(ratio, n_g))
+                assert np.array_equal(acc.cpu().numpy().reshape(-1), ref.reshape(-1))
+    fx.flexiq_check_status()
+    L.close()
