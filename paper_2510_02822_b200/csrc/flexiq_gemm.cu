@@ -1791,10 +1791,10 @@ extern "C" int flexiq_check_status(void *stream)
     unsigned int word = 0, zero = 0;
     FLEXIQ_CUDA_TRY(cudaStreamSynchronize(st));
     FLEXIQ_CUDA_TRY(cudaMemcpyFromSymbol(&word, g_status_word, sizeof(word)));
-    if (word != 0) {
-        FLEXIQ_CUDA_TRY(cudaMemcpyToSymbol(g_status_word, &zero, sizeof(zero)));
-        return set_error(FLEXIQ_ERR_TIMEOUT, "a bounded device-side wait expired (status word 0x%x)", word);
-    }
+    if (word != 0) FLEXIQ_CUDA_TRY(cudaMemcpyToSymbol(g_status_word, &zero, sizeof(zero)));
+    const unsigned int prologue_word = prologue_status();
+    if (word == 0) word = prologue_word;
+    if (word != 0) return set_error(FLEXIQ_ERR_TIMEOUT, "a bounded device-side wait expired (status word 0x%x)", word);
     return FLEXIQ_OK;
 }
 

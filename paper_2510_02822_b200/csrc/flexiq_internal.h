@@ -134,6 +134,9 @@ EncodeIm2colFn get_encode_im2col();
 int make_map_2d(CUtensorMap *map, const void *base, uint64_t row_bytes, uint64_t rows,
                 uint64_t pitch_bytes, uint32_t box_bytes, uint32_t box_rows, int swizzle_bytes);
 
+// status word of the prologue's bounded waits (0 = none expired), cleared when read
+unsigned prologue_status();
+
 int choose_bk(const Layer *L);
 int encode_weight_maps(Layer *L);
 

@@ -1,7 +1,7 @@
 // Activation prologue: quantize (Sec. 2.1, Eq. 1), bit-lower (Sec. 4.1, Fig. 3) and
 // gather the channel groups into slab order (Sec. 5), writing the low-bit slab and the
 // 8-bit slab that the mainloop consumes.  One pass over X (two in the dynamic
-// extraction-position mode), 128-bit loads and stores, one 16-channel chunk per thread.
+// extraction-position mode of the packed path), one 16-channel chunk per thread.
 #include "flexiq_internal.h"
 
 #include <cuda_bf16.h>
@@ -11,7 +11,7 @@
 #include "eq1_quantize.cuh"
 #include "straddle.cuh"
 
-#include <stdlib.h>
+#include <string.h>
 
 namespace flexiq {
 
@@ -64,12 +64,227 @@ __global__ void group_or_kernel(const void *__restrict__ X, long long M, int K, 
         if (or_s[i]) atomicOr(&or_words[i], or_s[i]);
 }
 
-// Phase 2 of the dynamic mode on the masked path: the low groups of the slab that phase 1 wrote are lowered in
-// place with the positions the OR words give -- clip to what four bits hold at the position, clear the bits below
-// it -- 16 bytes per thread; a group whose position is 0 is already what it should be and is not touched.  The
-// positions go to sx_out (slab order).  Blocks in front: the straddle block of the weights, as in the static kernel.
+// ---------------------------------------------------------------------------------
+// Masked path.
+//
+// Bound by HBM: every input byte is read once and one byte per value written.  A tile is a few whole rows, contiguous in
+// memory, which one bulk copy brings into a ring in shared memory; the gather into slab order is done from there.  Bulk
+// copies read at 6.7 TB/s where 128-bit loads by all threads, whatever their number and order, stay at 5.5 to 5.9 (206 MB,
+// read only; 38.7 MB: 7.5 us against 8.9 to 10), and the gather costs no sectors (a 16-byte int8 chunk is half of one).
+// A thread keeps its row within the tile and its slab chunk from tile to tile, so that a step is the 128-bit reads of its
+// chunk, the arithmetic and one 128-bit store; the stores of a warp are contiguous.  Measured, replayed from a graph on buffers
+// larger than L2, against one chunk per thread by plain loads: fp16 25216 x 4096 62.3 -> 51.8 us (6.0 TB/s; a plain
+// copy of the same bytes reaches 6.2), fp16 25216 x 1024 17.3 -> 15.6, fp32 12608 x 768 10.6 -> 9.4, int8 12608 x 3072 19.8 -> 14.8.
+constexpr int kRowWarps = 8;                     // consumer warps per block at most; one more issues the copies
+constexpr int kRowStages = 8;                    // ring stages at most
+constexpr int kRowRing = 49152;                  // bytes of ring a block aims at: four blocks per SM
+constexpr int kRowStageBytes = 65536;            // largest row the ring takes; wider rows go through the packed path's kernels
+constexpr int kRowSmem = 3 * kRowStageBytes + 32768;   // three stages of that and the tables of 65,536 channels (int8)
+constexpr uint32_t kCopyWaitLimit = 1u << 21;    // parked waits of at most a microsecond each: about two seconds
+
+__device__ unsigned int g_prologue_status = 0;
+
+// Bounded wait; false after the limit or when another warp already gave up.
+__device__ __forceinline__ bool wait_copy(uint32_t bar, uint32_t parity, volatile int *gave_up)
+{
+    if (ptx::mbar_try_wait_s(bar, parity)) return true;
+    for (uint32_t it = 0; it < kCopyWaitLimit; ++it) {
+        if (ptx::mbar_try_wait_hint_s(bar, parity, 1000u)) return true;
+        if (*gave_up) return false;
+    }
+    *gave_up = 1;
+    atomicMax(&g_prologue_status, 0x301u);
+    return false;
+}
+
+// Where slab chunk c comes from and how it is lowered: source chunk | shift << 28.  A low group keeps bits s..s+3 of
+// values clipped to what four bits hold at position s; an 8-bit group is the same at position 4 with nothing cleared,
+// which is told apart by shift 5: one instruction stream for both, since a warp spans the boundary in most rows.
+constexpr unsigned kShift8Bit = 5;
+__device__ __forceinline__ unsigned chunk_entry(int c, int G, int lo_c16, const int32_t *perm, const uint8_t *sx)
+{
+    const int cpg = G / 16, j = c / cpg;
+    const unsigned shift = c < lo_c16 ? (unsigned)__ldg(sx + j) : kShift8Bit;
+    return (unsigned)(__ldg(perm + j) * cpg + (c - j * cpg)) | (shift << 28);
+}
+
+struct RowsArgs {
+    const void *X;
+    int8_t *slab;
+    long long M, tiles;
+    int K, G, K_lo;
+    int rows;                  // rows per tile
+    int stages, stage_bytes;
+    float S;
+    QuotientPlan quot;
+    const int32_t *perm;
+    const uint8_t *sx;         // static positions, slab order
+    unsigned *or_words;        // dynamic: OR of the sign-folded values of every group
+    StraddleJob wp;
+};
+
+// DYN: phase 1 of the dynamic mode.  Every group is written at 8 bits and the OR of the sign-folded values of every
+// group is collected on the way, so that the input is read once.
+template <int DTYPE, bool DYN>
+__global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(const __grid_constant__ RowsArgs a)
+{
+    constexpr int kBytes = DTYPE == FLEXIQ_DTYPE_F32 ? 4 : (DTYPE == FLEXIQ_DTYPE_I8 ? 1 : 2);
+    constexpr int kPieces = kBytes;                  // 16-byte pieces per chunk: 4, 2 or 1
+    extern __shared__ __align__(128) uint8_t rows_smem[];
+    __shared__ uint64_t full_bar[kRowStages], empty_bar[kRowStages];
+    __shared__ int gave_up;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (blockDim.x >> 5) - 1;
+    const int n_c16 = a.K / 16, lo_c16 = DYN ? 0 : a.K_lo / 16, cpg = a.G / 16;
+    unsigned *table = reinterpret_cast<unsigned *>(rows_smem + a.stages * a.stage_bytes);
+    unsigned *or_s = table + n_c16;
+    ptx::pdl_launch_dependents();
+    if (blockIdx.x < a.wp.first_block) {
+        // Extra blocks in front of the quantizing ones (so that they run beside the first wave, not behind the
+        // last): the weight K block that max_4bit_ch falls into, for the GEMM that consumes these slabs -- the
+        // only weight data that depends on the ratio -- 16 bytes per thread.
+        ptx::pdl_wait();
+        const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (idx < (long long)a.wp.rows * (a.wp.BK >> 4)) straddle_write_unit(a.wp, idx);
+        return;
+    }
+    const long long first = blockIdx.x - a.wp.first_block, step = gridDim.x - a.wp.first_block;
+    const size_t row_bytes = (size_t)a.K * kBytes, tile_bytes = (size_t)a.rows * row_bytes;
+    auto copy = [&](long long tile, int stage) {
+        const uint32_t bytes = (uint32_t)(min((long long)a.rows, a.M - tile * a.rows) * (long long)row_bytes);
+        const uint32_t bar = ptx::smem_u32(&full_bar[stage]);
+        ptx::mbar_expect_tx_s(bar, bytes);
+        ptx::bulk_load(ptx::smem_u32(rows_smem) + (uint32_t)(stage * a.stage_bytes),
+                       reinterpret_cast<const char *>(a.X) + (size_t)tile * tile_bytes, bytes, bar);
+    };
+    long long next = first;                          // the copying thread's next tile
+    const bool copier = warp == warps && lane == 0;
+    if (copier) {
+        for (int i = 0; i < a.stages; ++i) {
+            ptx::mbar_init(&full_bar[i], 1);
+            ptx::mbar_init(&empty_bar[i], warps);
+        }
+        gave_up = 0;
+        ptx::fence_mbar_init();
+    }
+    ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
+    if (copier)
+        for (int i = 0; i < a.stages && next < a.tiles; ++i, next += step) copy(next, i);
+    for (int c = threadIdx.x; c < n_c16; c += blockDim.x) table[c] = chunk_entry(c, a.G, lo_c16, a.perm, a.sx);
+    if (DYN)
+        for (int j = threadIdx.x; j < a.K / a.G; j += blockDim.x) or_s[j] = 0;
+    __syncthreads();
+    if (warp == warps) {
+        if (lane == 0) {
+            // refill a stage when every warp has read it
+            int stage = 0;
+            uint32_t phase = 0;
+            for (; next < a.tiles; next += step) {
+                if (!wait_copy(ptx::smem_u32(&empty_bar[stage]), phase, &gave_up)) break;
+                copy(next, stage);
+                if (++stage == a.stages) { stage = 0; phase ^= 1; }
+            }
+        }
+    } else {
+        const int threads = 32 * warps, units = a.rows * n_c16;
+        const bool single = units <= threads;        // one chunk per thread and tile, the same in every tile
+        const int r0 = (int)threadIdx.x / n_c16, c0 = (int)threadIdx.x - r0 * n_c16;
+        unsigned src = 0, shift = kShift8Bit, mask = 0xffffffffu;
+        float lo = -128.f, hi = 127.f;
+        auto position = [&](int r, int c) {          // of the chunk at row r of a tile, slab chunk c
+            const unsigned ent = table[c];
+            src = (unsigned)r * (unsigned)row_bytes + (ent & 0x0fffffffu) * (16u * kBytes);
+            if (DYN) return;
+            shift = ent >> 28;
+            const float bound = (float)(8u << min(shift, 4u));
+            lo = -bound;
+            hi = bound - 1.f;
+            mask = shift == kShift8Bit ? 0xffffffffu : ((0xffu << shift) & 0xffu) * 0x01010101u;
+        };
+        if ((int)threadIdx.x < units) position(r0, c0);
+        int stage = 0;
+        uint32_t phase = 0;
+        for (long long tile = first; tile < a.tiles; tile += step) {
+            if (!__all_sync(0xffffffffu, wait_copy(ptx::smem_u32(&full_bar[stage]), phase, &gave_up))) break;
+            const uint32_t base = ptx::smem_u32(rows_smem) + (uint32_t)(stage * a.stage_bytes);
+            const int here = (int)min((long long)a.rows, a.M - tile * a.rows) * n_c16;
+            int r = r0, c = c0;
+            for (int u = threadIdx.x; u < here; u += threads) {
+                if (!single) position(r, c);
+                uint4 raw[kPieces];
+                // Neighbouring lanes start at different pieces of their chunks: with one order for all, the 16-byte reads
+                // of a quarter warp would share half (16-bit inputs) or a quarter (fp32) of the banks.
+                const unsigned turn = kPieces == 1 ? 0u : (unsigned)lane % kPieces;
+#pragma unroll
+                for (int p = 0; p < kPieces; ++p) raw[p] = ptx::ld_shared_128(base + src + ((p + turn) % kPieces) * 16);
+                unsigned w[4];
+                if constexpr (DTYPE == FLEXIQ_DTYPE_I8) {
+                    const unsigned in[4] = {raw[0].x, raw[0].y, raw[0].z, raw[0].w};
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) w[k] = DYN ? in[k] : clip_bytes(in[k], min(shift, 4u));
+                } else if (a.quot.form == kQuotGeneral) {
+                    quantize_raw<DTYPE>(raw, make_divider(a.S), lo, hi, w);
+                } else if constexpr (DTYPE == FLEXIQ_DTYPE_F32) {
+                    quantize_raw<DTYPE>(raw, TwoTerm{a.quot.r_hi, a.quot.r_lo}, lo, hi, w);
+                } else {
+                    quantize_raw_magic<DTYPE>(raw, a.quot.r_hi, lo, hi, w);
+                }
+                // back to channel order: piece p of the chunk is in place (p - turn) mod kPieces
+                if constexpr (kPieces == 4) {
+                    if (turn & 1) { const unsigned t = w[3]; w[3] = w[2]; w[2] = w[1]; w[1] = w[0]; w[0] = t; }
+                    if (turn & 2) { const unsigned t0 = w[0], t1 = w[1]; w[0] = w[2]; w[1] = w[3]; w[2] = t0; w[3] = t1; }
+                } else if constexpr (kPieces == 2) {
+                    if (turn) { const unsigned t0 = w[0], t1 = w[1]; w[0] = w[2]; w[1] = w[3]; w[2] = t0; w[3] = t1; }
+                }
+                if (DYN) {
+                    unsigned o = 0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {   // fold negatives per byte (q >= 0 ? q : ~q): xor with the byte's sign replicated
+                        unsigned sign;
+                        asm("prmt.b32 %0, %1, 0, 0xba98;" : "=r"(sign) : "r"(w[k]));
+                        o |= w[k] ^ sign;
+                    }
+                    o |= o >> 16;
+                    o = (o | (o >> 8)) & 0xffu;
+                    unsigned *seen = or_s + c / cpg;
+                    if (o & ~*reinterpret_cast<volatile unsigned *>(seen)) atomicOr(seen, o);   // rare after the first rows
+                }
+                *reinterpret_cast<uint4 *>(a.slab + (size_t)tile * (size_t)(units * 16) + (size_t)u * 16) =
+                    make_uint4(w[0] & mask, w[1] & mask, w[2] & mask, w[3] & mask);
+                if (!single) {
+                    c += threads;
+                    while (c >= n_c16) { c -= n_c16; ++r; }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&empty_bar[stage]);
+            if (++stage == a.stages) { stage = 0; phase ^= 1; }
+        }
+    }
+    __syncthreads();
+    if (gave_up) {
+        // the copies still in flight land before the block's shared memory is given back
+        if (copier)
+            for (int i = 0; i < a.stages; ++i)
+                for (uint32_t w = 0; w < (1u << 16) && !ptx::mbar_try_wait(&full_bar[i], 0) && !ptx::mbar_try_wait(&full_bar[i], 1); ++w) __nanosleep(64);
+        return;
+    }
+    if (DYN) {
+        // with many blocks most find nothing new in the end: a read saves the atomic
+        const bool look = gridDim.x > 128;
+        for (int j = threadIdx.x; j < a.K / a.G; j += blockDim.x) {
+            const unsigned o = or_s[j];
+            if (o & ~(look ? __ldcg(a.or_words + j) : 0u)) atomicOr(a.or_words + j, o);
+        }
+    }
+}
+
+// Phase 2 of the dynamic mode: the low groups of the slab that phase 1 wrote are lowered in place with the positions
+// the OR words give, 16 bytes per thread.  The positions cover every value of the call, so nothing saturates and
+// lowering is clearing the bits below the position; a group whose position is 0 is already what it should be and
+// is not touched.  The positions go to sx_out (slab order).  Blocks in front: the straddle block of the weights.
 __global__ void lower_inplace_kernel(int8_t *__restrict__ slab, long long M, int K, int G, int K_lo,
-                                     const unsigned *__restrict__ or_words, uint8_t *__restrict__ sx_out, StraddleJob wp)
+                                     const unsigned *__restrict__ or_words, uint8_t *__restrict__ sx_out, StraddleJob wp,
+                                     int step_m, int step_c)
 {
     ptx::pdl_launch_dependents();
     ptx::pdl_wait();  // phase 1 has written the slab and the OR words
@@ -78,119 +293,69 @@ __global__ void lower_inplace_kernel(int8_t *__restrict__ slab, long long M, int
         if (idx < (long long)wp.rows * (wp.BK >> 4)) straddle_write_unit(wp, idx);
         return;
     }
-    const unsigned qblock = blockIdx.x - wp.first_block, qblocks = gridDim.x - wp.first_block;
+    const unsigned qblock = blockIdx.x - wp.first_block;
     if (qblock == 0)
-        for (int j = threadIdx.x; j < K / G; j += blockDim.x) sx_out[j] = (uint8_t)position_from_or(or_words[j]);
+        for (int j = threadIdx.x; j < K / G; j += blockDim.x) sx_out[j] = (uint8_t)position_from_or(__ldcg(or_words + j));
     const int lo_c16 = K_lo / 16, c_per_g = G / 16;
-    const long long total = M * lo_c16;
-    for (long long idx = (long long)qblock * blockDim.x + threadIdx.x; idx < total; idx += (long long)qblocks * blockDim.x) {
-        const long long m = idx / lo_c16;
-        const int c16 = (int)(idx - m * lo_c16);
-        const int s = position_from_or(or_words[c16 / c_per_g]);
-        if (s == 0) continue;
-        uint4 *ptr = reinterpret_cast<uint4 *>(slab + (size_t)m * K + (size_t)c16 * 16);
-        const uint4 u = *ptr;
-        const unsigned in[4] = {u.x, u.y, u.z, u.w};
-        unsigned w[4];
-        const int hi = (8 << s) - 1, lo = -(8 << s);
-        const unsigned mask = ((0xffu << s) & 0xffu) * 0x01010101u;
+    if (lo_c16 == 0) return;
+    const long long idx = (long long)qblock * blockDim.x + threadIdx.x;
+    long long m = idx / lo_c16;
+    int c = (int)(idx - m * lo_c16);
+    while (m < M) {
+        // four units at a time: their loads are in flight together
+        uint4 *ptr[4];
+        uint4 v[4];
+        unsigned mask[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            int b[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) b[t] = max(lo, min(hi, (int)(signed char)((in[k] >> (8 * t)) & 0xff)));
-            w[k] = pack2_sat_s8(b[1], b[0], pack2_sat_s8(b[3], b[2], 0u)) & mask;
+        for (int i = 0; i < 4; ++i) {
+            ptr[i] = nullptr;
+            if (m < M) {
+                const int s = position_from_or(__ldcg(or_words + c / c_per_g));
+                mask[i] = ((0xffu << s) & 0xffu) * 0x01010101u;
+                if (s) {
+                    ptr[i] = reinterpret_cast<uint4 *>(slab + (size_t)m * K + (size_t)c * 16);
+                    v[i] = *ptr[i];
+                }
+            }
+            m += step_m;
+            c += step_c;
+            if (c >= lo_c16) { c -= lo_c16; ++m; }
         }
-        *ptr = make_uint4(w[0], w[1], w[2], w[3]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (ptr[i]) *ptr[i] = make_uint4(v[i].x & mask[i], v[i].y & mask[i], v[i].z & mask[i], v[i].w & mask[i]);
     }
 }
 
-// Quantize + lower + gather.  Thread <-> (row m, 16-channel slab chunk c16).
+// Packed path, and the masked path's rows that are too wide for the ring: quantize + lower + gather.  Thread <-> (row m,
+// 16-channel slab chunk c16).
 //   sx != nullptr : static positions (slab order);  else positions from or_words.
 // Lowering works on the packed int8 words: q is first clipped to the range the 4-bit value
 // at position s can hold, [-2^(s+3), 2^(s+3) - 1] (identical to clamping q >> s to [-8, 7],
-// the shift being monotone); then bits s..s+3 of every byte are the two's-complement nibble
-// (packed path), and clearing the s low bits of every byte is (q >> s) << s (masked path).
-// PACKED == 2 is phase 1 of the dynamic mode on the masked path: nothing is lowered yet (every group is written
-// at 8 bits, gathered into slab order) and the OR of the sign-folded values of every group is collected on the way
-// (or_acc; a thread keeps its chunk column from one grid stride to the next when the stride is a multiple of the
-// row's chunks, which the launch arranges, so it flushes its OR once), so that the input is read once.
-template <int DTYPE, int PACKED>
-__global__ void quantize_lower_kernel(const void *__restrict__ X, long long M, int K, int G, int K_lo, float S,
-                                      const int32_t *__restrict__ perm, const uint8_t *__restrict__ sx,
-                                      const unsigned *__restrict__ or_words, uint8_t *__restrict__ X4,
-                                      long long x4_pitch, int8_t *__restrict__ X8, long long x8_pitch, uint8_t *__restrict__ sx_out,
-                                      StraddleJob wp)
+// the shift being monotone); then bits s..s+3 of every byte are the two's-complement nibble (packed path), and
+// clearing the s low bits of every byte is (q >> s) << s (masked path: one slab, X8 lies behind the low groups of X4).
+template <int DTYPE, bool PACKED>
+__global__ void quantize_chunks_kernel(const void *__restrict__ X, long long M, int K, int G, int K_lo, float S,
+                                       const int32_t *__restrict__ perm, const uint8_t *__restrict__ sx,
+                                       const unsigned *__restrict__ or_words, uint8_t *__restrict__ X4,
+                                       long long x4_pitch, int8_t *__restrict__ X8, long long x8_pitch, uint8_t *__restrict__ sx_out)
 {
     const int n_c16 = K / 16, c_per_g = G / 16, lo_c16 = K_lo / 16;
     const long long total = M * n_c16;
     const Divider div = make_divider(S);
     ptx::pdl_launch_dependents();
     ptx::pdl_wait();  // the previous kernel may still read the slabs this one overwrites, or write X
-    if (blockIdx.x < wp.first_block) {
-        // Extra blocks in front of the quantizing ones (so that they run beside the first wave, not behind the
-        // last): the weight K block that max_4bit_ch falls into, for the GEMM that consumes these slabs -- the
-        // only weight data that depends on the ratio -- 16 bytes per thread.
-        const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-        if (idx < (long long)wp.rows * (wp.BK >> 4)) straddle_write_unit(wp, idx);
-        return;
-    }
-    const unsigned qblock = blockIdx.x - wp.first_block, qblocks = gridDim.x - wp.first_block;
-    if (PACKED == 2) {
-        extern __shared__ unsigned or_s[];
-        unsigned *or_acc = const_cast<unsigned *>(or_words);
-        const int n_g = K / G;
-        for (int i = threadIdx.x; i < n_g; i += blockDim.x) or_s[i] = 0;
-        __syncthreads();
-        unsigned o = 0;
-        int oj = -1;
-        for (long long idx = (long long)qblock * blockDim.x + threadIdx.x; idx < total; idx += (long long)qblocks * blockDim.x) {
-            const long long m = idx / n_c16;
-            const int c16 = (int)(idx - m * n_c16);
-            const int j = c16 / c_per_g;
-            if (j != oj) {   // another group (only when the stride is not a multiple of a row's chunks)
-                if (o) atomicOr(&or_s[oj], (o | (o >> 8) | (o >> 16) | (o >> 24)) & 0xffu);
-                o = 0;
-                oj = j;
-            }
-            const int src_c = perm[j] * G + (c16 % c_per_g) * 16;
-            unsigned w[4];
-            quantize16<DTYPE>(reinterpret_cast<const char *>(X) + ((size_t)m * K + src_c) * elem_bytes<DTYPE>(), div, -128.f, 127.f, w);
-            *reinterpret_cast<uint4 *>(X4 + m * x4_pitch + (size_t)c16 * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {   // fold negatives per byte (q >= 0 ? q : ~q): xor with the byte's sign replicated
-                const unsigned sign = (w[k] >> 7) & 0x01010101u;
-                o |= w[k] ^ (sign * 0xffu);
-            }
-        }
-        if (o) atomicOr(&or_s[oj], (o | (o >> 8) | (o >> 16) | (o >> 24)) & 0xffu);
-        __syncthreads();
-        for (int i = threadIdx.x; i < n_g; i += blockDim.x)
-            if (or_s[i]) atomicOr(&or_acc[i], or_s[i]);
-        return;
-    }
-    if (sx_out != nullptr && qblock == 0)
+    if (sx_out != nullptr && blockIdx.x == 0)
         for (int j = threadIdx.x; j < K / G; j += blockDim.x) sx_out[j] = (uint8_t)position_from_or(or_words[j]);
-    for (long long idx = (long long)qblock * blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)qblocks * blockDim.x) {
+    for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+         idx += (long long)gridDim.x * blockDim.x) {
         const long long m = idx / n_c16;
         const int c16 = (int)(idx - m * n_c16);
         const int j = c16 / c_per_g;
         const int src_c = perm[j] * G + (c16 % c_per_g) * 16;
         const void *src = reinterpret_cast<const char *>(X) + ((size_t)m * K + src_c) * elem_bytes<DTYPE>();
         unsigned w[4];
-        if (!PACKED) {
-            // Masked path: one instruction stream for both kinds of group (a warp spans the boundary in most rows).
-            // A low group keeps bits s..s+3 of values clipped to what four bits hold at position s; an 8-bit group
-            // is the same with the full range and nothing cleared.  The slab is [M][K]: X8 is X4 + K_lo.
-            const bool low = c16 < lo_c16;
-            const int s = low ? (sx ? (int)sx[j] : position_from_or(or_words[j])) : 4;
-            const float bound = (float)(8 << s);
-            quantize16<DTYPE>(src, div, -bound, bound - 1.f, w);
-            const unsigned mask = low ? ((0xffu << s) & 0xffu) * 0x01010101u : 0xffffffffu;
-            *reinterpret_cast<uint4 *>(X4 + m * x4_pitch + (size_t)c16 * 16) =
-                make_uint4(w[0] & mask, w[1] & mask, w[2] & mask, w[3] & mask);
-        } else if (c16 < lo_c16) {
+        if (c16 < lo_c16) {
             const int s = sx ? (int)sx[j] : position_from_or(or_words[j]);
             const float bound = (float)(8 << s);
             quantize16<DTYPE>(src, div, -bound, bound - 1.f, w);
@@ -204,8 +369,7 @@ __global__ void quantize_lower_kernel(const void *__restrict__ X, long long M, i
                 *reinterpret_cast<uint2 *>(X4 + m * x4_pitch + (size_t)c16 * 8) =
                     make_uint2(__byte_perm(h[0], h[1], 0x6420), __byte_perm(h[2], h[3], 0x6420));
             } else {
-                const unsigned keep = (0xffu << s) & 0xffu;
-                const unsigned mask = keep * 0x01010101u;
+                const unsigned mask = ((0xffu << s) & 0xffu) * 0x01010101u;
                 *reinterpret_cast<uint4 *>(X4 + m * x4_pitch + (size_t)c16 * 16) =
                     make_uint4(w[0] & mask, w[1] & mask, w[2] & mask, w[3] & mask);
             }
@@ -258,6 +422,69 @@ static cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned blocks, unsigne
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// plan_quotient (a few microseconds for 16-bit inputs), remembered by its two arguments for the scales in use
+static QuotientPlan quotient_plan(float S, int dtype)
+{
+    struct Known { float S; int dtype; QuotientPlan plan; };
+    static thread_local Known known[256] = {};
+    uint32_t bits;
+    memcpy(&bits, &S, sizeof(bits));
+    Known &k = known[((bits * 0x9E3779B1u) >> 24) ^ (unsigned)dtype];
+    if (k.S != S || k.dtype != dtype) k = Known{S, dtype, plan_quotient(S, dtype)};
+    return k.plan;
+}
+
+// The masked path's quantizing kernel, static (DYN = false) or phase 1 of the dynamic mode.
+template <int DTYPE, bool DYN>
+static int launch_rows(Layer *L, const void *X, long long M, float S, int8_t *slab, unsigned *or_words, const StraddleJob &job, cudaStream_t st)
+{
+    constexpr int kBytes = DTYPE == FLEXIQ_DTYPE_F32 ? 4 : (DTYPE == FLEXIQ_DTYPE_I8 ? 1 : 2);
+    const int n_c16 = L->C / 16, sms = device_sm_count(L->device);
+    RowsArgs a{};
+    a.X = X; a.slab = slab; a.M = M; a.K = L->C; a.G = L->G; a.K_lo = L->K_lo;
+    a.S = S;
+    a.quot = quotient_plan(S, DTYPE);
+    a.perm = L->perm; a.sx = L->sx; a.or_words = or_words;
+    a.wp = job;
+    // Rows per tile and consumer warps: as many chunks as the block has threads, with the fewest threads idle; a row of
+    // more than 256 chunks is a tile by itself.  Few rows: smaller tiles, so that they spread over the SMs (not in the
+    // dynamic mode, whose blocks meet at the OR words).
+    int warps = kRowWarps;
+    a.rows = 1;
+    if (n_c16 <= 32 * kRowWarps) {
+        double best = 0.0;
+        for (int w = kRowWarps; w >= 4; --w) {
+            const int r = 32 * w / n_c16;
+            const double used = (double)(r * n_c16) / (32 * w);
+            if (used > best + 1e-9) { best = used; warps = w; a.rows = r; }
+        }
+        if (!DYN && (M + a.rows - 1) / a.rows < sms) {
+            a.rows = (int)((M + sms - 1) / sms);
+            warps = (a.rows * n_c16 + 31) / 32;
+        }
+    }
+    a.tiles = (M + a.rows - 1) / a.rows;
+    a.stage_bytes = (a.rows * L->C * kBytes + 127) & ~127;
+    a.stages = kRowRing / a.stage_bytes;
+    if (a.stages > kRowStages) a.stages = kRowStages;
+    if (a.stages < 3) a.stages = 3;                   // wide rows: up to 192 KB, down to one block per SM
+    const size_t smem = (size_t)a.stages * a.stage_bytes + sizeof(unsigned) * (size_t)(n_c16 + (DYN ? L->n_g : 0));
+    long long per_sm = (long long)(220 * 1024 / (smem + 1280));
+    if (per_sm > 4) per_sm = 4;
+    if (per_sm < 1) per_sm = 1;
+    const long long blocks = a.tiles < sms * per_sm ? a.tiles : sms * per_sm;
+    const int threads = 32 * (warps + 1);
+    const unsigned extra = job.wst ? (unsigned)(((long long)job.rows * (job.BK >> 4) + threads - 1) / threads) : 0u;
+    a.wp.first_block = extra;   // the straddle blocks come first
+    static bool attr_set[64] = {};   // per instantiation
+    if (smem > 48 * 1024 && (L->device >= 64 || !attr_set[L->device])) {
+        FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(quantize_rows_kernel<DTYPE, DYN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem));
+        if (L->device < 64) attr_set[L->device] = true;
+    }
+    FLEXIQ_CUDA_TRY(launch_pdl(quantize_rows_kernel<DTYPE, DYN>, (unsigned)(blocks + extra), (unsigned)threads, smem, st, a));
+    return FLEXIQ_OK;
+}
+
 template <int DTYPE>
 static int launch_prologue(Layer *L, const void *X, long long M, float S, int dynamic, uint8_t *X4,
                            long long pitch, int8_t *X8, long long pitch8, uint8_t *sx_out, unsigned *scratch, cudaStream_t st)
@@ -267,66 +494,68 @@ static int launch_prologue(Layer *L, const void *X, long long M, float S, int dy
     const int sms = device_sm_count(L->device);
     const int threads = 256;
     const bool masked = L->lowbit_path == FLEXIQ_LOWBIT_MASKED_I8;
-    if (dynamic && masked) {
-        // the input is read once: phase 1 quantizes, gathers and collects the OR words, phase 2 lowers the low groups of
-        // the slab in place (from L2) with the positions those words give
-        FLEXIQ_CUDA_TRY(cudaMemsetAsync(scratch, 0, sizeof(unsigned) * L->n_g, st));
-        long long want1 = (M * n_c16 + threads - 1) / threads;
-        long long blocks1 = want1 < (long long)sms * 16 ? want1 : (long long)sms * 16;
-        // a grid stride that is a multiple of a row's chunks keeps every thread on its chunk column
-        int a = n_c16, b = threads;
-        while (b) { const int t = a % b; a = b; b = t; }
-        const long long unit = n_c16 / a;
-        if (blocks1 >= unit) blocks1 -= blocks1 % unit;
-        StraddleJob none{};
-        FLEXIQ_CUDA_TRY(launch_pdl(quantize_lower_kernel<DTYPE, 2>, (unsigned)blocks1, threads, sizeof(unsigned) * L->n_g, st, X, M, K, G, 0, S, L->perm,
-                                   static_cast<const uint8_t *>(nullptr), static_cast<const unsigned *>(scratch), X4, pitch, X8, pitch8,
-                                   static_cast<uint8_t *>(nullptr), none));
-    } else
+    constexpr size_t elem = DTYPE == FLEXIQ_DTYPE_F32 ? 4 : (DTYPE == FLEXIQ_DTYPE_I8 ? 1 : 2);
+    if (dynamic) FLEXIQ_CUDA_TRY(cudaMemsetAsync(scratch, 0, sizeof(unsigned) * L->n_g, st));
+    if (masked && (size_t)K * elem <= kRowStageBytes) {
+        StraddleJob job{};
+        if (straddle_in_use(L) && straddle_stale(L, st)) {
+            // the GEMM that consumes these slabs reads the straddle block of the same max_4bit_ch
+            job.wst = L->wst; job.w8m = L->w8m; job.w8 = L->w8;
+            job.rows = L->N * L->R * L->S;
+            job.C = L->C;
+            job.BK = choose_bk(L);
+            job.blk0 = (L->K_lo / job.BK) * job.BK;
+            job.K_lo = L->K_lo;
+        }
+        int8_t *slab = reinterpret_cast<int8_t *>(X4);
+        int rc;
+        if (!dynamic) rc = launch_rows<DTYPE, false>(L, X, M, S, slab, nullptr, job, st);
+        else {
+            // the input is read once: phase 1 quantizes, gathers and collects the OR words, phase 2 lowers the low groups of
+            // the slab in place (from L2) with the positions those words give
+            if ((rc = launch_rows<DTYPE, true>(L, X, M, S, slab, scratch, StraddleJob{}, st))) return rc;
+            const int lo_c16 = L->K_lo / 16;
+            const long long want = (M * lo_c16 + 4 * threads - 1) / (4 * threads);
+            long long blocks = want < (long long)sms * 8 ? want : (long long)sms * 8;
+            if (blocks < 1) blocks = 1;   // the positions are written even when no group is low
+            const long long extra = job.wst ? ((long long)job.rows * (job.BK >> 4) + threads - 1) / threads : 0;
+            job.first_block = (unsigned)extra;
+            FLEXIQ_CUDA_TRY(launch_pdl(lower_inplace_kernel, (unsigned)(blocks + extra), threads, 0, st, slab, M, K, G, L->K_lo,
+                                       static_cast<const unsigned *>(scratch), sx_out, job, lo_c16 ? (int)(blocks * threads / lo_c16) : 0,
+                                       lo_c16 ? (int)(blocks * threads % lo_c16) : 0));
+        }
+        if (rc) return rc;
+        if (job.wst) straddle_written(L, st);
+        record_slab(L, X4, L->K_lo);   // remember at which max_4bit_ch this buffer was written (the mixed_* calls check it)
+        return FLEXIQ_OK;
+    }
     if (dynamic) {
-        FLEXIQ_CUDA_TRY(cudaMemsetAsync(scratch, 0, sizeof(unsigned) * L->n_g, st));
         long long want = (M * n_c16 + threads - 1) / threads;
         long long blocks = want < (long long)sms * 8 ? want : (long long)sms * 8;
         // thread count must cover at least one full row of chunks
         while (blocks * threads < n_c16) ++blocks;
         FLEXIQ_CUDA_TRY(launch_pdl(group_or_kernel<DTYPE>, (unsigned)blocks, threads, sizeof(unsigned) * L->n_g, st, X, M, K, G, S, L->perm, scratch));
     }
-    long long want = (M * n_c16 + threads - 1) / threads;
-    long long blocks = want < (long long)sms * 16 ? want : (long long)sms * 16;
+    const long long want = (M * n_c16 + threads - 1) / threads;
+    const long long blocks = want < (long long)sms * 16 ? want : (long long)sms * 16;
     const uint8_t *sx = dynamic ? nullptr : L->sx;
-    StraddleJob wp{};
-    long long extra = 0;
-    if (straddle_in_use(L) && straddle_stale(L, st)) {
-        // the GEMM that consumes these slabs reads the straddle block of the same max_4bit_ch
-        wp.wst = L->wst; wp.w8m = L->w8m; wp.w8 = L->w8;
-        wp.rows = L->N * L->R * L->S;
-        wp.C = L->C;
-        wp.BK = choose_bk(L);
-        wp.blk0 = (L->K_lo / wp.BK) * wp.BK;
-        wp.K_lo = L->K_lo;
-        extra = ((long long)wp.rows * (wp.BK >> 4) + threads - 1) / threads;
-    }
-    wp.first_block = (unsigned)extra;   // the straddle blocks come first
-    if (dynamic && masked) {
-        long long want2 = (M * (L->K_lo / 16) + threads - 1) / threads;
-        long long blocks2 = want2 < (long long)sms * 16 ? want2 : (long long)sms * 16;
-        if (blocks2 < 1) blocks2 = 1;   // the positions are written even when no group is low
-        FLEXIQ_CUDA_TRY(launch_pdl(lower_inplace_kernel, (unsigned)(blocks2 + extra), threads, 0, st, reinterpret_cast<int8_t *>(X4), M, K, G, L->K_lo,
-                                   static_cast<const unsigned *>(scratch), sx_out, wp));
-        if (wp.wst) straddle_written(L, st);
-        record_slab(L, X4, L->K_lo);
-        return FLEXIQ_OK;
-    }
-    const unsigned grid = (unsigned)(blocks + extra);
-    if (!masked)
-        FLEXIQ_CUDA_TRY(launch_pdl(quantize_lower_kernel<DTYPE, 1>, grid, threads, 0, st, X, M, K, G, L->K_lo, S, L->perm, sx, scratch, X4, pitch, X8, pitch8, dynamic ? sx_out : nullptr, wp));
+    uint8_t *sx_to = dynamic ? sx_out : nullptr;
+    if (masked)   // (the straddle block of so wide a layer is left to the GEMM, which writes it when it is stale)
+        FLEXIQ_CUDA_TRY(launch_pdl(quantize_chunks_kernel<DTYPE, false>, (unsigned)blocks, threads, 0, st, X, M, K, G, L->K_lo, S, L->perm, sx, scratch, X4, pitch, X8, pitch8, sx_to));
     else
-        FLEXIQ_CUDA_TRY(launch_pdl(quantize_lower_kernel<DTYPE, 0>, grid, threads, 0, st, X, M, K, G, L->K_lo, S, L->perm, sx, scratch, X4, pitch, X8, pitch8, dynamic ? sx_out : nullptr, wp));
-    if (extra) straddle_written(L, st);
-    // remember at which max_4bit_ch these buffers were written (the mixed_* calls check it)
+        FLEXIQ_CUDA_TRY(launch_pdl(quantize_chunks_kernel<DTYPE, true>, (unsigned)blocks, threads, 0, st, X, M, K, G, L->K_lo, S, L->perm, sx, scratch, X4, pitch, X8, pitch8, sx_to));
     if (masked || L->K_lo > 0) record_slab(L, X4, L->K_lo);
     if (!masked && L->K_lo < L->C) record_slab(L, X8, L->K_lo);
     return FLEXIQ_OK;
+}
+
+unsigned prologue_status()
+{
+    unsigned word = 0;
+    const unsigned zero = 0;
+    if (cudaMemcpyFromSymbol(&word, g_prologue_status, sizeof(word)) != cudaSuccess) return 0;   // the caller's own read reports it
+    if (word) cudaMemcpyToSymbol(g_prologue_status, &zero, sizeof(zero));
+    return word;
 }
 
 }  // namespace flexiq
