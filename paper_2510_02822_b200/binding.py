@@ -1,8 +1,8 @@
-"""ctypes binding of libflexiq.so: argument marshalling only.
+"""Binding of libflexiq.so: argument marshalling only.
 
 Every function named ``flexiq_*`` here forwards to the C entry point of the same name
-(see ``include/flexiq.h``); ``Layer`` is a small convenience wrapper that owns a handle
-and allocates the slabs with torch.  Nothing here computes: every step of the path runs
+(see ``include/flexiq.h``) through ctypes; ``Layer`` is a small convenience wrapper that owns a handle
+and allocates the slabs with torch, and makes the calls of a forward pass through the native module ``_calls``.  Nothing here computes: every step of the path runs
 in the CUDA kernels of the library.
 """
 from __future__ import annotations
@@ -91,6 +91,21 @@ def lib():
         L.flexiq_sq_distance_i8.argtypes = [vp, vp, i64, vp, vp]
         _lib = L
     return _lib
+
+
+_calls_module = None
+
+
+def _native_calls():
+    """The native marshalling module (csrc/torch_calls.cpp), built beside the library; raises if it has not been."""
+    global _calls_module
+    if _calls_module is None:
+        import torch  # noqa: F401  (its libraries have to be loaded first)
+        lib()
+        from . import _calls
+        _calls.set_error_class(FlexiqError)
+        _calls_module = _calls
+    return _calls_module
 
 
 def last_error() -> str:
@@ -285,8 +300,16 @@ class Layer:
                                               perm, x_shift)
         self.device = Wq.device
         self._slabs = {}
+        # the calls of a forward pass go through native marshalling; what it answers NotImplemented to takes the Python code
+        # below it (a subclass with slabs of its own always does)
+        self._calls = None
+        if type(self).alloc_slabs is Layer.alloc_slabs:
+            st, pad = conv or (1, 0)
+            self._calls = _native_calls().Calls(self.h.value, self.K, self.N, G, int(conv is not None), st, pad, *((self.R, self.S) if conv else (1, 1)),
+                                                self.device.index, self._slabs)
 
     def close(self):
+        self._calls = None
         if self.h is not None:
             flexiq_layer_destroy(self.h)
             self.h = None
@@ -301,6 +324,8 @@ class Layer:
         flexiq_layer_set_lowbit_path(self.h, path)
 
     def set_lowbit_ratio(self, ratio):
+        if self._calls is not None and self._calls.set_lowbit_ratio(ratio) is not NotImplemented:
+            return
         flexiq_set_lowbit_ratio(self.h, ratio)
 
     def set_group_perm(self, Wq, group_perm, x_shift=None):
@@ -309,6 +334,16 @@ class Layer:
         perm = np.ascontiguousarray(group_perm, dtype=np.int32)
         xs = None if x_shift is None else np.ascontiguousarray(x_shift, dtype=np.uint8)
         _check(lib().flexiq_layer_set_group_perm(self.h, _ptr(Wq), _np_ptr(perm), None if xs is None else _np_ptr(xs), _stream()))
+
+    def select_groups(self, Wq, flags, x_shift):
+        """set_group_perm with the flagged groups (uint8 [n_g]) first, in index order, and the ratio that makes exactly them low."""
+        import numpy as np
+        if self._calls is not None and self._calls.select_groups(Wq, flags, x_shift) is not NotImplemented:
+            return
+        f = np.asarray(flags).astype(bool)
+        idx = np.arange(f.size, dtype=np.int32)
+        self.set_group_perm(Wq, np.concatenate([idx[f], idx[~f]]), x_shift)
+        self.set_lowbit_ratio(int(f.sum()) / f.size)
 
     def sync_ratio(self):
         """Writes the ratio-dependent weight K block for the ratio in force on the current stream, if it is not there yet."""
@@ -328,6 +363,10 @@ class Layer:
         return self._slabs[M]
 
     def quantize_lower(self, X, x_scale, dynamic=False, slabs=None):
+        if self._calls is not None:
+            r = self._calls.quantize_lower(X, x_scale, dynamic, slabs)
+            if r is not NotImplemented:
+                return r
         import torch
         M = X.numel() // self.K
         x4, x8 = slabs if slabs is not None else self.alloc_slabs(M)
@@ -339,6 +378,10 @@ class Layer:
         return x4, x8, shifts
 
     def mixed_gemm(self, x4, x8, M, x_scale, y_scale, out_mode, Y=None, x_shift=None):
+        if self._calls is not None:
+            r = self._calls.mixed_gemm(x4, x8, M, x_scale, y_scale, out_mode, Y, x_shift)
+            if r is not NotImplemented:
+                return r
         import torch
         if Y is None:
             dt = {OUT_ACC_I32: torch.int32, OUT_REQUANT_I8: torch.int8, OUT_DEQUANT_F32: torch.float32,
@@ -357,12 +400,20 @@ class Layer:
 
     def mixed_gemm_to_slab(self, x4, x8, M, x_scale, nxt, next_x_scale, relu=False, slab=None, x_shift=None, out_order=ORDER_ORIGINAL):
         """Mixed GEMM whose epilogue writes the masked slab of the layer `nxt` (fused layer boundary)."""
+        if self._calls is not None and nxt._calls is not None:
+            r = self._calls.mixed_gemm_to_slab(x4, x8, M, x_scale, nxt._calls, next_x_scale, relu, slab, x_shift, out_order)
+            if r is not NotImplemented:
+                return r
         if slab is None:
             slab = nxt.alloc_slabs(M)[0]
         flexiq_mixed_gemm_to_slab(self.h, x4, x8, x_shift, M, x_scale, nxt.h, next_x_scale, relu, out_order, slab)
         return slab
 
     def mixed_conv_to_slab(self, x4, x8, Nb, H, W, x_scale, nxt, next_x_scale, relu=False, slab=None, x_shift=None, out_order=ORDER_ORIGINAL):
+        if self._calls is not None and nxt._calls is not None:
+            r = self._calls.mixed_conv_to_slab(x4, x8, Nb, H, W, x_scale, nxt._calls, next_x_scale, relu, slab, x_shift, out_order)
+            if r is not NotImplemented:
+                return r
         stride, pad = self.conv
         P = (H + 2 * pad - self.R) // stride + 1
         Q = (W + 2 * pad - self.S) // stride + 1
@@ -372,6 +423,10 @@ class Layer:
         return slab
 
     def mixed_conv(self, x4, x8, Nb, H, W, x_scale, y_scale, out_mode, Y=None, x_shift=None):
+        if self._calls is not None:
+            r = self._calls.mixed_conv(x4, x8, Nb, H, W, x_scale, y_scale, out_mode, Y, x_shift)
+            if r is not NotImplemented:
+                return r
         import torch
         stride, pad = self.conv
         P = (H + 2 * pad - self.R) // stride + 1

@@ -1,13 +1,16 @@
-"""Builds libflexiq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libflexiq.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _calls.so (the Python side's native
+marshalling, which links against it and torch) with the host compiler."""
 from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 
 _DIR = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_DIR)
 CSRC = os.path.join(_DIR, "csrc")
 LIB = os.path.join(_DIR, "libflexiq.so")
+CALLS = os.path.join(_DIR, "_calls.so")
 SOURCES = ["flexiq_layer.cu", "flexiq_prologue.cu", "flexiq_gemm.cu", "flexiq_reorder.cu", "flexiq_calib.cu", "flexiq_serving.cu", "flexiq_evolution.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -17,9 +20,9 @@ NVCC_FLAGS = [
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(CALLS)):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(_ROOT, "include", "flexiq.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
@@ -37,7 +40,17 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         subprocess.run(cmd, check=True)
         objs.append(obj)
     subprocess.run([nvcc, "-shared", "-Wno-deprecated-gpu-targets", "-o", LIB, *objs, "-cudart", "static"], check=True)
+    _build_calls()
     return LIB
+
+
+def _build_calls():
+    from torch.utils.cpp_extension import include_paths, library_paths
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    include = [sysconfig.get_paths()["include"], *include_paths(), os.path.join(cuda, "include"), os.path.join(_ROOT, "include")]
+    subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", *(f"-I{d}" for d in include), os.path.join(CSRC, "torch_calls.cpp"), "-o", CALLS,
+                    f"-L{_DIR}", "-l:libflexiq.so", "-Wl,-rpath,$ORIGIN", *(f"-L{d}" for d in library_paths()), f"-L{os.path.join(cuda, 'lib64')}",
+                    "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-lcudart"], check=True)
 
 
 if __name__ == "__main__":

@@ -66,9 +66,13 @@ def static_preparation_device(Xcal: torch.Tensor, x_scale: float, Wq: torch.Tens
     (per-channel histograms, equal tails dropped) instead of the exact min / max.
     Returns (group_perm, x_shift, info) with info = {lo, hi, wmax, score, unused_hist} (torch tensors)."""
     from . import binding as fx
-    dev = Xcal.device
     C = Xcal.shape[-1]
     X2 = Xcal.reshape(-1, C)
+    r = fx._native_calls().static_preparation(X2, x_scale, Wq, G, conv, batches, coverage)
+    if r is not NotImplemented:
+        perm, x_shift, lo, hi, wmax, score, hist = r
+        return perm.numpy(), x_shift.numpy(), {"lo": lo, "hi": hi, "wmax": wmax, "score": score, "unused_hist": hist}
+    dev = Xcal.device
     lo = torch.empty(C, dtype=torch.int32, device=dev)
     hi = torch.empty(C, dtype=torch.int32, device=dev)
     rows = X2.shape[0]

@@ -62,37 +62,40 @@ class ChainFitness:
     def _layer(self, l, flags_layer):
         """The handle of layer l laid out for this selection: one handle per layer, re-laid out in place
         (flexiq_layer_set_group_perm: no allocation, no synchronisation) when the selection changes."""
-        key = bytes(np.asarray(flags_layer, dtype=np.uint8))
+        flags_layer = np.ascontiguousarray(flags_layer, dtype=np.uint8)
+        key = flags_layer.tobytes()
         h = self.handles[l]
         if key != self.current[l]:
-            perm, n_low = selection_perm(flags_layer)
             Wq, ws, b = self.dev_params[l]
-            xs = np.asarray(self.layers[l]["sx_group"], dtype=np.uint8)
+            xs = np.ascontiguousarray(self.layers[l]["sx_group"], dtype=np.uint8)
             if h is None:
+                perm, n_low = selection_perm(flags_layer)
                 h = self.handles[l] = fx.Layer(Wq, ws, b, perm, xs, self.layers[l]["G"])
+                h.set_lowbit_ratio(n_low / self.groups[l])
             else:
-                h.set_group_perm(Wq, perm, xs)
-            h.set_lowbit_ratio(n_low / self.groups[l])
+                h.select_groups(Wq, flags_layer, xs)
             self.current[l] = key
             self.created += 1
         return h
 
     def outputs(self, flags):
         """int8 outputs of the last layer under the selection `flags` (device tensor, reused by the next call)."""
-        src, dtype = self.X, fx.DTYPE_F32
+        src = self.X
         for l, L in enumerate(self.layers):
             h = self._layer(l, flags[self.off[l]:self.off[l + 1]])
-            fx.flexiq_quantize_lower(h.h, src, dtype, self.M, L["x_scale"], 0, self.slab[l], None)
-            fx.flexiq_mixed_gemm(h.h, self.slab[l], None, None, self.M, L["x_scale"], L["y_scale"], fx.OUT_REQUANT_I8, self.Y[l])
-            src, dtype = self.Y[l], fx.DTYPE_I8
+            h.quantize_lower(src, L["x_scale"], slabs=(self.slab[l], None))
+            src = h.mixed_gemm(self.slab[l], None, self.M, L["x_scale"], L["y_scale"], fx.OUT_REQUANT_I8, self.Y[l])
         self.evaluated += 1
         return self.Y[-1]
 
     def distances(self, pop):
         """Exact squared distances of every chromosome of `pop` (one device synchronisation in all)."""
+        calls = fx._native_calls()
         out = torch.zeros(len(pop), dtype=torch.int64, device=self.dev)
         for i, c in enumerate(pop):
-            fx.flexiq_sq_distance_i8(self.outputs(np.asarray(c, dtype=np.uint8)), self.Y8, out[i:i + 1])
+            Y = self.outputs(np.asarray(c, dtype=np.uint8))
+            if calls.sq_distance_i8(Y, self.Y8, out, i) is NotImplemented:
+                fx.flexiq_sq_distance_i8(Y, self.Y8, out[i:i + 1])
         return [int(v) for v in out.cpu().tolist()]
 
     def close(self):
