@@ -89,6 +89,8 @@ struct GemmParams {
     // patch then carries one more row.
     int pw_log2, TH, tiles_per_img, patch_stage;   // patch_stage: bytes of one ring stage (the patch, rounded up to 1 KB)
     int patch_rows;      // input rows of a patch: TH + R - 1, plus one when a tap's column index can pass the pitch (see above)
+    // Weight loads ahead of the dependency wait (see the kernel): whole blocks of w8 / w8m, and the straddle block
+    int early_w, early_st;
     // packed low-bit path only: positions the expander warps shift the 4-bit values back to
     const uint8_t *sx;   // [n_g] activation positions, slab order
     const uint8_t *sw;   // [n_g][N] weight positions
@@ -681,6 +683,14 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
     const uint32_t cta_rank = CG == 2 ? ptx::cluster_ctarank() : 0u;
     const bool leader = cta_rank == 0;
     const int first_tile = blockIdx.x / CG, tile_step = gridDim.x / CG;
+    // resident weights: all taps' weight tiles of this CTA's (only) column block, once
+    auto load_resident = [&]() {
+        const uint32_t bar = ptx::smem_u32(&raw_full[0]);
+        if (leader) ptx::mbar_expect_tx_s(bar, (uint32_t)(CG * p.T * b_sub));
+        const uint32_t bar_lead = CG == 2 ? ptx::mapa(bar, 0) : bar;
+        for (int t = 0; t < p.T; ++t)
+            ptx::tma_load_2d_s<CG>(ptx::smem_u32(stage_base) + t * b_sub, &mapB_hi, bar_lead, t * p.b_tap_step, (int)cta_rank * b_rows);
+    };
     // two accumulators (tiles in turn); SPLIT: two per tile, four in all
     const uint32_t buf_stride = BN <= 64 ? 64u : (BN <= 128 ? 128u : 256u);  // column offset from one accumulator to the next
     const uint32_t tmem_cols = ((SPLIT || kPatch) ? 4u : 2u) * buf_stride;
@@ -714,8 +724,37 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
     const uint32_t tmem_base = *tmem_ptr_s;
     // Everything above touched only this CTA's shared and tensor memory, so it may overlap the tail
     // of the previous kernel of the stream (programmatic dependent launch); wait for that kernel
-    // (the prologue that writes the slabs) before reading or writing global memory.  This kernel
-    // does not release its own successor early: a successor parked on the SMs slows the mainloop.
+    // (the prologue that writes the slabs) before reading or writing anything it may still touch.
+    // The weights are not among that: no prologue and no GEMM writes w8 or w8m, so the first tile's weight blocks, as many as
+    // the ring holds, are requested before the wait, and come from memory while the prologue still runs.  (The host says
+    // when it is not so: a layout or a straddle write not yet ordered by a call that has waited.)
+    // Only for the plain kind (and for resident weights): in the im2col kind's producer loop the extra selections cost
+    // more than they save (3x3 at 14 x 14: 13.7 -> 14.9 us).
+    uint32_t early = 0;                               // leading stages whose transaction bytes and weight loads are issued
+    TileWalk ptw;                                     // the producer's walk
+    if (warp == 0) {
+        ptw.init(first_tile, tile_step, num_tiles, p.n_tiles);
+        if (k_bres && p.early_w && p.early_st && ptw.left > 0) {
+            if (ptx::elect_one()) load_resident();
+        } else if (!PK && KIND == 0 && p.early_w && ptw.left > 0) {
+            const int slots = p.nb_lo + p.nb_hi;      // one tap
+            early = (uint32_t)(slots < p.stages ? slots : p.stages);
+            if (ptx::elect_one()) {
+                const uint32_t sb = ptx::smem_u32(stage_base) + (uint32_t)b_off, full0 = ptx::smem_u32(full_bar);
+                const uint32_t bar0 = CG == 2 ? ptx::mapa(full0, 0) : full0;
+                const int n0 = ptw.n_blk * BN + (int)cta_rank * b_rows;
+                for (uint32_t i = 0; i < early; ++i) {
+                    if (leader) ptx::mbar_expect_tx_s(full0 + 8 * i, (uint32_t)(CG * (BM * p.BK + b_rows * p.BK)));
+                    if ((int)i == p.st_cb) {
+                        if (p.early_st) ptx::tma_load_2d_s<CG>(sb + i * stage_bytes, &mapB_st, bar0 + 8 * i, 0, n0);
+                    } else {
+                        ptx::tma_load_2d_s<CG>(sb + i * stage_bytes, (int)i < p.nb_lo ? &mapB_lo : &mapB_hi, bar0 + 8 * i, (int)i * p.BK, n0);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+    }
     ptx::pdl_wait();
 
     if (warp == 0) {
@@ -742,16 +781,8 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         bool ok = true;
         PROF_DECL(prof_wait);
         PROF_T0(prof_start);
-        TileWalk tw;
-        tw.init(first_tile, tile_step, num_tiles, p.n_tiles);
-        if (k_bres && tw.left > 0 && ptx::elect_one()) {
-            // all taps' weight tiles of this CTA's (only) column block, once
-            const uint32_t bar = ptx::smem_u32(&raw_full[0]);
-            if (leader) ptx::mbar_expect_tx_s(bar, (uint32_t)(CG * p.T * b_sub));
-            const uint32_t bar_lead = CG == 2 ? ptx::mapa(bar, 0) : bar;
-            for (int t = 0; t < p.T; ++t)
-                ptx::tma_load_2d_s<CG>(ptx::smem_u32(stage_base) + t * b_sub, &mapB_hi, bar_lead, t * p.b_tap_step, (int)cta_rank * b_rows);
-        }
+        TileWalk &tw = ptw;
+        if (k_bres && !(p.early_w && p.early_st) && tw.left > 0 && ptx::elect_one()) load_resident();
         __syncwarp();
         // Output pixel (image, row, column) of this CTA's first row in the current tile, kept up to date by
         // additions: the divisions are done once per kernel, not once per tile, in this single-lane loop.
@@ -853,7 +884,8 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                         PROF_ADD(prof_wait, t0);
                         if (ptx::elect_one()) {
                             const uint32_t sa = stage0 + stage * stage_bytes;
-                            if (leader) ptx::mbar_expect_tx_s(full0 + 8 * stage, tx_bytes);
+                            const bool ahead = !PK && KIND == 0 && issued < (long long)early;
+                            if (leader && !ahead) ptx::mbar_expect_tx_s(full0 + 8 * stage, tx_bytes);
                             if (PK) ptx::mbar_arrive_count(&full_bar[stage], PK ? kExpWarps - 1 : 0);  // stand in for the expander warps
                             const uint32_t bar = full0_lead + 8 * stage;
                             if (k_im2col)
@@ -861,8 +893,11 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                             else
                                 ptx::tma_load_2d_s<CG>(sa, ma, bar, xa, (int)m0);
                             // the block that max_4bit_ch falls into comes from the straddle buffer [N][T][BK]
-                            if (!PK && part == 0 && cb == p.st_cb) ptx::tma_load_2d_s<CG>(sa + b_off, &mapB_st, bar, tap * p.BK, n0);
-                            else ptx::tma_load_2d_s<CG>(sa + b_off, mb, bar, xb, n0);
+                            if (!PK && part == 0 && cb == p.st_cb) {
+                                if (!(ahead && p.early_st)) ptx::tma_load_2d_s<CG>(sa + b_off, &mapB_st, bar, tap * p.BK, n0);
+                            } else if (!ahead) {
+                                ptx::tma_load_2d_s<CG>(sa + b_off, mb, bar, xb, n0);
+                            }
                         }
                         __syncwarp();
                         xa += p.BK;
@@ -875,11 +910,16 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                 }
             }
         }
+        // This CTA's loads are all issued: the next kernel of the stream may be launched as CTAs leave, and does what it can before
+        // its own dependency wait while the last tiles are computed and written (measured per layer, graph replay, prologue + GEMM: K = 1536
+        // at 197 rows 7.95 -> 7.67 us, ViT-B QKV 29.9 -> 29.5, 1x1 at 56 x 56 21.6 -> 20.6).
+        if (lane == 0) ptx::pdl_launch_dependents();
         PROF_STORE(0, prof_wait);
         PROF_STORE(1, clock64() - prof_start);
         PROF_STORE(2, issued);
         if (!ok && lane == 0) {
             // drain: let the copies already in flight land before the CTA retires
+            if (issued < (long long)early) __nanosleep(100000u);   // weight blocks whose stages will never fill
             const int n_back = issued < p.stages ? (int)issued : p.stages;
             int s = (int)stage;
             uint32_t ph = phase;
@@ -1672,6 +1712,11 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
         cm.slab = slab; cm.Y = staged ? Y : nullptr; cm.M = M; cm.Nb = Nb; cm.H = H; cm.W = W; cm.bk = p.BK; cm.im2col = (int)p.im2col + 2 * (int)patch;
         cm.staged = staged; cm.y_elem = y_elem; cm.a = a_hi; cm.y = y_map; cm.y16 = y_map16;
     }
+    // Early weight loads (see the kernel) are safe once some call on this handle has waited for whatever wrote the weights: this
+    // call's launches do, so the next may.  In a capture, or when one has written the straddle block, it is always late.
+    p.early_w = !L->weights_fresh;
+    p.early_st = p.st_cb < 0 || (!L->st_fresh && !L->st_graph_seen && stream_capture_id(st) == 0);
+    L->weights_fresh = L->st_fresh = 0;
     const int bi = weight_map_index(bn / cg);  // box rows = the B rows one CTA loads
     const bool conv_kind = p.im2col || p.tps > 1 || p.b_res;
     // One narrow tile per CTA and a long K: nothing overlaps across tiles, so the MMA warps share the tile

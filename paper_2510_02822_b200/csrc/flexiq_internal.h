@@ -47,6 +47,7 @@ struct Layer {
                                    // st_K_lo, so eager calls no longer trust it
     unsigned long long st_cap_id;  // capture sequence that last wrote wst, and for which max_4bit_ch
     int st_cap_K_lo;
+    int weights_fresh, st_fresh;   // w8 / w8m, or wst, written since the handle's last GEMM launch
     uint8_t *sw;     // [n_g][N] weight extraction positions
     uint8_t *sx;     // [n_g] static activation positions, slab order
     int32_t *perm;   // [n_g]

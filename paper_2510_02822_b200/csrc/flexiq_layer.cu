@@ -114,6 +114,7 @@ bool straddle_stale(const Layer *L, cudaStream_t st)
 }
 void straddle_written(Layer *L, cudaStream_t st)
 {
+    L->st_fresh = 1;
     const unsigned long long cap = stream_capture_id(st);
     if (cap) { L->st_cap_id = cap; L->st_cap_K_lo = L->K_lo; L->st_graph_seen = 1; L->st_K_lo = -1; }
     else L->st_K_lo = L->K_lo;
@@ -487,6 +488,7 @@ static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const u
     }
     FLEXIQ_CUDA_TRY(launch_prep(L, a, order, stream));
     L->st_K_lo = -1;   // the straddle block was cut from the previous order's weights
+    L->weights_fresh = 1;
     L->st_cap_id = 0;
     L->slab_next = 0;  // slabs written for the previous order are no longer this layer's
     memset(L->slab_seen, 0, sizeof(L->slab_seen));
