@@ -80,7 +80,7 @@ struct GemmParams {
     int b_res;
     // Patch mode (KIND 2: 3x3-like convolutions of stride 1 whose channels fit one K block and whose output
     // channels fit one tile): a tile is TH = 128 / PW whole output rows of one image, its 128 accumulator rows
-    // being the positions y * PW + x of a grid whose pitch PW (a power of two >= W + pad) leaves a few unused
+    // being the positions y * PW + x of a grid whose pitch PW (a power of two >= W + pad and >= Q) leaves a few unused
     // columns.  The input patch of TH + R - 1 rows x PW pixels is loaded ONCE per tile by a tiled 4-D copy
     // (halo and padding arrive as zeros); filter tap (r, s) is the same patch read from row offset r * PW + s,
     // so every input pixel crosses from L2 once instead of R * S times.  When W + 2 pad > PW the rightmost taps of the
@@ -1602,8 +1602,8 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
     // output channels fit one tile, the weights of all taps resident in shared memory.
     bool patch = false;
     int patch_pw = 8;
-    if (!packed && !g_forced_tile.cg && p.im2col && L->stride == 1 && L->C <= p.BK && L->N <= 128 && W + L->pad <= 128) {
-        while (patch_pw < W + L->pad) patch_pw *= 2;
+    if (!packed && !g_forced_tile.cg && p.im2col && L->stride == 1 && L->C <= p.BK && L->N <= 128 && W + L->pad <= 128 && p.Q <= 128) {
+        while (patch_pw < W + L->pad || patch_pw < p.Q) patch_pw *= 2;   // (padding wider than the filter: more output columns than input)
         const int th = BM / patch_pw, bn_p = L->N <= 64 ? 64 : 128;
         const int rows = th + L->R - 1 + (W + 2 * L->pad > patch_pw ? 1 : 0);
         const int stage = ((rows * patch_pw * p.BK) + 1023) & ~1023;
