@@ -89,6 +89,16 @@ struct GemmParams {
     // patch then carries one more row.
     int pw_log2, TH, tiles_per_img, patch_stage;   // patch_stage: bytes of one ring stage (the patch, rounded up to 1 KB)
     int patch_rows;      // input rows of a patch: TH + R - 1, plus one when a tap's column index can pass the pitch (see above)
+    // Streamed patch mode (KIND 3: the other stride-1 filters of more than one tap and at most three columns).  As in patch mode a
+    // tile is a grid of output positions whose input patch is loaded by one tiled copy and read by every tap as a row
+    // offset, but per K block of the channels (a ring of a_stages patches), with the weight tiles of a filter row at a
+    // time streaming through the operand ring.  Where an image is narrower and lower than the tile, 1 << img_log2 images lie
+    // side by side in each row of the grid ([y][image][x]): an image's right padding is its neighbour's left padding.
+    // What bounded these layers as im2col copies was the feed: every activation row fetched once per tap, 128 rows a copy.  Now it is
+    // shared memory: an MMA of a single CTA reads 4 KB of A and 2 or 4 KB of B, whose refill crosses it again (92
+    // cycles at 128 columns where the pipe needs 64); a CTA pair halves B for both.  Batch 32, prologue + convolution by graph
+    // replay: 256 channels at 14 x 14 13.5 -> 11.2 us, 512 at 7 x 7 16.7 -> 11.1, 144 at 28 x 28 24.7 -> 20.0.
+    int img_log2, nbt, a_stages, a_stage, patch_tx;   // K blocks per tap; ring of patches: depth, bytes per stage, bytes per copy
     // Weight loads ahead of the dependency wait (see the kernel): whole blocks of w8 / w8m, and the straddle block
     int early_w, early_st;
     // packed low-bit path only: positions the expander warps shift the 4-bit values back to
@@ -338,7 +348,7 @@ struct EpilogueCtx {
 template <int CG, int MODE, bool SPLIT, int KIND>
 __device__ __forceinline__ void epilogue_role(const GemmParams &p, const EpilogueCtx &x, int quad, int part, int lane)
 {
-    constexpr bool kPatch = KIND == 2;
+    constexpr bool kPatch = KIND == 2, kGrid = KIND >= 2;
     constexpr bool kScaled = MODE != FLEXIQ_OUT_ACC_I32;
     constexpr bool kHalf = MODE == FLEXIQ_OUT_DEQUANT_F16 || MODE == FLEXIQ_OUT_DEQUANT_BF16;
     constexpr int kElem = (MODE == FLEXIQ_OUT_REQUANT_I8 || MODE == kOutNextSlab) ? 1 : (kHalf ? 2 : 4);  // output bytes per element
@@ -369,17 +379,24 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
         // where the warp's 32 accumulator rows go: rows row0.. of Y, or in patch mode a box of bx x by pixels
         int st_x = 0, st_y = 0, st_n = 0;
         bool box_live = true;
-        if (kPatch) {
-            const int pw = 1 << p.pw_log2;
-            st_n = tw.m_blk / p.tiles_per_img;
-            const int y0 = (tw.m_blk - st_n * p.tiles_per_img) * p.TH;
+        if (kGrid) {
+            const int pw = 1 << p.pw_log2, ilog = KIND == 3 ? p.img_log2 : 0;
+            const int mt = KIND == 3 ? tw.m_blk * CG + (int)x.cta_rank : tw.m_blk;
+            st_n = mt / p.tiles_per_img;
+            const int y0 = (mt - st_n * p.tiles_per_img) * p.TH;
+            st_n <<= ilog;
             const int k = quad * 32 + lane;
-            const int yy = y0 + (k >> p.pw_log2), xx = k & (pw - 1);
-            row = (yy < p.P && xx < p.Q) ? ((long long)st_n * p.P + yy) * p.Q + xx : p.M;   // p.M: not an output pixel
-            st_y = y0 + ((quad * 32) >> p.pw_log2);
+            const int yy = y0 + (k >> (p.pw_log2 + ilog)), xx = k & (pw - 1), nn = st_n + ((k >> p.pw_log2) & ((1 << ilog) - 1));
+            row = (yy < p.P && xx < p.Q) ? ((long long)nn * p.P + yy) * p.Q + xx : p.M;   // p.M or more: not an output pixel
+            st_y = y0 + ((quad * 32) >> (p.pw_log2 + ilog));
             st_x = (quad * 32) & (pw - 1);
-            box_live = st_y < p.P && st_x < p.Q;
+            if (KIND == 3) st_n += ((quad * 32) >> p.pw_log2) & ((1 << ilog) - 1);
+            box_live = st_y < p.P && st_x < p.Q && (KIND == 2 || (long long)st_n * p.P * p.Q < p.M);
         }
+        auto store_box = [&](const CUtensorMap *map, int col) {
+            if (KIND == 3) ptx::tma_store_4d(map, x.store_stage, col, st_x, st_n, st_y);   // that map's order is (channels, x, image, y)
+            else ptx::tma_store_4d(map, x.store_stage, col, st_x, st_y, st_n);
+        };
         bool waited = false;
         for (int pass = 0; pass < passes; ++pass) {
             const int col0 = (part * passes + pass) * cols;  // first tile column of this warp in this pass
@@ -447,7 +464,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                 // Each warp stages 32 rows x 32 columns (1 KB, 32-byte swizzle: no bank conflicts) and one
                 // lane hands them to a tiled bulk store, which writes whole sectors asynchronously and
                 // drops the rows and columns that lie outside Y.
-                const long long row0 = kPatch ? (box_live ? 0 : p.M) : row - lane;
+                const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t *r = h == 0 ? ra : rb;
@@ -478,7 +495,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                         ptx::fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0) {
-                            if (kPatch) ptx::tma_store_4d(both ? x.map_y : x.map_y16, x.store_stage, n, st_x, st_y, st_n);
+                            if (kGrid) store_box(both ? x.map_y : x.map_y16, n);
                             else ptx::tma_store_2d(both ? x.map_y : x.map_y16, x.store_stage, n, (int)row0);
                             ptx::bulk_commit_group();
                         }
@@ -486,7 +503,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                 }
             } else if (kHalf && p.tma_store) {
                 // 16-bit outputs: 32 rows x 16 columns (32 bytes per row: the same 1 KB swizzled box) per store
-                const long long row0 = kPatch ? (box_live ? 0 : p.M) : row - lane;
+                const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t *r = h == 0 ? ra : rb;
@@ -508,7 +525,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                             ptx::fence_proxy_async_smem();
                             __syncwarp();
                             if (lane == 0) {
-                                if (kPatch) ptx::tma_store_4d(x.map_y, x.store_stage, 2 * n, st_x, st_y, st_n);
+                                if (kGrid) store_box(x.map_y, 2 * n);
                                 else ptx::tma_store_2d(x.map_y, x.store_stage, 2 * n, (int)row0);
                                 ptx::bulk_commit_group();
                             }
@@ -517,7 +534,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                 }
             } else if (kElem == 4 && p.tma_store) {
                 // 4-byte outputs: 32 rows x 8 columns per store (the same 32-byte rows)
-                const long long row0 = kPatch ? (box_live ? 0 : p.M) : row - lane;
+                const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t *r = h == 0 ? ra : rb;
@@ -538,7 +555,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                                 ptx::fence_proxy_async_smem();
                                 __syncwarp();
                                 if (lane == 0) {
-                                    if (kPatch) ptx::tma_store_4d(x.map_y, x.store_stage, 4 * (n + 8 * b), st_x, st_y, st_n);
+                                    if (kGrid) store_box(x.map_y, 4 * (n + 8 * b));
                                     else ptx::tma_store_2d(x.map_y, x.store_stage, 4 * (n + 8 * b), (int)row0);
                                     ptx::bulk_commit_group();
                                 }
@@ -677,12 +694,14 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
     const bool k_im2col = KIND != 0 && p.im2col;      // compile-time false for KIND 0: the branches below fold away
     const int k_tps = KIND != 0 ? p.tps : 1;
     const bool k_bres = KIND != 0 && p.b_res;
+    constexpr bool kStream = KIND == 3;           // a halo patch per K block, weights streamed a filter row at a time (see GemmParams)
     constexpr bool kPatch = KIND == 2;            // halo patch per tile, taps as row offsets (see GemmParams)
     const int b_rows = BN / CG;                       // rows of the B tile this CTA loads
     // one stage = tps sub-tiles of A (BM x BK each) followed by tps sub-tiles of B (b_rows x BK each)
     const int a_sub = BM * p.BK, b_sub = b_rows * p.BK, b_off = k_tps * a_sub;
-    const int stage_bytes = kPatch ? p.patch_stage : (k_bres ? k_tps * a_sub : k_tps * (a_sub + b_sub));
-    const int ring_off = k_bres ? ((p.T * b_sub + 1023) & ~1023) : 0;   // resident weight tiles lie in front of the ring
+    const int stage_bytes = kPatch ? p.patch_stage : kStream ? k_tps * b_sub : (k_bres ? k_tps * a_sub : k_tps * (a_sub + b_sub));
+    // resident weight tiles, or the ring of patches, lie in front of the ring
+    const int ring_off = kStream ? p.a_stages * p.a_stage : (k_bres ? ((p.T * b_sub + 1023) & ~1023) : 0);
     const int num_tiles = p.m_tiles * p.n_tiles;
     const uint32_t cta_rank = CG == 2 ? __shfl_sync(0xffffffffu, ptx::cluster_ctarank(), 0) : 0u;
     const bool leader = cta_rank == 0;
@@ -695,10 +714,28 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         for (int t = 0; t < p.T; ++t)
             ptx::tma_load_2d_s<CG>(ptx::smem_u32(stage_base) + t * b_sub, &mapB_hi, bar_lead, t * p.b_tap_step, (int)cta_rank * b_rows);
     };
+    // streamed patch mode: the weight tiles of filter row r and K block cb into a ring stage
+    auto stream_weights = [&](int n0, int cb, int r, uint32_t st, bool expect, bool load) {
+        uint32_t bar = ptx::smem_u32(&full_bar[st]);
+        const uint32_t dst = ptx::smem_u32(stage_base) + (uint32_t)ring_off + st * (uint32_t)stage_bytes;
+        if (expect && leader) ptx::mbar_expect_tx_s(bar, (uint32_t)(CG * p.S * b_sub));
+        if (!load) return;
+        if (CG == 2) bar = ptx::mapa(bar, 0);
+        const CUtensorMap *m = cb == p.st_cb ? &mapB_st : (cb < p.nb_lo ? &mapB_lo : &mapB_hi);
+        for (int t = 0; t < p.S; ++t) {
+            const int tap = r * p.S + t;
+            ptx::tma_load_2d_s<CG>(dst + t * b_sub, m, bar, cb == p.st_cb ? tap * p.BK : tap * p.C + cb * p.BK, n0 + (int)cta_rank * b_rows);
+        }
+    };
     // two accumulators (tiles in turn); SPLIT: two per tile, four in all
     const uint32_t buf_stride = BN <= 64 ? 64u : (BN <= 128 ? 128u : 256u);  // column offset from one accumulator to the next
     const uint32_t tmem_cols = ((SPLIT || kPatch) ? 4u : 2u) * buf_stride;
 
+    // The descriptors are fetched beside the rest of the preamble: a first copy waits for its map, 0.7 us each one after the other.
+    if (warp == 2 && lane < 6) {
+        const CUtensorMap *m = lane == 0 ? &mapB_lo : lane == 1 ? &mapB_hi : lane == 2 ? &mapA_hi : lane == 3 ? &mapA_lo : lane == 4 ? &mapB_st : &mapY;
+        ptx::prefetch_tmap(m);
+    }
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) {
             ptx::mbar_init(&full_bar[s], PK ? kExpWarps : 1);  // packed path: every fill counts eight arrivals
@@ -732,21 +769,30 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
     // The weights are not among that: no prologue and no GEMM writes w8 or w8m, so the first tile's weight blocks, as many as
     // the ring holds, are requested before the wait, and come from memory while the prologue still runs.  (The host says
     // when it is not so: a layout or a straddle write not yet ordered by a call that has waited.)
-    // Only for the plain kind (and for resident weights): in the im2col kind's producer loop the extra selections cost
-    // more than they save (3x3 at 14 x 14: 13.7 -> 14.9 us).
-    uint32_t early = 0;                               // leading stages whose transaction bytes and weight loads are issued
-    TileWalk ptw;                                     // the producer's walk
-    if (warp == 0) {
-        ptw.init(first_tile, tile_step, num_tiles, p.n_tiles);
-        if (k_bres && p.early_w && p.early_st && ptw.left > 0) {
-            if (ptx::elect_one()) load_resident();
-        } else if (!PK && KIND == 0 && p.early_w && ptw.left > 0) {
-            const int slots = p.nb_lo + p.nb_hi;      // one tap
-            early = (uint32_t)(slots < p.stages ? slots : p.stages);
+    // Not for the im2col kind: in its producer loop the extra selections cost more than they save.
+    // The second MMA warp, idle until then, issues the convolutions' copies, so that the producer is not late with the
+    // activations (a copy takes the issuing lane about 0.1 us; 3x3 at 7 x 7: 13.2 us from the producer, 11.1 so); the one copy per
+    // stage of the plain kind stays with the producer (197 x 384 x 384: 5.0 us against 5.25).
+    const int early_slots = KIND == 0 ? p.nb_lo + p.nb_hi : (kStream ? p.nbt * (p.T / p.S) : 0);
+    const bool early_on = !PK && p.early_w && first_tile < num_tiles;
+    const uint32_t early = early_on ? (uint32_t)(early_slots < p.stages ? early_slots : p.stages) : 0u;   // leading stages
+    if (early_on && warp == (KIND == 0 ? 0 : 2 + kNumWorkWarps)) {
+        const int n_blk = first_tile % p.n_tiles;
+        if (KIND != 0 && k_bres) {
+            if (p.early_st && ptx::elect_one()) load_resident();
+        } else if (kStream) {
+            if (ptx::elect_one()) {
+                int cb = 0, r = 0;
+                for (uint32_t i = 0; i < early; ++i) {
+                    stream_weights(n_blk * BN, cb, r, i, true, cb != p.st_cb || p.early_st);
+                    if (++r * p.S == p.T) { r = 0; ++cb; }
+                }
+            }
+        } else if (KIND == 0) {
             if (ptx::elect_one()) {
                 const uint32_t sb = ptx::smem_u32(stage_base) + (uint32_t)b_off, full0 = ptx::smem_u32(full_bar);
                 const uint32_t bar0 = CG == 2 ? ptx::mapa(full0, 0) : full0;
-                const int n0 = ptw.n_blk * BN + (int)cta_rank * b_rows;
+                const int n0 = n_blk * BN + (int)cta_rank * b_rows;
                 for (uint32_t i = 0; i < early; ++i) {
                     if (leader) ptx::mbar_expect_tx_s(full0 + 8 * i, (uint32_t)(CG * (BM * p.BK + b_rows * p.BK)));
                     if ((int)i == p.st_cb) {
@@ -765,13 +811,6 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         // ------------------------------------------------------------- TMA producer
         // The whole warp walks the loops; one elected lane issues the copies.  K blocks run
         // low slab first (every tap, every channel block), then the high slab.
-        if (ptx::elect_one()) {
-            ptx::prefetch_tmap(&mapA_lo);
-            ptx::prefetch_tmap(&mapA_hi);
-            ptx::prefetch_tmap(&mapB_lo);
-            ptx::prefetch_tmap(&mapB_hi);
-            if (!PK && p.st_cb >= 0) ptx::prefetch_tmap(&mapB_st);
-        }
         const uint32_t tx_bytes = (uint32_t)(CG * (BM * p.BK + b_rows * p.BK));  // both CTAs' loads
         const uint32_t stage0 = ptx::smem_u32(stage_base) + (uint32_t)ring_off;
         const uint32_t empty0 = ptx::smem_u32(empty_bar);
@@ -785,7 +824,8 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         bool ok = true;
         PROF_DECL(prof_wait);
         PROF_T0(prof_start);
-        TileWalk &tw = ptw;
+        TileWalk tw;
+        tw.init(first_tile, tile_step, num_tiles, p.n_tiles);
         if (k_bres && !(p.early_w && p.early_st) && tw.left > 0 && ptx::elect_one()) load_resident();
         __syncwarp();
         // Output pixel (image, row, column) of this CTA's first row in the current tile, kept up to date by
@@ -813,11 +853,39 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                     const int img = tw.m_blk / p.tiles_per_img;
                     const int y0 = (tw.m_blk - img * p.tiles_per_img) * p.TH;
                     ptx::mbar_expect_tx_s(full0 + 8 * stage, (uint32_t)((p.patch_rows << p.pw_log2) * p.BK));
-                    ptx::tma_load_4d_s(stage0 + stage * stage_bytes, &mapA_hi, full0 + 8 * stage, 0, -p.pad, y0 - p.pad, img);
+                    ptx::tma_load_4d_s<1>(stage0 + stage * stage_bytes, &mapA_hi, full0 + 8 * stage, 0, -p.pad, y0 - p.pad, img);
                 }
                 __syncwarp();
                 ++issued;
                 if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1; }
+                continue;
+            }
+            if (kStream) {
+                const int mt = tw.m_blk * CG + (int)cta_rank;
+                const int img = mt / p.tiles_per_img;
+                const int y0 = (mt - img * p.tiles_per_img) * p.TH;
+                for (int cb = 0; cb < p.nbt && ok; ++cb) {
+                    PROF_T0(tq0);
+                    if (!__all_sync(0xffffffffu, wait_bounded(&raw_empty[rstage], rphase ^ 1, abort_flag, 5))) { ok = false; break; }
+                    PROF_ADD(prof_wait, tq0);
+                    if (ptx::elect_one()) {
+                        const uint32_t bar = ptx::smem_u32(&raw_full[rstage]);
+                        if (leader) ptx::mbar_expect_tx_s(bar, (uint32_t)(CG * p.patch_tx));
+                        ptx::tma_load_4d_s<CG>(ptx::smem_u32(stage_base) + rstage * (uint32_t)p.a_stage, &mapA_hi, CG == 2 ? ptx::mapa(bar, 0) : bar, cb * p.BK, -p.pad, img << p.img_log2, y0 - p.pad);
+                    }
+                    __syncwarp();
+                    if (++rstage == (uint32_t)p.a_stages) { rstage = 0; rphase ^= 1; }
+                    for (int r = 0; r < p.T / p.S; ++r) {
+                        if (!__all_sync(0xffffffffu, wait_bounded(empty0 + 8 * stage, phase ^ 1, abort_flag, 1))) { ok = false; break; }
+                        if (ptx::elect_one()) {
+                            const bool ahead = issued < (long long)early;
+                            stream_weights(tw.n_blk * BN, cb, r, stage, !ahead, !ahead || (cb == p.st_cb && !p.early_st));
+                        }
+                        __syncwarp();
+                        ++issued;
+                        if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1; }
+                    }
+                }
                 continue;
             }
             if (k_tps > 1) {
@@ -966,7 +1034,8 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
             PROF_DECL(prof_wait_acc);
             PROF_DECL(prof_wait_full);
             PROF_T0(prof_start);
-            const int tile_slots = kPatch ? 1 : (k_tps > 1 ? (p.T + k_tps - 1) / k_tps : p.T * (p.nb_lo + p.nb_hi));  // ring stages per tile
+            uint32_t astage = 0, aphase = 0;                     // streamed patch mode: ring of patches
+            const int tile_slots = kPatch ? 1 : kStream ? p.nbt * (p.T / p.S) : (k_tps > 1 ? (p.T + k_tps - 1) / k_tps : p.T * (p.nb_lo + p.nb_hi));  // ring stages per tile
             int ti = 0;                                          // index of the tile in this CTA's sequence
             TileWalk tw;
             for (tw.init(first_tile, tile_step, num_tiles, p.n_tiles); tw.left > 0 && ok; tw.next(), ++ti) {
@@ -974,6 +1043,10 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                     // the other warp's tile: step over its ring stages
                     stage += (uint32_t)tile_slots;
                     while (stage >= (uint32_t)p.stages) { stage -= (uint32_t)p.stages; phase ^= 1; }
+                    if (kStream) {
+                        astage += (uint32_t)p.nbt;
+                        while (astage >= (uint32_t)p.a_stages) { astage -= (uint32_t)p.a_stages; aphase ^= 1; }
+                    }
                     continue;
                 }
                 int slot = 0;                                    // stages of this tile passed so far
@@ -1035,6 +1108,50 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                     }
                     __syncwarp();
                     if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1; }
+                } else if (kStream) {
+                    const uint32_t row16 = (uint32_t)(p.BK >> 4);                  // one position of the patch, in 16-byte units
+                    const uint32_t down = row16 << (p.pw_log2 + p.img_log2);       // one row of the grid
+                    const uint32_t b_step = (uint32_t)(b_sub >> 4);
+                    const int R = p.T / p.S;
+                    for (int cb = 0; cb < p.nbt && ok; ++cb) {
+                        PROF_T0(tq1);
+                        if (!__all_sync(0xffffffffu, wait_bounded(&raw_full[astage], aphase, abort_flag, 6))) { ok = false; break; }
+                        PROF_ADD(prof_wait_full, tq1);
+                        const int ks = cb == p.nbt - 1 ? p.ks_last_hi : ks_full;
+                        uint32_t a_row = bres_lo + astage * (uint32_t)(p.a_stage >> 4);
+                        for (int r = 0; r < R; ++r) {
+                            PROF_T0(tq2);
+                            if (!__all_sync(0xffffffffu, wait_bounded(full0 + 8 * stage, phase, abort_flag, 3))) { ok = false; break; }
+                            PROF_ADD(prof_wait_full, tq2);
+                            if (++slot == tile_slots && lane == 0) ptx::mbar_arrive(turn_bar);   // the other warp may go on
+                            ptx::tc_fence_after_sync();
+                            const uint32_t b_lo = a_lo0 + stage * stage_step;
+                            if (ptx::elect_one()) {
+                                if (p.S == 3 && ks == 4) {
+                                    // spelled out: twelve MMAs in a row issue at the pipe's own rate (48 cycles each at 64 columns, 64 at 128)
+#pragma unroll
+                                    for (int t = 0; t < 3; ++t)
+#pragma unroll
+                                        for (int k = 0; k < 4; ++k)
+                                            ptx::mma_i8_s<CG>(d_tmem, a_row + (uint32_t)t * row16 + 2 * k, b_lo + (uint32_t)t * b_step + 2 * k, desc_hi, idesc, (t | k) ? 1u : acc);
+                                } else {
+                                    uint32_t a2 = acc;
+                                    for (int t = 0; t < p.S; ++t)
+                                        for (int k = 0; k < ks; ++k) {
+                                            ptx::mma_i8_s<CG>(d_tmem, a_row + (uint32_t)t * row16 + 2 * k, b_lo + (uint32_t)t * b_step + 2 * k, desc_hi, idesc, a2);
+                                            a2 = 1;
+                                        }
+                                }
+                                ptx::mma_commit_s<CG>(empty0 + 8 * stage);
+                                if (r == R - 1) ptx::mma_commit_s<CG>(ptx::smem_u32(&raw_empty[astage]));   // every tap has read the patch
+                            }
+                            __syncwarp();
+                            acc = 1;
+                            a_row += down;
+                            if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1; }
+                        }
+                        if (++astage == (uint32_t)p.a_stages) { astage = 0; aphase ^= 1; }
+                    }
                 } else
                 if (k_tps > 1) {
                     const int ks = (p.C + 31) >> 5;  // K steps of one tap (C <= BK)
@@ -1076,7 +1193,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                         if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1; }
                     }
                 }
-                for (int part = 0; part < 2 && ok && k_tps == 1 && !kPatch; ++part) {
+                for (int part = 0; part < 2 && ok && k_tps == 1 && !kPatch && !kStream; ++part) {
                     const int nb = part ? p.nb_hi : p.nb_lo;
                     if (nb == 0) continue;
                     const int ks_last = part ? p.ks_last_hi : p.ks_last_lo;
@@ -1419,6 +1536,71 @@ static int make_map_nhwc(CUtensorMap *map, const void *base, uint64_t row_bytes,
     return FLEXIQ_OK;
 }
 
+// The same tensor with the images before the rows: (row_bytes, W, Nb, H), box (box_bytes, bx, bn, by).
+static int make_map_nhwc_by_row(CUtensorMap *map, const void *base, uint64_t row_bytes, int W, int H, int Nb, uint32_t box_bytes,
+                                uint32_t bx, uint32_t bn, uint32_t by, int swizzle_bytes)
+{
+    EncodeTiledFn enc = get_encode_tiled();
+    if (!enc) return set_error(FLEXIQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    if ((reinterpret_cast<uintptr_t>(base) & 15) != 0 || (row_bytes & 15) != 0)
+        return set_error(FLEXIQ_ERR_INVALID_ARG, "tensor base %p / pixel pitch %llu not 16-byte aligned", base, (unsigned long long)row_bytes);
+    cuuint64_t dims[4] = {row_bytes, (cuuint64_t)W, (cuuint64_t)Nb, (cuuint64_t)H};
+    cuuint64_t strides[3] = {row_bytes, row_bytes * W * H, row_bytes * W};
+    cuuint32_t box[4] = {box_bytes, bx, bn, by};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    const CUtensorMapSwizzle swz = swizzle_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                 : (swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                 : (swizzle_bytes == 32 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE));
+    CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS)
+        return set_error(FLEXIQ_ERR_CUDA, "cuTensorMapEncodeTiled (by row) failed with CUresult %d (box %u x %u x %u x %u)", (int)r, box_bytes, bx, bn, by);
+    return FLEXIQ_OK;
+}
+
+// Streamed patch mode for a stride-1 filter: geometry of the grid and the rings, and which column width, or none.
+struct StreamPlan { int cg, bn, pw_log2, img_log2, th, rows, a_stage, stages, tiles_per_img; long long m_tiles; };
+static bool plan_stream(const Layer *L, int Nb, int W, int P, int Q, int bk, int sms, StreamPlan *out)
+{
+    const int width = W + L->pad > Q ? W + L->pad : Q;   // columns a row of the grid has to hold
+    if (L->S > 3 || width > 128) return false;
+    StreamPlan s{};
+    s.pw_log2 = 3;
+    while ((1 << s.pw_log2) < width) ++s.pw_log2;
+    // images side by side: as many as make the grid's rows at least fit the image's, and there are images
+    const int rows_max = BM >> s.pw_log2;
+    while ((rows_max >> s.img_log2) >= 2 * P && (2 << s.img_log2) <= Nb) ++s.img_log2;
+    if ((rows_max >> s.img_log2) > P && (rows_max >> (s.img_log2 + 1)) >= 1 && (2 << s.img_log2) <= Nb) {
+        // one more doubling when it wastes fewer rows
+        const int t0 = rows_max >> s.img_log2, t1 = t0 >> 1;
+        if ((long long)((P + t1 - 1) / t1) * t1 < (long long)t0) ++s.img_log2;
+    }
+    s.th = rows_max >> s.img_log2;
+    s.rows = s.th + L->R - 1 + (W + 2 * L->pad > (1 << s.pw_log2) ? 1 : 0);
+    const long long patch = (long long)s.rows * (bk << (s.pw_log2 + s.img_log2));
+    if (s.rows > 256 || patch > 49152) return false;
+    s.a_stage = (int)((patch + 1023) & ~1023ll);
+    s.tiles_per_img = (P + s.th - 1) / s.th;
+    s.m_tiles = (long long)((Nb + (1 << s.img_log2) - 1) >> s.img_log2) * s.tiles_per_img;
+    // Tile by whole waves: cycles per 32-channel step of a tap as the shared memory delivers its operands and takes the
+    // refills (measured near: single CTA 128 columns 92, 64 columns 60; pair 128 columns 66, 64 columns 50), plus the tile's
+    // fixed part and a cluster launch's.
+    double best = 0.0;
+    const int nbt = (L->C + bk - 1) / bk;
+    for (int cg = 2; cg >= 1; --cg)
+        for (int bn = 128; bn >= 64; bn -= 64) {
+            const int st = (kStageRegion - 2 * s.a_stage) / (L->S * (bn / cg) * bk);
+            if (st < 2) continue;
+            const long long tiles = (s.m_tiles + cg - 1) / cg * ((L->N + bn - 1) / bn), waves = (tiles + sms / cg - 1) / (sms / cg);
+            const double per = cg == 2 ? (bn == 128 ? 66.0 : 50.0) : (bn == 128 ? 92.0 : 60.0);
+            const double cost = (double)waves * ((double)nbt * L->R * L->S * (bk / 32) * per + 1200.0) + (cg == 2 ? 800.0 : 0.0);
+            if (best == 0.0 || cost < best) { best = cost; s.cg = cg; s.bn = bn; s.stages = st < kMaxStages ? st : kMaxStages; }
+        }
+    if (!s.bn) return false;
+    *out = s;
+    return true;
+}
+
 template <int CG, int PK, int KIND, bool SPLIT>
 static int launch_kernel(const CUtensorMap &a_lo, const CUtensorMap &a_hi, const CUtensorMap &b_lo, const CUtensorMap &b_hi,
                          const CUtensorMap &b_st, const CUtensorMap &y_map, const CUtensorMap &y_map16, const GemmParams &p, int sms, cudaStream_t st)
@@ -1621,15 +1803,26 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
             p.tiles_per_img = (p.P + th - 1) / th;
         }
     }
+    // Streamed patch mode: the other stride-1 filters
+    bool stream = false;
+    StreamPlan sp{};
+    if (!packed && !patch && !g_forced_tile.cg && p.im2col && L->stride == 1 && plan_stream(L, Nb, W, p.P, p.Q, p.BK, sms, &sp)) {
+        stream = true;
+        tc.cg = sp.cg; tc.bn = sp.bn;
+        p.pw_log2 = sp.pw_log2; p.img_log2 = sp.img_log2; p.TH = sp.th; p.patch_rows = sp.rows; p.tiles_per_img = sp.tiles_per_img;
+        p.nbt = p.nb_lo + p.nb_hi; p.a_stages = 2; p.a_stage = sp.a_stage;
+        p.patch_tx = (sp.rows << (sp.pw_log2 + sp.img_log2)) * p.BK;
+    }
     const int bn = tc.bn, cg = tc.cg;
     p.sx = x_shift ? x_shift : L->sx;
     p.sw = L->sw;
     p.G = L->G;
-    p.m_tiles = patch ? Nb * p.tiles_per_img : (int)((M + (long long)BM * cg - 1) / ((long long)BM * cg));
+    p.m_tiles = patch ? Nb * p.tiles_per_img : stream ? (int)((sp.m_tiles + cg - 1) / cg) : (int)((M + (long long)BM * cg - 1) / ((long long)BM * cg));
     p.BN = bn;
     p.n_tiles = (L->N + bn - 1) / bn;
     p.tps = 1;
-    if (!packed && !patch && p.im2col && L->C <= p.BK && L->S > 1) {
+    if (stream) p.tps = L->S;
+    if (!packed && !patch && !stream && p.im2col && L->C <= p.BK && L->S > 1) {
         // convolution whose channels fit one K block: a stage holds up to a filter row of taps
         const int per_tap = (BM + bn / cg) * p.BK;
         const int limit = 49152 / per_tap;
@@ -1637,7 +1830,7 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
         if (p.tps < 1) p.tps = 1;
     }
     p.stages = kStageRegion / (p.tps * (BM + bn / cg) * p.BK);
-    if (p.tps > 1 && p.n_tiles == 1) {
+    if (!stream && p.tps > 1 && p.n_tiles == 1) {
         const int b_all = ((p.T * (bn / cg) * p.BK + 1023) / 1024) * 1024;
         const int st = (kStageRegion - b_all) / (p.tps * BM * p.BK);
         if (b_all <= 65536 && st >= 4) { p.b_res = 1; p.stages = st; }
@@ -1646,6 +1839,7 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
         p.b_res = 1;
         p.stages = (kStageRegion - (((p.T * bn * p.BK) + 1023) & ~1023)) / p.patch_stage;
     }
+    if (stream) p.stages = sp.stages;
     if (p.stages > kMaxStages) p.stages = kMaxStages;
     if (packed) {  // room for the ring of raw 4-bit tiles behind the operand ring
         const int raw = kRawStages * (BM + bn) * (p.BK / 2);
@@ -1662,13 +1856,15 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
     const void *slab = packed_path ? static_cast<const void *>(X8) : static_cast<const void *>(X4);
     Layer::CallMaps &cm = L->call_maps;
     const bool cached = !packed && cm.slab == slab && cm.M == M && cm.Nb == Nb && cm.H == H && cm.W == W && cm.bk == p.BK &&
-                        cm.im2col == (int)p.im2col + 2 * (int)patch && (!staged || (cm.staged && cm.Y == Y && cm.y_elem == y_elem));
+                        cm.im2col == (int)p.im2col + 2 * (int)patch + 4 * (int)stream && (!staged || (cm.staged && cm.Y == Y && cm.y_elem == y_elem));
     if (cached) {
         a_lo = a_hi = cm.a;
     } else if (!packed) {
         // one int8 slab [rows][C] (a packed-path layer at ratio 0 has it in X8_dev)
         if (patch) {
             if ((rc = make_map_nhwc(&a_hi, slab, (uint64_t)L->C, W, H, Nb, p.BK, 1u << p.pw_log2, p.patch_rows, p.BK))) return rc;
+        } else if (stream) {
+            if ((rc = make_map_nhwc_by_row(&a_hi, slab, (uint64_t)L->C, W, H, Nb, p.BK, 1u << p.pw_log2, 1u << p.img_log2, p.patch_rows, p.BK))) return rc;
         } else if (p.im2col) {
             if ((rc = make_map_im2col(&a_hi, slab, L->C, L->C, Nb, H, W, L->R, L->S, L->stride, L->pad, p.BK, p.BK))) return rc;
         } else {
@@ -1704,6 +1900,13 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
         if ((y_elem > 1 || L->N >= 32) && (rc = make_map_nhwc(&y_map, Y, rb, p.Q, p.P, Nb, 32, bx, by, 32))) return rc;
         if (y_elem > 1) y_map16 = y_map;
         else if ((rc = make_map_nhwc(&y_map16, Y, rb, p.Q, p.P, Nb, 16, bx, by, 0))) return rc;
+    } else if (staged && stream) {
+        // a warp's 32 accumulator rows are bx pixels of bi images of by rows
+        const uint32_t pw = 1u << p.pw_log2, bx = pw < 32u ? pw : 32u, ni = 1u << p.img_log2, bi = ni < 32u / bx ? ni : 32u / bx, by = 32u / (bx * bi);
+        const uint64_t rb = (uint64_t)L->N * y_elem;
+        if ((y_elem > 1 || L->N >= 32) && (rc = make_map_nhwc_by_row(&y_map, Y, rb, p.Q, p.P, Nb, 32, bx, bi, by, 32))) return rc;
+        if (y_elem > 1) y_map16 = y_map;
+        else if ((rc = make_map_nhwc_by_row(&y_map16, Y, rb, p.Q, p.P, Nb, 16, bx, bi, by, 0))) return rc;
     } else if (staged && y_elem > 1) {
         // rows of N 2- or 4-byte values addressed in bytes: a box is 32 bytes (16 or 8 columns) x 32 rows
         if ((rc = make_map_2d(&y_map, Y, (uint64_t)L->N * y_elem, (uint64_t)M, (uint64_t)L->N * y_elem, 32, 32, 32))) return rc;
@@ -1713,7 +1916,7 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
         if ((rc = make_map_2d(&y_map16, Y, (uint64_t)L->N, (uint64_t)M, (uint64_t)L->N, 16, 32, 0))) return rc;
     }
     if (!packed && !cached) {
-        cm.slab = slab; cm.Y = staged ? Y : nullptr; cm.M = M; cm.Nb = Nb; cm.H = H; cm.W = W; cm.bk = p.BK; cm.im2col = (int)p.im2col + 2 * (int)patch;
+        cm.slab = slab; cm.Y = staged ? Y : nullptr; cm.M = M; cm.Nb = Nb; cm.H = H; cm.W = W; cm.bk = p.BK; cm.im2col = (int)p.im2col + 2 * (int)patch + 4 * (int)stream;
         cm.staged = staged; cm.y_elem = y_elem; cm.a = a_hi; cm.y = y_map; cm.y16 = y_map16;
     }
     // Early weight loads (see the kernel) are safe once some call on this handle has waited for whatever wrote the weights: this
@@ -1726,14 +1929,17 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
     // One narrow tile per CTA and a long K: nothing overlaps across tiles, so the MMA warps share the tile
     // (SPLIT).  With several tiles per CTA the warps already work side by side on tiles of their own, and the
     // second accumulator's extra read in the epilogue would only cost (measured: +4 to +6 % on short-K shapes).
-    const bool split = !packed && !patch && bn <= 128 && p.tps == 1 && p.T * (p.nb_lo + p.nb_hi) >= 8 &&
+    const bool split = !packed && !patch && !stream && bn <= 128 && p.tps == 1 && p.T * (p.nb_lo + p.nb_hi) >= 8 &&
                        (long long)p.m_tiles * p.n_tiles <= sms / cg;
     if (next) record_slab(const_cast<Layer *>(next), Y, next->K_lo);   // the fused boundary writes the next layer's slab at its current ratio
     if (packed) return launch_kernel<1, 1, 1, false>(a_lo, a_hi, L->map_w4[bi], L->map_w8[bi], L->map_w8[bi], y_map, y_map16, p, sms, st);
     // multi-tap stages hold every channel in one K block: the whole weight operand is one of the three forms
-    const bool one_block = p.tps > 1 || patch;   // every channel in one K block: the weight operand is one of the three forms as a whole
+    const bool one_block = (p.tps > 1 && !stream) || patch;   // every channel in one K block: the weight operand is one of the three forms as a whole
     const CUtensorMap &b_hi_map = one_block ? (b_whole == 0 ? L->map_w8[bi] : (b_whole == 1 ? L->map_w8m[bi] : L->map_wst[bi])) : L->map_w8[bi];
     if (one_block && b_whole == 2) p.b_tap_step = p.BK;
+    if (stream)
+        return cg == 2 ? launch_kernel<2, 0, 3, false>(a_lo, a_hi, L->map_w8m[bi], L->map_w8[bi], L->map_wst[bi], y_map, y_map16, p, sms, st)
+                       : launch_kernel<1, 0, 3, false>(a_lo, a_hi, L->map_w8m[bi], L->map_w8[bi], L->map_wst[bi], y_map, y_map16, p, sms, st);
     if (patch) return launch_kernel<1, 0, 2, false>(a_lo, a_hi, L->map_w8m[bi], b_hi_map, L->map_wst[bi], y_map, y_map16, p, sms, st);
 #define FLEXIQ_LAUNCH(CG_, KIND_, SPLIT_) launch_kernel<CG_, 0, KIND_, SPLIT_>(a_lo, a_hi, L->map_w8m[bi], b_hi_map, L->map_wst[bi], y_map, y_map16, p, sms, st)
     if (cg == 2) {

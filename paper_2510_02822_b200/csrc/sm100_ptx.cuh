@@ -130,11 +130,17 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap *m, uint32_t src,
 }
 // Tiled load of a 4-D box (channel bytes, x, y, image).  x, y and n may start outside the tensor
 // (negative or beyond the end): those elements arrive as zeros; c must keep the 16-byte rule.
+template <int CG>
 __device__ __forceinline__ void tma_load_4d_s(uint32_t dst, const CUtensorMap *m, uint32_t bar, int c, int x, int y, int n)
 {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c), "r"(x), "r"(y), "r"(n) : "memory");
+    if (CG == 2)
+        asm volatile(
+            "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+            ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c), "r"(x), "r"(y), "r"(n) : "memory");
+    else
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+            ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c), "r"(x), "r"(y), "r"(n) : "memory");
 }
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // all of this thread's bulk groups have finished reading their shared-memory source

@@ -35,3 +35,16 @@ def check(Nb, H, W, C, N, R, S, stride, pad, G, ratio):
 @pytest.mark.parametrize("shape", [(2, 12, 15, 64, 64, 3, 1, 1, 1, 16, 0.5), (1, 9, 31, 128, 48, 2, 2, 1, 2, 16, 0.5), (2, 5, 7, 48, 32, 3, 1, 1, 1, 16, 1.0)])
 def test_padding_wider_than_the_filter(shape):
     check(*shape)
+
+
+# channels beyond a K block or outputs beyond a tile, one and several images per grid row, ragged channels and rows, wide
+# images, one- and two-column filters, odd numbers of tiles (the pair's second tile outside)
+@pytest.mark.parametrize("shape", [
+    (2, 14, 14, 256, 64, 3, 3, 1, 1, 16, 0.5), (3, 7, 7, 512, 128, 3, 3, 1, 1, 16, 0.3), (1, 7, 7, 256, 64, 3, 3, 1, 1, 16, 1.0),
+    (5, 7, 7, 144, 144, 3, 3, 1, 1, 16, 0.5), (4, 4, 4, 256, 80, 3, 3, 1, 1, 16, 0.0), (9, 3, 3, 128, 160, 3, 3, 1, 1, 16, 0.5),
+    (2, 28, 28, 160, 48, 3, 3, 1, 1, 32, 0.25), (2, 30, 27, 144, 64, 3, 3, 1, 1, 16, 0.6), (1, 56, 56, 192, 32, 3, 3, 1, 1, 64, 0.4),
+    (2, 12, 15, 256, 64, 3, 1, 1, 1, 16, 0.5), (2, 12, 15, 256, 64, 1, 3, 1, 1, 16, 0.5), (3, 9, 5, 208, 96, 5, 3, 1, 2, 16, 0.5),
+    (1, 5, 90, 256, 16, 3, 3, 1, 1, 16, 0.5), (2, 16, 16, 64, 256, 3, 3, 1, 1, 16, 0.5), (7, 13, 8, 272, 272, 3, 3, 1, 0, 16, 0.7),
+    (33, 7, 7, 256, 64, 2, 2, 1, 1, 16, 0.5), (32, 14, 14, 256, 256, 3, 3, 1, 1, 16, 0.5), (31, 7, 7, 512, 512, 3, 3, 1, 1, 16, 0.25)])
+def test_streamed_patches(shape):
+    check(*shape)
