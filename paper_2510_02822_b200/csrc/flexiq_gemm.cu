@@ -731,8 +731,8 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
     const uint32_t buf_stride = BN <= 64 ? 64u : (BN <= 128 ? 128u : 256u);  // column offset from one accumulator to the next
     const uint32_t tmem_cols = ((SPLIT || kPatch) ? 4u : 2u) * buf_stride;
 
-    // The descriptors are fetched beside the rest of the preamble: a first copy waits for its map, 0.7 us each one after the other.
-    if (warp == 2 && lane < 6) {
+    // The descriptors are fetched beside the rest of the preamble (the plain kind's by its producer).
+    if (KIND != 0 && warp == 2 && lane < 6) {
         const CUtensorMap *m = lane == 0 ? &mapB_lo : lane == 1 ? &mapB_hi : lane == 2 ? &mapA_hi : lane == 3 ? &mapA_lo : lane == 4 ? &mapB_st : &mapY;
         ptx::prefetch_tmap(m);
     }
@@ -772,35 +772,37 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
     // Not for the im2col kind: in its producer loop the extra selections cost more than they save.
     // The second MMA warp, idle until then, issues the convolutions' copies, so that the producer is not late with the
     // activations (a copy takes the issuing lane about 0.1 us; 3x3 at 7 x 7: 13.2 us from the producer, 11.1 so); the one copy per
-    // stage of the plain kind stays with the producer (197 x 384 x 384: 5.0 us against 5.25).
+    // stage of the plain kind stays with the producer.  The tile walk's divisions are done here too (behind the wait they cost
+    // 0.15 us: 384 -> 384 at 197 rows 5.25 us, here 5.07).
     const int early_slots = KIND == 0 ? p.nb_lo + p.nb_hi : (kStream ? p.nbt * (p.T / p.S) : 0);
-    const bool early_on = !PK && p.early_w && first_tile < num_tiles;
-    const uint32_t early = early_on ? (uint32_t)(early_slots < p.stages ? early_slots : p.stages) : 0u;   // leading stages
-    if (early_on && warp == (KIND == 0 ? 0 : 2 + kNumWorkWarps)) {
-        const int n_blk = first_tile % p.n_tiles;
-        if (KIND != 0 && k_bres) {
-            if (p.early_st && ptx::elect_one()) load_resident();
-        } else if (kStream) {
-            if (ptx::elect_one()) {
-                int cb = 0, r = 0;
-                for (uint32_t i = 0; i < early; ++i) {
-                    stream_weights(n_blk * BN, cb, r, i, true, cb != p.st_cb || p.early_st);
-                    if (++r * p.S == p.T) { r = 0; ++cb; }
+    uint32_t early = 0;                               // leading stages whose transaction bytes and weight loads are issued
+    TileWalk ptw;                                     // the producer's walk
+    if (warp == 0) {
+        ptw.init(first_tile, tile_step, num_tiles, p.n_tiles);
+        if (!PK && p.early_w && ptw.left > 0) early = (uint32_t)(early_slots < p.stages ? early_slots : p.stages);
+        if (KIND == 0 && early && ptx::elect_one()) {
+            const uint32_t sb = ptx::smem_u32(stage_base) + (uint32_t)b_off, full0 = ptx::smem_u32(full_bar);
+            const uint32_t bar0 = CG == 2 ? ptx::mapa(full0, 0) : full0;
+            const int n0 = ptw.n_blk * BN + (int)cta_rank * b_rows;
+            for (uint32_t i = 0; i < early; ++i) {
+                if (leader) ptx::mbar_expect_tx_s(full0 + 8 * i, (uint32_t)(CG * (BM * p.BK + b_rows * p.BK)));
+                if ((int)i == p.st_cb) {
+                    if (p.early_st) ptx::tma_load_2d_s<CG>(sb + i * stage_bytes, &mapB_st, bar0 + 8 * i, 0, n0);
+                } else {
+                    ptx::tma_load_2d_s<CG>(sb + i * stage_bytes, (int)i < p.nb_lo ? &mapB_lo : &mapB_hi, bar0 + 8 * i, (int)i * p.BK, n0);
                 }
             }
-        } else if (KIND == 0) {
-            if (ptx::elect_one()) {
-                const uint32_t sb = ptx::smem_u32(stage_base) + (uint32_t)b_off, full0 = ptx::smem_u32(full_bar);
-                const uint32_t bar0 = CG == 2 ? ptx::mapa(full0, 0) : full0;
-                const int n0 = n_blk * BN + (int)cta_rank * b_rows;
-                for (uint32_t i = 0; i < early; ++i) {
-                    if (leader) ptx::mbar_expect_tx_s(full0 + 8 * i, (uint32_t)(CG * (BM * p.BK + b_rows * p.BK)));
-                    if ((int)i == p.st_cb) {
-                        if (p.early_st) ptx::tma_load_2d_s<CG>(sb + i * stage_bytes, &mapB_st, bar0 + 8 * i, 0, n0);
-                    } else {
-                        ptx::tma_load_2d_s<CG>(sb + i * stage_bytes, (int)i < p.nb_lo ? &mapB_lo : &mapB_hi, bar0 + 8 * i, (int)i * p.BK, n0);
-                    }
-                }
+        }
+        __syncwarp();
+    } else if (KIND != 0 && !PK && warp == 2 + kNumWorkWarps && p.early_w && first_tile < num_tiles) {
+        if (k_bres) {
+            if (p.early_st && ptx::elect_one()) load_resident();
+        } else if (kStream && ptx::elect_one()) {
+            const int n_blk = first_tile % p.n_tiles, last = early_slots < p.stages ? early_slots : p.stages;
+            int cb = 0, r = 0;
+            for (int i = 0; i < last; ++i) {
+                stream_weights(n_blk * BN, cb, r, (uint32_t)i, true, cb != p.st_cb || p.early_st);
+                if (++r * p.S == p.T) { r = 0; ++cb; }
             }
         }
         __syncwarp();
@@ -811,6 +813,13 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         // ------------------------------------------------------------- TMA producer
         // The whole warp walks the loops; one elected lane issues the copies.  K blocks run
         // low slab first (every tap, every channel block), then the high slab.
+        if (KIND == 0 && ptx::elect_one()) {
+            ptx::prefetch_tmap(&mapA_lo);
+            ptx::prefetch_tmap(&mapA_hi);
+            ptx::prefetch_tmap(&mapB_lo);
+            ptx::prefetch_tmap(&mapB_hi);
+            if (!PK && p.st_cb >= 0) ptx::prefetch_tmap(&mapB_st);
+        }
         const uint32_t tx_bytes = (uint32_t)(CG * (BM * p.BK + b_rows * p.BK));  // both CTAs' loads
         const uint32_t stage0 = ptx::smem_u32(stage_base) + (uint32_t)ring_off;
         const uint32_t empty0 = ptx::smem_u32(empty_bar);
@@ -824,8 +833,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         bool ok = true;
         PROF_DECL(prof_wait);
         PROF_T0(prof_start);
-        TileWalk tw;
-        tw.init(first_tile, tile_step, num_tiles, p.n_tiles);
+        TileWalk &tw = ptw;
         if (k_bres && !(p.early_w && p.early_st) && tw.left > 0 && ptx::elect_one()) load_resident();
         __syncwarp();
         // Output pixel (image, row, column) of this CTA's first row in the current tile, kept up to date by
