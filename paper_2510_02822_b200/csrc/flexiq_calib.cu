@@ -64,9 +64,25 @@ __global__ void calib_ranges_kernel(const void *__restrict__ X, long long M, int
             float lo_f[8], hi_f[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) { lo_f[k] = 0.f; hi_f[k] = 0.f; }
-            for (long long m = (long long)slice * 8 + rl; m < M; m += (long long)slices * 8) {
+            const long long step = (long long)slices * 8;
+            long long m = (long long)slice * 8 + rl;
+            const char *src = reinterpret_cast<const char *>(X) + ((size_t)m * K + c8) * 4;
+            const size_t stride = (size_t)step * K * 4;
+            for (; m + 3 * step < M; m += 4 * step, src += 4 * stride) {   // four rows in flight: 96 KB per SM
+                float x[4][8];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) load8(src + r * stride, x[r]);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        lo_f[k] = fminf(lo_f[k], x[r][k]);
+                        hi_f[k] = fmaxf(hi_f[k], x[r][k]);
+                    }
+            }
+            for (; m < M; m += step, src += stride) {
                 float x[8];
-                load8(reinterpret_cast<const char *>(X) + ((size_t)m * K + c8) * 4, x);
+                load8(src, x);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     lo_f[k] = fminf(lo_f[k], x[k]);
@@ -145,36 +161,101 @@ __global__ void calib_hist_kernel(const void *__restrict__ X, long long M, int K
 }
 
 // Range of a channel after dropping at most `tail` samples from each end of its histogram, widened to
-// contain zero (lo <= 0 <= hi).  tail = 0 gives the exact min / max.
+// contain zero (lo <= 0 <= hi).  tail = 0 gives the exact min / max.  One warp per channel, eight bins per lane: the
+// ends are where the running sums from either side first pass `tail` (a thread walking a channel's 256 bins one after the
+// other took 31 us whatever the number of channels).
 __global__ void ranges_from_hist_kernel(const unsigned *__restrict__ hist, int K, long long tail, int32_t *__restrict__ lo,
                                         int32_t *__restrict__ hi)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (c >= K) return;
-    const unsigned *h = hist + (size_t)c * 256;
-    long long below = 0, above = 0;
-    int l = -128, u = 127;
-    while (l < 0 && below + h[l + 128] <= tail) { below += h[l + 128]; ++l; }
-    while (u > 0 && above + h[u + 128] <= tail) { above += h[u + 128]; --u; }
-    lo[c] = l;
-    hi[c] = u;
+    const unsigned *h = hist + (size_t)c * 256 + 8 * lane;
+    unsigned n[8];
+    long long mine = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { n[i] = h[i]; mine += n[i]; }
+    long long up = mine, down = mine;   // inclusive sums over lanes, from the lowest bin up and from the highest down
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long a = __shfl_up_sync(0xffffffffu, up, o), b = __shfl_down_sync(0xffffffffu, down, o);
+        if (lane >= o) up += a;
+        if (lane + o < 32) down += b;
+    }
+    int l = 0, u = 0;                    // this lane's candidates; a bin at or beyond zero ends the search there
+    long long sum = up - mine;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        sum += n[i];
+        if (l == 0 && sum > tail) l = min(8 * lane + i - 128, 0);
+    }
+    sum = down - mine;
+#pragma unroll
+    for (int i = 7; i >= 0; --i) {
+        sum += n[i];
+        if (u == 0 && sum > tail) u = max(8 * lane + i - 128, 0);
+    }
+    l = __reduce_min_sync(0xffffffffu, l);
+    u = __reduce_max_sync(0xffffffffu, u);
+    if (lane == 0) { lo[c] = l; hi[c] = u; }
 }
 
-// Largest |w| over the output channels (and taps) of every input channel.
+// Largest |w| over the output channels (and taps) of every input channel, sixteen weights per load where the rows
+// allow it (16-byte alignment, a row length that is a multiple of 16), else one.  Byte loads alone took 9.5 us for 768 x 3072 and
+// 12 us for 256 x 3 x 3 x 256.
+__device__ __forceinline__ unsigned absmax4(unsigned best, unsigned w) { return __vmaxu4(best, __vabs4(w)); }   // |-128| = 128 as an unsigned byte
+__device__ __forceinline__ int max_byte(unsigned w)
+{
+    return (int)max(max(w & 0xffu, (w >> 8) & 0xffu), max((w >> 16) & 0xffu, w >> 24));
+}
 // Linear weights [K][N]: one warp per input channel (row).
+template <bool WIDE>
 __global__ void weight_absmax_rows_kernel(const int8_t *__restrict__ W, int K, int N, int32_t *__restrict__ wmax)
 {
     const int row = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (row >= K) return;
     const int8_t *w = W + (size_t)row * N;
     int best = 0;
-    for (int n = lane; n < N; n += 32) best = max(best, abs((int)w[n]));
+    if (WIDE) {
+        unsigned b4 = 0;
+#pragma unroll 4
+        for (int n = 16 * lane; n < N; n += 512) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(w + n));
+            b4 = absmax4(absmax4(absmax4(absmax4(b4, v.x), v.y), v.z), v.w);
+        }
+        best = max_byte(b4);
+    } else {
+        for (int n = lane; n < N; n += 32) best = max(best, abs((int)w[n]));
+    }
     best = __reduce_max_sync(0xffffffffu, best);
     if (lane == 0) wmax[row] = best;
 }
-// Convolution weights [rows = Cout*R*S][Cin]: a thread per input channel, rows split over blockIdx.y.
+// Convolution weights [rows = Cout*R*S][Cin]: a thread per input channel (or sixteen of them), rows split over blockIdx.y and
+// in the wide form over the block's sixteen row lanes.
+template <bool WIDE>
 __global__ void weight_absmax_cols_kernel(const int8_t *__restrict__ W, long long rows, int C, int32_t *__restrict__ wmax)
 {
+    if (WIDE) {
+        __shared__ int best_s[256];
+        best_s[threadIdx.x] = 0;
+        __syncthreads();
+        const int chunk = threadIdx.x & 15, c0 = (blockIdx.x * 16 + chunk) * 16;
+        if (c0 < C) {
+            unsigned b[4] = {0, 0, 0, 0};
+            for (long long r = (long long)blockIdx.y * 16 + (threadIdx.x >> 4); r < rows; r += (long long)gridDim.y * 16) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(W + (size_t)r * C + c0));
+                b[0] = absmax4(b[0], v.x); b[1] = absmax4(b[1], v.y); b[2] = absmax4(b[2], v.z); b[3] = absmax4(b[3], v.w);
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int v = (int)((b[i >> 2] >> (8 * (i & 3))) & 0xffu);
+                if (v) atomicMax(&best_s[chunk * 16 + i], v);
+            }
+        }
+        __syncthreads();
+        const int c = blockIdx.x * 256 + threadIdx.x;
+        if (c < C && best_s[threadIdx.x] > 0) atomicMax(&wmax[c], best_s[threadIdx.x]);
+        return;
+    }
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= C) return;
     int best = 0;
@@ -194,36 +275,59 @@ __device__ __forceinline__ int used_bits(int lo, int hi)  // magnitude bits a ra
 // (position of its widest channel), the group's error-estimation score (largest activation range x
 // largest weight range over its channels, Sec. 4.2), the greedy order (ascending score, ties by
 // index; rank counting, one block) and the histogram of channels by unused magnitude bits (0..4+).
-__global__ void calib_prepare_kernel(const int32_t *__restrict__ lo, const int32_t *__restrict__ hi,
+// SHARED: the scores and bit counts meet in shared memory, one thread per channel (up to kPrepareShared groups); without it
+// one thread walks a group's channels and the ranking reads the scores from global memory.
+constexpr int kPrepareShared = 2048;
+template <bool SHARED>
+__global__ void __launch_bounds__(1024) calib_prepare_kernel(const int32_t *__restrict__ lo, const int32_t *__restrict__ hi,
                                      const int32_t *__restrict__ wmax, int K, int G, int32_t *__restrict__ perm,
                                      uint8_t *__restrict__ x_shift, long long *score, int32_t *__restrict__ hist)
 {
     __shared__ int hist_s[5];
+    __shared__ unsigned long long score_s[SHARED ? kPrepareShared : 1];
+    __shared__ int bits_s[SHARED ? kPrepareShared : 1];
     const int n_g = K / G;
     if (threadIdx.x < 5) hist_s[threadIdx.x] = 0;
+    if (SHARED)
+        for (int g = threadIdx.x; g < n_g; g += blockDim.x) { score_s[g] = 0; bits_s[g] = 0; }
     __syncthreads();
-    for (int g = threadIdx.x; g < n_g; g += blockDim.x) {
-        int L = 0;
-        long long best = 0;
-        for (int i = 0; i < G; ++i) {
-            const int c = g * G + i;
-            L = max(L, used_bits(lo[c], hi[c]));
-            const long long r = max(hi[c], -lo[c]);
-            best = max(best, r * (long long)wmax[c]);
+    if (SHARED) {
+        for (int c = threadIdx.x; c < K; c += blockDim.x) {
+            const int l = lo[c], h = hi[c], L = used_bits(l, h);
+            const long long v = (long long)max(h, -l) * (long long)wmax[c];
+            if (L) atomicMax(&bits_s[c / G], L);
+            if (v > 0) atomicMax(&score_s[c / G], (unsigned long long)v);
+            atomicAdd(&hist_s[min(4, 7 - L)], 1);
         }
-        x_shift[g] = (uint8_t)(L > 3 ? L - 3 : 0);
-        score[g] = best;
+    } else {
+        for (int g = threadIdx.x; g < n_g; g += blockDim.x) {
+            int L = 0;
+            long long best = 0;
+            for (int i = 0; i < G; ++i) {
+                const int c = g * G + i;
+                L = max(L, used_bits(lo[c], hi[c]));
+                const long long r = max(hi[c], -lo[c]);
+                best = max(best, r * (long long)wmax[c]);
+            }
+            x_shift[g] = (uint8_t)(L > 3 ? L - 3 : 0);
+            score[g] = best;
+        }
+        for (int c = threadIdx.x; c < K; c += blockDim.x) atomicAdd(&hist_s[min(4, 7 - used_bits(lo[c], hi[c]))], 1);
     }
-    for (int c = threadIdx.x; c < K; c += blockDim.x) atomicAdd(&hist_s[min(4, 7 - used_bits(lo[c], hi[c]))], 1);
     __syncthreads();  // the scores are complete (global writes of this block are visible to it after the barrier)
     for (int g = threadIdx.x; g < n_g; g += blockDim.x) {
-        const long long s = score[g];
+        const long long s = SHARED ? (long long)score_s[g] : score[g];
         int rank = 0;
         for (int o = 0; o < n_g; ++o) {
-            const long long so = score[o];
+            const long long so = SHARED ? (long long)score_s[o] : score[o];
             rank += (so < s) || (so == s && o < g);
         }
         perm[rank] = g;
+        if (SHARED) {
+            const int L = bits_s[g];
+            x_shift[g] = (uint8_t)(L > 3 ? L - 3 : 0);
+            score[g] = s;
+        }
     }
     if (threadIdx.x < 5) hist[threadIdx.x] = hist_s[threadIdx.x];
 }
@@ -282,14 +386,15 @@ extern "C" int flexiq_calib_channel_ranges(const void *X_dev, int x_dtype, int64
     if (rc) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (!accumulate) {
-        FLEXIQ_CUDA_TRY(cudaMemsetAsync(lo_dev, 0, sizeof(int32_t) * K, st));
-        FLEXIQ_CUDA_TRY(cudaMemsetAsync(hi_dev, 0, sizeof(int32_t) * K, st));
+        const bool one = hi_dev == lo_dev + K;   // neighbours: one clear
+        FLEXIQ_CUDA_TRY(cudaMemsetAsync(lo_dev, 0, sizeof(int32_t) * K * (one ? 2 : 1), st));
+        if (!one) FLEXIQ_CUDA_TRY(cudaMemsetAsync(hi_dev, 0, sizeof(int32_t) * K, st));
     }
     if (M == 0) return FLEXIQ_OK;
     if (!X_dev || (reinterpret_cast<uintptr_t>(X_dev) & 15)) return set_error(FLEXIQ_ERR_INVALID_ARG, "X_dev is NULL or not 16-byte aligned");
-    int dev = 0, sms = 148;
+    int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sm_count(dev);
     switch (x_dtype) {
         case FLEXIQ_DTYPE_F32: return launch_ranges<FLEXIQ_DTYPE_F32>(X_dev, M, K, x_scale, lo_dev, hi_dev, sms, st);
         case FLEXIQ_DTYPE_F16: return launch_ranges<FLEXIQ_DTYPE_F16>(X_dev, M, K, x_scale, lo_dev, hi_dev, sms, st);
@@ -336,7 +441,7 @@ extern "C" int flexiq_calib_ranges_from_histogram(const uint32_t *hist_dev, int 
     if (!hist_dev || !lo_dev || !hi_dev) return set_error(FLEXIQ_ERR_INVALID_ARG, "a device pointer is NULL");
     int rc = check_device_sm100();
     if (rc) return rc;
-    ranges_from_hist_kernel<<<(K + 127) / 128, 128, 0, reinterpret_cast<cudaStream_t>(stream)>>>(hist_dev, K, (long long)tail, lo_dev, hi_dev);
+    ranges_from_hist_kernel<<<(K + 3) / 4, 128, 0, reinterpret_cast<cudaStream_t>(stream)>>>(hist_dev, K, (long long)tail, lo_dev, hi_dev);
     FLEXIQ_CUDA_TRY(cudaGetLastError());
     return FLEXIQ_OK;
 }
@@ -349,13 +454,20 @@ extern "C" int flexiq_calib_weight_absmax(const int8_t *Wq_dev, int is_conv, int
     if (rc) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     if (!is_conv) {
-        const long long threads = (long long)K * 32;
-        weight_absmax_rows_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(Wq_dev, K, N, wmax_dev);
+        const unsigned blocks = (unsigned)(((long long)K * 32 + 127) / 128);
+        if (N % 16 == 0 && (reinterpret_cast<uintptr_t>(Wq_dev) & 15) == 0) weight_absmax_rows_kernel<true><<<blocks, 128, 0, st>>>(Wq_dev, K, N, wmax_dev);
+        else weight_absmax_rows_kernel<false><<<blocks, 128, 0, st>>>(Wq_dev, K, N, wmax_dev);
     } else {
         FLEXIQ_CUDA_TRY(cudaMemsetAsync(wmax_dev, 0, sizeof(int32_t) * K, st));
         const long long rows = (long long)N * taps;
-        const unsigned gy = (unsigned)(rows < 64 ? rows : 64);
-        weight_absmax_cols_kernel<<<dim3((K + 127) / 128, gy), 128, 0, st>>>(Wq_dev, rows, K, wmax_dev);
+        if (K % 16 == 0 && (reinterpret_cast<uintptr_t>(Wq_dev) & 15) == 0) {
+            const unsigned gx = (unsigned)((K + 255) / 256), most = gx < 296 ? 296 / gx : 1;   // four rows a lane, two blocks per SM
+            const long long want = (rows + 63) / 64;
+            weight_absmax_cols_kernel<true><<<dim3(gx, want < (long long)most ? (unsigned)want : most), 256, 0, st>>>(Wq_dev, rows, K, wmax_dev);
+        } else {
+            const unsigned gy = (unsigned)(rows < 64 ? rows : 64);
+            weight_absmax_cols_kernel<false><<<dim3((K + 127) / 128, gy), 128, 0, st>>>(Wq_dev, rows, K, wmax_dev);
+        }
     }
     FLEXIQ_CUDA_TRY(cudaGetLastError());
     return FLEXIQ_OK;
@@ -372,8 +484,10 @@ extern "C" int flexiq_calib_prepare(const int32_t *lo_dev, const int32_t *hi_dev
         return set_error(FLEXIQ_ERR_INVALID_ARG, "a device pointer is NULL");
     int rc = check_device_sm100();
     if (rc) return rc;
-    calib_prepare_kernel<<<1, 1024, 0, reinterpret_cast<cudaStream_t>(stream)>>>(lo_dev, hi_dev, wmax_dev, K, group_size, perm_dev, x_shift_dev,
-                                                                                 reinterpret_cast<long long *>(score_dev), unused_hist_dev);
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    long long *score = reinterpret_cast<long long *>(score_dev);
+    if (K / group_size <= kPrepareShared) calib_prepare_kernel<true><<<1, 1024, 0, st>>>(lo_dev, hi_dev, wmax_dev, K, group_size, perm_dev, x_shift_dev, score, unused_hist_dev);
+    else calib_prepare_kernel<false><<<1, 1024, 0, st>>>(lo_dev, hi_dev, wmax_dev, K, group_size, perm_dev, x_shift_dev, score, unused_hist_dev);
     FLEXIQ_CUDA_TRY(cudaGetLastError());
     return FLEXIQ_OK;
 }

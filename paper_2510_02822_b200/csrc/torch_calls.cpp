@@ -430,7 +430,8 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
         const long long rows = X.size(0), C = X.size(1), n_g = C / G, step = (rows + batches - 1) / batches;
         if (C < 1 || C > INT32_MAX || n_g < 1) throw Refused{};
         const at::TensorOptions opt = at::TensorOptions().device(X.device());
-        const at::Tensor lo = at::empty({C}, opt.dtype(at::kInt)), hi = at::empty({C}, opt.dtype(at::kInt)), wmax = at::empty({C}, opt.dtype(at::kInt));
+        const at::Tensor ranges = at::empty({2, C}, opt.dtype(at::kInt)), lo = ranges.select(0, 0), hi = ranges.select(0, 1);   // neighbours: one clear
+        const at::Tensor wmax = at::empty({C}, opt.dtype(at::kInt));
         const at::Tensor order = at::empty({5 * n_g}, opt.dtype(at::kByte));   // perm int32 [n_g], then x_shift [n_g]: one copy to the host
         const at::Tensor score = at::empty({n_g}, opt.dtype(at::kLong)), unused = at::empty({5}, opt.dtype(at::kInt));
         at::Tensor hist;

@@ -124,3 +124,38 @@ def test_front_end_with_coverage(dev):
     assert np.array_equal(xs, oracle.static_positions(lo, hi, case.G))
     perm_e, _ = oracle.greedy_order(lo, hi, oracle.weight_absmax_linear(case.Wq), case.G)
     assert np.array_equal(perm, perm_e)
+
+
+@pytest.mark.parametrize("K, N, taps, offset", [(16, 1, 0, 0), (48, 17, 0, 0), (33, 512, 0, 0), (70, 528, 0, 1), (768, 3072, 0, 0),
+                                                (16, 1, 9, 0), (272, 48, 9, 0), (260, 32, 1, 0), (512, 130, 9, 4), (4096, 3, 1, 0)])
+def test_weight_ranges_wide_and_byte_loads(dev, K, N, taps, offset):
+    """Rows that allow 16-byte loads and rows that do not (odd lengths, odd addresses), -128 among the weights."""
+    shape = (N, taps, K) if taps else (K, N)
+    w = ((inputs.uniform(77, K, int(np.prod(shape))) * 256).astype(np.int64) - 128).astype(np.int8)
+    w = (w >> (np.arange(w.size) % 5)).astype(np.int8)
+    w[-1] = -128
+    raw = torch.empty(w.size + 16, dtype=torch.int8, device=dev)
+    W = raw[offset:offset + w.size]
+    W.copy_(torch.from_numpy(w))
+    wmax = torch.full((K,), -1, dtype=torch.int32, device=dev)
+    fx.flexiq_calib_weight_absmax(W, bool(taps), K, N, max(taps, 1), wmax)
+    ref = np.abs(w.astype(np.int32).reshape(shape)).max(axis=(0, 1) if taps else 1)
+    assert np.array_equal(wmax.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("K, G", [(16, 16), (2048 * 16, 16), (2049 * 16, 16), (4096, 64)])
+def test_prepare_few_and_many_groups(dev, K, G):
+    """Group scores and order where they meet in shared memory and where they do not, ties included."""
+    lo = -(inputs.uniform(78, 0, K) * 129).astype(np.int32)
+    hi = (inputs.uniform(78, 1, K) * 128).astype(np.int32)
+    wm = (inputs.uniform(78, 2, K) * 3).astype(np.int32)
+    t = [torch.from_numpy(a).to(dev) for a in (lo, hi, wm)]
+    n_g = K // G
+    perm, xs = torch.empty(n_g, dtype=torch.int32, device=dev), torch.empty(n_g, dtype=torch.uint8, device=dev)
+    score, hist = torch.empty(n_g, dtype=torch.int64, device=dev), torch.empty(5, dtype=torch.int32, device=dev)
+    fx.flexiq_calib_prepare(*t, K, G, perm, xs, score, hist)
+    ref = (np.maximum(hi, -lo).astype(np.int64) * wm).reshape(n_g, G).max(1)
+    assert np.array_equal(score.cpu().numpy(), ref)
+    assert np.array_equal(perm.cpu().numpy(), np.argsort(ref, kind="stable"))
+    assert np.array_equal(xs.cpu().numpy(), oracle.static_positions(lo, hi, G))
+    assert np.array_equal(hist.cpu().numpy(), oracle.unused_bits_histogram(lo, hi))
