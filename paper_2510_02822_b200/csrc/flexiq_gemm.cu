@@ -651,7 +651,8 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
 // PK = 1 (single CTA only): the low slab arrives as packed 4-bit tiles; eight expander warps
 // widen them into the operand ring (eight epilogue warps remain).
 // KIND 0: linear layers and 1x1 convolutions (plain 2-D copies, one K block per stage); KIND 1: everything a
-// convolution may need (im2col copies, several taps per stage, resident weight tiles).  The issuing warps'
+// convolution may need (im2col copies, several taps per stage, resident weight tiles); KIND 2 and 3: halo patches, whole or
+// streamed per K block (see GemmParams).  The issuing warps'
 // instruction streams are on the critical path of a tile, so the first kind carries none of the second's code.
 // SPLIT (tiles of at most 128 columns, one K block per stage, at least two stages per tile): the two MMA warps
 // take the ring's stages in turn INSIDE a tile, each into an accumulator of its own, and the epilogue adds the
