@@ -327,6 +327,109 @@ __global__ void lower_inplace_kernel(int8_t *__restrict__ slab, long long M, int
     }
 }
 
+// Dynamic mode in one launch.  A cluster of eight CTAs owns a window of slab chunks (whole groups), each CTA an eighth of the
+// rows: it quantizes its part of the columns into shared memory, the CTAs read one another's OR words through
+// distributed shared memory, and each lowers and writes what it holds.  The input is read once, the slab written once, and
+// nothing is cleared beforehand or read back: 197 x 384 fp16 8.3 -> 3.3 us, 1576 x 1536 fp32 12.4 -> 9.0, 6304 x 768 fp16 14.4 -> 9.4 (graph
+// replay, against a clear and two launches).
+// The window is 32 bytes of a slab row (64 for groups of 64), so that a row's stores are whole sectors.
+constexpr int kColCluster = 8;
+constexpr int kColThreads = 256;
+constexpr int kColSmem = 102400;   // quantized rows a CTA may hold: two CTAs per SM
+
+struct ColumnsArgs {
+    const void *X;
+    int8_t *slab;
+    long long M;
+    int K, G, K_lo;
+    int window, rows;          // chunks per cluster, rows per CTA
+    float S;
+    QuotientPlan quot;
+    const int32_t *perm;
+    uint8_t *sx_out;
+    StraddleJob wp;
+};
+
+template <int DTYPE>
+__global__ void __launch_bounds__(kColThreads) dynamic_columns_kernel(const __grid_constant__ ColumnsArgs a)
+{
+    constexpr int kBytes = DTYPE == FLEXIQ_DTYPE_F32 ? 4 : (DTYPE == FLEXIQ_DTYPE_I8 ? 1 : 2);
+    constexpr int kPieces = kBytes, kAhead = DTYPE == FLEXIQ_DTYPE_F32 ? 2 : 4;   // rows in flight per thread
+    extern __shared__ __align__(128) uint8_t cols_smem[];
+    __shared__ unsigned or_s[4], all_s[4];
+    uint4 *held = reinterpret_cast<uint4 *>(cols_smem);
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
+    if (blockIdx.x < a.wp.first_block) {   // whole clusters: the straddle block of the weights
+        const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (idx < (long long)a.wp.rows * (a.wp.BK >> 4)) straddle_write_unit(a.wp, idx);
+        return;
+    }
+    const int n_c16 = a.K / 16, cpg = a.G / 16;
+    const int rank = (int)ptx::cluster_ctarank(), first = (int)((blockIdx.x - a.wp.first_block) / kColCluster) * a.window;
+    const int cl = threadIdx.x % a.window, c = first + cl, j = c / cpg;
+    const bool live = c < n_c16;
+    const int r0 = threadIdx.x / a.window, step = kColThreads / a.window;
+    const long long m_first = (long long)rank * a.rows;
+    const int rows = (int)max(0ll, min((long long)a.rows, a.M - m_first));
+    if (threadIdx.x < 4) { or_s[threadIdx.x] = 0; all_s[threadIdx.x] = 0; }
+    __syncthreads();
+    if (live) {
+        const size_t row_bytes = (size_t)a.K * kBytes;
+        const char *src = reinterpret_cast<const char *>(a.X) + (size_t)(m_first + r0) * row_bytes + ((size_t)__ldg(a.perm + j) * a.G + (c % cpg) * 16) * kBytes;
+        unsigned o = 0;
+        for (int r = r0; r < rows; r += kAhead * step, src += (size_t)(kAhead * step) * row_bytes) {
+            uint4 raw[kAhead][kPieces];
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i)
+                if (r + i * step < rows) {
+#pragma unroll
+                    for (int p = 0; p < kPieces; ++p) raw[i][p] = __ldg(reinterpret_cast<const uint4 *>(src + (size_t)(i * step) * row_bytes) + p);
+                }
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i)
+                if (r + i * step < rows) {
+                    unsigned w[4];
+                    if constexpr (DTYPE == FLEXIQ_DTYPE_I8) {
+                        w[0] = raw[i][0].x; w[1] = raw[i][0].y; w[2] = raw[i][0].z; w[3] = raw[i][0].w;
+                    } else if (a.quot.form == kQuotGeneral) {
+                        quantize_raw<DTYPE>(raw[i], make_divider(a.S), -128.f, 127.f, w);
+                    } else if constexpr (DTYPE == FLEXIQ_DTYPE_F32) {
+                        quantize_raw<DTYPE>(raw[i], TwoTerm{a.quot.r_hi, a.quot.r_lo}, -128.f, 127.f, w);
+                    } else {
+                        quantize_raw_magic<DTYPE>(raw[i], a.quot.r_hi, -128.f, 127.f, w);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {   // fold negatives per byte
+                        unsigned sign;
+                        asm("prmt.b32 %0, %1, 0, 0xba98;" : "=r"(sign) : "r"(w[k]));
+                        o |= w[k] ^ sign;
+                    }
+                    held[(r + i * step) * a.window + cl] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+        }
+        o |= o >> 16;
+        o = (o | (o >> 8)) & 0xffu;
+        if (o) atomicOr(&or_s[cl], o);
+    }
+    ptx::cluster_sync_all();       // every CTA's OR words are complete
+    if ((int)threadIdx.x < kColCluster * a.window) {
+        const unsigned o = ptx::ld_shared_cluster(ptx::mapa(ptx::smem_u32(&or_s[threadIdx.x % a.window]), threadIdx.x / a.window));
+        if (o) atomicOr(&all_s[threadIdx.x % a.window], o);
+    }
+    ptx::cluster_sync_all();       // and read: a CTA may leave
+    unsigned o = 0;
+    for (int i = 0; i < cpg; ++i) o |= all_s[cl / cpg * cpg + i];
+    const int s = position_from_or(o);
+    if (!live) return;
+    if (rank == 0 && r0 == 0 && c % cpg == 0) a.sx_out[j] = (uint8_t)s;
+    const unsigned mask = c < a.K_lo / 16 ? ((0xffu << s) & 0xffu) * 0x01010101u : 0xffffffffu;
+    for (int r = r0; r < rows; r += step) {
+        const uint4 v = held[r * a.window + cl];
+        *reinterpret_cast<uint4 *>(a.slab + (size_t)(m_first + r) * a.K + (size_t)c * 16) = make_uint4(v.x & mask, v.y & mask, v.z & mask, v.w & mask);
+    }
+}
+
 // Packed path, and the masked path's rows that are too wide for the ring: quantize + lower + gather.  Thread <-> (row m,
 // 16-channel slab chunk c16).
 //   sx != nullptr : static positions (slab order);  else positions from or_words.
@@ -485,6 +588,56 @@ static int launch_rows(Layer *L, const void *X, long long M, float S, int8_t *sl
     return FLEXIQ_OK;
 }
 
+// Does the one-launch dynamic kernel take M rows of this layer?  (rows per CTA, chunks per cluster)  The line lies where its columns'
+// short pieces (a chunk of each row at a time, rows far apart) begin to cost more than the two phases' launches: at 9.7 MB of
+// fp32, 1576 rows take 9.0 us against 12.4, 3152 10.5, 6304 12.1 and 12,608 17.9; 38.7 MB of fp16 in 6304 rows take 24, 77 MB 47 against 39.
+constexpr long long kColBytes = 10ll << 20, kColRows = 6144;   // of input; rows
+static bool columns_fit(const Layer *L, long long M, int elem, int *rows, int *window)
+{
+    if (M > kColRows || M * L->C * elem > kColBytes) return false;
+    *window = L->G == 64 ? 4 : 2;
+    const long long r = (M + kColCluster - 1) / kColCluster;
+    *rows = (int)(r < 1000000 ? r : 1000000);
+    return r * *window * 16 <= kColSmem;
+}
+
+template <int DTYPE>
+static int launch_columns(Layer *L, const void *X, long long M, float S, int8_t *slab, uint8_t *sx_out, const StraddleJob &job, int rows, int window, cudaStream_t st)
+{
+    ColumnsArgs a{};
+    a.X = X; a.slab = slab; a.M = M; a.K = L->C; a.G = L->G; a.K_lo = L->K_lo;
+    a.window = window; a.rows = rows;
+    a.S = S;
+    a.quot = quotient_plan(S, DTYPE);
+    a.perm = L->perm; a.sx_out = sx_out;
+    a.wp = job;
+    long long extra = job.wst ? ((long long)job.rows * (job.BK >> 4) + kColThreads - 1) / kColThreads : 0;
+    extra = (extra + kColCluster - 1) / kColCluster * kColCluster;   // whole clusters
+    a.wp.first_block = (unsigned)extra;
+    const size_t smem = (size_t)rows * window * 16;
+    static bool attr_set[64] = {};   // per instantiation
+    if (smem > 48 * 1024 - 64 && (L->device >= 64 || !attr_set[L->device])) {
+        FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(dynamic_columns_kernel<DTYPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kColSmem));
+        if (L->device < 64) attr_set[L->device] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(extra + (long long)((L->C / 16 + window - 1) / window) * kColCluster), 1, 1);
+    cfg.blockDim = dim3(kColThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kColCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    FLEXIQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, dynamic_columns_kernel<DTYPE>, a));
+    return FLEXIQ_OK;
+}
+
 template <int DTYPE>
 static int launch_prologue(Layer *L, const void *X, long long M, float S, int dynamic, uint8_t *X4,
                            long long pitch, int8_t *X8, long long pitch8, uint8_t *sx_out, unsigned *scratch, cudaStream_t st)
@@ -495,8 +648,10 @@ static int launch_prologue(Layer *L, const void *X, long long M, float S, int dy
     const int threads = 256;
     const bool masked = L->lowbit_path == FLEXIQ_LOWBIT_MASKED_I8;
     constexpr size_t elem = DTYPE == FLEXIQ_DTYPE_F32 ? 4 : (DTYPE == FLEXIQ_DTYPE_I8 ? 1 : 2);
-    if (dynamic) FLEXIQ_CUDA_TRY(cudaMemsetAsync(scratch, 0, sizeof(unsigned) * L->n_g, st));
-    if (masked && (size_t)K * elem <= kRowStageBytes) {
+    int col_rows = 0, col_window = 0;
+    const bool columns = dynamic && masked && columns_fit(L, M, (int)elem, &col_rows, &col_window);
+    if (dynamic && !columns) FLEXIQ_CUDA_TRY(cudaMemsetAsync(scratch, 0, sizeof(unsigned) * L->n_g, st));
+    if (masked && (columns || (size_t)K * elem <= kRowStageBytes)) {
         StraddleJob job{};
         if (straddle_in_use(L) && straddle_stale(L, st)) {
             // the GEMM that consumes these slabs reads the straddle block of the same max_4bit_ch
@@ -509,7 +664,8 @@ static int launch_prologue(Layer *L, const void *X, long long M, float S, int dy
         }
         int8_t *slab = reinterpret_cast<int8_t *>(X4);
         int rc;
-        if (!dynamic) rc = launch_rows<DTYPE, false>(L, X, M, S, slab, nullptr, job, st);
+        if (columns) rc = launch_columns<DTYPE>(L, X, M, S, slab, sx_out, job, col_rows, col_window, st);
+        else if (!dynamic) rc = launch_rows<DTYPE, false>(L, X, M, S, slab, nullptr, job, st);
         else {
             // the input is read once: phase 1 quantizes, gathers and collects the OR words, phase 2 lowers the low groups of
             // the slab in place (from L2) with the positions those words give

@@ -72,10 +72,10 @@ def test_fp32_next_to_every_boundary():
 
 
 # rows x channels: one row, one chunk, fewer tiles than SMs, ragged last tiles, rows of one chunk per thread and of many, the widest
-# rows of the ring for each type (65,536 bytes) and wider ones
+# rows of the ring for each type (65,536 bytes) and wider ones; rows beyond what the one-launch dynamic kernel holds
 @pytest.mark.parametrize("kind", ["f32", "f16", "bf16", "i8"])
 @pytest.mark.parametrize("M, K, G", [(1, 16, 16), (3, 144, 16), (197, 384, 32), (5000, 64, 64), (2111, 1360, 16), (2200, 1216, 64),
-                                     (9001, 96, 32), (333, 4112, 16), (151, 16384, 64), (2, 65536, 32), (2, 132000, 32)])
+                                     (9001, 96, 32), (26001, 32, 16), (13000, 64, 64), (333, 4112, 16), (151, 16384, 64), (2, 65536, 32), (2, 132000, 32)])
 def test_slab_matches_oracle(kind, M, K, G):
     n_g = K // G
     perm = np.argsort(inputs.uniform(11, K, n_g), kind="stable").astype(np.int32)
