@@ -335,7 +335,8 @@ __global__ void lower_inplace_kernel(int8_t *__restrict__ slab, long long M, int
 // The window is 32 bytes of a slab row (64 for groups of 64), so that a row's stores are whole sectors.
 constexpr int kColCluster = 8;
 constexpr int kColThreads = 256;
-constexpr int kColSmem = 102400;   // quantized rows a CTA may hold: two CTAs per SM
+constexpr long long kColBytes = 10ll << 20, kColRows = 6144;   // of input, rows: the largest calls it takes (see columns_fit)
+constexpr int kColSmem = (int)(kColRows / kColCluster) * 4 * 16;   // the quantized rows a CTA then holds, windows of four chunks
 
 struct ColumnsArgs {
     const void *X;
@@ -579,8 +580,8 @@ static int launch_rows(Layer *L, const void *X, long long M, float S, int8_t *sl
     const int threads = 32 * (warps + 1);
     const unsigned extra = job.wst ? (unsigned)(((long long)job.rows * (job.BK >> 4) + threads - 1) / threads) : 0u;
     a.wp.first_block = extra;   // the straddle blocks come first
-    static bool attr_set[64] = {};   // per instantiation
-    if (smem > 48 * 1024 && (L->device >= 64 || !attr_set[L->device])) {
+    static bool attr_set[64] = {};   // per instantiation, whatever the size: the 48 KB default covers the static part too
+    if (L->device >= 64 || !attr_set[L->device]) {
         FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(quantize_rows_kernel<DTYPE, DYN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem));
         if (L->device < 64) attr_set[L->device] = true;
     }
@@ -591,14 +592,12 @@ static int launch_rows(Layer *L, const void *X, long long M, float S, int8_t *sl
 // Does the one-launch dynamic kernel take M rows of this layer?  (rows per CTA, chunks per cluster)  The line lies where its columns'
 // short pieces (a chunk of each row at a time, rows far apart) begin to cost more than the two phases' launches: at 9.7 MB of
 // fp32, 1576 rows take 9.0 us against 12.4, 3152 10.5, 6304 12.1 and 12,608 17.9; 38.7 MB of fp16 in 6304 rows take 24, 77 MB 47 against 39.
-constexpr long long kColBytes = 10ll << 20, kColRows = 6144;   // of input; rows
 static bool columns_fit(const Layer *L, long long M, int elem, int *rows, int *window)
 {
     if (M > kColRows || M * L->C * elem > kColBytes) return false;
     *window = L->G == 64 ? 4 : 2;
-    const long long r = (M + kColCluster - 1) / kColCluster;
-    *rows = (int)(r < 1000000 ? r : 1000000);
-    return r * *window * 16 <= kColSmem;
+    *rows = (int)((M + kColCluster - 1) / kColCluster);
+    return true;
 }
 
 template <int DTYPE>
@@ -615,8 +614,8 @@ static int launch_columns(Layer *L, const void *X, long long M, float S, int8_t 
     extra = (extra + kColCluster - 1) / kColCluster * kColCluster;   // whole clusters
     a.wp.first_block = (unsigned)extra;
     const size_t smem = (size_t)rows * window * 16;
-    static bool attr_set[64] = {};   // per instantiation
-    if (smem > 48 * 1024 - 64 && (L->device >= 64 || !attr_set[L->device])) {
+    static bool attr_set[64] = {};   // per instantiation, as above
+    if (L->device >= 64 || !attr_set[L->device]) {
         FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(dynamic_columns_kernel<DTYPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kColSmem));
         if (L->device < 64) attr_set[L->device] = true;
     }
