@@ -436,6 +436,11 @@ int flexiq_choose_tile(int64_t M, int N, int k_blocks, int block_k, int sm_count
  * stays usable).  Nothing traps and nothing spins without bound.  The paper has no counterpart. */
 int flexiq_selftest_wait_expiry(int *result_dev, void *stream);
 
+/* Test hook, host-only: which weights the handle's last mixed_* call requested ahead of its wait for the kernel before it:
+ * *weights for the blocks of the two resident forms, *straddle for the block that max_4bit_ch falls into (1 = ahead;
+ * where no block does, that one follows *weights).  The paper has no counterpart. */
+int flexiq_layer_early_loads(flexiq_layer_t layer, int *weights, int *straddle);
+
 /* Reads and clears the device status word raised by a bounded wait that expired.
  * Synchronises `stream`. */
 int flexiq_check_status(void *stream);

@@ -30,7 +30,7 @@ EXPORTS = [
     "flexiq_calib_weight_absmax", "flexiq_calib_prepare", "flexiq_calib_absmax_ema",
     "flexiq_controller_create", "flexiq_controller_destroy", "flexiq_controller_level", "flexiq_controller_update",
     "flexiq_serving_simulate", "flexiq_evo_init", "flexiq_evo_next_generation", "flexiq_sq_distance_i8",
-    "flexiq_layer_export", "flexiq_selftest_wait_expiry", "flexiq_force_tile", "flexiq_choose_tile", "flexiq_check_status", "flexiq_last_error",
+    "flexiq_layer_export", "flexiq_layer_early_loads", "flexiq_selftest_wait_expiry", "flexiq_force_tile", "flexiq_choose_tile", "flexiq_check_status", "flexiq_last_error",
 ]
 
 _lib = None
@@ -77,6 +77,7 @@ def lib():
         L.flexiq_calib_prepare.argtypes = [vp, vp, vp, i32, i32, vp, vp, vp, vp, vp]
         L.flexiq_calib_absmax_ema.argtypes = [vp, i32, i64, f32, vp, vp]
         L.flexiq_layer_export.argtypes = [vp, vp, vp, vp]
+        L.flexiq_layer_early_loads.argtypes = [vp, C.POINTER(i32), C.POINTER(i32)]
         L.flexiq_check_status.argtypes = [vp]
         L.flexiq_selftest_wait_expiry.argtypes = [vp, vp]
         f64 = C.c_double
@@ -249,6 +250,13 @@ def flexiq_layer_export(h, sw_host=None, w8_host=None, w4_host=None):
     def hp(a):
         return None if a is None else a.ctypes.data_as(C.c_void_p)
     _check(lib().flexiq_layer_export(h, hp(sw_host), hp(w8_host), hp(w4_host)))
+
+
+def flexiq_layer_early_loads(h):
+    """(weights, straddle block): what the handle's last mixed_* call requested ahead of its dependency wait."""
+    w, s = C.c_int(), C.c_int()
+    _check(lib().flexiq_layer_early_loads(h, C.byref(w), C.byref(s)))
+    return bool(w.value), bool(s.value)
 
 
 def flexiq_force_tile(cta_group, tile_n):

@@ -1928,11 +1928,17 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
         cm.slab = slab; cm.Y = staged ? Y : nullptr; cm.M = M; cm.Nb = Nb; cm.H = H; cm.W = W; cm.bk = p.BK; cm.im2col = (int)p.im2col + 2 * (int)patch + 4 * (int)stream;
         cm.staged = staged; cm.y_elem = y_elem; cm.a = a_hi; cm.y = y_map; cm.y16 = y_map16;
     }
-    // Early weight loads (see the kernel) are safe once some call on this handle has waited for whatever wrote the weights: this
-    // call's launches do, so the next may.  In a capture, or when one has written the straddle block, it is always late.
-    p.early_w = !L->weights_fresh;
-    p.early_st = p.st_cb < 0 || (!L->st_fresh && !L->st_graph_seen && stream_capture_id(st) == 0);
-    L->weights_fresh = L->st_fresh = 0;
+    // Early weight loads (see the kernel) are safe once some launch on this handle has waited for whatever wrote the weights: this
+    // call's does, so the next may.  A captured call waits only within its own graph, which as a whole starts behind what the
+    // stream held before it: it answers for a layout of the same capture and leaves the marks of eager writes alone.  Once
+    // a layout has been captured, eager calls are always late; the straddle block is early neither in a capture nor after one
+    // that has written it.
+    const bool marked = L->weights_fresh || L->st_fresh || L->weights_graph_seen || p.st_cb >= 0;
+    const unsigned long long cap = marked ? stream_capture_id(st) : 0;
+    p.early_w = !L->weights_fresh && (cap ? L->weights_cap_id != cap : !L->weights_graph_seen);
+    p.early_st = p.st_cb < 0 || (!L->st_fresh && !L->st_graph_seen && cap == 0);
+    L->early_w = p.early_w;
+    L->early_st = p.early_w && p.early_st;
     const int bi = weight_map_index(bn / cg);  // box rows = the B rows one CTA loads
     const bool conv_kind = p.im2col || p.tps > 1 || p.b_res;
     // One narrow tile per CTA and a long K: nothing overlaps across tiles, so the MMA warps share the tile
@@ -1941,23 +1947,31 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
     const bool split = !packed && !patch && !stream && bn <= 128 && p.tps == 1 && p.T * (p.nb_lo + p.nb_hi) >= 8 &&
                        (long long)p.m_tiles * p.n_tiles <= sms / cg;
     if (next) record_slab(const_cast<Layer *>(next), Y, next->K_lo);   // the fused boundary writes the next layer's slab at its current ratio
-    if (packed) return launch_kernel<1, 1, 1, false>(a_lo, a_hi, L->map_w4[bi], L->map_w8[bi], L->map_w8[bi], y_map, y_map16, p, sms, st);
-    // multi-tap stages hold every channel in one K block: the whole weight operand is one of the three forms
-    const bool one_block = (p.tps > 1 && !stream) || patch;   // every channel in one K block: the weight operand is one of the three forms as a whole
-    const CUtensorMap &b_hi_map = one_block ? (b_whole == 0 ? L->map_w8[bi] : (b_whole == 1 ? L->map_w8m[bi] : L->map_wst[bi])) : L->map_w8[bi];
-    if (one_block && b_whole == 2) p.b_tap_step = p.BK;
-    if (stream)
-        return cg == 2 ? launch_kernel<2, 0, 3, false>(a_lo, a_hi, L->map_w8m[bi], L->map_w8[bi], L->map_wst[bi], y_map, y_map16, p, sms, st)
-                       : launch_kernel<1, 0, 3, false>(a_lo, a_hi, L->map_w8m[bi], L->map_w8[bi], L->map_wst[bi], y_map, y_map16, p, sms, st);
-    if (patch) return launch_kernel<1, 0, 2, false>(a_lo, a_hi, L->map_w8m[bi], b_hi_map, L->map_wst[bi], y_map, y_map16, p, sms, st);
+    auto launch = [&]() -> int {
+        if (packed) return launch_kernel<1, 1, 1, false>(a_lo, a_hi, L->map_w4[bi], L->map_w8[bi], L->map_w8[bi], y_map, y_map16, p, sms, st);
+        // multi-tap stages hold every channel in one K block: the whole weight operand is one of the three forms
+        const bool one_block = (p.tps > 1 && !stream) || patch;   // every channel in one K block: the weight operand is one of the three forms as a whole
+        const CUtensorMap &b_hi_map = one_block ? (b_whole == 0 ? L->map_w8[bi] : (b_whole == 1 ? L->map_w8m[bi] : L->map_wst[bi])) : L->map_w8[bi];
+        if (one_block && b_whole == 2) p.b_tap_step = p.BK;
+        if (stream)
+            return cg == 2 ? launch_kernel<2, 0, 3, false>(a_lo, a_hi, L->map_w8m[bi], L->map_w8[bi], L->map_wst[bi], y_map, y_map16, p, sms, st)
+                           : launch_kernel<1, 0, 3, false>(a_lo, a_hi, L->map_w8m[bi], L->map_w8[bi], L->map_wst[bi], y_map, y_map16, p, sms, st);
+        if (patch) return launch_kernel<1, 0, 2, false>(a_lo, a_hi, L->map_w8m[bi], b_hi_map, L->map_wst[bi], y_map, y_map16, p, sms, st);
 #define FLEXIQ_LAUNCH(CG_, KIND_, SPLIT_) launch_kernel<CG_, 0, KIND_, SPLIT_>(a_lo, a_hi, L->map_w8m[bi], b_hi_map, L->map_wst[bi], y_map, y_map16, p, sms, st)
-    if (cg == 2) {
-        if (conv_kind) return split ? FLEXIQ_LAUNCH(2, 1, true) : FLEXIQ_LAUNCH(2, 1, false);
-        return split ? FLEXIQ_LAUNCH(2, 0, true) : FLEXIQ_LAUNCH(2, 0, false);
-    }
-    if (conv_kind) return split ? FLEXIQ_LAUNCH(1, 1, true) : FLEXIQ_LAUNCH(1, 1, false);
-    return split ? FLEXIQ_LAUNCH(1, 0, true) : FLEXIQ_LAUNCH(1, 0, false);
+        if (cg == 2) {
+            if (conv_kind) return split ? FLEXIQ_LAUNCH(2, 1, true) : FLEXIQ_LAUNCH(2, 1, false);
+            return split ? FLEXIQ_LAUNCH(2, 0, true) : FLEXIQ_LAUNCH(2, 0, false);
+        }
+        if (conv_kind) return split ? FLEXIQ_LAUNCH(1, 1, true) : FLEXIQ_LAUNCH(1, 1, false);
+        return split ? FLEXIQ_LAUNCH(1, 0, true) : FLEXIQ_LAUNCH(1, 0, false);
 #undef FLEXIQ_LAUNCH
+    };
+    if ((rc = launch())) return rc;
+    if (marked) {
+        if (!cap) L->weights_fresh = L->st_fresh = 0;
+        else if (L->weights_cap_id == cap) L->weights_cap_id = 0;
+    }
+    return FLEXIQ_OK;
 }
 
 }  // namespace flexiq

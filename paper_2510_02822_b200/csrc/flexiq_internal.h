@@ -47,7 +47,12 @@ struct Layer {
                                    // st_K_lo, so eager calls no longer trust it
     unsigned long long st_cap_id;  // capture sequence that last wrote wst, and for which max_4bit_ch
     int st_cap_K_lo;
-    int weights_fresh, st_fresh;   // w8 / w8m, or wst, written since the handle's last GEMM launch
+    // w8 / w8m, or wst, written eagerly since the handle's last eager GEMM launch (one that is only captured runs, and waits
+    // for the writer, at the earliest when its graph is replayed)
+    int weights_fresh, st_fresh;
+    int weights_graph_seen;             // a layout was captured: replays rewrite w8 / w8m behind the mark above
+    unsigned long long weights_cap_id;  // capture sequence that holds a layout no GEMM of the same capture has waited for yet
+    int early_w, early_st;              // what the last mixed_* call requested ahead of its dependency wait (test hook)
     uint8_t *sw;     // [n_g][N] weight extraction positions
     uint8_t *sx;     // [n_g] static activation positions, slab order
     int32_t *perm;   // [n_g]

@@ -114,10 +114,9 @@ bool straddle_stale(const Layer *L, cudaStream_t st)
 }
 void straddle_written(Layer *L, cudaStream_t st)
 {
-    L->st_fresh = 1;
     const unsigned long long cap = stream_capture_id(st);
     if (cap) { L->st_cap_id = cap; L->st_cap_K_lo = L->K_lo; L->st_graph_seen = 1; L->st_K_lo = -1; }
-    else L->st_K_lo = L->K_lo;
+    else { L->st_K_lo = L->K_lo; L->st_fresh = 1; }
 }
 
 static void *driver_entry(const char *name)
@@ -488,8 +487,10 @@ static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const u
     }
     FLEXIQ_CUDA_TRY(launch_prep(L, a, order, stream));
     L->st_K_lo = -1;   // the straddle block was cut from the previous order's weights
-    L->weights_fresh = 1;
     L->st_cap_id = 0;
+    const unsigned long long cap = stream_capture_id(stream);
+    if (cap) { L->weights_cap_id = cap; L->weights_graph_seen = L->st_graph_seen = 1; }   // a replay makes both stale unseen
+    else L->weights_fresh = 1;
     L->slab_next = 0;  // slabs written for the previous order are no longer this layer's
     memset(L->slab_seen, 0, sizeof(L->slab_seen));
     return FLEXIQ_OK;
@@ -562,6 +563,7 @@ static int create_common(flexiq_layer_t *out, int is_conv, int C, int N, int R, 
     rc = layout_layer(L, Wq, perm, x_shift, stream);
     if (rc) { free_layer(L); return rc; }
     TRY_OR_FREE(cudaStreamSynchronize(stream));
+    L->weights_fresh = 0;   // waited for just now
 #undef TRY_OR_FREE
     rc = encode_weight_maps(L);
     if (rc) { free_layer(L); return rc; }
@@ -654,6 +656,15 @@ int flexiq_get_max_4bit_ch(flexiq_layer_t layer, int *K_lo)
     Layer *L = as_layer(layer);
     if (!L || !K_lo) return set_error(FLEXIQ_ERR_INVALID_ARG, "bad handle or NULL output");
     *K_lo = L->K_lo;
+    return FLEXIQ_OK;
+}
+
+int flexiq_layer_early_loads(flexiq_layer_t layer, int *weights, int *straddle)
+{
+    Layer *L = as_layer(layer);
+    if (!L || !weights || !straddle) return set_error(FLEXIQ_ERR_INVALID_ARG, "bad handle or NULL output");
+    *weights = L->early_w;
+    *straddle = L->early_st;
     return FLEXIQ_OK;
 }
 
