@@ -436,6 +436,13 @@ int flexiq_choose_tile(int64_t M, int N, int k_blocks, int block_k, int sm_count
  * stays usable).  Nothing traps and nothing spins without bound.  The paper has no counterpart. */
 int flexiq_selftest_wait_expiry(int *result_dev, void *stream);
 
+/* Test hook: what the prologue's copying thread does when it gives up.  A ring of two stages takes three copies of 16,384
+ * bytes of src_dev [49152]; a wait of about a millisecond on a barrier that nothing ever arrives on gives up (and raises the
+ * status word, as above); then the copies in flight are waited for.  result_dev [5] int32 receives {1, 0, 1, 1, 0}: a wait
+ * was served, one gave up, the block's give-up flag is set, all copies have landed, and no byte of the two stages differs
+ * from what was copied last.  The paper has no counterpart. */
+int flexiq_selftest_copy_drain(const uint8_t *src_dev, int *result_dev, void *stream);
+
 /* Test hook, host-only: which weights the handle's last mixed_* call requested ahead of its wait for the kernel before it:
  * *weights for the blocks of the two resident forms, *straddle for the block that max_4bit_ch falls into (1 = ahead;
  * where no block does, that one follows *weights).  The paper has no counterpart. */

@@ -8,6 +8,7 @@
 #include <cuda_fp16.h>
 
 #include "sm100_ptx.cuh"
+#include "copy_ring.cuh"
 #include "eq1_quantize.cuh"
 #include "straddle.cuh"
 
@@ -85,10 +86,10 @@ constexpr uint32_t kCopyWaitLimit = 1u << 21;    // parked waits of at most a mi
 __device__ unsigned int g_prologue_status = 0;
 
 // Bounded wait; false after the limit or when another warp already gave up.
-__device__ __forceinline__ bool wait_copy(uint32_t bar, uint32_t parity, volatile int *gave_up)
+__device__ __forceinline__ bool wait_copy(uint32_t bar, uint32_t parity, volatile int *gave_up, uint32_t limit = kCopyWaitLimit)
 {
     if (ptx::mbar_try_wait_s(bar, parity)) return true;
-    for (uint32_t it = 0; it < kCopyWaitLimit; ++it) {
+    for (uint32_t it = 0; it < limit; ++it) {
         if (ptx::mbar_try_wait_hint_s(bar, parity, 1000u)) return true;
         if (*gave_up) return false;
     }
@@ -262,10 +263,7 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
     }
     __syncthreads();
     if (gave_up) {
-        // the copies still in flight land before the block's shared memory is given back
-        if (copier)
-            for (int i = 0; i < a.stages; ++i)
-                for (uint32_t w = 0; w < (1u << 16) && !ptx::mbar_try_wait(&full_bar[i], 0) && !ptx::mbar_try_wait(&full_bar[i], 1); ++w) __nanosleep(64);
+        if (copier) drain_ring(full_bar, a.stages, (next - first) / step);   // the tiles it has requested
         return;
     }
     if (DYN) {
@@ -275,6 +273,42 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
             const unsigned o = or_s[j];
             if (o & ~(look ? __ldcg(a.or_words + j) : 0u)) atomicOr(a.or_words + j, o);
         }
+    }
+}
+
+// Test hook: a ring of two stages given up on with copies in flight.  Three copies are issued, the third into the first
+// one's stage; a wait of about a millisecond on a barrier that nothing arrives on gives up; after the drain the stages hold
+// what the last copies brought.
+constexpr int kDrainBytes = 16384;
+__global__ void drain_kernel(const uint8_t *src, int *result)
+{
+    __shared__ __align__(128) uint8_t ring[2][kDrainBytes];
+    __shared__ uint64_t full[2], never;
+    __shared__ int gave_up;
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 2; ++i) ptx::mbar_init(&full[i], 1);
+        ptx::mbar_init(&never, 1);
+        gave_up = 0;
+        ptx::fence_mbar_init();
+        auto copy = [&](int i) {
+            const uint32_t bar = ptx::smem_u32(&full[i & 1]);
+            ptx::mbar_expect_tx_s(bar, kDrainBytes);
+            ptx::bulk_load(ptx::smem_u32(ring[i & 1]), src + (size_t)i * kDrainBytes, kDrainBytes, bar);
+        };
+        copy(0);
+        const bool served = wait_copy(ptx::smem_u32(&full[0]), 0, &gave_up, 4096u);
+        const bool starved = wait_copy(ptx::smem_u32(&never), 0, &gave_up, 1024u);
+        copy(1);
+        if (served) copy(2);
+        const bool landed = drain_ring(full, 2, served ? 3 : 2);
+        int wrong = 0;
+        for (int s = 0; s < 2; ++s)
+            for (int b = 0; b < kDrainBytes; ++b) wrong += ring[s][b] != src[(size_t)(2 - s) * kDrainBytes + b];
+        result[0] = served;
+        result[1] = starved;
+        result[2] = gave_up;
+        result[3] = landed;
+        result[4] = wrong;
     }
 }
 
@@ -771,4 +805,15 @@ extern "C" int flexiq_quantize_lower_dynamic_noalloc(flexiq_layer_t layer, const
     unsigned *scratch = nullptr;
     if ((rc = static_scratch_address(&scratch))) return rc;
     return flexiq_quantize_lower(layer, X_dev, x_dtype, M, x_scale, 1, X4_dev, X8_dev, x_shift_out_dev, scratch, stream);
+}
+
+extern "C" int flexiq_selftest_copy_drain(const uint8_t *src_dev, int *result_dev, void *stream)
+{
+    if (!src_dev || !result_dev || (reinterpret_cast<uintptr_t>(src_dev) & 15))
+        return set_error(FLEXIQ_ERR_INVALID_ARG, "src_dev or result_dev is NULL, or src_dev is not 16-byte aligned");
+    int rc = check_device_sm100();
+    if (rc) return rc;
+    drain_kernel<<<1, 32, 0, reinterpret_cast<cudaStream_t>(stream)>>>(src_dev, result_dev);
+    FLEXIQ_CUDA_TRY(cudaGetLastError());
+    return FLEXIQ_OK;
 }

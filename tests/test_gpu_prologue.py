@@ -103,3 +103,14 @@ def test_slab_matches_oracle(kind, M, K, G):
                 assert np.array_equal(pos.cpu().numpy(), dyn_sx)
     fx.flexiq_check_status()
     L.close()
+
+
+def test_copies_in_flight_land_when_a_wait_expires():
+    src = torch.arange(49152, dtype=torch.int64, device="cuda").mul_(40503).bitwise_right_shift_(7).to(torch.uint8)
+    res = torch.zeros(5, dtype=torch.int32, device="cuda")
+    fx.flexiq_selftest_copy_drain(src, res)
+    with pytest.raises(fx.FlexiqError) as e:
+        fx.flexiq_check_status()
+    assert e.value.code == fx.ERR_TIMEOUT
+    assert res.cpu().tolist() == [1, 0, 1, 1, 0]
+    fx.flexiq_check_status()                             # reported once
