@@ -9,7 +9,7 @@ namespace flexiq {
 // A ring of `depth` stages that was filled `fills` times in order, full[] its barriers: waits for the last fill of every stage by
 // that fill's own parity (the parity before it is always the completed one and says nothing).  Bounded: about four
 // milliseconds a stage, for fills whose copies were never all issued.  True when all have landed.
-__device__ __noinline__ bool drain_ring(uint64_t *full, int depth, long long fills)
+static __device__ __noinline__ bool drain_ring(uint64_t *full, int depth, long long fills)
 {
     bool landed = true;
     for (long long i = fills > depth ? fills - depth : 0; i < fills; ++i) {

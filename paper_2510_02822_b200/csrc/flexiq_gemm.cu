@@ -23,6 +23,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include "sm100_ptx.cuh"
+#include "copy_ring.cuh"
 #include "straddle.cuh"
 #include "role_timers.cuh"   // PROF_* expand to nothing in the product build
 
@@ -830,7 +831,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         uint32_t rstage = 0, rphase = 0;                       // packed path: ring of raw 4-bit tiles
         const uint32_t raw0 = stage0 + (uint32_t)(p.stages * stage_bytes);
         const uint32_t raw_bytes = (uint32_t)((BM + BN) * (p.BK / 2));
-        long long issued = 0;
+        long long issued = 0, raw_issued = 0;                  // fills of the operand ring, and of the raw tiles or patches
         bool ok = true;
         PROF_DECL(prof_wait);
         PROF_T0(prof_start);
@@ -883,6 +884,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                         ptx::tma_load_4d_s<CG>(ptx::smem_u32(stage_base) + rstage * (uint32_t)p.a_stage, &mapA_hi, CG == 2 ? ptx::mapa(bar, 0) : bar, cb * p.BK, -p.pad, img << p.img_log2, y0 - p.pad);
                     }
                     __syncwarp();
+                    ++raw_issued;
                     if (++rstage == (uint32_t)p.a_stages) { rstage = 0; rphase ^= 1; }
                     for (int r = 0; r < p.T / p.S; ++r) {
                         if (!__all_sync(0xffffffffu, wait_bounded(empty0 + 8 * stage, phase ^ 1, abort_flag, 1))) { ok = false; break; }
@@ -953,6 +955,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
                                 ptx::tma_load_2d_s<1>(ra + BM * (p.BK / 2), mb, bar, xb >> 1, n0);
                             }
                             __syncwarp();
+                            ++raw_issued;
                             if (++rstage == kRawStages) { rstage = 0; rphase ^= 1; }
                             xa += p.BK;
                             xb += p.BK;
@@ -999,18 +1002,21 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         PROF_STORE(1, clock64() - prof_start);
         PROF_STORE(2, issued);
         if (!ok && lane == 0) {
-            // drain: let the copies already in flight land before the CTA retires
-            if (issued < (long long)early) __nanosleep(100000u);   // weight blocks whose stages will never fill
-            const int n_back = issued < p.stages ? (int)issued : p.stages;
-            int s = (int)stage;
-            uint32_t ph = phase;
-            for (int i = 0; i < n_back; ++i) {
-                if (--s < 0) { s = p.stages - 1; ph ^= 1; }
-                for (uint32_t w = 0; w < (1u << 16); ++w) {
-                    if (leader && ptx::mbar_try_wait(&full_bar[s], ph)) break;
-                    __nanosleep(64);
-                    if (!leader && w > 64) break;  // its loads credit the leader's barrier: give them a few microseconds
+            // drain: the copies already in flight land before the CTA retires.  Stages requested ahead that the walk has not come
+            // to (only the streamed kind can give up before it has, on its patches): what was held back of their weights is
+            // requested now, so that they fill.
+            long long fills = issued;
+            if (kStream)
+                for (; fills < (long long)early; ++fills) {
+                    const int R = p.T / p.S, cb = (int)fills / R;
+                    if (cb == p.st_cb && !p.early_st) stream_weights(first_tile % p.n_tiles * BN, cb, (int)fills - cb * R, (uint32_t)fills, false, true);
                 }
+            if (leader) {
+                drain_ring(full_bar, p.stages, fills);
+                if (PK || kStream) drain_ring(raw_full, kStream ? p.a_stages : kRawStages, raw_issued);
+                if (k_bres) drain_ring(raw_full, 1, 1);
+            } else {
+                for (int i = 0; i < p.stages; ++i) __nanosleep(4096u);  // its loads credit the leader's barrier: give them a few microseconds each
             }
         }
     } else if (warp == 1 || (!PK && warp == 2 + kNumWorkWarps)) {
