@@ -158,7 +158,8 @@ int flexiq_layer_set_slab_check(flexiq_layer_t layer, int enabled);
 int flexiq_x4_pitch(flexiq_layer_t layer, int K_lo, int64_t *pitch_bytes);
 
 /* Activation prologue (Sec. 2.1 Eq. 1, Sec. 4.1 bit-lowering, Sec. 5 layout):
- *   q  = clip(round_half_even(x / x_scale), -128, 127)          (skipped for I8 input)
+ *   q  = clip(round_half_even(x / x_scale), -128, 127)          (skipped for I8 input; infinities
+ *        saturate; a NaN, which Eq. 1 does not provide for, quantizes like +infinity)
  *   slab group j <  n_low : x4 = clamp(q >> sx[j], -8, 7)   -> X4_dev
  *   slab group j >= n_low : q                               -> X8_dev
  * with channels gathered into slab order.

@@ -18,10 +18,10 @@ namespace flexiq {
 // correctly rounded quotient RN(x/S) (Markstein's theorem), i.e. the IEEE division result,
 // at five instructions per element.  (Only the final integer matters here: results in the
 // subnormal range may differ but round to 0 either way.)  Infinite inputs, or inputs whose product with
-// r overflows, turn the corrections into NaN (inf - inf); the caller's clip fmaxf(NaN, lo) then yields lo,
+// r overflows, turn the corrections into NaN (inf - inf); the clip's fmaxf(NaN, lo) then yields lo,
 // which is right for the negative side only.  So x is first capped at 256 S from above -- every value
 // beyond it quantizes to 127 anyway -- and both infinities saturate as Eq. 1's clip says.  NaN inputs
-// are excluded.
+// have no place in Eq. 1; the cap replaces them too, so they quantize like +infinity, and the short forms below do the same.
 struct Divider {
     float S, r, lim;
     __device__ __forceinline__ float operator()(float x) const
@@ -32,6 +32,8 @@ struct Divider {
         t = __fmaf_rn(__fmaf_rn(-S, t, x), r, t);
         return t;
     }
+    // lo first: the quotient of -infinity is a NaN, see above (that of a NaN input is large, the cap has replaced it)
+    __device__ __forceinline__ static float clip(float t, float lo, float hi) { return fminf(fmaxf(t, lo), hi); }
 };
 __device__ __forceinline__ Divider make_divider(float scale)
 {
@@ -61,12 +63,14 @@ __device__ __forceinline__ Divider make_divider(float scale)
 // (both forms are odd in x): the same for 99.3 % of the scales with fp16 inputs and 99.9 % with bf16; the general
 // division serves the rest.
 //
-// Infinite x stay infinite with their sign in both forms (all factors are positive) and saturate.
+// Infinite x stay infinite with their sign in both forms (all factors are positive) and saturate.  NaN inputs stay NaN, which
+// the clip turns into its upper bound by taking the minimum first.
 constexpr float kRoundMagic = 12582912.0f;   // 1.5 * 2^23
 enum QuotientForm { kQuotGeneral = 0, kQuotTwoTerm = 1, kQuotMagic = 2 };
 struct TwoTerm {
     float r_hi, r_lo;
     __device__ __forceinline__ float operator()(float x) const { return __fmaf_rn(x, r_hi, __fmul_rn(x, r_lo)); }
+    __device__ __forceinline__ static float clip(float t, float lo, float hi) { return fmaxf(fminf(t, hi), lo); }
 };
 struct QuotientPlan { int form; float r_hi, r_lo; };
 inline QuotientPlan plan_quotient(float S, int dtype)
@@ -174,7 +178,7 @@ __device__ __forceinline__ void quantize16(const void *p, const Divider &div, fl
         for (int k = 0; k < 4; ++k) {
             float t[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) t[j] = fminf(fmaxf(div(x[4 * k + j]), lo), hi);
+            for (int j = 0; j < 4; ++j) t[j] = Divider::clip(div(x[4 * k + j]), lo, hi);
             w[k] = quant4(t[0], t[1], t[2], t[3]);
         }
     }
@@ -212,7 +216,7 @@ __device__ __forceinline__ void quantize_raw(const uint4 *raw, const Q &div, flo
         float x[4], t[4];
         widen4<DTYPE>(raw, k, x);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) t[j] = fminf(fmaxf(div(x[j]), lo), hi);
+        for (int j = 0; j < 4; ++j) t[j] = Q::clip(div(x[j]), lo, hi);
         w[k] = quant4(t[0], t[1], t[2], t[3]);
     }
 }
@@ -227,7 +231,7 @@ __device__ __forceinline__ void quantize_raw_magic(const uint4 *raw, float r, fl
         unsigned b[4];
         widen4<DTYPE>(raw, k, x);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = __float_as_uint(fminf(fmaxf(__fmaf_rn(x[j], r, kRoundMagic), mlo), mhi));
+        for (int j = 0; j < 4; ++j) b[j] = __float_as_uint(fmaxf(fminf(__fmaf_rn(x[j], r, kRoundMagic), mhi), mlo));
         w[k] = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
     }
 }

@@ -71,6 +71,34 @@ def test_fp32_next_to_every_boundary():
     L.close()
 
 
+@pytest.mark.parametrize("kind", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("M", [5, 40000])                # the one-launch dynamic kernel, and the two phases
+def test_infinities_and_nan(kind, M):
+    perm, sx = np.array([3, 0, 2, 1], np.int32), np.array([0, 1, 2, 4], np.uint8)
+    X = torch.zeros((M, 64))
+    X[0, ::16], X[1, ::16], X[2, ::16] = float("nan"), float("inf"), float("-inf")
+    X = X.to(DTYPES[kind]).cuda()
+    for path in (fx.LOWBIT_MASKED_I8, fx.LOWBIT_PACKED_U4):
+        L = make_layer(64, 16, perm, sx)
+        L.set_lowbit_path(path)
+        general = [np.float32(0.1) * np.float32(2.0 ** -110)]   # outside the short forms' range
+        for S in scales(kind) + general:
+            for ratio in (0.0, 0.5):
+                L.set_lowbit_ratio(ratio)
+                if path == fx.LOWBIT_MASKED_I8:
+                    for dynamic in (False, True):
+                        got, pos = slab(L, X, float(S), dynamic=dynamic)
+                        s = pos.cpu().numpy().astype(int) if dynamic else sx[perm].astype(int)
+                        lowered = np.arange(4) < 4 * ratio
+                        top, bottom = np.where(lowered, 7 << s, 127), np.where(lowered, -8 << s, -128)
+                        assert np.array_equal(got[:3, ::16], np.stack([top, top, bottom]).astype(np.int8)), (float(S), ratio, dynamic)
+                elif ratio == 0.0:
+                    _, x8, _ = L.quantize_lower(X, float(S))
+                    assert x8[:192].view(3, 64)[:, ::16].cpu().tolist() == [[127] * 4, [127] * 4, [-128] * 4], float(S)
+        L.close()
+    fx.flexiq_check_status()
+
+
 # rows x channels: one row, one chunk, fewer tiles than SMs, ragged last tiles, rows of one chunk per thread and of many, the widest
 # rows of the ring for each type (65,536 bytes) and wider ones; rows beyond what the one-launch dynamic kernel holds
 @pytest.mark.parametrize("kind", ["f32", "f16", "bf16", "i8"])
