@@ -430,6 +430,11 @@ int flexiq_force_tile(int cta_group, int tile_n);
  * SMs.  Writes the CTAs per tile (1 or 2) and the tile width.  The paper has no counterpart. */
 int flexiq_choose_tile(int64_t M, int N, int k_blocks, int block_k, int sm_count, int *cta_group_out, int *tile_n_out);
 
+/* Test hook, host-only: the form the automatic choice takes for a masked-path convolution on a GPU of sm_count SMs: 0 a plain
+ * GEMM (1x1, stride 1, no padding), 1 im2col copies, 2 halo patches with resident weights, 3 halo patches per K block with
+ * streamed weights.  The paper has no counterpart. */
+int flexiq_choose_conv_kind(int Nb, int H, int W, int Cin, int Cout, int R, int S, int stride, int pad, int sm_count, int *kind_out);
+
 /* Test hook: runs the mainloop's bounded wait, with a limit of about a millisecond instead of two seconds, once on
  * a barrier that completes and once on a barrier that nothing ever arrives on.  result_dev [3] int32 receives
  * {1, 0, 1}: the first wait was served, the second gave up, and the CTA's give-up flag is set; the status word is

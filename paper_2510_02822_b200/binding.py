@@ -30,7 +30,7 @@ EXPORTS = [
     "flexiq_calib_weight_absmax", "flexiq_calib_prepare", "flexiq_calib_absmax_ema",
     "flexiq_controller_create", "flexiq_controller_destroy", "flexiq_controller_level", "flexiq_controller_update",
     "flexiq_serving_simulate", "flexiq_evo_init", "flexiq_evo_next_generation", "flexiq_sq_distance_i8",
-    "flexiq_layer_export", "flexiq_layer_early_loads", "flexiq_selftest_wait_expiry", "flexiq_selftest_copy_drain", "flexiq_force_tile", "flexiq_choose_tile", "flexiq_check_status", "flexiq_last_error",
+    "flexiq_layer_export", "flexiq_layer_early_loads", "flexiq_selftest_wait_expiry", "flexiq_selftest_copy_drain", "flexiq_force_tile", "flexiq_choose_tile", "flexiq_choose_conv_kind", "flexiq_check_status", "flexiq_last_error",
 ]
 
 _lib = None
@@ -269,6 +269,13 @@ def flexiq_choose_tile(M, N, k_blocks, block_k=128, sm_count=148):
     cg, bn = C.c_int(0), C.c_int(0)
     _check(lib().flexiq_choose_tile(C.c_int64(M), N, k_blocks, block_k, sm_count, C.byref(cg), C.byref(bn)))
     return cg.value, bn.value
+
+
+def flexiq_choose_conv_kind(Nb, H, W, Cin, Cout, R, S, stride, pad, sm_count=148):
+    """0 plain, 1 im2col, 2 patches with resident weights, 3 streamed patches; host-only."""
+    kind = C.c_int()
+    _check(lib().flexiq_choose_conv_kind(Nb, H, W, Cin, Cout, R, S, stride, pad, sm_count, C.byref(kind)))
+    return kind.value
 
 
 def flexiq_selftest_wait_expiry(result_dev):

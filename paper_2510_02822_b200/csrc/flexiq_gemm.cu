@@ -1573,45 +1573,96 @@ static int make_map_nhwc_by_row(CUtensorMap *map, const void *base, uint64_t row
     return FLEXIQ_OK;
 }
 
-// Streamed patch mode for a stride-1 filter: geometry of the grid and the rings, and which column width, or none.
-struct StreamPlan { int cg, bn, pw_log2, img_log2, th, rows, a_stage, stages, tiles_per_img; long long m_tiles; };
-static bool plan_stream(const Layer *L, int Nb, int W, int P, int Q, int bk, int sms, StreamPlan *out)
+// What decides between the kinds a convolution can run as.
+struct ConvShape { int C, N, R, S, stride, pad, Nb, W, P, Q, bk; };
+
+// Patch mode (see GemmParams): stride-1 filters of more than one tap whose channels fit one K block and whose
+// output channels fit one tile, the weights of all taps resident in shared memory.
+struct PatchPlan { int bn, pw_log2, th, rows, stage, tiles_per_img; };
+static bool plan_patch(const ConvShape &c, PatchPlan *out)
 {
-    const int width = W + L->pad > Q ? W + L->pad : Q;   // columns a row of the grid has to hold
-    if (L->S > 3 || width > 128) return false;
+    if (c.stride != 1 || c.C > c.bk || c.N > 128 || c.W + c.pad > 128 || c.Q > 128) return false;
+    PatchPlan p{};
+    p.pw_log2 = 3;
+    while ((1 << p.pw_log2) < c.W + c.pad || (1 << p.pw_log2) < c.Q) ++p.pw_log2;   // (padding wider than the filter: more output columns than input)
+    p.th = BM >> p.pw_log2;
+    p.bn = c.N <= 64 ? 64 : 128;
+    p.rows = p.th + c.R - 1 + (c.W + 2 * c.pad > (1 << p.pw_log2) ? 1 : 0);
+    p.stage = (((p.rows << p.pw_log2) * c.bk) + 1023) & ~1023;
+    const int b_all = ((c.R * c.S * p.bn * c.bk) + 1023) & ~1023;
+    if (b_all + 2 * p.stage > kStageRegion || p.rows > 256) return false;
+    p.tiles_per_img = (c.P + p.th - 1) / p.th;
+    *out = p;
+    return true;
+}
+
+// Cycles that a convolution takes as im2col copies with a given tile, less what it has in common with the streamed form below.
+// Per K block of a tap the MMAs, or the copies: 128 pixels at 2.7 cycles each (three quarters of that where a stage takes several
+// taps), twice that where the pixels are an odd number of 16-byte chunks and so begin in the middle of a sector; the
+// weights at 115 bytes a cycle.
+static double im2col_cycles(const ConvShape &c, TileChoice t, int sms)
+{
+    const long long M = (long long)c.Nb * c.P * c.Q, tiles = (M + (long long)BM * t.cg - 1) / ((long long)BM * t.cg) * ((c.N + t.bn - 1) / t.bn);
+    const long long waves = (tiles + sms / t.cg - 1) / (sms / t.cg);
+    const double pixel = (c.C % 32 == 0 ? 2.7 : (c.bk == 128 ? 5.3 : 4.4)) * (c.C <= c.bk ? 0.75 : 1.0);
+    const double mma = 2.0 * t.bn * c.bk / 128.0, fill = 128.0 * pixel + (double)t.bn / t.cg * c.bk / 115.0;
+    return (double)waves * ((double)((c.C + c.bk - 1) / c.bk) * c.R * c.S * (mma > fill ? mma : fill) + 1700.0) + 600.0;
+}
+
+// Streamed patch mode for a stride-1 filter: geometry of the grid and the rings, and which column width, or none where the
+// filter has one column, the patch does not fit, or the im2col form (its tile: `im2col`) is the faster one.
+struct StreamPlan { int cg, bn, pw_log2, img_log2, th, rows, a_stage, stages, tiles_per_img; long long m_tiles; };
+static bool plan_stream(const ConvShape &c, TileChoice im2col, int sms, StreamPlan *out)
+{
+    const int width = c.W + c.pad > c.Q ? c.W + c.pad : c.Q;   // columns a row of the grid has to hold
+    if (c.stride != 1 || c.S > 3 || width > 128) return false;
+    // One column: nothing for the taps of a row to share, and a stage is a single weight tile.  Batch 12, 736 -> 208 channels, 3x1 at
+    // 16 x 16 13.7 us streamed, 12.1 as im2col copies; 256 -> 256 at 30 x 30, batch 16, 12.7 and 11.4; equal at best.
+    if (c.S == 1) return false;
     StreamPlan s{};
     s.pw_log2 = 3;
     while ((1 << s.pw_log2) < width) ++s.pw_log2;
     // images side by side: as many as make the grid's rows at least fit the image's, and there are images
     const int rows_max = BM >> s.pw_log2;
-    while ((rows_max >> s.img_log2) >= 2 * P && (2 << s.img_log2) <= Nb) ++s.img_log2;
-    if ((rows_max >> s.img_log2) > P && (rows_max >> (s.img_log2 + 1)) >= 1 && (2 << s.img_log2) <= Nb) {
+    while ((rows_max >> s.img_log2) >= 2 * c.P && (2 << s.img_log2) <= c.Nb) ++s.img_log2;
+    if ((rows_max >> s.img_log2) > c.P && (rows_max >> (s.img_log2 + 1)) >= 1 && (2 << s.img_log2) <= c.Nb) {
         // one more doubling when it wastes fewer rows
         const int t0 = rows_max >> s.img_log2, t1 = t0 >> 1;
-        if ((long long)((P + t1 - 1) / t1) * t1 < (long long)t0) ++s.img_log2;
+        if ((long long)((c.P + t1 - 1) / t1) * t1 < (long long)t0) ++s.img_log2;
     }
     s.th = rows_max >> s.img_log2;
-    s.rows = s.th + L->R - 1 + (W + 2 * L->pad > (1 << s.pw_log2) ? 1 : 0);
-    const long long patch = (long long)s.rows * (bk << (s.pw_log2 + s.img_log2));
+    s.rows = s.th + c.R - 1 + (c.W + 2 * c.pad > (1 << s.pw_log2) ? 1 : 0);
+    const long long patch = (long long)s.rows * (c.bk << (s.pw_log2 + s.img_log2));
     if (s.rows > 256 || patch > 49152) return false;
     s.a_stage = (int)((patch + 1023) & ~1023ll);
-    s.tiles_per_img = (P + s.th - 1) / s.th;
-    s.m_tiles = (long long)((Nb + (1 << s.img_log2) - 1) >> s.img_log2) * s.tiles_per_img;
+    s.tiles_per_img = (c.P + s.th - 1) / s.th;
+    s.m_tiles = (long long)((c.Nb + (1 << s.img_log2) - 1) >> s.img_log2) * s.tiles_per_img;
     // Tile by whole waves: cycles per 32-channel step of a tap as the shared memory delivers its operands and takes the
     // refills (measured near: single CTA 128 columns 92, 64 columns 60; pair 128 columns 66, 64 columns 50), plus the tile's
     // fixed part and a cluster launch's.
+    auto per_step = [](int cg, int bn) { return cg == 2 ? (bn == 128 ? 66.0 : 50.0) : (bn == 128 ? 92.0 : 60.0); };
     double best = 0.0;
-    const int nbt = (L->C + bk - 1) / bk;
+    long long best_waves = 0;
+    const int nbt = (c.C + c.bk - 1) / c.bk;
     for (int cg = 2; cg >= 1; --cg)
         for (int bn = 128; bn >= 64; bn -= 64) {
-            const int st = (kStageRegion - 2 * s.a_stage) / (L->S * (bn / cg) * bk);
+            const int st = (kStageRegion - 2 * s.a_stage) / (c.S * (bn / cg) * c.bk);
             if (st < 2) continue;
-            const long long tiles = (s.m_tiles + cg - 1) / cg * ((L->N + bn - 1) / bn), waves = (tiles + sms / cg - 1) / (sms / cg);
-            const double per = cg == 2 ? (bn == 128 ? 66.0 : 50.0) : (bn == 128 ? 92.0 : 60.0);
-            const double cost = (double)waves * ((double)nbt * L->R * L->S * (bk / 32) * per + 1200.0) + (cg == 2 ? 800.0 : 0.0);
-            if (best == 0.0 || cost < best) { best = cost; s.cg = cg; s.bn = bn; s.stages = st < kMaxStages ? st : kMaxStages; }
+            const long long tiles = (s.m_tiles + cg - 1) / cg * ((c.N + bn - 1) / bn), waves = (tiles + sms / cg - 1) / (sms / cg);
+            const double cost = (double)waves * ((double)nbt * c.R * c.S * (c.bk / 32) * per_step(cg, bn) + 1200.0) + (cg == 2 ? 800.0 : 0.0);
+            if (best == 0.0 || cost < best) { best = cost; best_waves = waves; s.cg = cg; s.bn = bn; s.stages = st < kMaxStages ? st : kMaxStages; }
         }
-    if (!s.bn) return false;
+    if (!s.bn || (c.R == 1 && best_waves > 1)) return false;   // one row: only where nothing waits behind a tile (192 of 64, 1x3 at 56 x 56, batch 32: 24.8 against 17.4)
+    // Streamed or im2col.  A grid whose pitch just misses the image (widths that are a power of two) computes up to twice the rows, and
+    // small filters do little with a patch.  Over 588 shapes (batch 1 to 64, 3 to 125 pixels wide, 32 to 1264 channels, 1x3 to 5x3,
+    // both forms measured) the choice is within 0.4 % of the faster one on average, 14 % at worst; the streamed form for all was 3.8 % off,
+    // up to 59 %.  A K block takes its MMAs, or 390 cycles a filter row and 95 bytes a cycle for the patch (1.3 times its
+    // bytes where the pixels begin in the middle of a sector) and the weights; a tile at least 2700: its epilogue.
+    const int last = (c.C - (nbt - 1) * c.bk + 31) >> 5;   // steps of a tap's last K block
+    const double fill = 390.0 * c.R + ((double)patch * (c.C % 32 ? 1.3 : 1.0) + (double)c.R * c.S * (s.bn / s.cg) * c.bk) / 95.0;
+    const double step = (double)c.R * c.S * per_step(s.cg, s.bn), whole = c.bk / 32 * step, end = last * step;
+    const double tile = (nbt - 1) * (whole > fill ? whole : fill) + (end > fill ? end : fill) + 800.0;
+    if ((double)best_waves * (tile > 2700.0 ? tile : 2700.0) > im2col_cycles(c, im2col, sms)) return false;
     *out = s;
     return true;
 }
@@ -1799,34 +1850,21 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
             }
         }
     }
-    // Patch mode (see GemmParams): stride-1 filters of more than one tap whose channels fit one K block and whose
-    // output channels fit one tile, the weights of all taps resident in shared memory.
-    bool patch = false;
-    int patch_pw = 8;
-    if (!packed && !g_forced_tile.cg && p.im2col && L->stride == 1 && L->C <= p.BK && L->N <= 128 && W + L->pad <= 128 && p.Q <= 128) {
-        while (patch_pw < W + L->pad || patch_pw < p.Q) patch_pw *= 2;   // (padding wider than the filter: more output columns than input)
-        const int th = BM / patch_pw, bn_p = L->N <= 64 ? 64 : 128;
-        const int rows = th + L->R - 1 + (W + 2 * L->pad > patch_pw ? 1 : 0);
-        const int stage = ((rows * patch_pw * p.BK) + 1023) & ~1023;
-        const int b_all = ((p.T * bn_p * p.BK) + 1023) & ~1023;
-        if (b_all + 2 * stage <= kStageRegion && rows <= 256) {
-            patch = true;
-            tc.cg = 1; tc.bn = bn_p;
-            p.TH = th; p.patch_stage = stage; p.patch_rows = rows;
-            p.pw_log2 = 0;
-            while ((1 << p.pw_log2) < patch_pw) ++p.pw_log2;
-            p.tiles_per_img = (p.P + th - 1) / th;
-        }
-    }
-    // Streamed patch mode: the other stride-1 filters
-    bool stream = false;
+    // the convolution's kind (see the plans above)
+    bool patch = false, stream = false;
     StreamPlan sp{};
-    if (!packed && !patch && !g_forced_tile.cg && p.im2col && L->stride == 1 && plan_stream(L, Nb, W, p.P, p.Q, p.BK, sms, &sp)) {
-        stream = true;
-        tc.cg = sp.cg; tc.bn = sp.bn;
-        p.pw_log2 = sp.pw_log2; p.img_log2 = sp.img_log2; p.TH = sp.th; p.patch_rows = sp.rows; p.tiles_per_img = sp.tiles_per_img;
-        p.nbt = p.nb_lo + p.nb_hi; p.a_stages = 2; p.a_stage = sp.a_stage;
-        p.patch_tx = (sp.rows << (sp.pw_log2 + sp.img_log2)) * p.BK;
+    if (!packed && !g_forced_tile.cg && p.im2col) {
+        const ConvShape shape{L->C, L->N, L->R, L->S, L->stride, L->pad, Nb, W, p.P, p.Q, p.BK};
+        PatchPlan pp{};
+        if ((patch = plan_patch(shape, &pp))) {
+            tc.cg = 1; tc.bn = pp.bn;
+            p.pw_log2 = pp.pw_log2; p.TH = pp.th; p.patch_stage = pp.stage; p.patch_rows = pp.rows; p.tiles_per_img = pp.tiles_per_img;
+        } else if ((stream = plan_stream(shape, tc, sms, &sp))) {
+            tc.cg = sp.cg; tc.bn = sp.bn;
+            p.pw_log2 = sp.pw_log2; p.img_log2 = sp.img_log2; p.TH = sp.th; p.patch_rows = sp.rows; p.tiles_per_img = sp.tiles_per_img;
+            p.nbt = p.nb_lo + p.nb_hi; p.a_stages = 2; p.a_stage = sp.a_stage;
+            p.patch_tx = (sp.rows << (sp.pw_log2 + sp.img_log2)) * p.BK;
+        }
     }
     const int bn = tc.bn, cg = tc.cg;
     p.sx = x_shift ? x_shift : L->sx;
@@ -2046,6 +2084,21 @@ extern "C" int flexiq_choose_tile(int64_t M, int N, int k_blocks, int block_k, i
     const TileChoice tc = choose_tile(M, N, k_blocks, block_k, sm_count);
     *cta_group_out = tc.cg;
     *tile_n_out = tc.bn;
+    return FLEXIQ_OK;
+}
+
+extern "C" int flexiq_choose_conv_kind(int Nb, int H, int W, int Cin, int Cout, int R, int S, int stride, int pad, int sm_count, int *kind_out)
+{
+    if (Nb <= 0 || H <= 0 || W <= 0 || Cin <= 0 || Cout <= 0 || R <= 0 || S <= 0 || stride <= 0 || pad < 0 || sm_count < 2 || !kind_out ||
+        H + 2 * pad < R || W + 2 * pad < S)
+        return set_error(FLEXIQ_ERR_INVALID_ARG, "flexiq_choose_conv_kind: sizes must be positive, the filter must fit the padded input, output non-NULL");
+    const int P = (H + 2 * pad - R) / stride + 1, Q = (W + 2 * pad - S) / stride + 1, bk = Cin >= 128 ? 128 : 64;
+    const ConvShape shape{Cin, Cout, R, S, stride, pad, Nb, W, P, Q, bk};
+    PatchPlan pp{};
+    StreamPlan sp{};
+    if (R == 1 && S == 1 && stride == 1 && pad == 0) *kind_out = 0;
+    else if (plan_patch(shape, &pp)) *kind_out = 2;
+    else *kind_out = plan_stream(shape, choose_tile((long long)Nb * P * Q, Cout, R * S * ((Cin + bk - 1) / bk), bk, sm_count), sm_count, &sp) ? 3 : 1;
     return FLEXIQ_OK;
 }
 

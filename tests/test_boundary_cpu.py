@@ -121,3 +121,24 @@ def test_tile_choice_host_logic(lib):
     for bad in [(0, 64, 1, 128, 148), (5, 0, 1, 128, 148), (5, 64, 0, 128, 148), (5, 64, 1, 96, 148), (5, 64, 1, 128, 0)]:
         with pytest.raises(fx.FlexiqError):
             fx.flexiq_choose_tile(*bad)
+
+
+# Nb, H, W, Cin, Cout, R, S: us as streamed patches and as im2col copies (prologue + convolution), and which of them runs
+@pytest.mark.parametrize("shape, streamed, im2col", [
+    ((32, 14, 14, 256, 256, 3, 3), 10.7, 12.9), ((32, 28, 28, 256, 256, 3, 3), 19.7, 20.9), ((8, 16, 16, 512, 512, 3, 3), 13.1, 16.4),
+    ((32, 28, 28, 144, 144, 3, 3), 18.0, 21.7), ((1, 64, 64, 256, 256, 3, 3), 10.4, 12.5), ((8, 28, 28, 128, 512, 3, 3), 10.0, 10.7),
+    ((32, 16, 16, 512, 512, 3, 3), 29.1, 20.7), ((32, 32, 32, 256, 256, 3, 3), 28.6, 22.3), ((8, 64, 64, 64, 256, 3, 3), 17.6, 12.5),
+    ((4, 120, 64, 160, 160, 3, 3), 25.6, 20.1), ((32, 56, 56, 64, 256, 3, 3), 27.4, 23.6), ((5, 77, 77, 672, 352, 2, 2), 57.0, 38.7),
+    ((12, 16, 16, 736, 208, 3, 1), 13.7, 12.1), ((32, 56, 56, 64, 192, 1, 3), 24.8, 17.4)])
+def test_conv_kind_is_the_faster_one(lib, shape, streamed, im2col):
+    assert fx.flexiq_choose_conv_kind(*shape, 1, shape[6] // 2) == (3 if streamed < im2col else 1)
+
+
+def test_conv_kind_host_logic(lib):
+    assert fx.flexiq_choose_conv_kind(32, 56, 56, 256, 64, 1, 1, 1, 0) == 0
+    assert fx.flexiq_choose_conv_kind(32, 56, 56, 64, 64, 3, 3, 1, 1) == 2       # channels in a K block, outputs in a tile
+    assert fx.flexiq_choose_conv_kind(32, 28, 28, 256, 256, 3, 3, 2, 1) == 1     # stride 2
+    assert fx.flexiq_choose_conv_kind(8, 128, 128, 256, 256, 3, 3, 1, 1) == 1    # rows wider than a tile
+    for bad in [(0, 8, 8, 64, 64, 3, 3, 1, 1), (1, 1, 8, 64, 64, 3, 3, 1, 0), (1, 8, 8, 64, 64, 3, 3, 0, 1), (1, 8, 8, 64, 64, 3, 3, 1, -1)]:
+        with pytest.raises(fx.FlexiqError):
+            fx.flexiq_choose_conv_kind(*bad)
