@@ -996,8 +996,10 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
         }
         // This CTA's loads are all issued: the next kernel of the stream may be launched as CTAs leave, and does what it can before
         // its own dependency wait while the last tiles are computed and written (measured per layer, graph replay, prologue + GEMM: K = 1536
-        // at 197 rows 7.95 -> 7.67 us, ViT-B QKV 29.9 -> 29.5, 1x1 at 56 x 56 21.6 -> 20.6).
-        if (lane == 0) ptx::pdl_launch_dependents();
+        // at 197 rows 7.95 -> 7.67 us, ViT-B QKV 29.9 -> 29.5, 1x1 at 56 x 56 21.6 -> 20.6).  Not on the packed path: what follows the
+        // loads is long there (the expander warps), and its prologue, which needs no shared memory, would crowd onto the few SMs
+        // that are free by then (224 -> 1920 at 2873 rows, fp32: 18.7 us so, 15.5 without; 208 -> 2144 at 6655 rows 26.7 and 24.2).
+        if (!PK && lane == 0) ptx::pdl_launch_dependents();
         PROF_STORE(0, prof_wait);
         PROF_STORE(1, clock64() - prof_start);
         PROF_STORE(2, issued);
