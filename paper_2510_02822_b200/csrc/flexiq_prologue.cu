@@ -572,6 +572,15 @@ static QuotientPlan quotient_plan(float S, int dtype)
     return k.plan;
 }
 
+// Dynamic shared memory with which no SM takes more than its share of a grid.  A GEMM releases the prologue behind it while some of
+// its CTAs still run; blocks go where there is room, so without this the SMs that are free first take as many as fit and
+// the others, when they come free, what is left.
+static size_t even_share_smem(long long blocks, long long sms)
+{
+    const long long share = (blocks + sms - 1) / sms;
+    return (size_t)(228 * 1024 / (share + 1)) - 1024;   // (an SM's 228 KB; each block takes 1 KB and the static part besides)
+}
+
 // The masked path's quantizing kernel, static (DYN = false) or phase 1 of the dynamic mode.
 template <int DTYPE, bool DYN>
 static int launch_rows(Layer *L, const void *X, long long M, float S, int8_t *slab, unsigned *or_words, const StraddleJob &job, cudaStream_t st)
@@ -606,7 +615,7 @@ static int launch_rows(Layer *L, const void *X, long long M, float S, int8_t *sl
     a.stages = kRowRing / a.stage_bytes;
     if (a.stages > kRowStages) a.stages = kRowStages;
     if (a.stages < 3) a.stages = 3;                   // wide rows: up to 192 KB, down to one block per SM
-    const size_t smem = (size_t)a.stages * a.stage_bytes + sizeof(unsigned) * (size_t)(n_c16 + (DYN ? L->n_g : 0));
+    size_t smem = (size_t)a.stages * a.stage_bytes + sizeof(unsigned) * (size_t)(n_c16 + (DYN ? L->n_g : 0));
     long long per_sm = (long long)(220 * 1024 / (smem + 1280));
     if (per_sm > 4) per_sm = 4;
     if (per_sm < 1) per_sm = 1;
@@ -614,6 +623,14 @@ static int launch_rows(Layer *L, const void *X, long long M, float S, int8_t *sl
     const int threads = 32 * (warps + 1);
     const unsigned extra = job.wst ? (unsigned)(((long long)job.rows * (job.BK >> 4) + threads - 1) / threads) : 0u;
     a.wp.first_block = extra;   // the straddle blocks come first
+    // Spread evenly where the bytes decide (prologue + GEMM by graph replay: int8 2033 x 2704 18.4 -> 15.7 us, fp16 38,332 x 528 in front
+    // of a 1x3 convolution 22.4 -> 20.0, fp32 14,843 x 832 16.9 -> 15.8, bf16 19,058 x 320 40.1 -> 38.8).  Below 8 MB a grid on few SMs is
+    // the better neighbour: the GEMM behind it finds free SMs and has its preamble and first weights done by then (1536 x 768 9.1 us
+    // crowded, 9.5 spread; int8 182 x 2224 10.2 and 10.8).
+    if (M * L->C * (kBytes + 1) >= 8ll << 20) {
+        const size_t even = even_share_smem(blocks, sms);
+        if (smem < even) smem = even;
+    }
     static bool attr_set[64] = {};   // per instantiation, whatever the size: the 48 KB default covers the static part too
     if (L->device >= 64 || !attr_set[L->device]) {
         FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(quantize_rows_kernel<DTYPE, DYN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem));
