@@ -305,6 +305,8 @@ def _dtype_code(t):
 class Layer:
     """Owns one flexiq layer handle plus reusable slab buffers (torch device memory)."""
 
+    _calls = None   # native marshalling; without it (subclasses that set themselves up, other objects as `nxt`) the Python code serves
+
     def __init__(self, Wq, w_scale, bias, perm, x_shift, G=16, conv=None):
         import numpy as np
         self.G = G
@@ -420,8 +422,9 @@ class Layer:
 
     def mixed_gemm_to_slab(self, x4, x8, M, x_scale, nxt, next_x_scale, relu=False, slab=None, x_shift=None, out_order=ORDER_ORIGINAL):
         """Mixed GEMM whose epilogue writes the masked slab of the layer `nxt` (fused layer boundary)."""
-        if self._calls is not None and nxt._calls is not None:
-            r = self._calls.mixed_gemm_to_slab(x4, x8, M, x_scale, nxt._calls, next_x_scale, relu, slab, x_shift, out_order)
+        nxt_calls = getattr(nxt, "_calls", None)
+        if self._calls is not None and nxt_calls is not None:
+            r = self._calls.mixed_gemm_to_slab(x4, x8, M, x_scale, nxt_calls, next_x_scale, relu, slab, x_shift, out_order)
             if r is not NotImplemented:
                 return r
         if slab is None:
@@ -430,8 +433,9 @@ class Layer:
         return slab
 
     def mixed_conv_to_slab(self, x4, x8, Nb, H, W, x_scale, nxt, next_x_scale, relu=False, slab=None, x_shift=None, out_order=ORDER_ORIGINAL):
-        if self._calls is not None and nxt._calls is not None:
-            r = self._calls.mixed_conv_to_slab(x4, x8, Nb, H, W, x_scale, nxt._calls, next_x_scale, relu, slab, x_shift, out_order)
+        nxt_calls = getattr(nxt, "_calls", None)
+        if self._calls is not None and nxt_calls is not None:
+            r = self._calls.mixed_conv_to_slab(x4, x8, Nb, H, W, x_scale, nxt_calls, next_x_scale, relu, slab, x_shift, out_order)
             if r is not NotImplemented:
                 return r
         stride, pad = self.conv

@@ -1,0 +1,45 @@
+"""The Python side of a layer without its native marshalling: objects that only look like a layer keep working."""
+import pytest
+
+from paper_2510_02822_b200 import binding as fx
+
+
+class Bare(fx.Layer):
+    """A subclass that sets itself up and never runs Layer.__init__."""
+
+    def __init__(self):
+        self.h, self.K, self.N, self.G, self.conv, self.R, self.S = "handle", 64, 64, 16, (1, 1), 3, 3
+
+
+class Next:
+    h = "next"
+
+    def alloc_slabs(self, M):
+        return f"slab of {M}", None
+
+
+@pytest.fixture
+def calls(monkeypatch):
+    seen = []
+    for name in ("flexiq_mixed_gemm_to_slab", "flexiq_mixed_conv_to_slab", "flexiq_set_lowbit_ratio", "flexiq_layer_destroy"):
+        monkeypatch.setattr(fx, name, lambda *a, name=name: seen.append((name, *a)))
+    return seen
+
+
+def test_next_layer_of_another_type(calls):
+    L = Bare()
+    assert L.mixed_gemm_to_slab("x4", None, 5, 0.5, Next(), 0.25) == "slab of 5"
+    assert L.mixed_conv_to_slab("x4", None, 2, 4, 4, 0.5, Next(), 0.25, relu=True) == "slab of 32"
+    L.set_lowbit_ratio(0.5)
+    assert [c[0] for c in calls] == ["flexiq_mixed_gemm_to_slab", "flexiq_mixed_conv_to_slab", "flexiq_set_lowbit_ratio"]
+    assert calls[0][1] == "handle" and calls[0][7] == "next" and calls[1][9] == "next"
+
+
+def test_native_layer_with_a_next_layer_of_another_type(calls):
+    class Native:
+        def __getattr__(self, name):
+            raise AssertionError(f"{name} was called with an object the native side does not know")
+    L = Bare()
+    L._calls = Native()
+    assert L.mixed_gemm_to_slab("x4", None, 5, 0.5, Next(), 0.25) == "slab of 5"
+    assert L.mixed_conv_to_slab("x4", None, 1, 4, 4, 0.5, Next(), 0.25) == "slab of 16"
