@@ -99,15 +99,22 @@ _calls_module = None
 
 
 def _native_calls():
-    """The native marshalling module (csrc/torch_calls.cpp), built beside the library; raises if it has not been."""
+    """The native marshalling module (csrc/torch_calls.cpp), built beside the library for one Python and one torch.  None, with a
+    warning, where it is missing or was built for others: the calls are then marshalled in Python, to the same kernels."""
     global _calls_module
     if _calls_module is None:
         import torch  # noqa: F401  (its libraries have to be loaded first)
         lib()
-        from . import _calls
-        _calls.set_error_class(FlexiqError)
-        _calls_module = _calls
-    return _calls_module
+        try:
+            from . import _calls
+            _calls.set_error_class(FlexiqError)
+            _calls_module = _calls
+        except ImportError as e:
+            import warnings
+            warnings.warn(f"the native marshalling module does not load ({e}): calls take about twice the host time; build it with "
+                          "python -m paper_2510_02822_b200.build", RuntimeWarning, stacklevel=3)
+            _calls_module = False
+    return _calls_module or None
 
 
 def last_error() -> str:
@@ -325,9 +332,10 @@ class Layer:
         # the calls of a forward pass go through native marshalling; what it answers NotImplemented to takes the Python code
         # below it (a subclass with slabs of its own always does)
         self._calls = None
-        if type(self).alloc_slabs is Layer.alloc_slabs:
+        native = _native_calls() if type(self).alloc_slabs is Layer.alloc_slabs else None
+        if native is not None:
             st, pad = conv or (1, 0)
-            self._calls = _native_calls().Calls(self.h.value, self.K, self.N, G, int(conv is not None), st, pad, *((self.R, self.S) if conv else (1, 1)),
+            self._calls = native.Calls(self.h.value, self.K, self.N, G, int(conv is not None), st, pad, *((self.R, self.S) if conv else (1, 1)),
                                                 self.device.index, self._slabs)
 
     def close(self):

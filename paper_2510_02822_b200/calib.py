@@ -68,7 +68,8 @@ def static_preparation_device(Xcal: torch.Tensor, x_scale: float, Wq: torch.Tens
     from . import binding as fx
     C = Xcal.shape[-1]
     X2 = Xcal.reshape(-1, C)
-    r = fx._native_calls().static_preparation(X2, x_scale, Wq, G, conv, batches, coverage)
+    native = fx._native_calls()
+    r = NotImplemented if native is None else native.static_preparation(X2, x_scale, Wq, G, conv, batches, coverage)
     if r is not NotImplemented:
         perm, x_shift, lo, hi, wmax, score, hist = r
         return perm.numpy(), x_shift.numpy(), {"lo": lo, "hi": hi, "wmax": wmax, "score": score, "unused_hist": hist}

@@ -94,7 +94,7 @@ class ChainFitness:
         out = torch.zeros(len(pop), dtype=torch.int64, device=self.dev)
         for i, c in enumerate(pop):
             Y = self.outputs(np.asarray(c, dtype=np.uint8))
-            if calls.sq_distance_i8(Y, self.Y8, out, i) is NotImplemented:
+            if calls is None or calls.sq_distance_i8(Y, self.Y8, out, i) is NotImplemented:
                 fx.flexiq_sq_distance_i8(Y, self.Y8, out[i:i + 1])
         return [int(v) for v in out.cpu().tolist()]
 

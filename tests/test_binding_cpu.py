@@ -2,6 +2,7 @@
 import pytest
 
 from paper_2510_02822_b200 import binding as fx
+from paper_2510_02822_b200 import build
 
 
 class Bare(fx.Layer):
@@ -18,12 +19,39 @@ class Next:
         return f"slab of {M}", None
 
 
+@pytest.fixture(scope="module")
+def lib_built():
+    build.build_library()
+
+
 @pytest.fixture
 def calls(monkeypatch):
     seen = []
     for name in ("flexiq_mixed_gemm_to_slab", "flexiq_mixed_conv_to_slab", "flexiq_set_lowbit_ratio", "flexiq_layer_destroy"):
         monkeypatch.setattr(fx, name, lambda *a, name=name: seen.append((name, *a)))
     return seen
+
+
+def test_without_the_native_module(monkeypatch, lib_built):
+    monkeypatch.setattr(fx, "_calls_module", None)
+    monkeypatch.setitem(__import__("sys").modules, "paper_2510_02822_b200._calls", None)      # import raises ImportError
+    monkeypatch.delattr(__import__("paper_2510_02822_b200"), "_calls", raising=False)
+    with pytest.warns(RuntimeWarning, match="native marshalling"):
+        assert fx._native_calls() is None
+    assert fx._native_calls() is None                                                         # and says so once
+
+
+def test_build_is_stale_for_another_torch_and_finds_nvcc_by_name(monkeypatch, lib_built, tmp_path):
+    assert not build._calls_stale()
+    monkeypatch.setattr(build, "_calls_for", lambda: "python 0.0, torch 0.0")
+    assert build._calls_stale() and build._stale()
+    tool = tmp_path / "bin" / "nvcc"
+    tool.parent.mkdir()
+    tool.write_text("#!/bin/sh\n")
+    tool.chmod(0o755)
+    monkeypatch.setenv("PATH", str(tool.parent))
+    monkeypatch.setenv("NVCC", "nvcc")
+    assert build._nvcc() == str(tool)
 
 
 def test_next_layer_of_another_type(calls):
