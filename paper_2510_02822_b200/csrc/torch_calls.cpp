@@ -14,6 +14,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <algorithm>
+#include <cmath>
 #include <optional>
 #include <vector>
 
@@ -425,7 +426,7 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
         const long long G = whole(args[3]), batches = whole(args[5]);
         const bool conv = truth(args[4]), cover = args[6] != Py_None;
         if (X.dim() != 2 || !X.is_contiguous() || !X.is_cuda() || !Wq.is_cuda() || Wq.dim() != (conv ? 4 : 2) || G < 1 || batches < 1) throw Refused{};
-        if (cover && !PyFloat_Check(args[6])) throw Refused{};
+        if (cover && !(PyFloat_Check(args[6]) && std::isfinite(PyFloat_AS_DOUBLE(args[6])))) throw Refused{};
         const int dtype = dtype_code(X);
         const long long rows = X.size(0), C = X.size(1), n_g = C / G, step = (rows + batches - 1) / batches;
         if (C < 1 || C > INT32_MAX || n_g < 1) throw Refused{};
@@ -471,6 +472,7 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
         });
         if (rc == FLEXIQ_OK && cuda) {
             Py_DECREF(result);
+            cudaGetLastError();   // reported here, not at whatever torch launches next
             PyErr_SetString(PyExc_RuntimeError, cudaGetErrorString((cudaError_t)cuda));
             return nullptr;
         }

@@ -159,3 +159,12 @@ def test_prepare_few_and_many_groups(dev, K, G):
     assert np.array_equal(perm.cpu().numpy(), np.argsort(ref, kind="stable"))
     assert np.array_equal(xs.cpu().numpy(), oracle.static_positions(lo, hi, G))
     assert np.array_equal(hist.cpu().numpy(), oracle.unused_bits_histogram(lo, hi))
+
+
+def test_coverage_that_is_no_number():
+    X, W = torch.randn((64, 32), device="cuda"), torch.ones((32, 16), dtype=torch.int8, device="cuda")
+    for coverage, error in ((float("nan"), ValueError), (float("-inf"), OverflowError)):
+        with pytest.raises(error):
+            calib.static_preparation_device(X, 0.1, W, 16, coverage=coverage)
+    perm, x_shift, _ = calib.static_preparation_device(X, 0.1, W, 16, coverage=0.99)
+    assert sorted(perm.tolist()) == [0, 1]
