@@ -370,7 +370,7 @@ __global__ void lower_inplace_kernel(int8_t *__restrict__ slab, long long M, int
 constexpr int kColCluster = 8;
 constexpr int kColThreads = 256;
 constexpr long long kColBytes = 10ll << 20, kColRows = 6144;   // of input, rows: the largest calls it takes (see columns_fit)
-constexpr int kColSmem = (int)(kColRows / kColCluster) * 4 * 16;   // the quantized rows a CTA then holds, windows of four chunks
+constexpr int kColSmem = 228 * 1024 / 2 - 1024;   // one CTA per SM at most (see launch_columns); the rows a CTA holds take up to 48 KB
 
 struct ColumnsArgs {
     const void *X;
@@ -664,14 +664,23 @@ static int launch_columns(Layer *L, const void *X, long long M, float S, int8_t 
     long long extra = job.wst ? ((long long)job.rows * (job.BK >> 4) + kColThreads - 1) / kColThreads : 0;
     extra = (extra + kColCluster - 1) / kColCluster * kColCluster;   // whole clusters
     a.wp.first_block = (unsigned)extra;
-    const size_t smem = (size_t)rows * window * 16;
+    const long long ctas = (long long)((L->C / 16 + window - 1) / window) * kColCluster;
+    size_t smem = (size_t)rows * window * 16;
+    // Spread evenly where there are rows enough for it to matter and so few clusters that they would crowd onto a part of the machine
+    // (clusters of eight find room on about 128 of the SMs): prologue + GEMM by graph replay, crowded and spread, fp32 6144 x 384
+    // 26.2 -> 12.8 us, 3152 x 768 20.5 -> 16.2, fp16 6144 x 192 14.3 -> 11.3, 1576 x 384 9.2 -> 8.8.  With fewer rows, or three and more
+    // CTAs per SM, the GEMM behind it gains more from the free SMs: 394 x 384 6.8 and 7.4, fp32 394 x 1536 8.6 and 10.7.
+    if (M >= 1024 && ctas <= 2 * 128) {
+        const size_t even = even_share_smem(ctas, 128);
+        if (smem < even) smem = even;
+    }
     static bool attr_set[64] = {};   // per instantiation, as above
     if (L->device >= 64 || !attr_set[L->device]) {
         FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(dynamic_columns_kernel<DTYPE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kColSmem));
         if (L->device < 64) attr_set[L->device] = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(extra + (long long)((L->C / 16 + window - 1) / window) * kColCluster), 1, 1);
+    cfg.gridDim = dim3((unsigned)(extra + ctas), 1, 1);
     cfg.blockDim = dim3(kColThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
