@@ -93,7 +93,14 @@ inline QuotientPlan plan_quotient(float S, int dtype)
         const int bits = dtype == FLEXIQ_DTYPE_F16 ? 10 : 7, emin = dtype == FLEXIQ_DTYPE_F16 ? -14 : -126;
         const double largest = dtype == FLEXIQ_DTYPE_F16 ? 65504.0 : 0x1.fep127;
         p.r_hi = (float)(1.0 / (double)S);
+        int exp;
+        const uint32_t s = (uint32_t)ldexpf(frexpf(S, &exp), 24);   // significand in [2^23, 2^24)
         for (int k = 0; k < 128; ++k) {
+            // Both quotients are within 2^-23 of x/S (r's rounding, and RN's), so only inputs that close to (k + 1/2) S can differ.  In units
+            // of half of S's last place that is v = (2k + 1) s, and the type's inputs near it are multiples of `unit` (or of more, where
+            // they are subnormal): few of the 128 have one near enough, which is then looked at.
+            const uint32_t v = (2u * (uint32_t)k + 1u) * s, unit = 1u << (31 - __builtin_clz(v) - bits), low = v & (unit - 1u);
+            if ((low < unit - low ? low : unit - low) > (v >> 21)) continue;
             const double at = ((double)k + 0.5) * (double)S;   // exact
             const int e = ilogb(at);
             const double ulp = ldexp(1.0, (e > emin ? e : emin) - bits), below = floor(at / ulp) * ulp;

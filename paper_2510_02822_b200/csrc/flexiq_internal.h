@@ -102,6 +102,8 @@ struct Layer {
     struct SlabRecord { const void *ptr; int K_lo; } slab_seen[8];
     int slab_next;
     int slab_check;  // 0 = the caller opted out
+    // how the prologue divides by the activation scale last used with each input type (eq1_quantize.cuh); S = 0: none yet
+    struct Quotient { float S; int form; float r_hi, r_lo; } quotient[4];
 };
 
 // the slab bookkeeping above

@@ -71,6 +71,20 @@ def test_fp32_next_to_every_boundary():
     L.close()
 
 
+def test_scales_and_types_in_turn_on_one_layer():
+    """The plan of the division belongs to a scale and a type: changing either between calls, scales far outside the inputs' range."""
+    rng = np.random.RandomState(4)
+    L = make_layer(64, 16)
+    tiny = [np.float32(1.0901 * 2.0 ** e) for e in (-71, -49, -24, 20, 60)]
+    for i, S in enumerate((tiny + scales("f16") + scales("bf16") + tiny) * 2):
+        kind = ("f16", "bf16", "f32", "i8")[(i * 7 + i // 4) % 4]
+        x = rng.randn(64, 64).astype(np.float32) * np.float32(min(max(float(S) * 90, 1e-6), 2e4))
+        t = torch.from_numpy(x).to(DTYPES[kind]) if kind != "i8" else torch.from_numpy(rng.randint(-128, 128, (64, 64)).astype(np.int8))
+        got, _ = slab(L, t.cuda(), float(S))
+        assert np.array_equal(got, ieee(t.float().numpy(), S) if kind != "i8" else t.numpy()), (kind, float(S))
+    L.close()
+
+
 @pytest.mark.parametrize("kind", ["f32", "f16", "bf16"])
 @pytest.mark.parametrize("M", [5, 40000])                # the one-launch dynamic kernel, and the two phases
 def test_infinities_and_nan(kind, M):
