@@ -47,6 +47,15 @@ constexpr int kSmemBytes = kStageRegion + kNumWorkWarps * (kFactorsPerWarp + kSt
 // next layer's masked slab (its channel order, its low groups lowered).
 constexpr int kOutNextSlab = 3;
 
+// A kernel serves one kind of output.  One kernel for all of them spilled registers in every epilogue (ptxas: 108 bytes stored and 244
+// loaded per thread in the plain CTA pair, against 8 and 8 now), and the epilogue is as long as the mainloop at short K.
+enum OutKind { kKindI8, kKindNext, kKindHalf, kKindWord };
+static OutKind out_kind(int out_mode)
+{
+    return out_mode == FLEXIQ_OUT_REQUANT_I8 ? kKindI8 : out_mode == kOutNextSlab ? kKindNext
+         : (out_mode == FLEXIQ_OUT_DEQUANT_F16 || out_mode == FLEXIQ_OUT_DEQUANT_BF16) ? kKindHalf : kKindWord;
+}
+
 struct GemmParams {
     long long M;         // rows of the implicit GEMM (tokens or output pixels)
     int N;               // output channels
@@ -660,7 +669,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
 // two: for narrow MMAs (64 cycles each) the issuing warp's bookkeeping, not the pipe, bounds a K block, and two
 // warps halve it.  No accumulator is shared, so no order between the warps' MMAs is needed; their waits on
 // the ring stay in ring order (one hand-over phase per stage).
-template <int CG, int PK, int KIND, bool SPLIT>
+template <int CG, int PK, int KIND, bool SPLIT, int OUT>
 __global__ void __launch_bounds__(kThreads, 1)
 mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_constant__ CUtensorMap mapA_hi,
                   const __grid_constant__ CUtensorMap mapB_lo, const __grid_constant__ CUtensorMap mapB_hi,
@@ -1288,12 +1297,15 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
             x.map_y = &mapY; x.map_y16 = &mapY16;
             x.first_tile = first_tile; x.tile_step = tile_step; x.num_tiles = num_tiles;
             x.parts = kEpiWarps / 4; x.arrivals_on = 1;
-            if (p.out_mode == FLEXIQ_OUT_REQUANT_I8) epilogue_role<CG, FLEXIQ_OUT_REQUANT_I8, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
-            else if (p.out_mode == FLEXIQ_OUT_DEQUANT_F32) epilogue_role<CG, FLEXIQ_OUT_DEQUANT_F32, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
-            else if (p.out_mode == kOutNextSlab) epilogue_role<CG, kOutNextSlab, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
-            else if (p.out_mode == FLEXIQ_OUT_DEQUANT_F16) epilogue_role<CG, FLEXIQ_OUT_DEQUANT_F16, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
-            else if (p.out_mode == FLEXIQ_OUT_DEQUANT_BF16) epilogue_role<CG, FLEXIQ_OUT_DEQUANT_BF16, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
-            else epilogue_role<CG, FLEXIQ_OUT_ACC_I32, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
+            if constexpr (OUT == kKindI8) epilogue_role<CG, FLEXIQ_OUT_REQUANT_I8, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
+            else if constexpr (OUT == kKindNext) epilogue_role<CG, kOutNextSlab, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
+            else if constexpr (OUT == kKindHalf) {
+                if (p.out_mode == FLEXIQ_OUT_DEQUANT_F16) epilogue_role<CG, FLEXIQ_OUT_DEQUANT_F16, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
+                else epilogue_role<CG, FLEXIQ_OUT_DEQUANT_BF16, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
+            } else {
+                if (p.out_mode == FLEXIQ_OUT_DEQUANT_F32) epilogue_role<CG, FLEXIQ_OUT_DEQUANT_F32, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
+                else epilogue_role<CG, FLEXIQ_OUT_ACC_I32, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
+            }
         } else if (PK && warp < 2 + kNumWorkWarps) {
             // --------------------------------------------------------- expanders (packed path)
             // Widen each raw 4-bit tile into the operand ring: 8 packed bytes -> one 16-byte unit
@@ -1676,16 +1688,17 @@ static bool plan_stream(const ConvShape &c, TileChoice im2col, int sms, StreamPl
     return true;
 }
 
-template <int CG, int PK, int KIND, bool SPLIT>
-static int launch_kernel(const CUtensorMap &a_lo, const CUtensorMap &a_hi, const CUtensorMap &b_lo, const CUtensorMap &b_hi,
-                         const CUtensorMap &b_st, const CUtensorMap &y_map, const CUtensorMap &y_map16, const GemmParams &p, int sms, cudaStream_t st)
+struct LaunchMaps { CUtensorMap a_lo, a_hi, b_lo, b_hi, b_st, y, y16; };
+
+template <int CG, int PK, int KIND, bool SPLIT, int OUT>
+static int launch_kernel(const LaunchMaps &m, const GemmParams &p, int sms, cudaStream_t st)
 {
     static bool attr_set[64] = {};   // per instantiation
     int dev = 0;
     cudaGetDevice(&dev);
-    if (dev < 64 && !attr_set[dev]) {
-        FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(mixed_gemm_kernel<CG, PK, KIND, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
-        attr_set[dev] = true;
+    if (dev >= 64 || !attr_set[dev]) {
+        FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(mixed_gemm_kernel<CG, PK, KIND, SPLIT, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+        if (dev < 64) attr_set[dev] = true;
     }
     const long long tiles = (long long)p.m_tiles * p.n_tiles;
     const long long slots = sms / CG;
@@ -1704,8 +1717,23 @@ static int launch_kernel(const CUtensorMap &a_lo, const CUtensorMap &a_hi, const
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    FLEXIQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, mixed_gemm_kernel<CG, PK, KIND, SPLIT>, a_lo, a_hi, b_lo, b_hi, b_st, y_map, y_map16, p));
+    FLEXIQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, mixed_gemm_kernel<CG, PK, KIND, SPLIT, OUT>, m.a_lo, m.a_hi, m.b_lo, m.b_hi, m.b_st, m.y, m.y16, p));
     return FLEXIQ_OK;
+}
+
+// What a launch is, beside its parameters.
+struct LaunchForm { int cg; bool packed, patch, stream, conv, split; };
+template <int OUT> static int launch_form(const LaunchForm &f, const LaunchMaps &m, const GemmParams &p, int sms, cudaStream_t st)
+{
+    if (f.packed) return launch_kernel<1, 1, 1, false, OUT>(m, p, sms, st);
+    if (f.stream) return f.cg == 2 ? launch_kernel<2, 0, 3, false, OUT>(m, p, sms, st) : launch_kernel<1, 0, 3, false, OUT>(m, p, sms, st);
+    if (f.patch) return launch_kernel<1, 0, 2, false, OUT>(m, p, sms, st);
+    if (f.cg == 2) {
+        if (f.conv) return f.split ? launch_kernel<2, 0, 1, true, OUT>(m, p, sms, st) : launch_kernel<2, 0, 1, false, OUT>(m, p, sms, st);
+        return f.split ? launch_kernel<2, 0, 0, true, OUT>(m, p, sms, st) : launch_kernel<2, 0, 0, false, OUT>(m, p, sms, st);
+    }
+    if (f.conv) return f.split ? launch_kernel<1, 0, 1, true, OUT>(m, p, sms, st) : launch_kernel<1, 0, 1, false, OUT>(m, p, sms, st);
+    return f.split ? launch_kernel<1, 0, 0, true, OUT>(m, p, sms, st) : launch_kernel<1, 0, 0, false, OUT>(m, p, sms, st);
 }
 
 // Masked path: writes the straddle block for the current max_4bit_ch when the stream does not hold it yet
@@ -2000,26 +2028,19 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
     const bool split = !packed && !patch && !stream && bn <= 128 && p.tps == 1 && p.T * (p.nb_lo + p.nb_hi) >= 8 &&
                        (long long)p.m_tiles * p.n_tiles <= sms / cg;
     if (next) record_slab(const_cast<Layer *>(next), Y, next->K_lo);   // the fused boundary writes the next layer's slab at its current ratio
-    auto launch = [&]() -> int {
-        if (packed) return launch_kernel<1, 1, 1, false>(a_lo, a_hi, L->map_w4[bi], L->map_w8[bi], L->map_w8[bi], y_map, y_map16, p, sms, st);
-        // multi-tap stages hold every channel in one K block: the whole weight operand is one of the three forms
-        const bool one_block = (p.tps > 1 && !stream) || patch;   // every channel in one K block: the weight operand is one of the three forms as a whole
-        const CUtensorMap &b_hi_map = one_block ? (b_whole == 0 ? L->map_w8[bi] : (b_whole == 1 ? L->map_w8m[bi] : L->map_wst[bi])) : L->map_w8[bi];
-        if (one_block && b_whole == 2) p.b_tap_step = p.BK;
-        if (stream)
-            return cg == 2 ? launch_kernel<2, 0, 3, false>(a_lo, a_hi, L->map_w8m[bi], L->map_w8[bi], L->map_wst[bi], y_map, y_map16, p, sms, st)
-                           : launch_kernel<1, 0, 3, false>(a_lo, a_hi, L->map_w8m[bi], L->map_w8[bi], L->map_wst[bi], y_map, y_map16, p, sms, st);
-        if (patch) return launch_kernel<1, 0, 2, false>(a_lo, a_hi, L->map_w8m[bi], b_hi_map, L->map_wst[bi], y_map, y_map16, p, sms, st);
-#define FLEXIQ_LAUNCH(CG_, KIND_, SPLIT_) launch_kernel<CG_, 0, KIND_, SPLIT_>(a_lo, a_hi, L->map_w8m[bi], b_hi_map, L->map_wst[bi], y_map, y_map16, p, sms, st)
-        if (cg == 2) {
-            if (conv_kind) return split ? FLEXIQ_LAUNCH(2, 1, true) : FLEXIQ_LAUNCH(2, 1, false);
-            return split ? FLEXIQ_LAUNCH(2, 0, true) : FLEXIQ_LAUNCH(2, 0, false);
-        }
-        if (conv_kind) return split ? FLEXIQ_LAUNCH(1, 1, true) : FLEXIQ_LAUNCH(1, 1, false);
-        return split ? FLEXIQ_LAUNCH(1, 0, true) : FLEXIQ_LAUNCH(1, 0, false);
-#undef FLEXIQ_LAUNCH
-    };
-    if ((rc = launch())) return rc;
+    // multi-tap stages hold every channel in one K block: the whole weight operand is one of the three forms
+    const bool one_block = (p.tps > 1 && !stream) || patch;
+    if (one_block && b_whole == 2) p.b_tap_step = p.BK;
+    LaunchMaps maps{a_lo, a_hi, packed ? L->map_w4[bi] : L->map_w8m[bi], L->map_w8[bi], packed ? L->map_w8[bi] : L->map_wst[bi], y_map, y_map16};
+    if (one_block && b_whole != 0) maps.b_hi = b_whole == 1 ? L->map_w8m[bi] : L->map_wst[bi];
+    const LaunchForm form{cg, packed, patch, stream, conv_kind, split};
+    switch (out_kind(out_mode)) {
+        case kKindI8: rc = launch_form<kKindI8>(form, maps, p, sms, st); break;
+        case kKindNext: rc = launch_form<kKindNext>(form, maps, p, sms, st); break;
+        case kKindHalf: rc = launch_form<kKindHalf>(form, maps, p, sms, st); break;
+        default: rc = launch_form<kKindWord>(form, maps, p, sms, st); break;
+    }
+    if (rc) return rc;
     if (marked) {
         if (!cap) L->weights_fresh = L->st_fresh = 0;
         else if (L->weights_cap_id == cap) L->weights_cap_id = 0;
