@@ -46,13 +46,15 @@ constexpr int kSmemBytes = kStageRegion + kNumWorkWarps * (kFactorsPerWarp + kSt
 // Internal epilogue mode of the fused layer boundary: the int8 result goes straight into the
 // next layer's masked slab (its channel order, its low groups lowered).
 constexpr int kOutNextSlab = 3;
+// The same with the chunks of the producer's own channel order scattered to their places (a mode of the epilogue only).
+constexpr int kOutScatter = 6;
 
 // A kernel serves one kind of output.  One kernel for all of them spilled registers in every epilogue (ptxas: 108 bytes stored and 244
 // loaded per thread in the plain CTA pair, against 8 and 8 now), and the epilogue is as long as the mainloop at short K.
-enum OutKind { kKindI8, kKindNext, kKindHalf, kKindWord };
-static OutKind out_kind(int out_mode)
+enum OutKind { kKindI8, kKindNext, kKindScatter, kKindHalf, kKindWord };
+static OutKind out_kind(int out_mode, bool staged)
 {
-    return out_mode == FLEXIQ_OUT_REQUANT_I8 ? kKindI8 : out_mode == kOutNextSlab ? kKindNext
+    return out_mode == FLEXIQ_OUT_REQUANT_I8 ? kKindI8 : out_mode == kOutNextSlab ? (staged ? kKindNext : kKindScatter)
          : (out_mode == FLEXIQ_OUT_DEQUANT_F16 || out_mode == FLEXIQ_OUT_DEQUANT_BF16) ? kKindHalf : kKindWord;
 }
 
@@ -83,7 +85,6 @@ struct GemmParams {
     const int32_t *next_ent;   // [N/16] slab position (in chunks) of original chunk c | its group's position << 24
     int next_K_lo;             // the next layer's max_4bit_ch
     int relu;                  // clamp at zero before the re-quantization
-    int tma_store;             // int8 output leaves through shared memory and tiled bulk stores (mapY)
     // Resident weights (convolutions on the multi-tap path whose output channels fit one tile): every tap's
     // weight tile is loaded once per CTA and stays in shared memory in front of the ring, whose stages then hold
     // activation taps only: half as many copies per tile for the producer lane, which bounds these layers.
@@ -361,14 +362,14 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
     constexpr bool kPatch = KIND == 2, kGrid = KIND >= 2;
     constexpr bool kScaled = MODE != FLEXIQ_OUT_ACC_I32;
     constexpr bool kHalf = MODE == FLEXIQ_OUT_DEQUANT_F16 || MODE == FLEXIQ_OUT_DEQUANT_BF16;
-    constexpr int kElem = (MODE == FLEXIQ_OUT_REQUANT_I8 || MODE == kOutNextSlab) ? 1 : (kHalf ? 2 : 4);  // output bytes per element
+    constexpr int kElem = (MODE == FLEXIQ_OUT_REQUANT_I8 || MODE == kOutNextSlab || MODE == kOutScatter) ? 1 : (kHalf ? 2 : 4);  // output bytes per element
     const int BN = p.BN;
     // Columns per warp and pass: 64 (tiles of 192 or 256 columns) or 32 (128 or 64), so that every staged
     // box is 32 columns = whole sectors; with 192 or 64 columns the last column slot of a lane quadrant has no
     // columns and its warp only keeps step with the accumulator barriers.
     const int cols = BN >= 192 ? 64 : 32;
-    const bool y32 = (reinterpret_cast<uintptr_t>(p.Y) & 31) == 0;
-    const bool wide = y32 && (p.N & 31) == 0;    // int8 rows are 32-byte aligned: 256-bit stores
+    constexpr bool kStaged = MODE != kOutScatter;                 // 32 x 32-byte boxes through shared memory and bulk stores
+    constexpr bool kSlab = MODE == kOutNextSlab || MODE == kOutScatter;
     // lane l keeps factors 4l..4l+3 of the table alpha[64] | beta[64]
     const float *fsrc = (lane < 16 ? p.alpha : p.beta) + 4 * (lane & 15);
     int buf = 0;
@@ -429,7 +430,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
             float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
             if (kScaled && nw + 4 * (lane & 15) < p.N) f = __ldg(reinterpret_cast<const float4 *>(fsrc + nw));
             int ent = 0;                                     // fused boundary: lane g fetches chunk g's slab entry
-            if (MODE == kOutNextSlab && lane < 4 && nw + 16 * lane < p.N) ent = __ldg(p.next_ent + (nw >> 4) + lane);
+            if (kSlab && lane < 4 && nw + 16 * lane < p.N) ent = __ldg(p.next_ent + (nw >> 4) + lane);
             if (!waited) {
                 PROF_T0(t0);
                 const bool ok = wait_bounded(&x.tmem_full[buf], buf_phase, x.abort_flag, 4);
@@ -466,11 +467,11 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                 }
             }
             int ents[4] = {0, 0, 0, 0};
-            if (MODE == kOutNextSlab) {
+            if (kSlab) {
 #pragma unroll
                 for (int g = 0; g < 4; ++g) ents[g] = __shfl_sync(0xffffffffu, ent, g);
             }
-            if ((MODE == FLEXIQ_OUT_REQUANT_I8 || MODE == kOutNextSlab) && p.tma_store) {
+            if (MODE == FLEXIQ_OUT_REQUANT_I8 || MODE == kOutNextSlab) {
                 // Each warp stages 32 rows x 32 columns (1 KB, 32-byte swizzle: no bank conflicts) and one
                 // lane hands them to a tiled bulk store, which writes whole sectors asynchronously and
                 // drops the rows and columns that lie outside Y.
@@ -511,7 +512,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                         }
                     }
                 }
-            } else if (kHalf && p.tma_store) {
+            } else if (kHalf) {
                 // 16-bit outputs: 32 rows x 16 columns (32 bytes per row: the same 1 KB swizzled box) per store
                 const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
 #pragma unroll
@@ -542,7 +543,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                         }
                     }
                 }
-            } else if (kElem == 4 && p.tma_store) {
+            } else if (kElem == 4) {
                 // 4-byte outputs: 32 rows x 8 columns per store (the same 32-byte rows)
                 const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
 #pragma unroll
@@ -573,75 +574,29 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                         }
                     }
                 }
-            } else
-            if (row < p.M) {
-                uint8_t *yrow = static_cast<uint8_t *>(p.Y) + (row * p.N + nw) * kElem;
+            } else if (MODE == kOutScatter && row < p.M) {
+                // each 16-channel chunk goes to its place in the next layer's slab row
+                uint8_t *srow = static_cast<uint8_t *>(p.Y) + row * p.N;
+                const bool wide = ((reinterpret_cast<uintptr_t>(p.Y) | (uintptr_t)p.N) & 31) == 0;   // rows are 32-byte aligned: 256-bit stores
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {                       // two halves of 32 columns
                     const uint32_t *r = h == 0 ? ra : rb;
                     const int n = nw + 32 * h;
                     if (32 * h < cols && n < p.N) {
                         const bool second = n + 16 < p.N;  // columns 16..31 of this half are live
-                        if (MODE == kOutNextSlab) {
-                            // each 16-channel chunk goes to its place in the next layer's slab row
-                            uint32_t w[8];
-                            int pos[2] = {0, 0};
+                        uint32_t w[8];
+                        int pos[2] = {0, 0};
 #pragma unroll
-                            for (int g = 0; g < 2; ++g) {
-                                if (g == 0 || second) {
-                                    pos[g] = ents[2 * h + g] & 0xffffff;
-                                    next_slab16(p, ents[2 * h + g], r + 16 * g, x.fac + 32 * h + 16 * g, x.fac + 64 + 32 * h + 16 * g, w + 4 * g);
-                                }
+                        for (int g = 0; g < 2; ++g) {
+                            if (g == 0 || second) {
+                                pos[g] = ents[2 * h + g] & 0xffffff;
+                                next_slab16(p, ents[2 * h + g], r + 16 * g, x.fac + 32 * h + 16 * g, x.fac + 64 + 32 * h + 16 * g, w + 4 * g);
                             }
-                            uint8_t *srow = static_cast<uint8_t *>(p.Y) + row * p.N;
-                            if (second && wide && pos[1] == pos[0] + 1 && (pos[0] & 1) == 0) st_global_256(srow + pos[0] * 16, w);
-                            else {
-                                st_global_128(srow + pos[0] * 16, w[0], w[1], w[2], w[3]);
-                                if (second) st_global_128(srow + pos[1] * 16, w[4], w[5], w[6], w[7]);
-                            }
-                        } else if (MODE == FLEXIQ_OUT_REQUANT_I8) {
-                            uint32_t w[8];
-                            finish16<MODE>(r, x.fac + 32 * h, x.fac + 64 + 32 * h, w);
-                            if (second) finish16<MODE>(r + 16, x.fac + 32 * h + 16, x.fac + 64 + 32 * h + 16, w + 4);
-                            if (second && wide && ((nw & 31) == 0)) st_global_256(yrow + 32 * h, w);  // 32-byte aligned only then
-                            else {
-                                st_global_128(yrow + 32 * h, w[0], w[1], w[2], w[3]);
-                                if (second) st_global_128(yrow + 32 * h + 16, w[4], w[5], w[6], w[7]);
-                            }
-                        } else if (kHalf) {
-                            // 16-bit floating-point outputs: the fp32 result of the fma, rounded once more (to nearest even)
-#pragma unroll
-                            for (int g = 0; g < 2; ++g) {
-                                if (g == 0 || second) {
-                                    uint32_t w[16], hw[8];
-                                    finish16<FLEXIQ_OUT_DEQUANT_F32>(r + 16 * g, x.fac + 32 * h + 16 * g, x.fac + 64 + 32 * h + 16 * g, w);
-#pragma unroll
-                                    for (int q = 0; q < 8; ++q)
-                                        hw[q] = pack2_f16<MODE == FLEXIQ_OUT_DEQUANT_BF16>(__uint_as_float(w[2 * q]), __uint_as_float(w[2 * q + 1]));
-                                    uint8_t *dst = yrow + (32 * h + 16 * g) * 2;
-                                    if (y32) st_global_256(dst, hw);    // rows of 2-byte elements with N % 16 == 0 are 32-byte aligned
-                                    else {
-                                        st_global_128(dst, hw[0], hw[1], hw[2], hw[3]);
-                                        st_global_128(dst + 16, hw[4], hw[5], hw[6], hw[7]);
-                                    }
-                                }
-                            }
-                        } else {
-#pragma unroll
-                            for (int g = 0; g < 2; ++g) {
-                                if (g == 0 || second) {
-                                    uint32_t w[16];
-                                    finish16<MODE>(r + 16 * g, x.fac + 32 * h + 16 * g, x.fac + 64 + 32 * h + 16 * g, w);
-                                    uint8_t *dst = yrow + (32 * h + 16 * g) * 4;
-                                    if (y32) {                      // rows of 4-byte elements with N % 16 == 0 are 64-byte aligned
-                                        st_global_256(dst, w);
-                                        st_global_256(dst + 32, w + 8);
-                                    } else {
-#pragma unroll
-                                        for (int q = 0; q < 4; ++q) st_global_128(dst + 16 * q, w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-                                    }
-                                }
-                            }
+                        }
+                        if (second && wide && pos[1] == pos[0] + 1 && (pos[0] & 1) == 0) st_global_256(srow + pos[0] * 16, w);
+                        else {
+                            st_global_128(srow + pos[0] * 16, w[0], w[1], w[2], w[3]);
+                            if (second) st_global_128(srow + pos[1] * 16, w[4], w[5], w[6], w[7]);
                         }
                     }
                 }
@@ -650,7 +605,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
         }
         if (!kPatch && (buf ^= 1) == 0) buf_phase ^= 1;
     }
-    if (p.tma_store && lane == 0) ptx::bulk_wait_all();  // the staged stores are performed
+    if (kStaged && lane == 0) ptx::bulk_wait_all();  // the staged stores are performed
     if (quad == 2 && part == 0 && lane == 0) { PROF_STORE(8, prof_wait); PROF_STORE(9, clock64() - prof_start); PROF_STORE(10, prof_ld); PROF_STORE(11, prof_math); }
 }
 
@@ -1299,6 +1254,7 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
             x.parts = kEpiWarps / 4; x.arrivals_on = 1;
             if constexpr (OUT == kKindI8) epilogue_role<CG, FLEXIQ_OUT_REQUANT_I8, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
             else if constexpr (OUT == kKindNext) epilogue_role<CG, kOutNextSlab, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
+            else if constexpr (OUT == kKindScatter) epilogue_role<CG, kOutScatter, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
             else if constexpr (OUT == kKindHalf) {
                 if (p.out_mode == FLEXIQ_OUT_DEQUANT_F16) epilogue_role<CG, FLEXIQ_OUT_DEQUANT_F16, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
                 else epilogue_role<CG, FLEXIQ_OUT_DEQUANT_BF16, SPLIT, KIND>(p, x, warp & 3, e >> 2, lane);
@@ -1979,7 +1935,6 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
     }
     // int8 output leaves through staged tiled bulk stores
     CUtensorMap y_map = a_hi, y_map16 = a_hi;
-    p.tma_store = staged;
     if (staged && cached) {
         y_map = cm.y;
         y_map16 = cm.y16;
@@ -2034,8 +1989,9 @@ static int run_mixed(Layer *L, const uint8_t *X4, const int8_t *X8, const uint8_
     LaunchMaps maps{a_lo, a_hi, packed ? L->map_w4[bi] : L->map_w8m[bi], L->map_w8[bi], packed ? L->map_w8[bi] : L->map_wst[bi], y_map, y_map16};
     if (one_block && b_whole != 0) maps.b_hi = b_whole == 1 ? L->map_w8m[bi] : L->map_wst[bi];
     const LaunchForm form{cg, packed, patch, stream, conv_kind, split};
-    switch (out_kind(out_mode)) {
+    switch (out_kind(out_mode, staged)) {
         case kKindI8: rc = launch_form<kKindI8>(form, maps, p, sms, st); break;
+        case kKindScatter: rc = launch_form<kKindScatter>(form, maps, p, sms, st); break;
         case kKindNext: rc = launch_form<kKindNext>(form, maps, p, sms, st); break;
         case kKindHalf: rc = launch_form<kKindHalf>(form, maps, p, sms, st); break;
         default: rc = launch_form<kKindWord>(form, maps, p, sms, st); break;
