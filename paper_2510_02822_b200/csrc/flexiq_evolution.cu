@@ -13,10 +13,9 @@ namespace flexiq {
 // ---------------------------------------------------------------------------------- device: fitness
 // sum over i of (A[i] - B[i])^2 for int8 tensors, exact in int64.  (a - b)^2 = a.a - 2 a.b + b.b,
 // four elements per dp4a; one 16-byte unit of each tensor per thread and step, four steps in flight.
-__global__ void sq_distance_i8_kernel(const int8_t *__restrict__ A, const int8_t *__restrict__ B, long long n,
-                                      unsigned long long *__restrict__ out)
+// Returns the block's sum in thread 0.
+__device__ __forceinline__ long long block_sq_distance(const int8_t *__restrict__ A, const int8_t *__restrict__ B, long long n)
 {
-    ptx::pdl_wait();  // A may be the previous kernel's output
     const long long units = n >> 4;
     const uint4 *a4 = reinterpret_cast<const uint4 *>(A), *b4 = reinterpret_cast<const uint4 *>(B);
     const long long step = (long long)gridDim.x * blockDim.x;
@@ -49,14 +48,45 @@ __global__ void sq_distance_i8_kernel(const int8_t *__restrict__ A, const int8_t
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    __shared__ long long warp_sum[8];
+    __shared__ long long warp_sum[32];
     if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = acc;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        long long t = 0;
+    long long t = 0;
+    if (threadIdx.x == 0)
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += warp_sum[w];
-        if (t) atomicAdd(out, (unsigned long long)t);
+    return t;
+}
+__global__ void sq_distance_i8_kernel(const int8_t *__restrict__ A, const int8_t *__restrict__ B, long long n,
+                                      unsigned long long *__restrict__ out)
+{
+    const long long t = block_sq_distance(A, B, n);
+    if (threadIdx.x == 0 && t) atomicAdd(out, (unsigned long long)t);
+}
+
+// The same by one cluster of sixteen blocks, whose sums meet in the first one's shared memory: one launch, which may start while
+// the GEMM before it ends, and nothing cleared beforehand.  Larger tensors need more than sixteen SMs: the grid above and its clear.
+constexpr int kDistCluster = 16, kDistThreads = 512;
+constexpr int kDistSmem = 228 * 1024 / 2 - 1024;   // one block per SM: the cluster is launched while the GEMM before it still runs on some
+constexpr long long kDistClusterMax = 2ll << 20;
+__global__ void __launch_bounds__(kDistThreads) sq_distance_i8_cluster_kernel(const int8_t *A, const int8_t *B, long long n, long long *out)
+{
+    __shared__ unsigned sum_s[2];
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();   // A may be the previous kernel's output, and out its to read
+    const long long t = block_sq_distance(A, B, n);
+    if (threadIdx.x == 0) { sum_s[0] = (unsigned)t; sum_s[1] = (unsigned)(t >> 32); }
+    ptx::cluster_sync_all();
+    if (ptx::cluster_ctarank() == 0 && threadIdx.x < 32) {
+        long long v = 0;
+        if (threadIdx.x < kDistCluster) {
+            const unsigned at = ptx::mapa(ptx::smem_u32(sum_s), threadIdx.x);
+            v = (long long)ptx::ld_shared_cluster(at) | (long long)ptx::ld_shared_cluster(at + 4) << 32;
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (threadIdx.x == 0) *out = v;
     }
+    ptx::cluster_sync_all();   // read: the others may leave
 }
 
 // ---------------------------------------------------------------------------------- host: operators
@@ -276,10 +306,34 @@ extern "C" int flexiq_sq_distance_i8(const int8_t *A_dev, const int8_t *B_dev, i
     int rc = check_device_sm100();
     if (rc) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    FLEXIQ_CUDA_TRY(cudaMemsetAsync(out_dev, 0, sizeof(int64_t), st));
-    if (n == 0) return FLEXIQ_OK;
     int dev = 0;
     FLEXIQ_CUDA_TRY(cudaGetDevice(&dev));
+    if (n <= kDistClusterMax && n > 0) {
+        static bool attr_set[64] = {};
+        if (dev >= 64 || !attr_set[dev]) {
+            FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(sq_distance_i8_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(sq_distance_i8_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDistSmem));
+            if (dev < 64) attr_set[dev] = true;
+        }
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kDistCluster, 1, 1);
+        cfg.blockDim = dim3(kDistThreads, 1, 1);
+        cfg.dynamicSmemBytes = kDistSmem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kDistCluster;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        FLEXIQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, sq_distance_i8_cluster_kernel, A_dev, B_dev, (long long)n, reinterpret_cast<long long *>(out_dev)));
+        return FLEXIQ_OK;
+    }
+    FLEXIQ_CUDA_TRY(cudaMemsetAsync(out_dev, 0, sizeof(int64_t), st));
+    if (n == 0) return FLEXIQ_OK;
     const int sms = device_sm_count(dev);
     const int threads = 256;
     long long blocks = ((n >> 4) + 4 * threads - 1) / (4 * threads);

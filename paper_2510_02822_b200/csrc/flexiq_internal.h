@@ -157,4 +157,31 @@ int encode_weight_maps(Layer *L);
                                        cudaGetErrorString(e__));                      \
     } while (0)
 
+// Dynamic shared memory with which no SM takes more than its share of a grid.  A GEMM releases the launch behind it while some of
+// its CTAs still run; blocks go where there is room, so without this the SMs that are free first take as many as fit and
+// the others, when they come free, what is left.
+inline size_t even_share_smem(long long blocks, long long sms)
+{
+    const long long share = (blocks + sms - 1) / sms;
+    return (size_t)(228 * 1024 / (share + 1)) - 1024;   // (an SM's 228 KB; each block takes 1 KB and the static part besides)
+}
+
+// Launch with programmatic stream serialization allowed: the kernel may start before its predecessor in the stream has
+// ended and waits for it itself (ptx::pdl_wait).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 blocks, unsigned threads, size_t smem, cudaStream_t st, const Args &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = blocks;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 }  // namespace flexiq

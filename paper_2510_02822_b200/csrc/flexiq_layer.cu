@@ -3,6 +3,8 @@
 // 4-bit weights (Sec. 7), and the run-time ratio knob max_4bit_ch (Sec. 7).
 #include "flexiq_internal.h"
 
+#include "sm100_ptx.cuh"
+
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -202,6 +204,9 @@ struct PrepArgs {
     uint8_t *w4;
     int w4_pitch;
     uint8_t *sw;
+    // linear layers: the straddle block (straddle.cuh) of the max_4bit_ch in force, NULL where that needs none
+    int8_t *wst;
+    int st_blk0, BK, K_lo;
 };
 
 // bytes with their sign folded away (v >= 0 ? v : ~v): the OR of a range's folded values has the bit length of the
@@ -256,9 +261,12 @@ __device__ __forceinline__ void write_tables(const PrepArgs &a, const InlineOrde
 // channels of 4 output channels, so that 16 lanes cover 64 contiguous bytes of a row.  64 and not 128 output channels: 288 blocks
 // instead of 144 for 768 x 3072, and 18 for 384 x 384.
 constexpr int kPrepN = 64, kPrepChunks = 8;
+constexpr int kPrepStatic = 9 * 1024, kPrepSmem = 228 * 1024 / 2 - 1024;   // the kernel's own shared memory, rounded up; what it asks for at most
 __global__ void __launch_bounds__(kPrepN / 4 * kPrepChunks)
 prep_linear_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ InlineOrder order)
 {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();   // what runs before may still read the previous layout, or write Wq
     __shared__ uint4 tile[kPrepN * kPrepChunks];      // [n][chunk ^ (n / 4)]: neither the writes nor the reads share a bank
     __shared__ uint32_t fold_s[kPrepChunks][kPrepN / 4];
     const int quad = threadIdx.x % (kPrepN / 4), chunk = threadIdx.x / (kPrepN / 4);
@@ -314,11 +322,19 @@ prep_linear_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ I
         const int u = threadIdx.x + it * (kPrepN / 4 * kPrepChunks);
         const int nl = u / kPrepChunks, ch = u % kPrepChunks;
         const int n = blockIdx.x * kPrepN + nl, c = blockIdx.y * kPrepChunks + ch;
-        if (n < a.N && c < a.C / 16) {
-            const uint4 v = tile[nl * kPrepChunks + (ch ^ ((nl >> 2) & 7))];
+        const bool here = n < a.N && c < a.C / 16;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        uint32_t mask = 0;
+        if (here) {
+            v = tile[nl * kPrepChunks + (ch ^ ((nl >> 2) & 7))];
             const int s = (int)((fold_s[ch][nl >> 2] >> (8 * (nl & 3))) & 0xffu);
             write_forms(a, (long long)n * a.C, (long long)n * a.w4_pitch, c * 16, v, s);
+            mask = c * 16 < a.K_lo ? ((0xffu << s) & 0xffu) * 0x01010101u : 0xffffffffu;
         }
+        // the block that max_4bit_ch falls into, from the same registers: channels below it masked, zeros beyond C
+        const int col = c * 16 - a.st_blk0;
+        if (a.wst != nullptr && n < a.N && col >= 0 && col < a.BK)
+            *reinterpret_cast<uint4 *>(a.wst + (long long)n * a.BK + col) = make_uint4(v.x & mask, v.y & mask, v.z & mask, v.w & mask);
     }
 }
 
@@ -328,6 +344,8 @@ prep_linear_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ I
 constexpr int kPrepGroups = 2048;   // groups per window: bounds the shared memory; one window up to 32,768 channels
 __global__ void __launch_bounds__(256) prep_conv_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ InlineOrder order, int nb)
 {
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();   // as above
     extern __shared__ uint32_t prep_s[];                // folded OR [nb][window], then the window's order
     const int g0 = blockIdx.y * kPrepGroups, n_g = min(kPrepGroups, a.C / a.G - g0);
     const int cpg = a.G / 16, n_c16 = n_g * cpg, units = a.T * n_c16;
@@ -374,8 +392,16 @@ static cudaError_t launch_prep(const Layer *L, const PrepArgs &a, const InlineOr
 {
     if (!L->is_conv) {
         const dim3 grid((a.N + kPrepN - 1) / kPrepN, (a.C / 16 + kPrepChunks - 1) / kPrepChunks);
-        prep_linear_kernel<<<grid, kPrepN / 4 * kPrepChunks, 0, stream>>>(a, order);
-        return cudaGetLastError();
+        // spread evenly over the SMs: it is launched while the GEMM before it still runs on most of them
+        static bool attr_set[64] = {};
+        if (L->device >= 64 || !attr_set[L->device]) {
+            const cudaError_t e = cudaFuncSetAttribute(prep_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepSmem);
+            if (e != cudaSuccess) return e;
+            if (L->device < 64) attr_set[L->device] = true;
+        }
+        size_t smem = even_share_smem((long long)grid.x * grid.y, device_sm_count(L->device));
+        smem = smem > kPrepStatic ? smem - kPrepStatic : 0;
+        return launch_pdl(prep_linear_kernel, grid, kPrepN / 4 * kPrepChunks, smem, stream, a, order);
     }
     // as many output channels per block as give every thread a chunk, but blocks enough for the machine
     const int sms = device_sm_count(L->device), window = L->n_g < kPrepGroups ? L->n_g : kPrepGroups;
@@ -383,8 +409,7 @@ static cudaError_t launch_prep(const Layer *L, const PrepArgs &a, const InlineOr
     if (nb > (a.N + sms - 1) / sms) nb = (a.N + sms - 1) / sms;
     if (nb < 1) nb = 1;
     const dim3 grid((a.N + nb - 1) / nb, (L->n_g + kPrepGroups - 1) / kPrepGroups);
-    prep_conv_kernel<<<grid, 256, sizeof(uint32_t) * (size_t)(nb + 1) * window, stream>>>(a, order, nb);
-    return cudaGetLastError();
+    return launch_pdl(prep_conv_kernel, grid, 256, sizeof(uint32_t) * (size_t)(nb + 1) * window, stream, a, order, nb);
 }
 
 static int validate_perm(const int32_t *perm, int n_g)
@@ -460,6 +485,13 @@ static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const u
     a.perm = L->perm; a.inv_perm = L->inv_perm; a.chunk_ent = L->chunk_ent; a.chunk_ent_slab = L->chunk_ent_slab; a.sx = L->sx;
     a.w8 = L->w8; a.w8m = L->w8m; a.w4 = L->w4; a.w4_pitch = L->w4_pitch; a.sw = L->sw;
     a.inline_order = n_g <= kInlineGroups;
+    a.K_lo = L->K_lo;
+    const bool straddle = !L->is_conv && straddle_in_use(L);
+    if (straddle) {
+        a.wst = L->wst;
+        a.BK = choose_bk(L);
+        a.st_blk0 = L->K_lo / a.BK * a.BK;
+    }
     if (a.inline_order) {
         for (int j = 0; j < n_g; ++j) {
             order.perm[j] = (uint16_t)perm[j];
@@ -488,6 +520,7 @@ static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const u
     FLEXIQ_CUDA_TRY(launch_prep(L, a, order, stream));
     L->st_K_lo = -1;   // the straddle block was cut from the previous order's weights
     L->st_cap_id = 0;
+    if (straddle) straddle_written(L, stream);   // ... and this layout has cut it again
     const unsigned long long cap = stream_capture_id(stream);
     if (cap) { L->weights_cap_id = cap; L->weights_graph_seen = L->st_graph_seen = 1; }   // a replay makes both stale unseen
     else L->weights_fresh = 1;

@@ -549,23 +549,6 @@ static int static_scratch_address(unsigned **out)
     return FLEXIQ_OK;
 }
 
-// Launch with programmatic stream serialization allowed (see pdl_wait in the kernels).
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks, 1, 1);
-    cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
 // The plan of the layer's scale (plan_quotient takes about half a microsecond for 16-bit inputs), one per input type.
 static QuotientPlan quotient_plan(Layer *L, float S, int dtype)
 {
@@ -575,15 +558,6 @@ static QuotientPlan quotient_plan(Layer *L, float S, int dtype)
         k = Layer::Quotient{S, p.form, p.r_hi, p.r_lo};
     }
     return QuotientPlan{k.form, k.r_hi, k.r_lo};
-}
-
-// Dynamic shared memory with which no SM takes more than its share of a grid.  A GEMM releases the prologue behind it while some of
-// its CTAs still run; blocks go where there is room, so without this the SMs that are free first take as many as fit and
-// the others, when they come free, what is left.
-static size_t even_share_smem(long long blocks, long long sms)
-{
-    const long long share = (blocks + sms - 1) / sms;
-    return (size_t)(228 * 1024 / (share + 1)) - 1024;   // (an SM's 228 KB; each block takes 1 KB and the static part besides)
 }
 
 // The masked path's quantizing kernel, static (DYN = false) or phase 1 of the dynamic mode.

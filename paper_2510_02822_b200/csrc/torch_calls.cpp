@@ -363,8 +363,14 @@ PyObject *calls_select_groups(PyObject *self, PyObject *const *args, Py_ssize_t 
         for (Py_ssize_t g = 0; g < n_g; ++g)
             if (!flags.data()[g]) perm[(size_t)at++] = (int32_t)g;
         void *st = current_stream();
-        int rc = released([&] { return flexiq_layer_set_group_perm(c->h, static_cast<const int8_t *>(Wq), perm.data(), positions.data(), st); });
+        // the ratio first, so that the layout cuts the weight block that depends on it; a refused layout leaves both as they were
+        int before = 0;
+        int rc = flexiq_get_max_4bit_ch(c->h, &before);
         if (rc == FLEXIQ_OK) rc = flexiq_set_lowbit_ratio(c->h, (float)((double)low / (double)n_g));
+        if (rc == FLEXIQ_OK) {
+            rc = released([&] { return flexiq_layer_set_group_perm(c->h, static_cast<const int8_t *>(Wq), perm.data(), positions.data(), st); });
+            if (rc != FLEXIQ_OK) flexiq_set_lowbit_ratio(c->h, (float)((double)before / (double)c->K));
+        }
         return finish(rc, Py_NewRef(Py_None));
     });
 }

@@ -32,6 +32,15 @@ def test_sq_distance_is_exact(dev, n):
     assert int(out.item()) == int(((a - b) ** 2).sum())
 
 
+@pytest.mark.parametrize("n", [15, 16 * 8192 * 4 + 16, (2 << 20) - 1, 2 << 20, (2 << 20) + 1])   # one cluster, and beyond its largest tensor
+def test_sq_distance_of_either_form(dev, n):
+    g = torch.Generator(device=dev).manual_seed(n)
+    A, B = (torch.randint(-128, 128, (n,), generator=g, device=dev, dtype=torch.int8) for _ in range(2))
+    out = torch.full((2,), -5, dtype=torch.int64, device=dev)
+    fx.flexiq_sq_distance_i8(A, B, out[1:])
+    assert out.tolist() == [-5, int(((A.long() - B.long()) ** 2).sum())]
+
+
 def test_chain_fitness_matches_oracle(dev):
     layers, X, groups, y8 = helpers.tiny_stack(M=200, dims=(128, 192, 96))
     fit = gpu_ev.ChainFitness(layers, X, dev)

@@ -67,3 +67,27 @@ def test_layout_matches_oracle(shape, G, offset):
                 assert np.array_equal(acc.cpu().numpy().reshape(-1), ref.reshape(-1))
     fx.flexiq_check_status()
     L.close()
+
+
+@pytest.mark.parametrize("K, N, G", [(112, 48, 16), (144, 80, 16), (400, 64, 16), (192, 208, 64), (128, 16, 16)])
+def test_layout_cuts_the_block_of_the_ratio_in_force(K, N, G):
+    """A layout made at a ratio inside a K block: the weight block that holds both kinds of channels is the new order's, and a GEMM
+    that follows without another prologue reads it."""
+    dev = torch.device("cuda:0")
+    n_g = K // G
+    W, X = draw(700 + K, (K, N)), draw(701 + K, (70, K))
+    Wd, Xd, ones = torch.from_numpy(W).to(dev), torch.from_numpy(X).to(dev), torch.ones(N, device=dev)
+    sx = (np.arange(n_g) % 5).astype(np.uint8)
+    L = fx.Layer(Wd, ones, None, np.arange(n_g, dtype=np.int32), sx, G)
+    for low in range(n_g + 1):
+        perm = np.argsort(inputs.uniform(70 + low, 2, n_g), kind="stable").astype(np.int32)
+        flags = np.zeros(n_g, np.uint8)
+        flags[perm[:low]] = 1
+        L.select_groups(Wd, flags, sx)
+        order = np.concatenate([np.flatnonzero(flags), np.flatnonzero(flags == 0)]).astype(np.int32)
+        sw = oracle.weight_positions_linear(W, G, order)
+        x4, x8, _ = L.quantize_lower(Xd, 1.0)
+        acc = L.mixed_gemm(x4, x8, 70, 1.0, 1.0, fx.OUT_ACC_I32)
+        assert np.array_equal(acc.cpu().numpy(), oracle.mixed_gemm_acc(X, W, G, order, sx[order].copy(), sw, low)), low
+    fx.flexiq_check_status()
+    L.close()
