@@ -295,6 +295,9 @@ int flexiq_mixed_conv_to_slab(flexiq_layer_t layer, const uint8_t *X4_dev, const
  *     unused_hist_dev [5] number of channels with 0, 1, 2, 3, >= 4 unused magnitude bits (Sec. 8.4)
  *   perm_dev and x_shift_dev, copied to the host, are the group_perm_host / x_shift_host of
  *   flexiq_layer_create_*.
+ * flexiq_calib_static: channel ranges (of one batch, or with hist_dev from its histogram and `tail`), weight ranges and
+ *   preparation of a layer in one launch.  work_dev: [3 K + 1] int32, receives lo | hi | wmax and a scratch word; perm and
+ *   x_shift may also lie in page-locked host memory that the device can write.  Same results and refusals as the calls it stands for.
  * flexiq_calib_absmax_ema: activation range across batches by exponential moving average
  *   (Sec. 7: momentum 0.99).  state_dev: 4 floats, zeroed by the caller before the first batch;
  *   after each call state_dev[0] = momentum * previous + (1 - momentum) * max|x| of this batch
@@ -312,6 +315,9 @@ int flexiq_calib_weight_absmax(const int8_t *Wq_dev, int is_conv, int K, int N, 
 int flexiq_calib_prepare(const int32_t *lo_dev, const int32_t *hi_dev, const int32_t *wmax_dev, int K,
                          int group_size, int32_t *perm_dev, uint8_t *x_shift_dev, int64_t *score_dev,
                          int32_t *unused_hist_dev, void *stream);
+int flexiq_calib_static(const void *X_dev, int x_dtype, int64_t M, float x_scale, const uint32_t *hist_dev, int64_t tail, int K,
+                        const int8_t *Wq_dev, int is_conv, int N, int taps, int group_size, int32_t *work_dev, int32_t *perm,
+                        uint8_t *x_shift, int64_t *score_dev, int32_t *unused_hist_dev, void *stream);
 int flexiq_calib_absmax_ema(const void *X_dev, int x_dtype, int64_t count, float momentum,
                             float *state_dev, void *stream);
 

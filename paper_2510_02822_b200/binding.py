@@ -27,7 +27,7 @@ EXPORTS = [
     "flexiq_x4_pitch", "flexiq_quantize_lower", "flexiq_quantize_lower_dynamic_noalloc", "flexiq_mixed_gemm", "flexiq_mixed_conv",
     "flexiq_mixed_gemm_to_slab", "flexiq_mixed_conv_to_slab", "flexiq_reorder_channels",
     "flexiq_calib_channel_ranges", "flexiq_calib_channel_histogram", "flexiq_calib_ranges_from_histogram",
-    "flexiq_calib_weight_absmax", "flexiq_calib_prepare", "flexiq_calib_absmax_ema",
+    "flexiq_calib_weight_absmax", "flexiq_calib_prepare", "flexiq_calib_static", "flexiq_calib_absmax_ema",
     "flexiq_controller_create", "flexiq_controller_destroy", "flexiq_controller_level", "flexiq_controller_update",
     "flexiq_serving_simulate", "flexiq_evo_init", "flexiq_evo_next_generation", "flexiq_sq_distance_i8",
     "flexiq_layer_export", "flexiq_layer_early_loads", "flexiq_selftest_wait_expiry", "flexiq_selftest_copy_drain", "flexiq_force_tile", "flexiq_choose_tile", "flexiq_choose_conv_kind", "flexiq_check_status", "flexiq_last_error",

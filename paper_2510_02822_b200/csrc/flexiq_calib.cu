@@ -22,14 +22,13 @@ __device__ __forceinline__ void load8(const void *p, float x[8])
 // memory, then one global atomic per channel of the window.
 constexpr int kCalibWindow = 256;
 template <int DTYPE>
-__global__ void calib_ranges_kernel(const void *__restrict__ X, long long M, int K, float S, int slices,
-                                    int32_t *__restrict__ lo, int32_t *__restrict__ hi)
+__device__ __forceinline__ void ranges_block(int block, const void *__restrict__ X, long long M, int K, float S, int slices, int *lo_s, int *hi_s,
+                                             int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
-    __shared__ int lo_s[kCalibWindow], hi_s[kCalibWindow];
     lo_s[threadIdx.x] = 0;
     hi_s[threadIdx.x] = 0;
     __syncthreads();
-    const int win = blockIdx.x / slices, slice = blockIdx.x - win * slices;
+    const int win = block / slices, slice = block - win * slices;
     const int chunk = threadIdx.x & 15, rlane = threadIdx.x >> 4;
     const int c0 = win * kCalibWindow + 16 * chunk;
     const Divider div = make_divider(S);
@@ -125,6 +124,14 @@ __global__ void calib_ranges_kernel(const void *__restrict__ X, long long M, int
     }
 }
 
+template <int DTYPE>
+__global__ void calib_ranges_kernel(const void *__restrict__ X, long long M, int K, float S, int slices,
+                                    int32_t *__restrict__ lo, int32_t *__restrict__ hi)
+{
+    __shared__ int lo_s[kCalibWindow], hi_s[kCalibWindow];
+    ranges_block<DTYPE>(blockIdx.x, X, M, K, S, slices, lo_s, hi_s, lo, hi);
+}
+
 // Per-channel histogram of the Eq. 1-quantized activations (256 bins, bin = q + 128), the input of
 // coverage-based ranges (Sec. 8.4: ranges that cover 99 % of a channel's values).  A block owns 32
 // channels and a slice of the rows and counts in shared memory; one global atomic per non-empty bin.
@@ -164,11 +171,9 @@ __global__ void calib_hist_kernel(const void *__restrict__ X, long long M, int K
 // contain zero (lo <= 0 <= hi).  tail = 0 gives the exact min / max.  One warp per channel, eight bins per lane: the
 // ends are where the running sums from either side first pass `tail` (a thread walking a channel's 256 bins one after the
 // other took 31 us whatever the number of channels).
-__global__ void ranges_from_hist_kernel(const unsigned *__restrict__ hist, int K, long long tail, int32_t *__restrict__ lo,
-                                        int32_t *__restrict__ hi)
+__device__ __forceinline__ void range_from_hist(int c, int lane, const unsigned *__restrict__ hist, long long tail, int32_t *__restrict__ lo,
+                                                int32_t *__restrict__ hi)
 {
-    const int c = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (c >= K) return;
     const unsigned *h = hist + (size_t)c * 256 + 8 * lane;
     unsigned n[8];
     long long mine = 0;
@@ -198,6 +203,12 @@ __global__ void ranges_from_hist_kernel(const unsigned *__restrict__ hist, int K
     u = __reduce_max_sync(0xffffffffu, u);
     if (lane == 0) { lo[c] = l; hi[c] = u; }
 }
+__global__ void ranges_from_hist_kernel(const unsigned *__restrict__ hist, int K, long long tail, int32_t *__restrict__ lo,
+                                        int32_t *__restrict__ hi)
+{
+    const int c = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (c < K) range_from_hist(c, threadIdx.x & 31, hist, tail, lo, hi);
+}
 
 // Largest |w| over the output channels (and taps) of every input channel, sixteen weights per load where the rows
 // allow it (16-byte alignment, a row length that is a multiple of 16), else one.  Byte loads alone took 9.5 us for 768 x 3072 and
@@ -209,10 +220,8 @@ __device__ __forceinline__ int max_byte(unsigned w)
 }
 // Linear weights [K][N]: one warp per input channel (row).
 template <bool WIDE>
-__global__ void weight_absmax_rows_kernel(const int8_t *__restrict__ W, int K, int N, int32_t *__restrict__ wmax)
+__device__ __forceinline__ void absmax_row(int row, int lane, const int8_t *__restrict__ W, int N, int32_t *__restrict__ wmax)
 {
-    const int row = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (row >= K) return;
     const int8_t *w = W + (size_t)row * N;
     int best = 0;
     if (WIDE) {
@@ -229,31 +238,42 @@ __global__ void weight_absmax_rows_kernel(const int8_t *__restrict__ W, int K, i
     best = __reduce_max_sync(0xffffffffu, best);
     if (lane == 0) wmax[row] = best;
 }
+template <bool WIDE>
+__global__ void weight_absmax_rows_kernel(const int8_t *__restrict__ W, int K, int N, int32_t *__restrict__ wmax)
+{
+    const int row = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (row < K) absmax_row<WIDE>(row, threadIdx.x & 31, W, N, wmax);
+}
 // Convolution weights [rows = Cout*R*S][Cin]: a thread per input channel (or sixteen of them), rows split over blockIdx.y and
 // in the wide form over the block's sixteen row lanes.
+// The wide form: block (bx, by) of 256 threads, by one of `gy`.
+__device__ __forceinline__ void absmax_cols_block(int bx, int by, int gy, const int8_t *__restrict__ W, long long rows, int C, int *best_s, int32_t *__restrict__ wmax)
+{
+    best_s[threadIdx.x] = 0;
+    __syncthreads();
+    const int chunk = threadIdx.x & 15, c0 = (bx * 16 + chunk) * 16;
+    if (c0 < C) {
+        unsigned b[4] = {0, 0, 0, 0};
+        for (long long r = (long long)by * 16 + (threadIdx.x >> 4); r < rows; r += (long long)gy * 16) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(W + (size_t)r * C + c0));
+            b[0] = absmax4(b[0], v.x); b[1] = absmax4(b[1], v.y); b[2] = absmax4(b[2], v.z); b[3] = absmax4(b[3], v.w);
+        }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int v = (int)((b[i >> 2] >> (8 * (i & 3))) & 0xffu);
+            if (v) atomicMax(&best_s[chunk * 16 + i], v);
+        }
+    }
+    __syncthreads();
+    const int c = bx * 256 + threadIdx.x;
+    if (c < C && best_s[threadIdx.x] > 0) atomicMax(&wmax[c], best_s[threadIdx.x]);
+}
 template <bool WIDE>
 __global__ void weight_absmax_cols_kernel(const int8_t *__restrict__ W, long long rows, int C, int32_t *__restrict__ wmax)
 {
     if (WIDE) {
         __shared__ int best_s[256];
-        best_s[threadIdx.x] = 0;
-        __syncthreads();
-        const int chunk = threadIdx.x & 15, c0 = (blockIdx.x * 16 + chunk) * 16;
-        if (c0 < C) {
-            unsigned b[4] = {0, 0, 0, 0};
-            for (long long r = (long long)blockIdx.y * 16 + (threadIdx.x >> 4); r < rows; r += (long long)gridDim.y * 16) {
-                const uint4 v = __ldg(reinterpret_cast<const uint4 *>(W + (size_t)r * C + c0));
-                b[0] = absmax4(b[0], v.x); b[1] = absmax4(b[1], v.y); b[2] = absmax4(b[2], v.z); b[3] = absmax4(b[3], v.w);
-            }
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int v = (int)((b[i >> 2] >> (8 * (i & 3))) & 0xffu);
-                if (v) atomicMax(&best_s[chunk * 16 + i], v);
-            }
-        }
-        __syncthreads();
-        const int c = blockIdx.x * 256 + threadIdx.x;
-        if (c < C && best_s[threadIdx.x] > 0) atomicMax(&wmax[c], best_s[threadIdx.x]);
+        absmax_cols_block(blockIdx.x, blockIdx.y, gridDim.y, W, rows, C, best_s, wmax);
         return;
     }
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -332,6 +352,80 @@ __global__ void __launch_bounds__(1024) calib_prepare_kernel(const int32_t *__re
     if (threadIdx.x < 5) hist[threadIdx.x] = hist_s[threadIdx.x];
 }
 
+// The static preparation of a layer in one launch: the blocks in front take the weights' ranges, the others the activations'
+// (from the rows, or with HIST from their histogram, a warp per channel), and the block that finishes last does what
+// calib_prepare_kernel does, from the tables the others have left in L2.  perm and x_shift may lie in mapped host memory: the
+// stream's end is then all that the host waits for.
+constexpr int kStaticGroups = 512;   // the last block ranks them with 256 threads
+struct StaticArgs {
+    const void *X;                   // or the histogram
+    long long M, tail;
+    int K, G;
+    float S;
+    int slices;
+    const int8_t *W;
+    int is_conv, N;
+    long long w_rows;
+    int w_blocks, w_gx, w_gy;
+    int32_t *lo, *hi, *wmax;
+    unsigned *done;                  // blocks that have finished, cleared beforehand
+    int32_t *perm;
+    uint8_t *x_shift;
+    long long *score;
+    int32_t *unused;
+};
+template <int DTYPE, bool HIST>
+__global__ void __launch_bounds__(kCalibWindow) calib_static_kernel(const __grid_constant__ StaticArgs a)
+{
+    __shared__ int lo_s[kCalibWindow], hi_s[kCalibWindow], hist_s[5], last_s;
+    __shared__ unsigned long long score_s[kStaticGroups];
+    __shared__ int bits_s[kStaticGroups];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, block = (int)blockIdx.x - a.w_blocks;
+    if (block < 0) {
+        if (a.is_conv) absmax_cols_block(blockIdx.x % a.w_gx, blockIdx.x / a.w_gx, a.w_gy, a.W, a.w_rows, a.K, lo_s, a.wmax);
+        else {
+            const int row = (int)blockIdx.x * (kCalibWindow / 32) + warp;
+            if (row < a.K) absmax_row<true>(row, lane, a.W, a.N, a.wmax);
+        }
+    } else if (HIST) {
+        const int c = block * (kCalibWindow / 32) + warp;
+        if (c < a.K) range_from_hist(c, lane, static_cast<const unsigned *>(a.X), a.tail, a.lo, a.hi);
+    } else {
+        ranges_block<DTYPE>(block, a.X, a.M, a.K, a.S, a.slices, lo_s, hi_s, a.lo, a.hi);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last_s = atomicAdd(a.done, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (!last_s) return;
+    __threadfence();
+    const int n_g = a.K / a.G;
+    if (threadIdx.x < 5) hist_s[threadIdx.x] = 0;
+    for (int g = threadIdx.x; g < n_g; g += blockDim.x) { score_s[g] = 0; bits_s[g] = 0; }
+    __syncthreads();
+    for (int c = threadIdx.x; c < a.K; c += blockDim.x) {
+        const int l = __ldcg(a.lo + c), h = __ldcg(a.hi + c), L = used_bits(l, h);
+        const long long v = (long long)max(h, -l) * (long long)__ldcg(a.wmax + c);
+        if (L) atomicMax(&bits_s[c / a.G], L);
+        if (v > 0) atomicMax(&score_s[c / a.G], (unsigned long long)v);
+        atomicAdd(&hist_s[min(4, 7 - L)], 1);
+    }
+    __syncthreads();
+    for (int g = threadIdx.x; g < n_g; g += blockDim.x) {
+        const unsigned long long s = score_s[g];
+        int rank = 0;
+        for (int o = 0; o < n_g; ++o) {
+            const unsigned long long so = score_s[o];
+            rank += (so < s) || (so == s && o < g);
+        }
+        const int L = bits_s[g];
+        a.perm[rank] = g;
+        a.x_shift[g] = (uint8_t)(L > 3 ? L - 3 : 0);
+        a.score[g] = (long long)s;
+    }
+    if (threadIdx.x < 5) a.unused[threadIdx.x] = hist_s[threadIdx.x];
+}
+
 // Activation range by exponential moving average (Sec. 7): absmax of the batch, then
 // state[0] <- momentum * state[0] + (1 - momentum) * absmax (the first batch initialises it).
 // state = { ema, batches seen, scratch (absmax bits), unused }.
@@ -358,14 +452,26 @@ __global__ void ema_update_kernel(float *state, float momentum)
     state[2] = 0.f;
 }
 
+// wide form of the convolution weights' ranges: four rows a lane, two blocks per SM
+static dim3 cols_grid(int C, long long rows)
+{
+    const unsigned gx = (unsigned)((C + 255) / 256), most = gx < 296 ? 296 / gx : 1;
+    const long long want = (rows + 63) / 64;
+    return dim3(gx, want < (long long)most ? (unsigned)want : most);
+}
+// about three blocks per SM: few, long-lived blocks amortise the merge (fewer rows than lanes leave lanes idle, nothing more)
+static int range_slices(long long M, int K, int sms)
+{
+    const int windows = (K + kCalibWindow - 1) / kCalibWindow;
+    const long long slices = ((long long)sms * 3 + windows - 1) / windows, most = (M + 15) / 16;
+    return (int)(slices < most ? slices : most);
+}
 template <int DTYPE>
 static int launch_ranges(const void *X, long long M, int K, float S, int32_t *lo, int32_t *hi, int sms, cudaStream_t st)
 {
     const int windows = (K + kCalibWindow - 1) / kCalibWindow;
-    long long slices = ((long long)sms * 3 + windows - 1) / windows;   // about three blocks per SM: few, long-lived blocks amortise the merge
-    const long long max_slices = (M + 15) / 16;   // (fewer rows than lanes leave lanes idle, nothing more)
-    if (slices > max_slices) slices = max_slices;
-    calib_ranges_kernel<DTYPE><<<(unsigned)(windows * slices), kCalibWindow, 0, st>>>(X, M, K, S, (int)slices, lo, hi);
+    const int slices = range_slices(M, K, sms);
+    calib_ranges_kernel<DTYPE><<<(unsigned)(windows * slices), kCalibWindow, 0, st>>>(X, M, K, S, slices, lo, hi);
     FLEXIQ_CUDA_TRY(cudaGetLastError());
     return FLEXIQ_OK;
 }
@@ -461,9 +567,8 @@ extern "C" int flexiq_calib_weight_absmax(const int8_t *Wq_dev, int is_conv, int
         FLEXIQ_CUDA_TRY(cudaMemsetAsync(wmax_dev, 0, sizeof(int32_t) * K, st));
         const long long rows = (long long)N * taps;
         if (K % 16 == 0 && (reinterpret_cast<uintptr_t>(Wq_dev) & 15) == 0) {
-            const unsigned gx = (unsigned)((K + 255) / 256), most = gx < 296 ? 296 / gx : 1;   // four rows a lane, two blocks per SM
-            const long long want = (rows + 63) / 64;
-            weight_absmax_cols_kernel<true><<<dim3(gx, want < (long long)most ? (unsigned)want : most), 256, 0, st>>>(Wq_dev, rows, K, wmax_dev);
+            const dim3 grid = cols_grid(K, rows);
+            weight_absmax_cols_kernel<true><<<grid, 256, 0, st>>>(Wq_dev, rows, K, wmax_dev);
         } else {
             const unsigned gy = (unsigned)(rows < 64 ? rows : 64);
             weight_absmax_cols_kernel<false><<<dim3((K + 127) / 128, gy), 128, 0, st>>>(Wq_dev, rows, K, wmax_dev);
@@ -488,6 +593,58 @@ extern "C" int flexiq_calib_prepare(const int32_t *lo_dev, const int32_t *hi_dev
     long long *score = reinterpret_cast<long long *>(score_dev);
     if (K / group_size <= kPrepareShared) calib_prepare_kernel<true><<<1, 1024, 0, st>>>(lo_dev, hi_dev, wmax_dev, K, group_size, perm_dev, x_shift_dev, score, unused_hist_dev);
     else calib_prepare_kernel<false><<<1, 1024, 0, st>>>(lo_dev, hi_dev, wmax_dev, K, group_size, perm_dev, x_shift_dev, score, unused_hist_dev);
+    FLEXIQ_CUDA_TRY(cudaGetLastError());
+    return FLEXIQ_OK;
+}
+
+extern "C" int flexiq_calib_static(const void *X_dev, int x_dtype, int64_t M, float x_scale, const uint32_t *hist_dev, int64_t tail, int K,
+                                   const int8_t *Wq_dev, int is_conv, int N, int taps, int group_size, int32_t *work_dev, int32_t *perm,
+                                   uint8_t *x_shift, int64_t *score_dev, int32_t *unused_hist_dev, void *stream)
+{
+    if (K <= 0 || !work_dev) return set_error(FLEXIQ_ERR_INVALID_ARG, "K = %d must be positive, work_dev not NULL", K);
+    int32_t *lo = work_dev, *hi = lo + K, *wmax = hi + K;
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const bool group_ok = (group_size == 16 || group_size == 32 || group_size == 64) && K % group_size == 0;
+    const bool x_ok = hist_dev ? tail >= 0
+                               : X_dev && (reinterpret_cast<uintptr_t>(X_dev) & 15) == 0 && M > 0 && x_dtype >= FLEXIQ_DTYPE_F32 && x_dtype <= FLEXIQ_DTYPE_I8 &&
+                                     (x_dtype == FLEXIQ_DTYPE_I8 || x_scale > 0.0f);
+    const bool w_ok = Wq_dev && (reinterpret_cast<uintptr_t>(Wq_dev) & 15) == 0 && N > 0 && (is_conv ? taps > 0 : N % 16 == 0);
+    if (!(group_ok && x_ok && w_ok && K / group_size <= kStaticGroups && perm && x_shift && score_dev && unused_hist_dev)) {
+        // what the one launch does not take, and what is refused: the calls it stands for, one after the other
+        int rc = hist_dev ? flexiq_calib_ranges_from_histogram(hist_dev, K, tail, lo, hi, stream)
+                          : flexiq_calib_channel_ranges(X_dev, x_dtype, M, K, x_scale, 0, lo, hi, stream);
+        if (rc == FLEXIQ_OK) rc = flexiq_calib_weight_absmax(Wq_dev, is_conv, K, N, taps, wmax, stream);
+        if (rc == FLEXIQ_OK) rc = flexiq_calib_prepare(lo, hi, wmax, K, group_size, perm, x_shift, score_dev, unused_hist_dev, stream);
+        return rc;
+    }
+    int rc = check_device_sm100();
+    if (rc) return rc;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int sms = device_sm_count(dev);
+    StaticArgs a{};
+    a.X = hist_dev ? static_cast<const void *>(hist_dev) : X_dev;
+    a.M = M; a.tail = tail; a.K = K; a.G = group_size; a.S = x_scale;
+    a.W = Wq_dev; a.is_conv = is_conv != 0; a.N = N; a.w_rows = (long long)N * (is_conv ? taps : 1);
+    const dim3 cols = cols_grid(K, a.w_rows);
+    a.w_gx = (int)cols.x; a.w_gy = (int)cols.y;
+    constexpr int kWarps = kCalibWindow / 32;
+    a.w_blocks = is_conv ? (int)(cols.x * cols.y) : (K + kWarps - 1) / kWarps;
+    a.lo = lo; a.hi = hi; a.wmax = wmax; a.done = reinterpret_cast<unsigned *>(wmax + K);
+    a.perm = perm; a.x_shift = x_shift; a.score = reinterpret_cast<long long *>(score_dev); a.unused = unused_hist_dev;
+    FLEXIQ_CUDA_TRY(cudaMemsetAsync(work_dev, 0, sizeof(int32_t) * (3 * (size_t)K + 1), st));
+    if (hist_dev) {
+        calib_static_kernel<FLEXIQ_DTYPE_I8, true><<<(unsigned)(a.w_blocks + (K + kWarps - 1) / kWarps), kCalibWindow, 0, st>>>(a);
+    } else {
+        a.slices = range_slices(M, K, sms);
+        const unsigned grid = (unsigned)(a.w_blocks + (K + kCalibWindow - 1) / kCalibWindow * a.slices);
+        switch (x_dtype) {
+            case FLEXIQ_DTYPE_F32: calib_static_kernel<FLEXIQ_DTYPE_F32, false><<<grid, kCalibWindow, 0, st>>>(a); break;
+            case FLEXIQ_DTYPE_F16: calib_static_kernel<FLEXIQ_DTYPE_F16, false><<<grid, kCalibWindow, 0, st>>>(a); break;
+            case FLEXIQ_DTYPE_BF16: calib_static_kernel<FLEXIQ_DTYPE_BF16, false><<<grid, kCalibWindow, 0, st>>>(a); break;
+            default: calib_static_kernel<FLEXIQ_DTYPE_I8, false><<<grid, kCalibWindow, 0, st>>>(a); break;
+        }
+    }
     FLEXIQ_CUDA_TRY(cudaGetLastError());
     return FLEXIQ_OK;
 }

@@ -437,9 +437,12 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
         const long long rows = X.size(0), C = X.size(1), n_g = C / G, step = (rows + batches - 1) / batches;
         if (C < 1 || C > INT32_MAX || n_g < 1) throw Refused{};
         const at::TensorOptions opt = at::TensorOptions().device(X.device());
-        const at::Tensor ranges = at::empty({2, C}, opt.dtype(at::kInt)), lo = ranges.select(0, 0), hi = ranges.select(0, 1);   // neighbours: one clear
-        const at::Tensor wmax = at::empty({C}, opt.dtype(at::kInt));
-        const at::Tensor order = at::empty({5 * n_g}, opt.dtype(at::kByte));   // perm int32 [n_g], then x_shift [n_g]: one copy to the host
+        const at::Tensor work = at::empty({3 * C + 1}, opt.dtype(at::kInt));
+        const at::Tensor lo = work.narrow(0, 0, C), hi = work.narrow(0, C, C), wmax = work.narrow(0, 2 * C, C);
+        // perm int32 [n_g], then x_shift [n_g]: page-locked, written by the device, so that the stream's end is all there is to wait for
+        const at::Tensor order = at::empty({5 * n_g}, at::TensorOptions().dtype(at::kByte).pinned_memory(true));
+        void *order_dev = nullptr;
+        if (cudaHostGetDevicePointer(&order_dev, order.data_ptr(), 0) != cudaSuccess) { cudaGetLastError(); throw Refused{}; }
         const at::Tensor score = at::empty({n_g}, opt.dtype(at::kLong)), unused = at::empty({5}, opt.dtype(at::kInt));
         at::Tensor hist;
         if (cover) hist = at::empty({C, 256}, opt.dtype(at::kInt));
@@ -449,11 +452,10 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
         const int N = (int)(conv ? Wq.size(0) : Wq.size(1)), taps = (int)(conv ? Wq.size(1) * Wq.size(2) : 1);
         int32_t *lo_p = lo.data_ptr<int32_t>(), *hi_p = hi.data_ptr<int32_t>(), *wmax_p = wmax.data_ptr<int32_t>();
         uint32_t *hist_p = cover ? reinterpret_cast<uint32_t *>(hist.data_ptr<int32_t>()) : nullptr;
-        int32_t *perm_p = static_cast<int32_t *>(order.data_ptr());
-        uint8_t *shift_p = static_cast<uint8_t *>(order.data_ptr()) + 4 * n_g;
+        int32_t *perm_p = static_cast<int32_t *>(order_dev);
+        uint8_t *shift_p = static_cast<uint8_t *>(order_dev) + 4 * n_g;
         const long long tail = cover ? (long long)((double)rows * (1.0 - PyFloat_AS_DOUBLE(args[6])) / 2.0) : 0;
         void *st = current_stream();
-        std::vector<char> host((size_t)(5 * n_g));
         PyObject *out[] = {THPVariable_Wrap(perm), THPVariable_Wrap(shift), THPVariable_Wrap(lo), THPVariable_Wrap(hi),
                            THPVariable_Wrap(wmax), THPVariable_Wrap(score), THPVariable_Wrap(unused)};
         PyObject *result = PyTuple_Pack(7, out[0], out[1], out[2], out[3], out[4], out[5], out[6]);
@@ -462,18 +464,22 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
         int cuda = 0;
         const int rc = released([&] {
             int r = FLEXIQ_OK;
-            for (long long b = 0; b < batches && r == FLEXIQ_OK; ++b) {
+            const bool rows_too = batches == 1 && !cover;   // one launch for everything
+            for (long long b = 0; b < batches && r == FLEXIQ_OK && !rows_too; ++b) {
                 const long long from = std::min(b * step, rows), part = std::min(step, rows - from);
                 const void *p = x + (size_t)from * C * X.element_size();
                 r = cover ? flexiq_calib_channel_histogram(p, dtype, part, (int)C, scale, b > 0, hist_p, st)
                           : flexiq_calib_channel_ranges(p, dtype, part, (int)C, scale, b > 0, lo_p, hi_p, st);
             }
-            if (r == FLEXIQ_OK && cover) r = flexiq_calib_ranges_from_histogram(hist_p, (int)C, tail, lo_p, hi_p, st);
-            if (r == FLEXIQ_OK) r = flexiq_calib_weight_absmax(w, conv, (int)C, N, taps, wmax_p, st);
-            if (r == FLEXIQ_OK) r = flexiq_calib_prepare(lo_p, hi_p, wmax_p, (int)C, (int)G, perm_p, shift_p, score.data_ptr<int64_t>(), unused.data_ptr<int32_t>(), st);
+            if (r == FLEXIQ_OK && (cover || rows_too)) {
+                r = flexiq_calib_static(x, dtype, rows, scale, hist_p, tail, (int)C, w, conv, N, taps, (int)G, lo_p, perm_p, shift_p,
+                                        score.data_ptr<int64_t>(), unused.data_ptr<int32_t>(), st);
+            } else if (r == FLEXIQ_OK) {
+                r = flexiq_calib_weight_absmax(w, conv, (int)C, N, taps, wmax_p, st);
+                if (r == FLEXIQ_OK) r = flexiq_calib_prepare(lo_p, hi_p, wmax_p, (int)C, (int)G, perm_p, shift_p, score.data_ptr<int64_t>(), unused.data_ptr<int32_t>(), st);
+            }
             if (r != FLEXIQ_OK) return r;
-            cuda = (int)cudaMemcpyAsync(host.data(), order.data_ptr(), host.size(), cudaMemcpyDeviceToHost, static_cast<cudaStream_t>(st));
-            if (!cuda) cuda = (int)cudaStreamSynchronize(static_cast<cudaStream_t>(st));
+            cuda = (int)cudaStreamSynchronize(static_cast<cudaStream_t>(st));
             return r;
         });
         if (rc == FLEXIQ_OK && cuda) {
@@ -482,8 +488,9 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
             PyErr_SetString(PyExc_RuntimeError, cudaGetErrorString((cudaError_t)cuda));
             return nullptr;
         }
-        std::copy(host.begin(), host.begin() + 4 * n_g, static_cast<char *>(perm.data_ptr()));
-        std::copy(host.begin() + 4 * n_g, host.end(), static_cast<char *>(shift.data_ptr()));
+        const char *host = static_cast<const char *>(order.data_ptr());
+        std::copy(host, host + 4 * n_g, static_cast<char *>(perm.data_ptr()));
+        std::copy(host + 4 * n_g, host + 5 * n_g, static_cast<char *>(shift.data_ptr()));
         return finish(rc, result);
     });
 }

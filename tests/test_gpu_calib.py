@@ -168,3 +168,32 @@ def test_coverage_that_is_no_number():
             calib.static_preparation_device(X, 0.1, W, 16, coverage=coverage)
     perm, x_shift, _ = calib.static_preparation_device(X, 0.1, W, 16, coverage=0.99)
     assert sorted(perm.tolist()) == [0, 1]
+
+
+@pytest.mark.parametrize("K,N,G,rows,shape,dtype,coverage,offset", [
+    (128, 128, 16, 256, "linear", torch.float32, None, 0), (272, 48, 16, 257, "linear", torch.float16, None, 0), (4096, 64, 64, 1000, "linear", torch.bfloat16, None, 0),
+    (512 * 16, 16, 16, 33, "linear", torch.int8, None, 0), (513 * 16, 16, 16, 33, "linear", torch.float32, None, 0),   # the most groups in one launch, and one more
+    (768, 80, 16, 300, "linear", torch.float32, None, 1), (256, 48, 32, 999, "conv", torch.float16, None, 0), (48, 16, 16, 5, "conv", torch.float32, None, 3),
+    (720, 1104, 16, 2000, "linear", torch.float32, 0.99, 0), (160, 32, 32, 500, "conv", torch.bfloat16, 0.9, 0)])
+def test_one_launch_equals_the_calls_it_stands_for(dev, K, N, G, rows, shape, dtype, coverage, offset):
+    g = torch.Generator(device=dev).manual_seed(K + rows)
+    X = torch.randn((rows, K), generator=g, device=dev) * torch.exp(torch.randn(K, generator=g, device=dev))
+    X = torch.clamp(X * 30, -128, 127).to(dtype) if dtype == torch.int8 else X.to(dtype)
+    size = (N, 3, 3, K) if shape == "conv" else (K, N)
+    raw = torch.randint(-128, 128, (int(np.prod(size)) + 16,), generator=g, device=dev, dtype=torch.int8)
+    W = raw[offset:offset + int(np.prod(size))].view(size)
+    perm, xs, info = calib.static_preparation_device(X, 0.05, W, G, conv=shape == "conv", coverage=coverage)
+    lo, hi, wmax = (torch.empty(K, dtype=torch.int32, device=dev) for _ in range(3))
+    if coverage is None:
+        fx.flexiq_calib_channel_ranges(X, fx._dtype_code(X), rows, K, 0.05, False, lo, hi)
+    else:
+        hist = torch.empty((K, 256), dtype=torch.int32, device=dev)
+        fx.flexiq_calib_channel_histogram(X, fx._dtype_code(X), rows, K, 0.05, False, hist)
+        fx.flexiq_calib_ranges_from_histogram(hist, K, int(rows * (1.0 - coverage) / 2.0), lo, hi)
+    fx.flexiq_calib_weight_absmax(W, shape == "conv", K, N, 9 if shape == "conv" else 1, wmax)
+    perm_e, xs_e = torch.empty(K // G, dtype=torch.int32, device=dev), torch.empty(K // G, dtype=torch.uint8, device=dev)
+    score, unused = torch.empty(K // G, dtype=torch.int64, device=dev), torch.empty(5, dtype=torch.int32, device=dev)
+    fx.flexiq_calib_prepare(lo, hi, wmax, K, G, perm_e, xs_e, score, unused)
+    assert np.array_equal(perm, perm_e.cpu().numpy()) and np.array_equal(xs, xs_e.cpu().numpy())
+    for name, want in (("lo", lo), ("hi", hi), ("wmax", wmax), ("score", score), ("unused_hist", unused)):
+        assert torch.equal(info[name], want), name
