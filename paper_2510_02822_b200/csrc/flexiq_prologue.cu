@@ -21,6 +21,13 @@ __device__ __forceinline__ int position_from_or(unsigned o)
     return used > 3 ? used - 3 : 0;
 }
 
+__global__ void clear_words_kernel(unsigned *words, int n)
+{
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) words[i] = 0;
+}
+
 // Phase 1 of the dynamic mode (Sec. 4.1): OR of the sign-folded quantized values of each
 // slab group over all rows.  A thread keeps one chunk column and walks rows; lanes that
 // hold the same group merge with a warp reduction, then one shared and one global atomic.
@@ -691,7 +698,8 @@ static int launch_prologue(Layer *L, const void *X, long long M, float S, int dy
     constexpr size_t elem = DTYPE == FLEXIQ_DTYPE_F32 ? 4 : (DTYPE == FLEXIQ_DTYPE_I8 ? 1 : 2);
     int col_rows = 0, col_window = 0;
     const bool columns = dynamic && masked && columns_fit(L, M, (int)elem, &col_rows, &col_window);
-    if (dynamic && !columns) FLEXIQ_CUDA_TRY(cudaMemsetAsync(scratch, 0, sizeof(unsigned) * L->n_g, st));
+    // a launch, not a memset: the kernel behind it may then start (and ask for its first rows) while the one before it ends
+    if (dynamic && !columns) FLEXIQ_CUDA_TRY(launch_pdl(clear_words_kernel, 1, 256, 0, st, scratch, L->n_g));
     if (masked && (columns || (size_t)K * elem <= kRowStageBytes)) {
         StraddleJob job{};
         if (straddle_in_use(L) && straddle_stale(L, st)) {
