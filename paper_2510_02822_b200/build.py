@@ -71,7 +71,7 @@ def _build_calls():
     include = [sysconfig.get_paths()["include"], *include_paths(), os.path.join(cuda, "include"), os.path.join(_ROOT, "include")]
     subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", *(f"-I{d}" for d in include), os.path.join(CSRC, "torch_calls.cpp"), "-o", CALLS,
                     f"-L{_DIR}", "-l:libflexiq.so", "-Wl,-rpath,$ORIGIN", *(f"-L{d}" for d in library_paths()), f"-L{os.path.join(cuda, 'lib64')}",
-                    "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-lcudart"], check=True)
+                    "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda", "-lcudart"], check=True)
     with open(CALLS_FOR, "w") as f:
         f.write(_calls_for())
 
