@@ -114,6 +114,10 @@ int flexiq_layer_destroy(flexiq_layer_t layer);
  * ratio in force is kept.  Slabs written for the previous order no longer fit the handle. */
 int flexiq_layer_set_group_perm(flexiq_layer_t layer, const int8_t *Wq_dev, const int32_t *group_perm_host,
                                 const uint8_t *x_shift_host, void *stream);
+/* The same for n different handles, with as few launches as their sizes allow (up to four linear layers of together 1024 groups in
+ * one).  The arguments are arrays of n; x_shift_host may be NULL, or hold NULLs.  Everything is checked before anything is enqueued. */
+int flexiq_layers_set_group_perm(int n, const flexiq_layer_t *layers, const int8_t *const *Wq_dev, const int32_t *const *group_perm_host,
+                                 const uint8_t *const *x_shift_host, void *stream);
 
 /* Chooses FLEXIQ_LOWBIT_MASKED_I8 (default) or FLEXIQ_LOWBIT_PACKED_U4 for the layer.
  * Must be the same for a flexiq_quantize_lower call and the mixed_* call that consumes

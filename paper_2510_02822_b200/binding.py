@@ -23,7 +23,7 @@ REORDER_TO_SLAB, REORDER_FROM_SLAB = 0, 1
 
 EXPORTS = [
     "flexiq_layer_create_linear", "flexiq_layer_create_conv", "flexiq_layer_destroy",
-    "flexiq_layer_set_group_perm", "flexiq_layer_set_lowbit_path", "flexiq_layer_sync_ratio", "flexiq_layer_set_slab_check", "flexiq_set_lowbit_ratio", "flexiq_get_max_4bit_ch",
+    "flexiq_layer_set_group_perm", "flexiq_layers_set_group_perm", "flexiq_layer_set_lowbit_path", "flexiq_layer_sync_ratio", "flexiq_layer_set_slab_check", "flexiq_set_lowbit_ratio", "flexiq_get_max_4bit_ch",
     "flexiq_x4_pitch", "flexiq_quantize_lower", "flexiq_quantize_lower_dynamic_noalloc", "flexiq_mixed_gemm", "flexiq_mixed_conv",
     "flexiq_mixed_gemm_to_slab", "flexiq_mixed_conv_to_slab", "flexiq_reorder_channels",
     "flexiq_calib_channel_ranges", "flexiq_calib_channel_histogram", "flexiq_calib_ranges_from_histogram",
@@ -367,13 +367,7 @@ class Layer:
 
     def select_groups(self, Wq, flags, x_shift):
         """set_group_perm with the flagged groups (uint8 [n_g]) first, in index order, and the ratio that makes exactly them low."""
-        import numpy as np
-        if self._calls is not None and self._calls.select_groups(Wq, flags, x_shift) is not NotImplemented:
-            return
-        f = np.asarray(flags).astype(bool)
-        idx = np.arange(f.size, dtype=np.int32)
-        self.set_group_perm(Wq, np.concatenate([idx[f], idx[~f]]), x_shift)
-        self.set_lowbit_ratio(int(f.sum()) / f.size)
+        select_groups([(self, Wq, flags, x_shift)])
 
     def sync_ratio(self):
         """Writes the ratio-dependent weight K block for the ratio in force on the current stream, if it is not there yet."""
@@ -469,6 +463,20 @@ class Layer:
             Y = torch.empty((Nb, P, Q, self.N), dtype=dt, device=self.device)
         flexiq_mixed_conv(self.h, x4, x8, x_shift, Nb, H, W, x_scale, y_scale, out_mode, Y)
         return Y
+
+
+def select_groups(selections):
+    """Layer.select_groups for several different layers, [(layer, Wq, flags, x_shift), ...], with fewer launches."""
+    import numpy as np
+    native = _native_calls()
+    if native is not None and all(s[0]._calls is not None for s in selections):
+        if native.select_groups([(layer._calls, *rest) for layer, *rest in selections]) is not NotImplemented:
+            return
+    for layer, Wq, flags, x_shift in selections:
+        f = np.asarray(flags).astype(bool)
+        idx = np.arange(f.size, dtype=np.int32)
+        layer.set_group_perm(Wq, np.concatenate([idx[f], idx[~f]]), x_shift)
+        layer.set_lowbit_ratio(int(f.sum()) / f.size)
 
 
 # ------------------------------------------------------------------ ratio controller and request queue (host only)

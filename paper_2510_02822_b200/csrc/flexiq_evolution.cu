@@ -64,8 +64,10 @@ __global__ void sq_distance_i8_kernel(const int8_t *__restrict__ A, const int8_t
 }
 
 // The same by one cluster of sixteen blocks, whose sums meet in the first one's shared memory: one launch, which may start while
-// the GEMM before it ends, and nothing cleared beforehand.  Larger tensors need more than sixteen SMs: the grid above and its clear.
-constexpr int kDistCluster = 16, kDistThreads = 512;
+// the GEMM before it ends, and nothing cleared beforehand.  Larger tensors need more than sixteen SMs: the grid above and its clear
+// (graph replay, clear and grid against this: 0.6 MB 6.0 and 3.4 us, 1.2 MB 6.0 and 4.4, 2 MB 5.9 and 4.7; with 512 threads a block 3 MB took
+// 8.1 where the grid takes 6.2).
+constexpr int kDistCluster = 16, kDistThreads = 1024;
 constexpr int kDistSmem = 228 * 1024 / 2 - 1024;   // one block per SM: the cluster is launched while the GEMM before it still runs on some
 constexpr long long kDistClusterMax = 2ll << 20;
 __global__ void __launch_bounds__(kDistThreads) sq_distance_i8_cluster_kernel(const int8_t *A, const int8_t *B, long long n, long long *out)

@@ -238,13 +238,13 @@ __device__ __forceinline__ void write_forms(const PrepArgs &a, long long row8, l
     *reinterpret_cast<uint4 *>(a.w8m + row8 + col) = make_uint4(w[0] & mask, w[1] & mask, w[2] & mask, w[3] & mask);
     *reinterpret_cast<uint2 *>(a.w4 + row4 + (col >> 1)) = make_uint2(__byte_perm(h[0], h[1], 0x6420), __byte_perm(h[2], h[3], 0x6420));
 }
-// the tables of an inline order, by one block
-__device__ __forceinline__ void write_tables(const PrepArgs &a, const InlineOrder &o)
+// the tables of an inline order that begins at `at`, by one block
+__device__ __forceinline__ void write_tables(const PrepArgs &a, const InlineOrder &o, int at)
 {
     const int n_g = a.C / a.G, cpg = a.G / 16;
     for (int j = threadIdx.x; j < n_g; j += blockDim.x) {
-        const int g = o.perm[j];
-        const int sx = o.sx[j];
+        const int g = o.perm[at + j];
+        const int sx = o.sx[at + j];
         a.perm[j] = g;
         a.inv_perm[g] = j;
         a.sx[j] = (uint8_t)sx;
@@ -262,22 +262,33 @@ __device__ __forceinline__ void write_tables(const PrepArgs &a, const InlineOrde
 // instead of 144 for 768 x 3072, and 18 for 384 x 384.
 constexpr int kPrepN = 64, kPrepChunks = 8;
 constexpr int kPrepStatic = 9 * 1024, kPrepSmem = 228 * 1024 / 2 - 1024;   // the kernel's own shared memory, rounded up; what it asks for at most
+// Several layers at once (a selection search lays a chain out per chromosome): a layer's blocks are too few to fill the machine, and
+// four launches of 3 us each stood before every chain.
+constexpr int kPrepLayers = 4;
+struct PrepMany {
+    PrepArgs a[kPrepLayers];
+    int n, first_block[kPrepLayers], first_group[kPrepLayers], nx[kPrepLayers];   // nx: blocks across the output channels
+};
 __global__ void __launch_bounds__(kPrepN / 4 * kPrepChunks)
-prep_linear_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ InlineOrder order)
+prep_linear_kernel(const __grid_constant__ PrepMany many, const __grid_constant__ InlineOrder order)
 {
     ptx::pdl_launch_dependents();
     ptx::pdl_wait();   // what runs before may still read the previous layout, or write Wq
+    int which = 0;
+    while (which + 1 < many.n && (int)blockIdx.x >= many.first_block[which + 1]) ++which;
+    const PrepArgs &a = many.a[which];
+    const int rel = (int)blockIdx.x - many.first_block[which], by = rel / many.nx[which], bx = rel - by * many.nx[which], at = many.first_group[which];
     __shared__ uint4 tile[kPrepN * kPrepChunks];      // [n][chunk ^ (n / 4)]: neither the writes nor the reads share a bank
     __shared__ uint32_t fold_s[kPrepChunks][kPrepN / 4];
     const int quad = threadIdx.x % (kPrepN / 4), chunk = threadIdx.x / (kPrepN / 4);
-    const int n0 = blockIdx.x * kPrepN + 4 * quad, c16 = blockIdx.y * kPrepChunks + chunk;
+    const int n0 = bx * kPrepN + 4 * quad, c16 = by * kPrepChunks + chunk;
     const int cpg = a.G / 16, j = c16 / cpg;
-    if (a.inline_order && blockIdx.x == 0 && blockIdx.y == 0) write_tables(a, order);
+    if (a.inline_order && rel == 0) write_tables(a, order, at);
     uint32_t r[16];
     uint32_t o = 0;
     const bool live = c16 < a.C / 16 && n0 < a.N;
     if (live) {
-        const int g = a.inline_order ? (int)order.perm[j] : a.perm[j];
+        const int g = a.inline_order ? (int)order.perm[at + j] : a.perm[j];
         const int8_t *src = a.Wq + (long long)(g * a.G + (c16 % cpg) * 16) * a.N + n0;
         if (a.aligned) {
 #pragma unroll
@@ -321,7 +332,7 @@ prep_linear_kernel(const __grid_constant__ PrepArgs a, const __grid_constant__ I
     for (int it = 0; it < 4; ++it) {
         const int u = threadIdx.x + it * (kPrepN / 4 * kPrepChunks);
         const int nl = u / kPrepChunks, ch = u % kPrepChunks;
-        const int n = blockIdx.x * kPrepN + nl, c = blockIdx.y * kPrepChunks + ch;
+        const int n = bx * kPrepN + nl, c = by * kPrepChunks + ch;
         const bool here = n < a.N && c < a.C / 16;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
         uint32_t mask = 0;
@@ -351,7 +362,7 @@ __global__ void __launch_bounds__(256) prep_conv_kernel(const __grid_constant__ 
     const int cpg = a.G / 16, n_c16 = n_g * cpg, units = a.T * n_c16;
     const int n_first = blockIdx.x * nb, n_here = min(nb, a.N - n_first);
     uint32_t *perm_s = prep_s + nb * n_g;
-    if (a.inline_order && blockIdx.x == 0) write_tables(a, order);   // an inline order is one window
+    if (a.inline_order && blockIdx.x == 0) write_tables(a, order, 0);   // an inline order is one window
     for (int i = threadIdx.x; i < nb * n_g; i += blockDim.x) prep_s[i] = 0;
     for (int i = threadIdx.x; i < n_g; i += blockDim.x) perm_s[i] = a.inline_order ? (uint32_t)order.perm[i] : (uint32_t)a.perm[g0 + i];
     __syncthreads();
@@ -388,21 +399,34 @@ __global__ void __launch_bounds__(256) prep_conv_kernel(const __grid_constant__ 
     }
 }
 
-static cudaError_t launch_prep(const Layer *L, const PrepArgs &a, const InlineOrder &order, cudaStream_t stream)
+// layers[0 .. n): linear, their orders one after the other in `order`
+static cudaError_t launch_prep_linear(const Layer *const *layers, const PrepArgs *args, int n, const InlineOrder &order, cudaStream_t stream)
 {
-    if (!L->is_conv) {
-        const dim3 grid((a.N + kPrepN - 1) / kPrepN, (a.C / 16 + kPrepChunks - 1) / kPrepChunks);
-        // spread evenly over the SMs: it is launched while the GEMM before it still runs on most of them
-        static bool attr_set[64] = {};
-        if (L->device >= 64 || !attr_set[L->device]) {
-            const cudaError_t e = cudaFuncSetAttribute(prep_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepSmem);
-            if (e != cudaSuccess) return e;
-            if (L->device < 64) attr_set[L->device] = true;
-        }
-        size_t smem = even_share_smem((long long)grid.x * grid.y, device_sm_count(L->device));
-        smem = smem > kPrepStatic ? smem - kPrepStatic : 0;
-        return launch_pdl(prep_linear_kernel, grid, kPrepN / 4 * kPrepChunks, smem, stream, a, order);
+    PrepMany many{};
+    many.n = n;
+    int blocks = 0, groups = 0;
+    for (int i = 0; i < n; ++i) {
+        const PrepArgs &a = many.a[i] = args[i];
+        many.first_block[i] = blocks;
+        many.first_group[i] = groups;
+        many.nx[i] = (a.N + kPrepN - 1) / kPrepN;
+        blocks += many.nx[i] * ((a.C / 16 + kPrepChunks - 1) / kPrepChunks);
+        groups += a.C / a.G;
     }
+    // spread evenly over the SMs: it is launched while the GEMM before it still runs on most of them
+    const int device = layers[0]->device;
+    static bool attr_set[64] = {};
+    if (device >= 64 || !attr_set[device]) {
+        const cudaError_t e = cudaFuncSetAttribute(prep_linear_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepSmem);
+        if (e != cudaSuccess) return e;
+        if (device < 64) attr_set[device] = true;
+    }
+    size_t smem = even_share_smem(blocks, device_sm_count(device));
+    smem = smem > kPrepStatic ? smem - kPrepStatic : 0;
+    return launch_pdl(prep_linear_kernel, (unsigned)blocks, kPrepN / 4 * kPrepChunks, smem, stream, many, order);
+}
+static cudaError_t launch_prep_conv(const Layer *L, const PrepArgs &a, const InlineOrder &order, cudaStream_t stream)
+{
     // as many output channels per block as give every thread a chunk, but blocks enough for the machine
     const int sms = device_sm_count(L->device), window = L->n_g < kPrepGroups ? L->n_g : kPrepGroups;
     int nb = 256 / (a.T * window * (a.G / 16));
@@ -470,15 +494,14 @@ int encode_weight_maps(Layer *L)
     return FLEXIQ_OK;
 }
 
-// The layout post-processing of a handle for a group order (Sec. 5): the order, the activation positions in slab
+// The layout post-processing of handles for a group order (Sec. 5): the order, the activation positions in slab
 // order and the chunk tables, the slab-order weights, their positions and the 4-bit cache, all from the
 // original-order weights.  Stream-ordered, allocates nothing on the device, does not wait for the stream: one launch
-// that carries the order in its parameters, or beyond kInlineGroups groups an upload from a pinned mirror before it.
-static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const uint8_t *x_shift, cudaStream_t stream)
+// that carries the orders in its parameters, or beyond kInlineGroups groups an upload from a pinned mirror before it.
+static int plan_layout(Layer *L, const int8_t *Wq, const int32_t *perm, const uint8_t *x_shift, PrepArgs &a, InlineOrder &order, int at, cudaStream_t stream)
 {
     const int n_g = L->n_g, C = L->C, G = L->G;
-    InlineOrder order;
-    PrepArgs a{};
+    a = PrepArgs{};
     a.Wq = Wq;
     a.aligned = (reinterpret_cast<uintptr_t>(Wq) & (L->is_conv ? 15u : 3u)) == 0;
     a.C = C; a.N = L->N; a.G = G; a.T = L->R * L->S;
@@ -486,16 +509,15 @@ static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const u
     a.w8 = L->w8; a.w8m = L->w8m; a.w4 = L->w4; a.w4_pitch = L->w4_pitch; a.sw = L->sw;
     a.inline_order = n_g <= kInlineGroups;
     a.K_lo = L->K_lo;
-    const bool straddle = !L->is_conv && straddle_in_use(L);
-    if (straddle) {
+    if (!L->is_conv && straddle_in_use(L)) {
         a.wst = L->wst;
         a.BK = choose_bk(L);
         a.st_blk0 = L->K_lo / a.BK * a.BK;
     }
     if (a.inline_order) {
         for (int j = 0; j < n_g; ++j) {
-            order.perm[j] = (uint16_t)perm[j];
-            order.sx[j] = x_shift ? x_shift[perm[j]] : 0;
+            order.perm[at + j] = (uint16_t)perm[j];
+            order.sx[at + j] = x_shift ? x_shift[perm[j]] : 0;
         }
     } else {
         // the pinned mirror is free again once the previous upload has read it (normally long ago)
@@ -517,15 +539,27 @@ static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const u
         FLEXIQ_CUDA_TRY(cudaEventRecord(L->tables_event, stream));
         L->tables_in_flight = 1;
     }
-    FLEXIQ_CUDA_TRY(launch_prep(L, a, order, stream));
+    return FLEXIQ_OK;
+}
+static void layout_done(Layer *L, const PrepArgs &a, cudaStream_t stream)
+{
     L->st_K_lo = -1;   // the straddle block was cut from the previous order's weights
     L->st_cap_id = 0;
-    if (straddle) straddle_written(L, stream);   // ... and this layout has cut it again
+    if (a.wst) straddle_written(L, stream);   // ... and this layout has cut it again
     const unsigned long long cap = stream_capture_id(stream);
     if (cap) { L->weights_cap_id = cap; L->weights_graph_seen = L->st_graph_seen = 1; }   // a replay makes both stale unseen
     else L->weights_fresh = 1;
     L->slab_next = 0;  // slabs written for the previous order are no longer this layer's
     memset(L->slab_seen, 0, sizeof(L->slab_seen));
+}
+static int layout_layer(Layer *L, const int8_t *Wq, const int32_t *perm, const uint8_t *x_shift, cudaStream_t stream)
+{
+    InlineOrder order;
+    PrepArgs a;
+    const int rc = plan_layout(L, Wq, perm, x_shift, a, order, 0, stream);
+    if (rc) return rc;
+    FLEXIQ_CUDA_TRY(L->is_conv ? launch_prep_conv(L, a, order, stream) : launch_prep_linear(&L, &a, 1, order, stream));
+    layout_done(L, a, stream);
     return FLEXIQ_OK;
 }
 
@@ -629,10 +663,8 @@ int flexiq_layer_create_conv(flexiq_layer_t *out, int Cin, int Cout, int R, int 
                          group_perm_host, x_shift_host, stream);
 }
 
-int flexiq_layer_set_group_perm(flexiq_layer_t layer, const int8_t *Wq_dev, const int32_t *group_perm_host,
-                                const uint8_t *x_shift_host, void *stream)
+static int check_layout(Layer *L, const int8_t *Wq_dev, const int32_t *group_perm_host, const uint8_t *x_shift_host)
 {
-    Layer *L = as_layer(layer);
     if (!L) return set_error(FLEXIQ_ERR_INVALID_ARG, "not a live flexiq layer handle");
     if (!Wq_dev || !group_perm_host) return set_error(FLEXIQ_ERR_INVALID_ARG, "Wq_dev and group_perm_host must not be NULL");
     int rc = validate_perm(group_perm_host, L->n_g);
@@ -640,9 +672,54 @@ int flexiq_layer_set_group_perm(flexiq_layer_t layer, const int8_t *Wq_dev, cons
     if (x_shift_host)
         for (int g = 0; g < L->n_g; ++g)
             if (x_shift_host[g] > 4) return set_error(FLEXIQ_ERR_INVALID_ARG, "x_shift_host[%d] = %d exceeds 4", g, x_shift_host[g]);
-    rc = check_layer_device(L);
+    return check_layer_device(L);
+}
+
+int flexiq_layer_set_group_perm(flexiq_layer_t layer, const int8_t *Wq_dev, const int32_t *group_perm_host,
+                                const uint8_t *x_shift_host, void *stream)
+{
+    Layer *L = as_layer(layer);
+    const int rc = check_layout(L, Wq_dev, group_perm_host, x_shift_host);
     if (rc) return rc;
     return layout_layer(L, Wq_dev, group_perm_host, x_shift_host, reinterpret_cast<cudaStream_t>(stream));
+}
+
+int flexiq_layers_set_group_perm(int n, const flexiq_layer_t *layers, const int8_t *const *Wq_dev, const int32_t *const *group_perm_host,
+                                 const uint8_t *const *x_shift_host, void *stream)
+{
+    if (n < 0 || (n > 0 && (!layers || !Wq_dev || !group_perm_host)))
+        return set_error(FLEXIQ_ERR_INVALID_ARG, "n = %d is negative, or an array is NULL", n);
+    int rc;
+    for (int i = 0; i < n; ++i) {
+        if ((rc = check_layout(as_layer(layers[i]), Wq_dev[i], group_perm_host[i], x_shift_host ? x_shift_host[i] : nullptr))) return rc;
+        for (int k = 0; k < i; ++k)
+            if (layers[k] == layers[i]) return set_error(FLEXIQ_ERR_INVALID_ARG, "layers[%d] and layers[%d] are the same handle", k, i);
+    }
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    InlineOrder order;
+    PrepArgs args[kPrepLayers];
+    for (int i = 0; i < n;) {
+        // as many linear layers as one launch takes
+        Layer *taken[kPrepLayers];
+        int count = 0, groups = 0;
+        for (; i + count < n && count < kPrepLayers; ++count) {
+            Layer *L = as_layer(layers[i + count]);
+            if (L->is_conv || groups + L->n_g > kInlineGroups) break;
+            taken[count] = L;
+            groups += L->n_g;
+        }
+        if (count < 2) {   // nothing to share a launch with
+            if ((rc = layout_layer(as_layer(layers[i]), Wq_dev[i], group_perm_host[i], x_shift_host ? x_shift_host[i] : nullptr, st))) return rc;
+            ++i;
+            continue;
+        }
+        for (int k = 0, at = 0; k < count; at += taken[k]->n_g, ++k)
+            if ((rc = plan_layout(taken[k], Wq_dev[i + k], group_perm_host[i + k], x_shift_host ? x_shift_host[i + k] : nullptr, args[k], order, at, st))) return rc;
+        FLEXIQ_CUDA_TRY(launch_prep_linear(taken, args, count, order, st));
+        for (int k = 0; k < count; ++k) layout_done(taken[k], args[k], st);
+        i += count;
+    }
+    return FLEXIQ_OK;
 }
 
 int flexiq_layer_destroy(flexiq_layer_t layer)

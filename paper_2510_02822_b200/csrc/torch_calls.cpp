@@ -16,6 +16,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <memory>
 #include <optional>
 #include <vector>
 
@@ -355,31 +356,60 @@ struct Bytes {   // a contiguous buffer of single bytes
     const uint8_t *data() const { return static_cast<const uint8_t *>(view.buf); }
 };
 
-// select_groups(Wq, flags, positions): the layer laid out with the flagged groups first (index order), at the ratio that
+// The flagged groups first (index order), then the others; *low = their number.
+std::vector<int32_t> selection(const Bytes &flags, Py_ssize_t n_g, int32_t *low)
+{
+    std::vector<int32_t> perm((size_t)n_g);
+    *low = 0;
+    for (Py_ssize_t g = 0; g < n_g; ++g)
+        if (flags.data()[g]) perm[(size_t)(*low)++] = (int32_t)g;
+    int32_t at = *low;
+    for (Py_ssize_t g = 0; g < n_g; ++g)
+        if (!flags.data()[g]) perm[(size_t)at++] = (int32_t)g;
+    return perm;
+}
+
+// select_groups([(calls, Wq, flags, positions), ...]): every layer laid out with its flagged groups first, at the ratio that
 // makes exactly them low -> None
-PyObject *calls_select_groups(PyObject *self, PyObject *const *args, Py_ssize_t n)
+PyObject *select_groups(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     return guarded([&]() -> PyObject * {
-        if (n != 3) throw Refused{};
-        Calls *c = reinterpret_cast<Calls *>(self);
-        const void *Wq = pointer(args[0]);
-        const Py_ssize_t n_g = (Py_ssize_t)(c->K / c->G);
-        const Bytes flags(args[1], n_g), positions(args[2], n_g);
-        std::vector<int32_t> perm((size_t)n_g);
-        int32_t low = 0;
-        for (Py_ssize_t g = 0; g < n_g; ++g)
-            if (flags.data()[g]) perm[(size_t)low++] = (int32_t)g;
-        int32_t at = low;
-        for (Py_ssize_t g = 0; g < n_g; ++g)
-            if (!flags.data()[g]) perm[(size_t)at++] = (int32_t)g;
+        if (n != 1 || !PyList_Check(args[0])) throw Refused{};
+        const Py_ssize_t count = PyList_GET_SIZE(args[0]);
+        std::vector<Calls *> calls;
+        std::vector<flexiq_layer_t> layers;
+        std::vector<const int8_t *> weights;
+        std::vector<std::vector<int32_t>> perms;
+        std::vector<const int32_t *> perm_ptrs;
+        std::vector<std::unique_ptr<Bytes>> positions;
+        std::vector<const uint8_t *> position_ptrs;
+        std::vector<int> low, before((size_t)count);
+        for (Py_ssize_t i = 0; i < count; ++i) {
+            PyObject *t = PyList_GET_ITEM(args[0], i);
+            if (!PyTuple_Check(t) || PyTuple_GET_SIZE(t) != 4) throw Refused{};
+            Calls *c = calls_of(PyTuple_GET_ITEM(t, 0));
+            const Py_ssize_t n_g = (Py_ssize_t)(c->K / c->G);
+            calls.push_back(c);
+            layers.push_back(c->h);
+            weights.push_back(static_cast<const int8_t *>(pointer(PyTuple_GET_ITEM(t, 1))));
+            const Bytes flags(PyTuple_GET_ITEM(t, 2), n_g);
+            int32_t l;
+            perms.push_back(selection(flags, n_g, &l));
+            perm_ptrs.push_back(perms.back().data());
+            low.push_back(l);
+            positions.push_back(std::make_unique<Bytes>(PyTuple_GET_ITEM(t, 3), n_g));
+            position_ptrs.push_back(positions.back()->data());
+        }
+        auto set_low = [](const Calls *c, int groups) { return flexiq_set_lowbit_ratio(c->h, (float)((double)groups / (double)(c->K / c->G))); };
+        // the ratios first, so that the layouts cut the weight blocks that depend on them; a refused layout leaves both as they were
+        int rc = FLEXIQ_OK;
+        for (size_t i = 0; i < calls.size() && rc == FLEXIQ_OK; ++i) rc = flexiq_get_max_4bit_ch(calls[i]->h, &before[i]);
+        for (size_t i = 0; i < calls.size() && rc == FLEXIQ_OK; ++i) rc = set_low(calls[i], low[i]);
         void *st = current_stream();
-        // the ratio first, so that the layout cuts the weight block that depends on it; a refused layout leaves both as they were
-        int before = 0;
-        int rc = flexiq_get_max_4bit_ch(c->h, &before);
-        if (rc == FLEXIQ_OK) rc = flexiq_set_lowbit_ratio(c->h, (float)((double)low / (double)n_g));
         if (rc == FLEXIQ_OK) {
-            rc = released([&] { return flexiq_layer_set_group_perm(c->h, static_cast<const int8_t *>(Wq), perm.data(), positions.data(), st); });
-            if (rc != FLEXIQ_OK) flexiq_set_lowbit_ratio(c->h, (float)((double)before / (double)c->K));
+            rc = released([&] { return flexiq_layers_set_group_perm((int)count, layers.data(), weights.data(), perm_ptrs.data(), position_ptrs.data(), st); });
+            if (rc != FLEXIQ_OK)
+                for (size_t i = 0; i < calls.size(); ++i) set_low(calls[i], before[i] / (int)calls[i]->G);
         }
         return finish(rc, Py_NewRef(Py_None));
     });
@@ -392,7 +422,6 @@ PyMethodDef calls_methods[] = {
     {"mixed_gemm_to_slab", (PyCFunction)(void (*)(void))calls_mixed_gemm_to_slab, METH_FASTCALL, nullptr},
     {"mixed_conv_to_slab", (PyCFunction)(void (*)(void))calls_mixed_conv_to_slab, METH_FASTCALL, nullptr},
     {"set_lowbit_ratio", calls_set_lowbit_ratio, METH_O, nullptr},
-    {"select_groups", (PyCFunction)(void (*)(void))calls_select_groups, METH_FASTCALL, nullptr},
     {nullptr, nullptr, 0, nullptr},
 };
 
@@ -541,6 +570,7 @@ PyObject *set_error_class(PyObject *, PyObject *cls)
 
 PyMethodDef module_methods[] = {
     {"static_preparation", (PyCFunction)(void (*)(void))static_preparation, METH_FASTCALL, nullptr},
+    {"select_groups", (PyCFunction)(void (*)(void))select_groups, METH_FASTCALL, nullptr},
     {"sq_distance_i8", (PyCFunction)(void (*)(void))sq_distance, METH_FASTCALL, nullptr},
     {"set_error_class", set_error_class, METH_O, nullptr},
     {nullptr, nullptr, 0, nullptr},

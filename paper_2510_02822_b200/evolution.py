@@ -59,30 +59,38 @@ class ChainFitness:
         self.evaluated = 0
         self.Y8 = self.outputs(np.zeros(int(self.off[-1]), dtype=np.uint8)).clone()
 
-    def _layer(self, l, flags_layer):
-        """The handle of layer l laid out for this selection: one handle per layer, re-laid out in place
-        (flexiq_layer_set_group_perm: no allocation, no synchronisation) when the selection changes."""
-        flags_layer = np.ascontiguousarray(flags_layer, dtype=np.uint8)
-        key = flags_layer.tobytes()
-        h = self.handles[l]
-        if key != self.current[l]:
+    def _lay_out(self, flags):
+        """Every layer laid out for this selection: one handle per layer, re-laid out in place (no allocation, no synchronisation) where
+        the selection has changed."""
+        changed = []
+        for l, L in enumerate(self.layers):
+            f = np.ascontiguousarray(flags[self.off[l]:self.off[l + 1]], dtype=np.uint8)
+            if f.tobytes() == self.current[l]:
+                continue
             Wq, ws, b = self.dev_params[l]
-            xs = np.ascontiguousarray(self.layers[l]["sx_group"], dtype=np.uint8)
-            if h is None:
-                perm, n_low = selection_perm(flags_layer)
-                h = self.handles[l] = fx.Layer(Wq, ws, b, perm, xs, self.layers[l]["G"])
+            xs = np.ascontiguousarray(L["sx_group"], dtype=np.uint8)
+            if self.handles[l] is None:
+                perm, n_low = selection_perm(f)
+                h = self.handles[l] = fx.Layer(Wq, ws, b, perm, xs, L["G"])
                 h.set_lowbit_ratio(n_low / self.groups[l])
+                self.current[l] = f.tobytes()
+                self.created += 1
             else:
-                h.select_groups(Wq, flags_layer, xs)
-            self.current[l] = key
-            self.created += 1
-        return h
+                changed.append((l, Wq, f, xs))
+        if changed:
+            for l, *_ in changed:
+                self.current[l] = None
+            fx.select_groups([(self.handles[l], *rest) for l, *rest in changed])
+            for l, _, f, _ in changed:
+                self.current[l] = f.tobytes()
+            self.created += len(changed)
 
     def outputs(self, flags):
         """int8 outputs of the last layer under the selection `flags` (device tensor, reused by the next call)."""
         src = self.X
+        self._lay_out(flags)
         for l, L in enumerate(self.layers):
-            h = self._layer(l, flags[self.off[l]:self.off[l + 1]])
+            h = self.handles[l]
             h.quantize_lower(src, L["x_scale"], slabs=(self.slab[l], None))
             src = h.mixed_gemm(self.slab[l], None, self.M, L["x_scale"], L["y_scale"], fx.OUT_REQUANT_I8, self.Y[l])
         self.evaluated += 1

@@ -91,3 +91,41 @@ def test_layout_cuts_the_block_of_the_ratio_in_force(K, N, G):
         assert np.array_equal(acc.cpu().numpy(), oracle.mixed_gemm_acc(X, W, G, order, sx[order].copy(), sw, low)), low
     fx.flexiq_check_status()
     L.close()
+
+
+@pytest.mark.parametrize("shapes", [
+    [(144, 80, 16), (112, 48, 16)], [(192, 208, 64), (128, 16, 16), (400, 64, 16), (64, 64, 16), (768, 96, 16)],      # two in a launch; four and one
+    [(600 * 16, 16, 16), (500 * 16, 16, 16), (32, 16, 16)], [(1025 * 16, 16, 16), (64, 32, 32)]])   # more groups than a launch carries, together and alone
+def test_several_layers_laid_out_at_once(shapes):
+    dev = torch.device("cuda:0")
+    made = []
+    for i, (K, N, G) in enumerate(shapes):
+        W, n_g = draw(800 + i, (K, N)), K // G
+        sx = (np.arange(n_g) % 5).astype(np.uint8)
+        Wd = torch.from_numpy(W).to(dev)
+        made.append((W, Wd, G, n_g, sx, fx.Layer(Wd, torch.ones(N, device=dev), None, np.arange(n_g, dtype=np.int32), sx, G)))
+    for turn in range(2):
+        flags = [(inputs.uniform(80 + turn, i, m[3]) < 0.4).astype(np.uint8) for i, m in enumerate(made)]
+        fx.select_groups([(m[5], m[1], f, m[4]) for m, f in zip(made, flags)])
+        for (W, Wd, G, n_g, sx, L), f in zip(made, flags):
+            order, low = np.concatenate([np.flatnonzero(f), np.flatnonzero(f == 0)]).astype(np.int32), int(f.sum())
+            assert L.K_lo == low * G
+            X = draw(850, (5, W.shape[0]))
+            sw = oracle.weight_positions_linear(W, G, order)
+            x4, x8, _ = L.quantize_lower(torch.from_numpy(X).to(dev), 1.0)
+            acc = L.mixed_gemm(x4, x8, 5, 1.0, 1.0, fx.OUT_ACC_I32)
+            assert np.array_equal(acc.cpu().numpy(), oracle.mixed_gemm_acc(X, W, G, order, sx[order].copy(), sw, low))
+            sw_g, w8, w4 = np.empty((n_g, W.shape[1]), np.uint8), np.empty((W.shape[1], W.shape[0]), np.int8), np.empty((W.shape[1], W.shape[0] // 2), np.uint8)
+            fx.flexiq_layer_export(L.h, sw_g, w8, w4)
+            assert np.array_equal(sw_g, sw.reshape(n_g, -1))
+    # one handle twice, or a position that is none: refused, and nothing has changed
+    m, before = made[0], made[0][5].K_lo
+    bad = m[4].copy()
+    bad[0] = 5
+    for args in ([(m[5], m[1], np.ones(m[3], np.uint8), m[4])] * 2, [(m[5], m[1], np.ones(m[3], np.uint8), bad)]):
+        with pytest.raises(fx.FlexiqError):
+            fx.select_groups(args)
+        assert m[5].K_lo == before
+    fx.flexiq_check_status()
+    for m in made:
+        m[5].close()
