@@ -441,46 +441,50 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
             }
             const uint32_t taddr = x.tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(SPLIT ? 2 * buf : buf) * x.buf_stride + (uint32_t)col0;
             PROF_T0(te0);
-            uint32_t ra[32], rb[32];
-            ptx::tmem_ld_32x32(taddr, ra);
-            if (SPLIT) ptx::tmem_ld_32x32(taddr + x.buf_stride, rb);   // the other MMA warp's partial sums (32-column passes only)
-            else if (cols == 64) ptx::tmem_ld_32x32(taddr + 32, rb);
             if (kScaled) {
                 __syncwarp();                                      // the previous reads of the table are done
                 reinterpret_cast<float4 *>(x.fac)[lane] = f;
                 __syncwarp();
-            }
-            ptx::tmem_ld_wait();
-            if (SPLIT) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) ra[i] += rb[i];
-            }
-            PROF_ADD(prof_ld, te0);
-            PROF_T0(te1);
-            if (pass + 1 == passes) {
-                // the accumulator slice is in registers: hand it back to the MMA warp before the math
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) {
-                    if (CG == 2) ptx::mbar_arrive_cluster_relaxed(ptx::mapa(ptx::smem_u32(&x.tmem_empty[buf]), 0));
-                    else ptx::mbar_arrive_relaxed(&x.tmem_empty[buf]);
-                }
             }
             int ents[4] = {0, 0, 0, 0};
             if (kSlab) {
 #pragma unroll
                 for (int g = 0; g < 4; ++g) ents[g] = __shfl_sync(0xffffffffu, ent, g);
             }
-            if (MODE == FLEXIQ_OUT_REQUANT_I8 || MODE == kOutNextSlab) {
-                // Each warp stages 32 rows x 32 columns (1 KB, 32-byte swizzle: no bank conflicts) and one
-                // lane hands them to a tiled bulk store, which writes whole sectors asynchronously and
-                // drops the rows and columns that lie outside Y.
-                const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
+            const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
+            // 32 columns at a time, in a loop: both halves' registers at once spilled, and the small launches pay for every
+            // instruction that has to be fetched (the waits' slow path inlined: DeiT-S at batch 1 275 -> 284 us).
+#pragma unroll 1
+            for (int h = 0; 32 * h < cols; ++h) {
+                uint32_t r[32];
+                ptx::tmem_ld_32x32(taddr + 32 * h, r);
+                if (SPLIT) {                                       // the other MMA warp's partial sums (32-column passes only)
+                    uint32_t rb[32];
+                    ptx::tmem_ld_32x32(taddr + x.buf_stride, rb);
+                    ptx::tmem_ld_wait();
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t *r = h == 0 ? ra : rb;
+                    for (int i = 0; i < 32; ++i) r[i] += rb[i];
+                } else {
+                    ptx::tmem_ld_wait();
+                }
+                PROF_ADD(prof_ld, te0);
+                PROF_T0(te1);
+                if (pass + 1 == passes && 32 * h + 32 >= cols) {
+                    // the accumulator slice is in registers: hand it back to the MMA warp before the math
+                    ptx::tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (CG == 2) ptx::mbar_arrive_cluster_relaxed(ptx::mapa(ptx::smem_u32(&x.tmem_empty[buf]), 0));
+                        else ptx::mbar_arrive_relaxed(&x.tmem_empty[buf]);
+                    }
+                }
+                const float *fac = x.fac + 32 * h;                 // alpha of these columns; their beta lies 64 further on
+                if (MODE == FLEXIQ_OUT_REQUANT_I8 || MODE == kOutNextSlab) {
+                    // Each warp stages 32 rows x 32 columns (1 KB, 32-byte swizzle: no bank conflicts) and one
+                    // lane hands them to a tiled bulk store, which writes whole sectors asynchronously and
+                    // drops the rows and columns that lie outside Y.
                     const int n = nw + 32 * h;
-                    if (32 * h < cols && n < p.N && row0 < p.M) {   // warp-uniform
+                    if (n < p.N && row0 < p.M) {   // warp-uniform
                         const bool both = n + 16 < p.N;  // a 32-column box, else (last 16 channels of N) a 16-column one
                         uint32_t w[8];
                         if (MODE == kOutNextSlab) {
@@ -488,10 +492,10 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                             // is lowered when it lies below the next layer's max_4bit_ch
 #pragma unroll
                             for (int g = 0; g < 2; ++g)
-                                if (g == 0 || both) next_slab16(p, ents[2 * h + g], r + 16 * g, x.fac + 32 * h + 16 * g, x.fac + 64 + 32 * h + 16 * g, w + 4 * g);
+                                if (g == 0 || both) next_slab16(p, (h ? ents[2 + g] : ents[g]), r + 16 * g, fac + 16 * g, fac + 64 + 16 * g, w + 4 * g);
                         } else {
-                            finish16<FLEXIQ_OUT_REQUANT_I8>(r, x.fac + 32 * h, x.fac + 64 + 32 * h, w);
-                            if (both) finish16<FLEXIQ_OUT_REQUANT_I8>(r + 16, x.fac + 32 * h + 16, x.fac + 64 + 32 * h + 16, w + 4);
+                            finish16<FLEXIQ_OUT_REQUANT_I8>(r, fac, fac + 64, w);
+                            if (both) finish16<FLEXIQ_OUT_REQUANT_I8>(r + 16, fac + 16, fac + 64 + 16, w + 4);
                         }
                         if (lane == 0) ptx::bulk_wait_read_all();    // the previous store has read the buffer
                         __syncwarp();
@@ -511,19 +515,14 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                             ptx::bulk_commit_group();
                         }
                     }
-                }
-            } else if (kHalf) {
-                // 16-bit outputs: 32 rows x 16 columns (32 bytes per row: the same 1 KB swizzled box) per store
-                const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t *r = h == 0 ? ra : rb;
+                } else if (kHalf) {
+                    // 16-bit outputs: 32 rows x 16 columns (32 bytes per row: the same 1 KB swizzled box) per store
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
                         const int n = nw + 32 * h + 16 * g;
-                        if (32 * h < cols && n < p.N && row0 < p.M) {   // warp-uniform
+                        if (n < p.N && row0 < p.M) {   // warp-uniform
                             uint32_t w[16], hw[8];
-                            finish16<FLEXIQ_OUT_DEQUANT_F32>(r + 16 * g, x.fac + 32 * h + 16 * g, x.fac + 64 + 32 * h + 16 * g, w);
+                            finish16<FLEXIQ_OUT_DEQUANT_F32>(r + 16 * g, fac + 16 * g, fac + 64 + 16 * g, w);
 #pragma unroll
                             for (int q = 0; q < 8; ++q)
                                 hw[q] = pack2_f16<MODE == FLEXIQ_OUT_DEQUANT_BF16>(__uint_as_float(w[2 * q]), __uint_as_float(w[2 * q + 1]));
@@ -542,19 +541,14 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                             }
                         }
                     }
-                }
-            } else if (kElem == 4) {
-                // 4-byte outputs: 32 rows x 8 columns per store (the same 32-byte rows)
-                const long long row0 = kGrid ? (box_live ? 0 : p.M) : row - lane;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t *r = h == 0 ? ra : rb;
+                } else if (kElem == 4 && MODE != kOutScatter) {
+                    // 4-byte outputs: 32 rows x 8 columns per store (the same 32-byte rows)
 #pragma unroll
                     for (int g = 0; g < 2; ++g) {
                         const int n = nw + 32 * h + 16 * g;
-                        if (32 * h < cols && n < p.N && row0 < p.M) {   // warp-uniform
+                        if (n < p.N && row0 < p.M) {   // warp-uniform
                             uint32_t w[16];
-                            finish16<MODE>(r + 16 * g, x.fac + 32 * h + 16 * g, x.fac + 64 + 32 * h + 16 * g, w);
+                            finish16<MODE>(r + 16 * g, fac + 16 * g, fac + 64 + 16 * g, w);
                             const uint32_t dst = x.store_stage + (uint32_t)lane * 32u;
                             const uint32_t sw16 = ((uint32_t)lane >> 2 & 1u) << 4;
 #pragma unroll
@@ -573,24 +567,20 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                             }
                         }
                     }
-                }
-            } else if (MODE == kOutScatter && row < p.M) {
-                // each 16-channel chunk goes to its place in the next layer's slab row
-                uint8_t *srow = static_cast<uint8_t *>(p.Y) + row * p.N;
-                const bool wide = ((reinterpret_cast<uintptr_t>(p.Y) | (uintptr_t)p.N) & 31) == 0;   // rows are 32-byte aligned: 256-bit stores
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {                       // two halves of 32 columns
-                    const uint32_t *r = h == 0 ? ra : rb;
+                } else if (MODE == kOutScatter && row < p.M) {
+                    // each 16-channel chunk goes to its place in the next layer's slab row
+                    uint8_t *srow = static_cast<uint8_t *>(p.Y) + row * p.N;
+                    const bool wide = ((reinterpret_cast<uintptr_t>(p.Y) | (uintptr_t)p.N) & 31) == 0;   // rows are 32-byte aligned: 256-bit stores
                     const int n = nw + 32 * h;
-                    if (32 * h < cols && n < p.N) {
+                    if (n < p.N) {
                         const bool second = n + 16 < p.N;  // columns 16..31 of this half are live
                         uint32_t w[8];
                         int pos[2] = {0, 0};
 #pragma unroll
                         for (int g = 0; g < 2; ++g) {
                             if (g == 0 || second) {
-                                pos[g] = ents[2 * h + g] & 0xffffff;
-                                next_slab16(p, ents[2 * h + g], r + 16 * g, x.fac + 32 * h + 16 * g, x.fac + 64 + 32 * h + 16 * g, w + 4 * g);
+                                pos[g] = (h ? ents[2 + g] : ents[g]) & 0xffffff;
+                                next_slab16(p, (h ? ents[2 + g] : ents[g]), r + 16 * g, fac + 16 * g, fac + 64 + 16 * g, w + 4 * g);
                             }
                         }
                         if (second && wide && pos[1] == pos[0] + 1 && (pos[0] & 1) == 0) st_global_256(srow + pos[0] * 16, w);
@@ -600,8 +590,9 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                         }
                     }
                 }
+                PROF_ADD(prof_math, te1);
+                if (MODE == kOutScatter) __syncwarp();              // rows beyond M rejoin for the next columns' load
             }
-            PROF_ADD(prof_math, te1);
         }
         if (!kPatch && (buf ^= 1) == 0) buf_phase ^= 1;
     }
