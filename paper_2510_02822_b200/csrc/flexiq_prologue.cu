@@ -215,6 +215,13 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
             mask = shift == kShift8Bit ? 0xffffffffu : ((0xffu << shift) & 0xffu) * 0x01010101u;
         };
         if ((int)threadIdx.x < units) position(r0, c0);
+        unsigned held = 0;                           // DYN: OR of the folded words this thread has seen, four bytes wide
+        auto merge = [&](unsigned o, int c) {
+            o |= o >> 16;
+            o = (o | (o >> 8)) & 0xffu;
+            unsigned *seen = or_s + c / cpg;
+            if (o & ~*reinterpret_cast<volatile unsigned *>(seen)) atomicOr(seen, o);   // rare after the first rows
+        };
         int stage = 0;
         uint32_t phase = 0;
         for (long long tile = first; tile < a.tiles; tile += step) {
@@ -257,10 +264,8 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
                         asm("prmt.b32 %0, %1, 0, 0xba98;" : "=r"(sign) : "r"(w[k]));
                         o |= w[k] ^ sign;
                     }
-                    o |= o >> 16;
-                    o = (o | (o >> 8)) & 0xffu;
-                    unsigned *seen = or_s + c / cpg;
-                    if (o & ~*reinterpret_cast<volatile unsigned *>(seen)) atomicOr(seen, o);   // rare after the first rows
+                    if (single) held |= o;      // its own chunk in every tile: merged once, behind the last
+                    else merge(o, c);
                 }
                 *reinterpret_cast<uint4 *>(a.slab + (size_t)tile * (size_t)(units * 16) + (size_t)u * 16) =
                     make_uint4(w[0] & mask, w[1] & mask, w[2] & mask, w[3] & mask);
@@ -273,6 +278,7 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
             if (lane == 0) ptx::mbar_arrive(&empty_bar[stage]);
             if (++stage == a.stages) { stage = 0; phase ^= 1; }
         }
+        if (DYN && single && (int)threadIdx.x < units) merge(held, c0);
     }
     __syncthreads();
     if (gave_up) {
