@@ -478,7 +478,8 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
         const at::TensorOptions opt = at::TensorOptions().device(X.device());
         const at::Tensor work = at::empty({3 * C + 1}, opt.dtype(at::kInt));   // lo, hi, wmax and a scratch word
         // perm int32 [n_g], then x_shift [n_g]: page-locked, written by the device, so that the stream's end is all there is to wait for
-        const at::Tensor order = at::empty({5 * n_g}, at::TensorOptions().dtype(at::kByte).pinned_memory(true));
+        // (one size for most layers: the allocator keeps a block per power of two, and the first of each is a call to the driver)
+        const at::Tensor order = at::empty({std::max(5 * n_g, 4096ll)}, at::TensorOptions().dtype(at::kByte).pinned_memory(true));
         void *order_dev = nullptr;
         if (cudaHostGetDevicePointer(&order_dev, order.data_ptr(), 0) != cudaSuccess) { cudaGetLastError(); throw Refused{}; }
         const at::Tensor score = at::empty({n_g}, opt.dtype(at::kLong)), unused = at::empty({5}, opt.dtype(at::kInt));
