@@ -374,6 +374,12 @@ struct StaticArgs {
     long long *score;
     int32_t *unused;
 };
+__global__ void clear_static_kernel(int32_t *work, int n)
+{
+    ptx::pdl_launch_dependents();
+    ptx::pdl_wait();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) work[i] = 0;
+}
 template <int DTYPE, bool HIST>
 __global__ void __launch_bounds__(kCalibWindow) calib_static_kernel(const __grid_constant__ StaticArgs a)
 {
@@ -381,6 +387,7 @@ __global__ void __launch_bounds__(kCalibWindow) calib_static_kernel(const __grid
     __shared__ unsigned long long score_s[kStaticGroups];
     __shared__ int bits_s[kStaticGroups];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, block = (int)blockIdx.x - a.w_blocks;
+    ptx::pdl_wait();   // the clear, and what wrote X and W before it
     if (block < 0) {
         if (a.is_conv) absmax_cols_block(blockIdx.x % a.w_gx, blockIdx.x / a.w_gx, a.w_gy, a.W, a.w_rows, a.K, lo_s, a.wmax);
         else {
@@ -632,20 +639,20 @@ extern "C" int flexiq_calib_static(const void *X_dev, int x_dtype, int64_t M, fl
     a.w_blocks = is_conv ? (int)(cols.x * cols.y) : (K + kWarps - 1) / kWarps;
     a.lo = lo; a.hi = hi; a.wmax = wmax; a.done = reinterpret_cast<unsigned *>(wmax + K);
     a.perm = perm; a.x_shift = x_shift; a.score = reinterpret_cast<long long *>(score_dev); a.unused = unused_hist_dev;
-    FLEXIQ_CUDA_TRY(cudaMemsetAsync(work_dev, 0, sizeof(int32_t) * (3 * (size_t)K + 1), st));
+    // a launch, not a memset: the blocks behind it are resident when it ends
+    FLEXIQ_CUDA_TRY(launch_pdl(clear_static_kernel, 1, 1024, 0, st, work_dev, 3 * K + 1));
     if (hist_dev) {
-        calib_static_kernel<FLEXIQ_DTYPE_I8, true><<<(unsigned)(a.w_blocks + (K + kWarps - 1) / kWarps), kCalibWindow, 0, st>>>(a);
+        FLEXIQ_CUDA_TRY(launch_pdl(calib_static_kernel<FLEXIQ_DTYPE_I8, true>, (unsigned)(a.w_blocks + (K + kWarps - 1) / kWarps), kCalibWindow, 0, st, a));
     } else {
         a.slices = range_slices(M, K, sms);
         const unsigned grid = (unsigned)(a.w_blocks + (K + kCalibWindow - 1) / kCalibWindow * a.slices);
         switch (x_dtype) {
-            case FLEXIQ_DTYPE_F32: calib_static_kernel<FLEXIQ_DTYPE_F32, false><<<grid, kCalibWindow, 0, st>>>(a); break;
-            case FLEXIQ_DTYPE_F16: calib_static_kernel<FLEXIQ_DTYPE_F16, false><<<grid, kCalibWindow, 0, st>>>(a); break;
-            case FLEXIQ_DTYPE_BF16: calib_static_kernel<FLEXIQ_DTYPE_BF16, false><<<grid, kCalibWindow, 0, st>>>(a); break;
-            default: calib_static_kernel<FLEXIQ_DTYPE_I8, false><<<grid, kCalibWindow, 0, st>>>(a); break;
+            case FLEXIQ_DTYPE_F32: FLEXIQ_CUDA_TRY(launch_pdl(calib_static_kernel<FLEXIQ_DTYPE_F32, false>, grid, kCalibWindow, 0, st, a)); break;
+            case FLEXIQ_DTYPE_F16: FLEXIQ_CUDA_TRY(launch_pdl(calib_static_kernel<FLEXIQ_DTYPE_F16, false>, grid, kCalibWindow, 0, st, a)); break;
+            case FLEXIQ_DTYPE_BF16: FLEXIQ_CUDA_TRY(launch_pdl(calib_static_kernel<FLEXIQ_DTYPE_BF16, false>, grid, kCalibWindow, 0, st, a)); break;
+            default: FLEXIQ_CUDA_TRY(launch_pdl(calib_static_kernel<FLEXIQ_DTYPE_I8, false>, grid, kCalibWindow, 0, st, a)); break;
         }
     }
-    FLEXIQ_CUDA_TRY(cudaGetLastError());
     return FLEXIQ_OK;
 }
 
