@@ -1428,9 +1428,8 @@ __global__ void wait_expiry_kernel(int *result)
 // The straddle block of the masked path (straddle.cuh) for a GEMM that no prologue launch precedes.
 __global__ void straddle_kernel(const StraddleJob job)
 {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     ptx::pdl_wait();  // the previous kernel of the stream may still read the block
-    if (idx < (long long)job.rows * (job.BK >> 4)) straddle_write_unit(job, idx);
+    StraddleUnit(job, (long long)blockIdx.x * blockDim.x + threadIdx.x).write();
 }
 
 // ------------------------------------------------------------------------------------

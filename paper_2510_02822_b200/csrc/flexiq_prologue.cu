@@ -150,9 +150,10 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
         // Extra blocks in front of the quantizing ones (so that they run beside the first wave, not behind the
         // last): the weight K block that max_4bit_ch falls into, for the GEMM that consumes these slabs -- the
         // only weight data that depends on the ratio -- 16 bytes per thread.
+        const StraddleUnit unit(a.wp, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+        unit.ask();
         ptx::pdl_wait();
-        const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-        if (idx < (long long)a.wp.rows * (a.wp.BK >> 4)) straddle_write_unit(a.wp, idx);
+        unit.write();
         return;
     }
     const long long first = blockIdx.x - a.wp.first_block, step = gridDim.x - a.wp.first_block;
@@ -340,12 +341,14 @@ __global__ void lower_inplace_kernel(int8_t *__restrict__ slab, long long M, int
                                      int step_m, int step_c)
 {
     ptx::pdl_launch_dependents();
-    ptx::pdl_wait();  // phase 1 has written the slab and the OR words
     if (blockIdx.x < wp.first_block) {
-        const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-        if (idx < (long long)wp.rows * (wp.BK >> 4)) straddle_write_unit(wp, idx);
+        const StraddleUnit unit(wp, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+        unit.ask();
+        ptx::pdl_wait();
+        unit.write();
         return;
     }
+    ptx::pdl_wait();  // phase 1 has written the slab and the OR words
     const unsigned qblock = blockIdx.x - wp.first_block;
     if (qblock == 0)
         for (int j = threadIdx.x; j < K / G; j += blockDim.x) sx_out[j] = (uint8_t)position_from_or(__ldcg(or_words + j));
@@ -413,12 +416,14 @@ __global__ void __launch_bounds__(kColThreads) dynamic_columns_kernel(const __gr
     __shared__ unsigned or_s[4], all_s[4];
     uint4 *held = reinterpret_cast<uint4 *>(cols_smem);
     ptx::pdl_launch_dependents();
-    ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
     if (blockIdx.x < a.wp.first_block) {   // whole clusters: the straddle block of the weights
-        const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-        if (idx < (long long)a.wp.rows * (a.wp.BK >> 4)) straddle_write_unit(a.wp, idx);
+        const StraddleUnit unit(a.wp, (long long)blockIdx.x * blockDim.x + threadIdx.x);
+        unit.ask();
+        ptx::pdl_wait();
+        unit.write();
         return;
     }
+    ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
     const int n_c16 = a.K / 16, cpg = a.G / 16;
     const int rank = (int)ptx::cluster_ctarank(), first = (int)((blockIdx.x - a.wp.first_block) / kColCluster) * a.window;
     const int cl = threadIdx.x % a.window, c = first + cl, j = c / cpg;

@@ -22,16 +22,26 @@ struct StraddleJob {
     unsigned first_block;  // prologue launches: number of straddle blocks, which come in front of the quantizing blocks
 };
 
-// one 16-byte unit of the straddle block; idx < rows * (BK / 16)
-__device__ __forceinline__ void straddle_write_unit(const StraddleJob &j, long long idx)
-{
-    const int upb = j.BK >> 4;
-    const int u = (int)(idx % upb);
-    const long long row = idx / upb;
-    const int c = j.blk0 + 16 * u;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (c < j.C) v = *reinterpret_cast<const uint4 *>((c < j.K_lo ? j.w8m : j.w8) + (size_t)row * j.C + c);
-    *reinterpret_cast<uint4 *>(j.wst + (size_t)row * j.BK + 16 * u) = v;
-}
+// One 16-byte unit of the straddle block, idx < rows * (BK / 16).  Where it comes from (nowhere: zeros) and goes to, and its source asked
+// into L2, can all be done before a dependency wait: nothing is read early.
+struct StraddleUnit {
+    const uint4 *src;
+    uint4 *dst;
+    __device__ __forceinline__ StraddleUnit(const StraddleJob &j, long long idx)
+    {
+        const int log_upb = j.BK == 128 ? 3 : 2, u = (int)idx & ((1 << log_upb) - 1), c = j.blk0 + 16 * u;
+        const long long row = idx >> log_upb;
+        dst = idx < ((long long)j.rows << log_upb) ? reinterpret_cast<uint4 *>(j.wst) + idx : nullptr;   // [row][BK]: unit after unit
+        src = dst && c < j.C ? reinterpret_cast<const uint4 *>((c < j.K_lo ? j.w8m : j.w8) + (size_t)row * j.C + c) : nullptr;
+    }
+    __device__ __forceinline__ void ask() const
+    {
+        if (src) asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
+    }
+    __device__ __forceinline__ void write() const
+    {
+        if (dst) *dst = src ? *src : make_uint4(0u, 0u, 0u, 0u);
+    }
+};
 
 }  // namespace flexiq
