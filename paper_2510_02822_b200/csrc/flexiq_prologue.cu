@@ -108,11 +108,11 @@ __device__ __forceinline__ bool wait_copy(uint32_t bar, uint32_t parity, volatil
 // values clipped to what four bits hold at position s; an 8-bit group is the same at position 4 with nothing cleared,
 // which is told apart by shift 5: one instruction stream for both, since a warp spans the boundary in most rows.
 constexpr unsigned kShift8Bit = 5;
-__device__ __forceinline__ unsigned chunk_entry(int c, int G, int lo_c16, const int32_t *perm, const uint8_t *sx)
+__device__ __forceinline__ unsigned chunk_entry(int c, int log_cpg, int lo_c16, const int32_t *perm, const uint8_t *sx)   // 1 << log_cpg chunks a group
 {
-    const int cpg = G / 16, j = c / cpg;
+    const int j = c >> log_cpg;
     const unsigned shift = c < lo_c16 ? (unsigned)__ldg(sx + j) : kShift8Bit;
-    return (unsigned)(__ldg(perm + j) * cpg + (c - j * cpg)) | (shift << 28);
+    return (unsigned)((__ldg(perm + j) << log_cpg) + (c - (j << log_cpg))) | (shift << 28);
 }
 
 struct RowsArgs {
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
     __shared__ uint64_t full_bar[kRowStages], empty_bar[kRowStages];
     __shared__ int gave_up;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (blockDim.x >> 5) - 1;
-    const int n_c16 = a.K / 16, lo_c16 = DYN ? 0 : a.K_lo / 16, cpg = a.G / 16;
+    const int n_c16 = a.K / 16, lo_c16 = DYN ? 0 : a.K_lo / 16, log_cpg = a.G == 16 ? 0 : a.G == 32 ? 1 : 2;
     unsigned *table = reinterpret_cast<unsigned *>(rows_smem + a.stages * a.stage_bytes);
     unsigned *or_s = table + n_c16;
     ptx::pdl_launch_dependents();
@@ -166,6 +166,10 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
         ptx::bulk_load(ptx::smem_u32(rows_smem) + (uint32_t)(stage * a.stage_bytes),
                        reinterpret_cast<const char *>(a.X) + (size_t)tile * tile_bytes, bytes, bar);
     };
+    // Everything that needs no global memory comes before the dependency wait: a small launch is one chain of latencies behind it.
+    const int threads = 32 * warps, units = a.rows * n_c16;
+    const bool single = units <= threads;            // one chunk per thread and tile, the same in every tile
+    const int r0 = (int)threadIdx.x / n_c16, c0 = (int)threadIdx.x - r0 * n_c16;
     long long next = first;                          // the copying thread's next tile
     const bool copier = warp == warps && lane == 0;
     if (copier) {
@@ -181,13 +185,20 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
         for (int i = 0; i < a.ahead && t < a.tiles; ++i, t += step)
             ptx::bulk_prefetch_l2(reinterpret_cast<const char *>(a.X) + (size_t)t * tile_bytes, bytes_of(t));
     }
-    ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
-    if (copier)
-        for (int i = 0; i < a.stages && next < a.tiles; ++i, next += step) copy(next, i);
-    for (int c = threadIdx.x; c < n_c16; c += blockDim.x) table[c] = chunk_entry(c, a.G, lo_c16, a.perm, a.sx);
     if (DYN)
         for (int j = threadIdx.x; j < a.K / a.G; j += blockDim.x) or_s[j] = 0;
     __syncthreads();
+    ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
+    if (copier)
+        for (int i = 0; i < a.stages && next < a.tiles; ++i, next += step) copy(next, i);
+    // A thread with one chunk fetches that chunk's entry itself; otherwise the block makes a table.
+    unsigned ent = 0;
+    if (single) {
+        if ((int)threadIdx.x < units) ent = chunk_entry(c0, log_cpg, lo_c16, a.perm, a.sx);
+    } else {
+        for (int c = threadIdx.x; c < n_c16; c += blockDim.x) table[c] = chunk_entry(c, log_cpg, lo_c16, a.perm, a.sx);
+        __syncthreads();
+    }
     if (warp == warps) {
         if (lane == 0) {
             // refill a stage when every warp has read it
@@ -200,13 +211,9 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
             }
         }
     } else {
-        const int threads = 32 * warps, units = a.rows * n_c16;
-        const bool single = units <= threads;        // one chunk per thread and tile, the same in every tile
-        const int r0 = (int)threadIdx.x / n_c16, c0 = (int)threadIdx.x - r0 * n_c16;
         unsigned src = 0, shift = kShift8Bit, mask = 0xffffffffu;
         float lo = -128.f, hi = 127.f;
-        auto position = [&](int r, int c) {          // of the chunk at row r of a tile, slab chunk c
-            const unsigned ent = table[c];
+        auto position = [&](int r, unsigned ent) {   // of the chunk of this entry in row r of a tile
             src = (unsigned)r * (unsigned)row_bytes + (ent & 0x0fffffffu) * (16u * kBytes);
             if (DYN) return;
             shift = ent >> 28;
@@ -215,12 +222,12 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
             hi = bound - 1.f;
             mask = shift == kShift8Bit ? 0xffffffffu : ((0xffu << shift) & 0xffu) * 0x01010101u;
         };
-        if ((int)threadIdx.x < units) position(r0, c0);
+        if (single) position(r0, ent);
         unsigned held = 0;                           // DYN: OR of the folded words this thread has seen, four bytes wide
         auto merge = [&](unsigned o, int c) {
             o |= o >> 16;
             o = (o | (o >> 8)) & 0xffu;
-            unsigned *seen = or_s + c / cpg;
+            unsigned *seen = or_s + (c >> log_cpg);
             if (o & ~*reinterpret_cast<volatile unsigned *>(seen)) atomicOr(seen, o);   // rare after the first rows
         };
         int stage = 0;
@@ -231,7 +238,7 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
             const int here = (int)min((long long)a.rows, a.M - tile * a.rows) * n_c16;
             int r = r0, c = c0;
             for (int u = threadIdx.x; u < here; u += threads) {
-                if (!single) position(r, c);
+                if (!single) position(r, table[c]);
                 uint4 raw[kPieces];
                 // Neighbouring lanes start at different pieces of their chunks: with one order for all, the 16-byte reads
                 // of a quarter warp would share half (16-bit inputs) or a quarter (fp32) of the banks.
@@ -423,7 +430,6 @@ __global__ void __launch_bounds__(kColThreads) dynamic_columns_kernel(const __gr
         unit.write();
         return;
     }
-    ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
     const int n_c16 = a.K / 16, cpg = a.G / 16;
     const int rank = (int)ptx::cluster_ctarank(), first = (int)((blockIdx.x - a.wp.first_block) / kColCluster) * a.window;
     const int cl = threadIdx.x % a.window, c = first + cl, j = c / cpg;
@@ -433,6 +439,7 @@ __global__ void __launch_bounds__(kColThreads) dynamic_columns_kernel(const __gr
     const int rows = (int)max(0ll, min((long long)a.rows, a.M - m_first));
     if (threadIdx.x < 4) { or_s[threadIdx.x] = 0; all_s[threadIdx.x] = 0; }
     __syncthreads();
+    ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
     if (live) {
         const size_t row_bytes = (size_t)a.K * kBytes;
         const char *src = reinterpret_cast<const char *>(a.X) + (size_t)(m_first + r0) * row_bytes + ((size_t)__ldg(a.perm + j) * a.G + (c % cpg) * 16) * kBytes;
