@@ -159,11 +159,12 @@ int encode_weight_maps(Layer *L);
 
 // Dynamic shared memory with which no SM takes more than its share of a grid.  A GEMM releases the launch behind it while some of
 // its CTAs still run; blocks go where there is room, so without this the SMs that are free first take as many as fit and
-// the others, when they come free, what is left.
+// the others, when they come free, what is left.  None where a share is more blocks than that could hold apart.
 inline size_t even_share_smem(long long blocks, long long sms)
 {
     const long long share = (blocks + sms - 1) / sms;
-    return (size_t)(228 * 1024 / (share + 1)) - 1024;   // (an SM's 228 KB; each block takes 1 KB and the static part besides)
+    const long long each = 228 * 1024 / (share + 1);   // (an SM's 228 KB; each block takes 1 KB and the static part besides)
+    return each > 1024 ? (size_t)(each - 1024) : 0;
 }
 
 // Launch with programmatic stream serialization allowed: the kernel may start before its predecessor in the stream has

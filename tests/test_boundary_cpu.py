@@ -3,6 +3,7 @@ every symbol the header declares, and rejects bad arguments before touching a de
 import ctypes as C
 import os
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -142,3 +143,29 @@ def test_conv_kind_host_logic(lib):
     for bad in [(0, 8, 8, 64, 64, 3, 3, 1, 1), (1, 1, 8, 64, 64, 3, 3, 1, 0), (1, 8, 8, 64, 64, 3, 3, 0, 1), (1, 8, 8, 64, 64, 3, 3, 1, -1)]:
         with pytest.raises(fx.FlexiqError):
             fx.flexiq_choose_conv_kind(*bad)
+
+
+def test_even_share_of_any_grid(tmp_path):
+    """The shared memory that spreads a grid over the SMs: with it a share of the blocks and no more fits an SM, whatever the grid."""
+    src = tmp_path / "share.cpp"
+    src.write_text("""
+#include "flexiq_internal.h"
+#include <stdio.h>
+int main()
+{
+    for (long long sms : {1ll, 74ll, 148ll})
+        for (long long blocks = 1; blocks <= 1000000; blocks += 1 + blocks / 5000) {
+            const long long smem = (long long)flexiq::even_share_smem(blocks, sms), share = (blocks + sms - 1) / sms;
+            if (smem < 0 || smem > 113 * 1024 || (smem && (smem + 1024) * share > 228 * 1024) || (share < 200 && (smem + 1024) * (share + 2) < 228 * 1024)) {
+                printf("%lld blocks on %lld SMs: %lld bytes\\n", blocks, sms, smem);
+                return 1;
+            }
+        }
+    return 0;
+}
+""")
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(fxbuild._nvcc())))
+    exe = str(tmp_path / "share")
+    subprocess.run(["g++", "-std=c++17", *(f"-I{d}" for d in (fxbuild.CSRC, os.path.join(ROOT, "include"), os.path.join(cuda, "include"))), str(src), "-o", exe], check=True)
+    r = subprocess.run([exe], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout

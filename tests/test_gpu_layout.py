@@ -129,3 +129,37 @@ def test_several_layers_laid_out_at_once(shapes):
     fx.flexiq_check_status()
     for m in made:
         m[5].close()
+
+
+@pytest.mark.parametrize("widths", [(67264,), (34304, 34304)])   # 33,632 and 2 x 17,152 blocks of one launch: more than 227 an SM
+def test_layout_of_very_large_layers(widths):
+    """Each alone when it is created, and together in one launch; a few output columns against the oracle."""
+    dev, K, G = torch.device("cuda:0"), 4096, 64
+    n_g = K // G
+    gen = torch.Generator(device=dev).manual_seed(widths[0])
+    sx = (np.arange(n_g) % 5).astype(np.uint8)
+    X = draw(860, (5, K))
+    made = []
+    for N in widths:
+        W = torch.randint(-128, 128, (K, N), generator=gen, device=dev, dtype=torch.int8)
+        W >>= torch.randint(0, 6, (n_g, N), generator=gen, device=dev, dtype=torch.int8).repeat_interleave(G, 0)
+        made.append((W, fx.Layer(W, torch.ones(N, device=dev), None, np.arange(n_g, dtype=np.int32), sx, G)))
+
+    def check(L, W, order, low):
+        cols = np.unique(np.concatenate([np.arange(16), np.linspace(0, L.N - 1, 97).astype(np.int64), np.arange(L.N - 16, L.N)]))
+        Wc = np.ascontiguousarray(W[:, torch.from_numpy(cols).to(dev)].cpu().numpy())
+        x4, x8, _ = L.quantize_lower(torch.from_numpy(X).to(dev), 1.0)
+        acc = L.mixed_gemm(x4, x8, 5, 1.0, 1.0, fx.OUT_ACC_I32).cpu().numpy()
+        sw = oracle.weight_positions_linear(Wc, G, order)
+        assert np.array_equal(acc[:, cols], oracle.mixed_gemm_acc(X, Wc, G, order, sx[order].copy(), sw, low))
+
+    for W, L in made:
+        L.set_lowbit_ratio(0.5)
+        check(L, W, np.arange(n_g, dtype=np.int32), n_g // 2)
+    flags = [(inputs.uniform(90, i, n_g) < 0.4).astype(np.uint8) for i in range(len(made))]
+    fx.select_groups([(L, W, f, sx) for (W, L), f in zip(made, flags)])
+    for (W, L), f in zip(made, flags):
+        check(L, W, np.concatenate([np.flatnonzero(f), np.flatnonzero(f == 0)]).astype(np.int32), int(f.sum()))
+    fx.flexiq_check_status()
+    for _, L in made:
+        L.close()
