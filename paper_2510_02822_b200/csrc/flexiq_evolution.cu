@@ -64,9 +64,9 @@ __global__ void sq_distance_i8_kernel(const int8_t *__restrict__ A, const int8_t
 }
 
 // The same by one cluster of sixteen blocks, whose sums meet in the first one's shared memory: one launch, which may start while
-// the GEMM before it ends, and nothing cleared beforehand.  Larger tensors need more than sixteen SMs: the grid above and its clear
-// (graph replay, clear and grid against this: 0.6 MB 6.0 and 3.4 us, 1.2 MB 6.0 and 4.4, 2 MB 5.9 and 4.7; with 512 threads a block 3 MB took
-// 8.1 where the grid takes 6.2).
+// the GEMM before it ends, and nothing cleared beforehand.  Larger tensors need more than sixteen SMs, and not every device has sixteen
+// of one GPC to give: the grid above and its clear (graph replay, clear and grid against this: 0.6 MB 6.0 and 3.4 us, 1.2 MB 6.0 and 4.4,
+// 2 MB 5.9 and 4.7; with 512 threads a block 3 MB took 8.1 where the grid takes 6.2).
 constexpr int kDistCluster = 16, kDistThreads = 1024;
 constexpr int kDistSmem = 228 * 1024 / 2 - 1024;   // one block per SM: the cluster is launched while the GEMM before it still runs on some
 constexpr long long kDistClusterMax = 2ll << 20;
@@ -311,12 +311,6 @@ extern "C" int flexiq_sq_distance_i8(const int8_t *A_dev, const int8_t *B_dev, i
     int dev = 0;
     FLEXIQ_CUDA_TRY(cudaGetDevice(&dev));
     if (n <= kDistClusterMax && n > 0) {
-        static bool attr_set[64] = {};
-        if (dev >= 64 || !attr_set[dev]) {
-            FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(sq_distance_i8_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            FLEXIQ_CUDA_TRY(cudaFuncSetAttribute(sq_distance_i8_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDistSmem));
-            if (dev < 64) attr_set[dev] = true;
-        }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(kDistCluster, 1, 1);
         cfg.blockDim = dim3(kDistThreads, 1, 1);
@@ -330,9 +324,25 @@ extern "C" int flexiq_sq_distance_i8(const int8_t *A_dev, const int8_t *B_dev, i
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = 2;
-        FLEXIQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, sq_distance_i8_cluster_kernel, A_dev, B_dev, (long long)n, reinterpret_cast<long long *>(out_dev)));
-        return FLEXIQ_OK;
+        cfg.numAttrs = 1;   // what decides where it fits; the launch takes both
+        // A cluster of sixteen is more than is promised (a partition of a device may have fewer SMs): asked once per device.
+        static signed char resident[64] = {};   // 1: they are there, -1: they are not
+        signed char fits = dev < 64 ? resident[dev] : 0;
+        if (!fits) {
+            int clusters = 0;
+            const bool ok = cudaFuncSetAttribute(sq_distance_i8_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                            cudaFuncSetAttribute(sq_distance_i8_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDistSmem) == cudaSuccess &&
+                            cudaOccupancyMaxActiveClusters(&clusters, sq_distance_i8_cluster_kernel, &cfg) == cudaSuccess;
+            fits = ok && clusters > 0 ? 1 : -1;
+            if (!ok) cudaGetLastError();
+            if (dev < 64) resident[dev] = fits;
+        }
+        if (fits > 0) {
+            cfg.numAttrs = 2;
+            if (cudaLaunchKernelEx(&cfg, sq_distance_i8_cluster_kernel, A_dev, B_dev, (long long)n, reinterpret_cast<long long *>(out_dev)) == cudaSuccess)
+                return FLEXIQ_OK;
+            cudaGetLastError();   // refused where the device as a whole would take it (a context with fewer SMs): the grid below goes anywhere
+        }
     }
     FLEXIQ_CUDA_TRY(cudaMemsetAsync(out_dev, 0, sizeof(int64_t), st));
     if (n == 0) return FLEXIQ_OK;
