@@ -60,6 +60,7 @@ def lib():
         L.flexiq_layer_sync_ratio.argtypes = [vp, vp]
         L.flexiq_layer_set_slab_check.argtypes = [vp, i32]
         L.flexiq_layer_set_group_perm.argtypes = [vp, vp, vp, vp, vp]
+        L.flexiq_layers_set_group_perm.argtypes = [i32, vp, vp, vp, vp, vp]
         L.flexiq_set_lowbit_ratio.argtypes = [vp, f32]
         L.flexiq_get_max_4bit_ch.argtypes = [vp, C.POINTER(i32)]
         L.flexiq_x4_pitch.argtypes = [vp, i32, C.POINTER(i64)]
@@ -75,6 +76,7 @@ def lib():
         L.flexiq_calib_ranges_from_histogram.argtypes = [vp, i32, i64, vp, vp, vp]
         L.flexiq_calib_weight_absmax.argtypes = [vp, i32, i32, i32, i32, vp, vp]
         L.flexiq_calib_prepare.argtypes = [vp, vp, vp, i32, i32, vp, vp, vp, vp, vp]
+        L.flexiq_calib_static.argtypes = [vp, i32, i64, f32, vp, i64, i32, vp, i32, i32, i32, i32, vp, vp, vp, vp, vp, vp]
         L.flexiq_calib_absmax_ema.argtypes = [vp, i32, i64, f32, vp, vp]
         L.flexiq_layer_export.argtypes = [vp, vp, vp, vp]
         L.flexiq_layer_early_loads.argtypes = [vp, C.POINTER(i32), C.POINTER(i32)]
@@ -174,6 +176,14 @@ def flexiq_layer_set_lowbit_path(h, path):
 
 def flexiq_layer_set_slab_check(h, enabled):
     _check(lib().flexiq_layer_set_slab_check(h, int(bool(enabled))))
+
+
+def flexiq_layers_set_group_perm(handles, Wq_dev, perms_host, x_shifts_host):
+    """Lists of the same length; a position array may be None."""
+    n = len(handles)
+    array = C.c_void_p * n
+    _check(lib().flexiq_layers_set_group_perm(n, array(*handles), array(*(_ptr(w) for w in Wq_dev)), array(*(_np_ptr(p) for p in perms_host)),
+                                              array(*(None if x is None else _np_ptr(x) for x in x_shifts_host)), _stream()))
 
 
 def flexiq_set_lowbit_ratio(h, ratio):
@@ -472,11 +482,20 @@ def select_groups(selections):
     if native is not None and all(s[0]._calls is not None for s in selections):
         if native.select_groups([(layer._calls, *rest) for layer, *rest in selections]) is not NotImplemented:
             return
-    for layer, Wq, flags, x_shift in selections:
-        f = np.asarray(flags).astype(bool)
-        idx = np.arange(f.size, dtype=np.int32)
-        layer.set_group_perm(Wq, np.concatenate([idx[f], idx[~f]]), x_shift)
-        layer.set_lowbit_ratio(int(f.sum()) / f.size)
+    layers = [s[0] for s in selections]
+    flags = [np.asarray(s[2]).astype(bool) for s in selections]
+    perms = [np.concatenate([np.flatnonzero(f), np.flatnonzero(~f)]).astype(np.int32) for f in flags]
+    shifts = [None if s[3] is None else np.ascontiguousarray(s[3], np.uint8) for s in selections]
+    # the ratios first, so that the layouts cut the weight blocks that depend on them; a refused call leaves both as they were
+    before = [layer.K_lo / layer.K for layer in layers]
+    try:
+        for layer, f in zip(layers, flags):
+            layer.set_lowbit_ratio(int(f.sum()) / f.size)
+        flexiq_layers_set_group_perm([layer.h for layer in layers], [s[1] for s in selections], perms, shifts)
+    except Exception:
+        for layer, ratio in zip(layers, before):
+            layer.set_lowbit_ratio(ratio)
+        raise
 
 
 # ------------------------------------------------------------------ ratio controller and request queue (host only)

@@ -1,4 +1,5 @@
 """The Python side of a layer without its native marshalling: objects that only look like a layer keep working."""
+import numpy as np
 import pytest
 
 from paper_2510_02822_b200 import binding as fx
@@ -71,3 +72,34 @@ def test_native_layer_with_a_next_layer_of_another_type(calls):
     L._calls = Native()
     assert L.mixed_gemm_to_slab("x4", None, 5, 0.5, Next(), 0.25) == "slab of 5"
     assert L.mixed_conv_to_slab("x4", None, 1, 4, 4, 0.5, Next(), 0.25) == "slab of 16"
+
+
+def test_selections_without_the_native_module(monkeypatch, lib_built):
+    """Checked and enqueued in one call, with the ratios set before it and put back where it is refused."""
+    seen, low = [], {"a": 16, "b": 48}
+    monkeypatch.setattr(fx, "_native_calls", lambda: None)
+    monkeypatch.setattr(fx, "flexiq_get_max_4bit_ch", lambda h: low[h])
+
+    def set_ratio(h, ratio):
+        low[h] = int(np.ceil(ratio * 4 - 1e-4)) * 16
+    monkeypatch.setattr(fx, "flexiq_set_lowbit_ratio", set_ratio)
+
+    def lay_out(*args):
+        seen.append((args, dict(low)))
+        if args[0][-1] == "a":
+            raise fx.FlexiqError(fx.ERR_INVALID_ARG, "refused")
+    monkeypatch.setattr(fx, "flexiq_layers_set_group_perm", lay_out)
+    A, B = Bare(), Bare()
+    A.h, B.h = "a", "b"
+    flags = np.array([0, 1, 0, 1], np.uint8), [1, 0, 0, 0]
+    fx.select_groups([(A, "Wa", flags[0], None), (B, "Wb", flags[1], [0, 1, 2, 3])])
+    ((handles, weights, perms, shifts), then), = seen
+    assert handles == ["a", "b"] and weights == ["Wa", "Wb"] and then == low == {"a": 32, "b": 16}
+    assert [p.tolist() for p in perms] == [[1, 3, 0, 2], [0, 1, 2, 3]] and all(p.dtype == np.int32 for p in perms)
+    assert shifts[0] is None and shifts[1].dtype == np.uint8 and shifts[1].tolist() == [0, 1, 2, 3]
+    with pytest.raises(fx.FlexiqError):
+        fx.select_groups([(B, "Wb", flags[0], None), (A, "Wa", [1, 1, 1, 1], None)])
+    assert seen[1][1] == {"a": 64, "b": 32} and low == {"a": 32, "b": 16}
+    B.select_groups("Wb", [0, 0, 0, 0], None)
+    assert seen[2][0][0] == ["b"] and low == {"a": 32, "b": 0}
+    A.h = B.h = None

@@ -163,3 +163,38 @@ def test_layout_of_very_large_layers(widths):
     fx.flexiq_check_status()
     for _, L in made:
         L.close()
+
+
+def test_selections_in_python_as_in_native_code():
+    """Without the native module: the same layouts in the same call, and a refused one changes nothing."""
+    dev = torch.device("cuda:0")
+    pairs = []
+    for i, (K, N, G) in enumerate([(144, 80, 16), (192, 208, 64), (112, 48, 16)]):
+        Wd, n_g = torch.from_numpy(draw(870 + i, (K, N))).to(dev), K // G
+        sx = (np.arange(n_g) % 5).astype(np.uint8)
+        pair = [fx.Layer(Wd, torch.ones(N, device=dev), None, np.arange(n_g, dtype=np.int32), sx, G) for _ in range(2)]
+        pair[1]._calls = None
+        pairs.append((pair, Wd, (inputs.uniform(95, i, n_g) < 0.4).astype(np.uint8), sx))
+
+    def same():
+        for (a, b), Wd, _, _ in pairs:
+            assert a.K_lo == b.K_lo
+            X = torch.from_numpy(draw(880, (7, a.K))).to(dev)
+            ya, yb = (L.mixed_gemm(*L.quantize_lower(X, 1.0)[:2], 7, 1.0, 1.0, fx.OUT_ACC_I32) for L in (a, b))
+            assert torch.equal(ya, yb)
+    for k in (0, 1):
+        fx.select_groups([(pair[k], Wd, f, sx) for pair, Wd, f, sx in pairs])
+    same()
+    first, last = pairs[0], pairs[-1]
+    bad = last[3].copy()
+    bad[-1] = 5
+    ones = [np.ones_like(p[2]) for p in pairs]
+    for args in ([(p[0][1], p[1], o, p[3]) for p, o in zip(pairs[:-1], ones)] + [(last[0][1], last[1], ones[-1], bad)],
+                 [(first[0][1], first[1], ones[0], first[3])] * 2):
+        with pytest.raises(fx.FlexiqError):
+            fx.select_groups(args)
+        same()
+    fx.flexiq_check_status()
+    for pair, *_ in pairs:
+        for L in pair:
+            L.close()
