@@ -137,14 +137,14 @@ __device__ __forceinline__ void load16(const void *p, float x[16])
         const float4 *v = reinterpret_cast<const float4 *>(p);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const float4 f = __ldg(v + i);
+            const float4 f = v[i];
             x[4 * i + 0] = f.x; x[4 * i + 1] = f.y; x[4 * i + 2] = f.z; x[4 * i + 3] = f.w;
         }
     } else {
         const uint4 *v = reinterpret_cast<const uint4 *>(p);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const uint4 u = __ldg(v + i);
+            const uint4 u = v[i];
             const unsigned w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -168,7 +168,7 @@ template <int DTYPE>
 __device__ __forceinline__ void quantize16(const void *p, const Divider &div, float lo, float hi, unsigned w[4])
 {
     if (DTYPE == FLEXIQ_DTYPE_I8) {
-        const uint4 u = __ldg(reinterpret_cast<const uint4 *>(p));
+        const uint4 u = *reinterpret_cast<const uint4 *>(p);
         const unsigned in[4] = {u.x, u.y, u.z, u.w};
         const int ilo = (int)lo, ihi = (int)hi;
 #pragma unroll

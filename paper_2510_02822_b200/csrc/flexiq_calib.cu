@@ -12,7 +12,7 @@ namespace flexiq {
 // Loads 8 fp32 channels starting at p.
 __device__ __forceinline__ void load8(const void *p, float x[8])
 {
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(p)), b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
+    const float4 a = reinterpret_cast<const float4 *>(p)[0], b = reinterpret_cast<const float4 *>(p)[1];
     x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
 }
 
@@ -22,7 +22,7 @@ __device__ __forceinline__ void load8(const void *p, float x[8])
 // memory, then one global atomic per channel of the window.
 constexpr int kCalibWindow = 256;
 template <int DTYPE>
-__device__ __forceinline__ void ranges_block(int block, const void *__restrict__ X, long long M, int K, float S, int slices, int *lo_s, int *hi_s,
+__device__ __forceinline__ void ranges_block(int block, const void *X, long long M, int K, float S, int slices, int *lo_s, int *hi_s,
                                              int32_t *__restrict__ lo, int32_t *__restrict__ hi)
 {
     lo_s[threadIdx.x] = 0;
@@ -35,7 +35,7 @@ __device__ __forceinline__ void ranges_block(int block, const void *__restrict__
     if (c0 < K && DTYPE == FLEXIQ_DTYPE_I8) {
         unsigned lo_w[4] = {0, 0, 0, 0}, hi_w[4] = {0, 0, 0, 0};
         for (long long m = (long long)slice * 16 + rlane; m < M; m += (long long)slices * 16) {
-            const uint4 u = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const char *>(X) + (size_t)m * K + c0));
+            const uint4 u = *reinterpret_cast<const uint4 *>(reinterpret_cast<const char *>(X) + (size_t)m * K + c0);
             const unsigned w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -171,7 +171,7 @@ __global__ void calib_hist_kernel(const void *__restrict__ X, long long M, int K
 // contain zero (lo <= 0 <= hi).  tail = 0 gives the exact min / max.  One warp per channel, eight bins per lane: the
 // ends are where the running sums from either side first pass `tail` (a thread walking a channel's 256 bins one after the
 // other took 31 us whatever the number of channels).
-__device__ __forceinline__ void range_from_hist(int c, int lane, const unsigned *__restrict__ hist, long long tail, int32_t *__restrict__ lo,
+__device__ __forceinline__ void range_from_hist(int c, int lane, const unsigned *hist, long long tail, int32_t *__restrict__ lo,
                                                 int32_t *__restrict__ hi)
 {
     const unsigned *h = hist + (size_t)c * 256 + 8 * lane;
@@ -220,7 +220,7 @@ __device__ __forceinline__ int max_byte(unsigned w)
 }
 // Linear weights [K][N]: one warp per input channel (row).
 template <bool WIDE>
-__device__ __forceinline__ void absmax_row(int row, int lane, const int8_t *__restrict__ W, int N, int32_t *__restrict__ wmax)
+__device__ __forceinline__ void absmax_row(int row, int lane, const int8_t *W, int N, int32_t *__restrict__ wmax)
 {
     const int8_t *w = W + (size_t)row * N;
     int best = 0;
@@ -228,7 +228,7 @@ __device__ __forceinline__ void absmax_row(int row, int lane, const int8_t *__re
         unsigned b4 = 0;
 #pragma unroll 4
         for (int n = 16 * lane; n < N; n += 512) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(w + n));
+            const uint4 v = *reinterpret_cast<const uint4 *>(w + n);
             b4 = absmax4(absmax4(absmax4(absmax4(b4, v.x), v.y), v.z), v.w);
         }
         best = max_byte(b4);
@@ -247,7 +247,7 @@ __global__ void weight_absmax_rows_kernel(const int8_t *__restrict__ W, int K, i
 // Convolution weights [rows = Cout*R*S][Cin]: a thread per input channel (or sixteen of them), rows split over blockIdx.y and
 // in the wide form over the block's sixteen row lanes.
 // The wide form: block (bx, by) of 256 threads, by one of `gy`.
-__device__ __forceinline__ void absmax_cols_block(int bx, int by, int gy, const int8_t *__restrict__ W, long long rows, int C, int *best_s, int32_t *__restrict__ wmax)
+__device__ __forceinline__ void absmax_cols_block(int bx, int by, int gy, const int8_t *W, long long rows, int C, int *best_s, int32_t *__restrict__ wmax)
 {
     best_s[threadIdx.x] = 0;
     __syncthreads();
@@ -255,7 +255,7 @@ __device__ __forceinline__ void absmax_cols_block(int bx, int by, int gy, const 
     if (c0 < C) {
         unsigned b[4] = {0, 0, 0, 0};
         for (long long r = (long long)by * 16 + (threadIdx.x >> 4); r < rows; r += (long long)gy * 16) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(W + (size_t)r * C + c0));
+            const uint4 v = *reinterpret_cast<const uint4 *>(W + (size_t)r * C + c0);
             b[0] = absmax4(b[0], v.x); b[1] = absmax4(b[1], v.y); b[2] = absmax4(b[2], v.z); b[3] = absmax4(b[3], v.w);
         }
 #pragma unroll

@@ -14,7 +14,7 @@ namespace flexiq {
 // sum over i of (A[i] - B[i])^2 for int8 tensors, exact in int64.  (a - b)^2 = a.a - 2 a.b + b.b,
 // four elements per dp4a; one 16-byte unit of each tensor per thread and step, four steps in flight.
 // Returns the block's sum in thread 0.
-__device__ __forceinline__ long long block_sq_distance(const int8_t *__restrict__ A, const int8_t *__restrict__ B, long long n)
+__device__ __forceinline__ long long block_sq_distance(const int8_t *A, const int8_t *B, long long n)
 {
     const long long units = n >> 4;
     const uint4 *a4 = reinterpret_cast<const uint4 *>(A), *b4 = reinterpret_cast<const uint4 *>(B);
@@ -25,7 +25,7 @@ __device__ __forceinline__ long long block_sq_distance(const int8_t *__restrict_
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const long long u = base + q * step;
-            if (u < units) { va[q] = __ldg(a4 + u); vb[q] = __ldg(b4 + u); }
+            if (u < units) { va[q] = a4[u]; vb[q] = b4[u]; }
             else { va[q] = make_uint4(0, 0, 0, 0); vb[q] = make_uint4(0, 0, 0, 0); }
         }
         int s = 0;

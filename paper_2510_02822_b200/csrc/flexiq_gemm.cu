@@ -370,7 +370,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
     const int cols = BN >= 192 ? 64 : 32;
     constexpr bool kStaged = MODE != kOutScatter;                 // 32 x 32-byte boxes through shared memory and bulk stores
     constexpr bool kSlab = MODE == kOutNextSlab || MODE == kOutScatter;
-    // lane l keeps factors 4l..4l+3 of the table alpha[64] | beta[64]
+    // lane l keeps factors 4l..4l+3 of the table alpha[64] | beta[64]  (__ldg: their writer releases no launch before it has ended)
     const float *fsrc = (lane < 16 ? p.alpha : p.beta) + 4 * (lane & 15);
     int buf = 0;
     uint32_t buf_phase = 0;
@@ -430,7 +430,7 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
             float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
             if (kScaled && nw + 4 * (lane & 15) < p.N) f = __ldg(reinterpret_cast<const float4 *>(fsrc + nw));
             int ent = 0;                                     // fused boundary: lane g fetches chunk g's slab entry
-            if (kSlab && lane < 4 && nw + 16 * lane < p.N) ent = __ldg(p.next_ent + (nw >> 4) + lane);
+            if (kSlab && lane < 4 && nw + 16 * lane < p.N) ent = p.next_ent[(nw >> 4) + lane];
             if (!waited) {
                 PROF_T0(t0);
                 const bool ok = wait_bounded(&x.tmem_full[buf], buf_phase, x.abort_flag, 4);
@@ -1293,12 +1293,12 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
 #pragma unroll
                             for (int u = 0; u < 8; ++u) {
                                 const int chunk = min(cb * upr + (u < upr ? u : 0), last_chunk);
-                                nxB[u] = __ldg(p.sw + (size_t)(chunk >> cpg_log2) * p.N + colB);
+                                nxB[u] = p.sw[(size_t)(chunk >> cpg_log2) * p.N + colB];
                             }
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
                                 const int chunk = min(cb * upr + uA0 + (k < (upr >> 1) ? k : 0), last_chunk);
-                                nxA[k] = __ldg(p.sx + (chunk >> cpg_log2));
+                                nxA[k] = p.sx[chunk >> cpg_log2];
                             }
                         };
                         if (part == 0 && nb > 0) request(0);
@@ -1389,8 +1389,8 @@ mixed_gemm_kernel(const __grid_constant__ CUtensorMap mapA_lo, const __grid_cons
 
 // Per-output-channel factors of a call: REQUANT alpha = (S_x * S_w[n]) / S_y, beta = bias[n] / S_y;
 // DEQUANT alpha = S_x * S_w[n], beta = bias[n].  Each operation rounds once, in fp32.
-__global__ void scale_vectors_kernel(int N, float x_scale, float y_scale, int requant, const float *__restrict__ w_scale,
-                                     const float *__restrict__ bias, float *__restrict__ alpha, float *__restrict__ beta)
+__global__ void scale_vectors_kernel(int N, float x_scale, float y_scale, int requant, const float *w_scale,
+                                     const float *bias, float *__restrict__ alpha, float *__restrict__ beta)
 {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     ptx::pdl_wait();  // the previous kernel of the stream may still read the table

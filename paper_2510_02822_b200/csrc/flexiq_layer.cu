@@ -292,7 +292,7 @@ prep_linear_kernel(const __grid_constant__ PrepMany many, const __grid_constant_
         const int8_t *src = a.Wq + (long long)(g * a.G + (c16 % cpg) * 16) * a.N + n0;
         if (a.aligned) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) r[i] = __ldg(reinterpret_cast<const uint32_t *>(src + (long long)i * a.N));
+            for (int i = 0; i < 16; ++i) r[i] = *reinterpret_cast<const uint32_t *>(src + (long long)i * a.N);
         } else {
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(256) prep_conv_kernel(const __grid_constant__ 
             const int nl = idx / units, u = idx - nl * units, t = u / n_c16, c = u - t * n_c16, j = c / cpg;
             const int8_t *src = a.Wq + ((long long)(n_first + nl) * a.T + t) * a.C + perm_s[j] * a.G + (c % cpg) * 16;
             uint4 v;
-            if (a.aligned) v = __ldg(reinterpret_cast<const uint4 *>(src));
+            if (a.aligned) v = *reinterpret_cast<const uint4 *>(src);
             else {
                 uint32_t w[4];
 #pragma unroll

@@ -32,8 +32,8 @@ __global__ void clear_words_kernel(unsigned *words, int n)
 // slab group over all rows.  A thread keeps one chunk column and walks rows; lanes that
 // hold the same group merge with a warp reduction, then one shared and one global atomic.
 template <int DTYPE>
-__global__ void group_or_kernel(const void *__restrict__ X, long long M, int K, int G, float S,
-                                const int32_t *__restrict__ perm, unsigned *__restrict__ or_words)
+__global__ void group_or_kernel(const void *X, long long M, int K, int G, float S,
+                                const int32_t *perm, unsigned *__restrict__ or_words)
 {
     extern __shared__ unsigned or_s[];
     const int n_c16 = K / 16, c_per_g = G / 16, n_g = K / G;
@@ -111,8 +111,8 @@ constexpr unsigned kShift8Bit = 5;
 __device__ __forceinline__ unsigned chunk_entry(int c, int log_cpg, int lo_c16, const int32_t *perm, const uint8_t *sx)   // 1 << log_cpg chunks a group
 {
     const int j = c >> log_cpg;
-    const unsigned shift = c < lo_c16 ? (unsigned)__ldg(sx + j) : kShift8Bit;
-    return (unsigned)((__ldg(perm + j) << log_cpg) + (c - (j << log_cpg))) | (shift << 28);
+    const unsigned shift = c < lo_c16 ? (unsigned)sx[j] : kShift8Bit;
+    return (unsigned)((perm[j] << log_cpg) + (c - (j << log_cpg))) | (shift << 28);
 }
 
 struct RowsArgs {
@@ -344,7 +344,7 @@ __global__ void drain_kernel(const uint8_t *src, int *result)
 // lowering is clearing the bits below the position; a group whose position is 0 is already what it should be and
 // is not touched.  The positions go to sx_out (slab order).  Blocks in front: the straddle block of the weights.
 __global__ void lower_inplace_kernel(int8_t *__restrict__ slab, long long M, int K, int G, int K_lo,
-                                     const unsigned *__restrict__ or_words, uint8_t *__restrict__ sx_out, StraddleJob wp,
+                                     const unsigned *or_words, uint8_t *__restrict__ sx_out, StraddleJob wp,
                                      int step_m, int step_c)
 {
     ptx::pdl_launch_dependents();
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(kColThreads) dynamic_columns_kernel(const __gr
     ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
     if (live) {
         const size_t row_bytes = (size_t)a.K * kBytes;
-        const char *src = reinterpret_cast<const char *>(a.X) + (size_t)(m_first + r0) * row_bytes + ((size_t)__ldg(a.perm + j) * a.G + (c % cpg) * 16) * kBytes;
+        const char *src = reinterpret_cast<const char *>(a.X) + (size_t)(m_first + r0) * row_bytes + ((size_t)a.perm[j] * a.G + (c % cpg) * 16) * kBytes;
         unsigned o = 0;
         for (int r = r0; r < rows; r += kAhead * step, src += (size_t)(kAhead * step) * row_bytes) {
             uint4 raw[kAhead][kPieces];
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(kColThreads) dynamic_columns_kernel(const __gr
             for (int i = 0; i < kAhead; ++i)
                 if (r + i * step < rows) {
 #pragma unroll
-                    for (int p = 0; p < kPieces; ++p) raw[i][p] = __ldg(reinterpret_cast<const uint4 *>(src + (size_t)(i * step) * row_bytes) + p);
+                    for (int p = 0; p < kPieces; ++p) raw[i][p] = reinterpret_cast<const uint4 *>(src + (size_t)(i * step) * row_bytes)[p];
                 }
 #pragma unroll
             for (int i = 0; i < kAhead; ++i)
@@ -504,9 +504,9 @@ __global__ void __launch_bounds__(kColThreads) dynamic_columns_kernel(const __gr
 // the shift being monotone); then bits s..s+3 of every byte are the two's-complement nibble (packed path), and
 // clearing the s low bits of every byte is (q >> s) << s (masked path: one slab, X8 lies behind the low groups of X4).
 template <int DTYPE, bool PACKED>
-__global__ void quantize_chunks_kernel(const void *__restrict__ X, long long M, int K, int G, int K_lo, float S,
-                                       const int32_t *__restrict__ perm, const uint8_t *__restrict__ sx,
-                                       const unsigned *__restrict__ or_words, uint8_t *__restrict__ X4,
+__global__ void quantize_chunks_kernel(const void *X, long long M, int K, int G, int K_lo, float S,
+                                       const int32_t *perm, const uint8_t *sx,
+                                       const unsigned *or_words, uint8_t *__restrict__ X4,
                                        long long x4_pitch, int8_t *__restrict__ X8, long long x8_pitch, uint8_t *__restrict__ sx_out)
 {
     const int n_c16 = K / 16, c_per_g = G / 16, lo_c16 = K_lo / 16;

@@ -11,8 +11,8 @@ namespace flexiq {
 
 // Y[m][j*G + i] = X[m][src_group[j]*G + i] for every row m, group j, channel i < G.
 // units_per_group = G * elem_bytes / 16; units_per_row = C * elem_bytes / 16.
-__global__ void reorder_channels_kernel(const uint4 *__restrict__ X, uint4 *__restrict__ Y, long long M, int units_per_row,
-                                        int units_per_group, const int32_t *__restrict__ src_group)
+__global__ void reorder_channels_kernel(const uint4 *X, uint4 *__restrict__ Y, long long M, int units_per_row,
+                                        int units_per_group, const int32_t *src_group)
 {
     ptx::pdl_wait();  // X may be the previous kernel's output
     const long long total = M * units_per_row;
@@ -27,8 +27,8 @@ __global__ void reorder_channels_kernel(const uint4 *__restrict__ X, uint4 *__re
                 const long long m = idx / units_per_row;
                 const int u = (int)(idx - m * units_per_row);
                 const int j = u / units_per_group;
-                const int src = __ldg(src_group + j) * units_per_group + (u - j * units_per_group);
-                v[q] = __ldg(X + m * units_per_row + src);
+                const int src = src_group[j] * units_per_group + (u - j * units_per_group);
+                v[q] = X[m * units_per_row + src];
             }
         }
 #pragma unroll

@@ -17,6 +17,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
 // memory the predecessor writes (or reads, if it overwrites it) before pdl_wait() returns.
 // pdl_launch_dependents() lets the successor start its own preamble.  Both are no-ops for
 // a plain launch.
+// What a predecessor may write is read with ordinary loads: a non-coherent one (__ldg, a const __restrict__ argument) is defined only
+// for memory that nobody writes while the kernel is resident, and the compiler may move it ahead of the wait.
 __device__ __forceinline__ void pdl_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");

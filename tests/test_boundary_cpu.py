@@ -169,3 +169,23 @@ int main()
     subprocess.run(["g++", "-std=c++17", *(f"-I{d}" for d in (fxbuild.CSRC, os.path.join(ROOT, "include"), os.path.join(cuda, "include"))), str(src), "-o", exe], check=True)
     r = subprocess.run([exe], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+def test_kernels_that_overlap_their_predecessor_read_with_coherent_loads():
+    """A non-coherent load is defined for memory that nobody writes while its kernel is resident; a kernel with a dependency wait is
+    resident while the launches before it still write its inputs, its layer's tables (a layout) and its positions (a prologue)."""
+    waiting = 0
+    for name in sorted(os.listdir(fxbuild.CSRC)):
+        if not name.endswith((".cu", ".cuh")):
+            continue
+        text = open(os.path.join(fxbuild.CSRC, name)).read()
+        code = re.sub(r"//[^\n]*", "", text)
+        for line in code.splitlines():
+            assert ("__ldg(" not in line or "fsrc" in line) and "ld.global.nc" not in line, (name, line)
+        for kernel in re.split(r"\b__global__\b", code)[1:]:
+            head, body = kernel.split("{", 1)
+            body = body.split("\n}\n", 1)[0]
+            if "pdl_wait" in body:
+                waiting += 1
+                assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", head), (name, head)
+    assert waiting >= 12
