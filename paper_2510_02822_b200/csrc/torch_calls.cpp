@@ -117,7 +117,7 @@ template <class F> PyObject *guarded(F f)
     try {
         return f();
     } catch (...) {
-        return not_implemented();   // before any library call: those do not throw
+        return not_implemented();   // what is refused here is refused before a library call, or where the same calls may be made again
     }
 }
 // the library call with the interpreter released, as ctypes makes it
@@ -539,7 +539,10 @@ PyObject *static_preparation(PyObject *, PyObject *const *args, Py_ssize_t n)
             PyErr_SetString(PyExc_RuntimeError, cudaGetErrorString((cudaError_t)cuda));
             return nullptr;
         }
-        if (!result.o) throw Refused{};
+        if (!result.o) {
+            if (PyErr_Occurred()) return nullptr;   // the interpreter's own error (no memory) is the caller's to see
+            throw Refused{};                        // torch's: the general path makes the calls again, into tensors of its own
+        }
         const char *host = static_cast<const char *>(order.data_ptr());
         std::copy(host, host + 4 * n_g, perm_host);
         std::copy(host + 4 * n_g, host + 5 * n_g, shift_host);

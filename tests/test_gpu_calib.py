@@ -197,3 +197,29 @@ def test_one_launch_equals_the_calls_it_stands_for(dev, K, N, G, rows, shape, dt
     assert np.array_equal(perm, perm_e.cpu().numpy()) and np.array_equal(xs, xs_e.cpu().numpy())
     for name, want in (("lo", lo), ("hi", hi), ("wmax", wmax), ("score", score), ("unused_hist", unused)):
         assert torch.equal(info[name], want), name
+
+
+def test_interpreter_out_of_memory_is_reported(dev):
+    """An allocation of Python's that fails behind the launch is a MemoryError: not swallowed, not answered with "take the general path"."""
+    testcapi = pytest.importorskip("_testcapi")
+    native = fx._native_calls()
+    if native is None:
+        pytest.skip("built without the native module")
+    X, W = torch.randn((64, 64), device=dev), torch.randint(-128, 128, (64, 48), device=dev, dtype=torch.int8)
+    args = (X, 0.1, W, 16, False, 1, None)
+    call, arm, disarm = native.static_preparation, testcapi.set_nomemory, testcapi.remove_mem_hooks
+    want = call(*args)
+    failed = 0
+    for k in range(40):
+        got = None
+        arm(k, k + 1)
+        try:
+            got = call(*args)
+        except MemoryError:
+            failed += 1
+        finally:
+            disarm()
+        assert got is not NotImplemented, k
+        if got is not None:
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
+    assert failed
