@@ -2,6 +2,8 @@
 (group, output channel) against the oracle and a plain gather, at the edges of the kernels' tiles (64 output
 channels x 128 input channels; whole convolution rows), for every group size, for weights at odd addresses and
 for more groups than a launch's parameters carry."""
+import contextlib
+
 import numpy as np
 import pytest
 import torch
@@ -89,6 +91,18 @@ def test_layout_cuts_the_block_of_the_ratio_in_force(K, N, G):
         x4, x8, _ = L.quantize_lower(Xd, 1.0)
         acc = L.mixed_gemm(x4, x8, 70, 1.0, 1.0, fx.OUT_ACC_I32)
         assert np.array_equal(acc.cpu().numpy(), oracle.mixed_gemm_acc(X, W, G, order, sx[order].copy(), sw, low)), low
+        # other weights in the same order, so that the slab stays what it is: the GEMM finds the block cut and launches nothing for it
+        W2 = draw(702 + low, (K, N))
+        L.select_groups(torch.from_numpy(W2).to(dev), flags, sx)
+        watched = low in (1, n_g // 2, n_g - 1)
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) if watched else contextlib.nullcontext() as seen:
+            acc = L.mixed_gemm(x4, x8, 70, 1.0, 1.0, fx.OUT_ACC_I32)
+            torch.cuda.synchronize()
+        if watched:
+            launched = [e.key for e in seen.key_averages() if "flexiq::" in e.key]
+            assert len(launched) == 1 and "mixed_gemm_kernel" in launched[0], launched
+        sw = oracle.weight_positions_linear(W2, G, order)
+        assert np.array_equal(acc.cpu().numpy(), oracle.mixed_gemm_acc(X, W2, G, order, sx[order].copy(), sw, low)), low
     fx.flexiq_check_status()
     L.close()
 
