@@ -49,8 +49,9 @@ constexpr int kOutNextSlab = 3;
 // The same with the chunks of the producer's own channel order scattered to their places (a mode of the epilogue only).
 constexpr int kOutScatter = 6;
 
-// A kernel serves one kind of output.  One kernel for all of them spilled registers in every epilogue (ptxas: 108 bytes stored and 244
-// loaded per thread in the plain CTA pair, against 8 and 8 now), and the epilogue is as long as the mainloop at short K.
+// A kernel serves one kind of output.  One kernel for all of them spilled registers in every epilogue (ptxas, per thread: 160 bytes stored
+// and 180 loaded in the plain CTA pair, 108 and 244 in the single CTA, none in either now), and the epilogue is as long as the mainloop
+// at short K.  Packed path, 768 -> 3072 at 12,608 rows 60.7 -> 57.1 us, 384 -> 1536 at 1576 8.9 -> 7.8.
 enum OutKind { kKindI8, kKindNext, kKindScatter, kKindHalf, kKindWord };
 static OutKind out_kind(int out_mode, bool staged)
 {
@@ -353,9 +354,10 @@ struct EpilogueCtx {
 
 // One epilogue warp: TMEM lane quadrant `quad` (32 rows, lane = row), column slot `part` (32 or 64
 // columns per pass; two passes when only eight warps drain the tile) of every tile of this CTA.
-// Per pass: fetch the columns' factors, read the whole slice of the accumulator into registers,
-// hand the accumulator back, then scale / round / clip; the results are staged in shared memory (32 rows
-// x 32 bytes: 32 int8, 16 half-precision or 8 four-byte columns) and leave through tiled bulk stores.
+// Per pass: fetch the columns' factors, then 32 columns at a time: read the accumulator into registers (and hand it back with the last
+// of them), scale / round / clip; the results are staged in shared memory (32 rows x 32 bytes: 32 int8, 16 half-precision or
+// 8 four-byte columns) and leave through tiled bulk stores.  That the first half is stored before the accumulator goes back costs
+// nothing: against the one kernel for all, which read the whole slice first, int8 ViT-B QKV 19.2 -> 18.0 us, fc2 22.3 -> 21.7, ViT-L fc2 72-82 and 71-82 us (the power cap).
 template <int CG, int MODE, bool SPLIT, int KIND>
 __device__ __forceinline__ void epilogue_role(const GemmParams &p, const EpilogueCtx &x, int quad, int part, int lane)
 {
@@ -568,7 +570,8 @@ __device__ __forceinline__ void epilogue_role(const GemmParams &p, const Epilogu
                         }
                     }
                 } else if (MODE == kOutScatter && row < p.M) {
-                    // each 16-channel chunk goes to its place in the next layer's slab row
+                    // each 16-channel chunk goes to its place in the next layer's slab row (768 -> 3072 at 12,608 rows 38.4 -> 32.5 us as a
+                    // kernel of its own, 384 -> 1536 at 1576 6.4 -> 5.5)
                     uint8_t *srow = static_cast<uint8_t *>(p.Y) + row * p.N;
                     const bool wide = ((reinterpret_cast<uintptr_t>(p.Y) | (uintptr_t)p.N) & 31) == 0;   // rows are 32-byte aligned: 256-bit stores
                     const int n = nw + 32 * h;

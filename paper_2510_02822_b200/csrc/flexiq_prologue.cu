@@ -191,7 +191,9 @@ __global__ void __launch_bounds__(32 * (kRowWarps + 1)) quantize_rows_kernel(con
     ptx::pdl_wait();  // the previous kernel may still read the slab this one overwrites, or write X
     if (copier)
         for (int i = 0; i < a.stages && next < a.tiles; ++i, next += step) copy(next, i);
-    // A thread with one chunk fetches that chunk's entry itself; otherwise the block makes a table.
+    // A thread with one chunk fetches that chunk's entry itself; otherwise the block makes a table.  (With the entries by shifts and
+    // all that needs no memory ahead of the wait: DeiT-S at batch 1, 48 layers, 265.9 -> 254.3 us, one block at batch 8 28.9 -> 27.9,
+    // 1001 x 720 bf16 with its GEMM 7.8 -> 7.45; ViT-B sweep level.)
     unsigned ent = 0;
     if (single) {
         if ((int)threadIdx.x < units) ent = chunk_entry(c0, log_cpg, lo_c16, a.perm, a.sx);
@@ -716,7 +718,7 @@ static int launch_prologue(Layer *L, const void *X, long long M, float S, int dy
     constexpr size_t elem = DTYPE == FLEXIQ_DTYPE_F32 ? 4 : (DTYPE == FLEXIQ_DTYPE_I8 ? 1 : 2);
     int col_rows = 0, col_window = 0;
     const bool columns = dynamic && masked && columns_fit(L, M, (int)elem, &col_rows, &col_window);
-    // a launch, not a memset: the kernel behind it may then start (and ask for its first rows) while the one before it ends
+    // a launch, not a memset: the kernel behind it may then start, and do all that comes before its wait, while the one before it ends
     if (dynamic && !columns) FLEXIQ_CUDA_TRY(launch_pdl(clear_words_kernel, 1, 256, 0, st, scratch, L->n_g));
     if (masked && (columns || (size_t)K * elem <= kRowStageBytes)) {
         StraddleJob job{};
