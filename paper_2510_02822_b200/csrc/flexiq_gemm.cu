@@ -356,8 +356,9 @@ struct EpilogueCtx {
 // columns per pass; two passes when only eight warps drain the tile) of every tile of this CTA.
 // Per pass: fetch the columns' factors, then 32 columns at a time: read the accumulator into registers (and hand it back with the last
 // of them), scale / round / clip; the results are staged in shared memory (32 rows x 32 bytes: 32 int8, 16 half-precision or
-// 8 four-byte columns) and leave through tiled bulk stores.  That the first half is stored before the accumulator goes back costs
-// nothing: against the one kernel for all, which read the whole slice first, int8 ViT-B QKV 19.2 -> 18.0 us, fc2 22.3 -> 21.7, ViT-L fc2 72-82 and 71-82 us (the power cap).
+// 8 four-byte columns) and leave through tiled bulk stores.  The first half is stored before the accumulator goes back; against the one
+// kernel for all outputs, which read the whole slice first, no shape is slower for it (int8, GEMM alone: ViT-B QKV 19.2 -> 18.0 us,
+// fc2 22.3 -> 21.7, ViT-L fc2 70-83 and 70-86 us under the power cap).
 template <int CG, int MODE, bool SPLIT, int KIND>
 __device__ __forceinline__ void epilogue_role(const GemmParams &p, const EpilogueCtx &x, int quad, int part, int lane)
 {
